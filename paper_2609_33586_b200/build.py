@@ -5,12 +5,13 @@ import os
 import shutil
 import subprocess
 import sys
+import tempfile
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libattn_b200.so"
-SOURCES = ["api.cu", "attn_fwd_sm100.cu"]
+SOURCES = ["api.cu", "attn_fwd_sm100.cu", "attn_rows_sm100.cu"]
 HEADERS = ["ptx.cuh", "weight_map.cuh", "attn_kernel_common.cuh", "softmax_math.cuh", "../../include/attn.h"]
 
 
@@ -32,14 +33,22 @@ def build(force: bool = False, verbose: bool = False) -> Path:
     if not force and not needs_build():
         return LIB
     tmp = LIB.with_suffix(f".so.tmp{os.getpid()}")
-    cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-Xcompiler", "-fPIC", "-shared", "--ptxas-options=-v" if verbose else "-w",
-           "-o", str(tmp)] + [str(CSRC / f) for f in SOURCES] + ["-lcudart"]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+    flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
+             "--ptxas-options=-v" if verbose else "-w"]
+    with tempfile.TemporaryDirectory() as objs:
+        # one compiler per source file, side by side
+        jobs = [(f, subprocess.Popen([_nvcc(), *flags, "-c", "-o", f"{objs}/{f}.o", str(CSRC / f)],
+                                     stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)) for f in SOURCES]
+        logs = [job.communicate()[0] for _, job in jobs]
+        for (f, job), log in zip(jobs, logs):
+            if job.returncode != 0:
+                raise RuntimeError(f"nvcc failed on {f}:\n{log}")
+        link = subprocess.run([_nvcc(), "-shared", "-o", str(tmp), *(f"{objs}/{f}.o" for f in SOURCES), "-lcudart"],
+                              capture_output=True, text=True)
+        if link.returncode != 0:
+            raise RuntimeError("nvcc failed at the link:\n" + link.stdout + link.stderr)
     if verbose:
-        print(res.stdout + res.stderr)
+        print("".join(logs))
     os.replace(tmp, LIB)
     return LIB
 

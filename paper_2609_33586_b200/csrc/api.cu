@@ -12,6 +12,9 @@
 namespace rowmax {
 cudaError_t launch_attn_fwd(int D, int in_type, int mode, const CUtensorMap& tq, const CUtensorMap& tk,
                             const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream);
+bool use_rows_kernel(int in_type, int mode, const AttnParams& p);
+cudaError_t launch_attn_rows(int D, int in_type, int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q,
+                             const AttnParams& p, cudaStream_t stream);
 cudaError_t launch_weight_map(const float* x, float* w, size_t n, int mode, cudaStream_t stream);
 cudaError_t launch_weight_map_pot(const float* x, float* w, size_t n, int kmax, int drop, cudaStream_t stream);
 cudaError_t launch_weight_map_fused(const float* x, float* w, size_t n, int mode, int in_type, float pot_neg_cap,
@@ -178,12 +181,6 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     rc = status_word(&p.status);
     if (rc != ATTN_OK) return rc;
 
-    CUtensorMap tq, tk, tv;
-    const bool half_in = in_dtype == ATTN_IN_FP16;
-    if ((rc = make_tile_map(&tq, q, fp8, half_in, B, Sq, Hq, D)) != ATTN_OK) return rc;
-    if ((rc = make_tile_map(&tk, k, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
-    if ((rc = make_tile_map(&tv, v, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
-
     static_assert(ATTN_IN_BF16 == rowmax::kInBF16 && ATTN_IN_FP8_E4M3 == rowmax::kInFP8 && ATTN_IN_FP16 == rowmax::kInFP16,
                   "the kernel's storage-type codes are those of the C interface");
     int kernel_mode = (weight_mode == ATTN_W_POT && drop) ? rowmax::kPotDrop : weight_mode;
@@ -192,7 +189,17 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
         const int by_share[5] = {0, rowmax::kExactPoly1, rowmax::kExactPoly, rowmax::kExactPoly3, rowmax::kExactPoly4};
         kernel_mode = by_share[poly_eighths];
     }
-    cudaError_t e = rowmax::launch_attn_fwd(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
+    CUtensorMap tq, tk, tv;
+    const bool half_in = in_dtype == ATTN_IN_FP16;
+    if ((rc = make_tile_map(&tk, k, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
+    if ((rc = make_tile_map(&tv, v, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
+    cudaError_t e;
+    if (rowmax::use_rows_kernel(in_dtype, kernel_mode, p)) {
+        e = rowmax::launch_attn_rows(D, in_dtype, kernel_mode, tk, tv, q, p, static_cast<cudaStream_t>(stream));
+    } else {
+        if ((rc = make_tile_map(&tq, q, fp8, half_in, B, Sq, Hq, D)) != ATTN_OK) return rc;
+        e = rowmax::launch_attn_fwd(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
+    }
     if (e != cudaSuccess) {
         g_last_cuda_error = static_cast<int>(e);
         return e == cudaErrorInvalidValue ? ATTN_ERR_UNSUPPORTED : ATTN_ERR_CUDA;

@@ -508,7 +508,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     const float big_r = masked_tile ? kRm : kR;
                     const float inv_r = masked_tile ? 1.0f / kRm : 1.0f / kR;
                     rs.su = -c_eff * inv_r;
-                    rs.ou = (m_use * c_eff) * inv_r;
+                    const float ou = (m_use * c_eff) * inv_r;
+                    rs.ou = make_float2(ou, ou);
                     rs.sat_mul = -big_r;
 #pragma unroll
                     for (int cc = 0; cc < 4; ++cc) {
@@ -777,7 +778,7 @@ __global__ void weight_map_fused_kernel(const float* __restrict__ x, float* __re
             // 16-bit inputs: the saturating form, as in a key tile without masked scores
             constexpr float kR = 126.0f * (1 << kFam);
             rs.su = -static_cast<float>(1 << kFam) * (1.0f / kR);
-            rs.ou = 0.0f;
+            rs.ou = make_float2(0.0f, 0.0f);
             rs.sat_mul = -kR;
             weights_chunk32<FP8, MODE, false, true, HALF, true>(s, rs, 32, acc, pw);
         } else {

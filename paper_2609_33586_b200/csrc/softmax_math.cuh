@@ -191,7 +191,8 @@ struct RowScale {
     float pot_drop_x;   // pot, dropped tail: offsets at or below this (-(K_max + 1/2)) weigh zero
     // saturating form (SAT, h15 family): u = sat(score * su + ou) is the distance below the anchor as a fraction
     // of the clamp distance R = 2^K * 126 (2^K * 127 in a tile with masked scores); sat_mul = -R
-    float su, ou, sat_mul;
+    float su, sat_mul;
+    float2 ou;     // both lanes
 };
 
 // fma with saturation to [0, 1] (NaN gives 0)
@@ -199,6 +200,47 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
     float d;
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
+}
+
+// The weights (times 2^kOffLog2) of a pair of scores; `i` is the pair's position, which selects the route of the
+// partly emulated exact mode.  The two lanes may belong to one score row or to two rows with anchors of their own.
+template <bool FP8, int MODE, bool CLAMP, bool SAT>
+__device__ __forceinline__ float2 weight_pair(float2 sv, const RowScale& rs, int i) {
+    constexpr int kOff = PFormat<FP8, MODE>::kOffLog2;
+    float2 x = make_float2(0.f, 0.f);
+    if constexpr (!SAT) x = ffma2(sv, rs.c, rs.nmc);
+    float2 w;
+    if constexpr (SAT && h15_family_k(MODE) > 0) {
+        float2 t;
+        t.x = fmaf(fma_sat(sv.x, rs.su, rs.ou.x), rs.sat_mul, kH15Magic);
+        t.y = fmaf(fma_sat(sv.y, rs.su, rs.ou.y), rs.sat_mul, kH15Magic);
+        w = h15_weight_pair_from_t<kOff, h15_family_k(MODE)>(t, rs.two22);
+    } else if constexpr (exact_poly_eighths(MODE) > 0) {
+        // e eighths of the pairs, spread evenly, take the polynomial route, the rest the hardware ex2; a masked
+        // score (-inf) weighs nothing on either route
+        constexpr int e = exact_poly_eighths(MODE);
+        if (((i * e) & 7) < e) {
+            w.x = w_exact_poly3(x.x);
+            w.y = w_exact_poly3(x.y);
+        } else {
+            w.x = w_exact(x.x);
+            w.y = w_exact(x.y);
+        }
+    } else if constexpr (is_exact_like(MODE)) {
+        w.x = w_exact(x.x);  // masked scores are -inf -> weight 0
+        w.y = w_exact(x.y);
+    } else if constexpr (h15_family_k(MODE) > 0) {
+        // Eq. h15 on the input scaled by 2^K (K = 1: doubled): clamp, add 2^23 + 2^22 (rounds to the
+        // integer n, ties to even), then (bits << (23 - K)) + bias builds the weight times 2^kOff.
+        w = w_h15_doubled_pair<kOff, CLAMP, h15_family_k(MODE)>(x, rs.two22, rs.clamp_lo);
+    } else {
+        w = pot_weight_pair_rne<kOff>(x, rs.pot_neg_cap, rs.two22 << 1);
+        if constexpr (MODE == kPotDrop) {   // the index K_max + 1 stands for everything beyond K_max: weight zero
+            if (x.x <= rs.pot_drop_x) w.x = 0.f;
+            if (x.y <= rs.pot_drop_x) w.y = 0.f;
+        }
+    }
+    return w;
 }
 
 // Turns 32 consecutive scores of one row into weights.  Adds them (times 2^kOffLog2) into `acc`
@@ -217,45 +259,12 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
 template <bool FP8, int MODE, bool MASKED, bool CLAMP = true, bool HALFP = false, bool SAT = false>
 __device__ __forceinline__ void weights_chunk32(const uint32_t (&s)[32], const RowScale& rs, int limit,
                                                 float2 (&acc)[2], uint32_t* pw) {
-    constexpr int kOff = PFormat<FP8, MODE>::kOffLog2;
     uint32_t half16[16];
     float2 w_even = make_float2(0.f, 0.f);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
         const float2 sv = make_float2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1]));
-        float2 x = make_float2(0.f, 0.f);
-        if constexpr (!SAT) x = ffma2(sv, rs.c, rs.nmc);
-        float2 w;
-        if constexpr (SAT && h15_family_k(MODE) > 0) {
-            float2 t;
-            t.x = fmaf(fma_sat(sv.x, rs.su, rs.ou), rs.sat_mul, kH15Magic);
-            t.y = fmaf(fma_sat(sv.y, rs.su, rs.ou), rs.sat_mul, kH15Magic);
-            w = h15_weight_pair_from_t<kOff, h15_family_k(MODE)>(t, rs.two22);
-        } else if constexpr (exact_poly_eighths(MODE) > 0) {
-            // e eighths of the pairs, spread evenly, take the polynomial route, the rest the hardware ex2; a masked
-            // score (-inf) weighs nothing on either route
-            constexpr int e = exact_poly_eighths(MODE);
-            if (((i * e) & 7) < e) {
-                w.x = w_exact_poly3(x.x);
-                w.y = w_exact_poly3(x.y);
-            } else {
-                w.x = w_exact(x.x);
-                w.y = w_exact(x.y);
-            }
-        } else if constexpr (is_exact_like(MODE)) {
-            w.x = w_exact(x.x);  // masked scores are -inf -> weight 0
-            w.y = w_exact(x.y);
-        } else if constexpr (h15_family_k(MODE) > 0) {
-            // Eq. h15 on the input scaled by 2^K (K = 1: doubled): clamp, add 2^23 + 2^22 (rounds to the
-            // integer n, ties to even), then (bits << (23 - K)) + bias builds the weight times 2^kOff.
-            w = w_h15_doubled_pair<kOff, CLAMP, h15_family_k(MODE)>(x, rs.two22, rs.clamp_lo);
-        } else {
-            w = pot_weight_pair_rne<kOff>(x, rs.pot_neg_cap, rs.two22 << 1);
-            if constexpr (MODE == kPotDrop) {   // the index K_max + 1 stands for everything beyond K_max: weight zero
-                if (x.x <= rs.pot_drop_x) w.x = 0.f;
-                if (x.y <= rs.pot_drop_x) w.y = 0.f;
-            }
-        }
+        float2 w = weight_pair<FP8, MODE, CLAMP, SAT>(sv, rs, i);
         if constexpr (!is_exact_like(MODE) && MASKED) {
             if (2 * i >= limit) w.x = 0.f;
             if (2 * i + 1 >= limit) w.y = 0.f;
