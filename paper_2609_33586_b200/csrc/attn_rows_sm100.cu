@@ -57,12 +57,16 @@ struct RowsCfg {
     static constexpr int kFixedBytes = kMiscOff + 16 + 1024;    // + alignment slack
     static_assert(kQBytes % 1024 == 0 && kPBytes % 1024 == 0, "operand tiles start on a swizzle atom");
     static_assert(kMaxSlots <= 31, "one lane per slot sets up the ring's barriers");
-    static_assert(N * D * 4 <= 4 * C::kTileBytes, "the partial result is parked in the (at least four) ring slots");
 };
 
 // Query rows that the softmax warps take at a time: work is skipped in these steps (rows up to the next multiple are
 // computed on zero queries and never stored).
 template <int N> constexpr int kRowGroup = N == 16 ? 4 : 8;
+
+// TMEM columns of a CTA.  Two CTAs share an SM where the row tile leaves room for two in shared memory: each of them waits
+// for hand-offs most of the time (4 x 16K context, e4m3, D = 64: 22 us against 32 us with one; the others 3 to 20 %
+// faster or equal). 
+template <int N> constexpr int kRowsCols = N == 64 ? 512 : 256;
 
 template <int MODE> struct ModeTag { static constexpr int value = MODE; };
 
@@ -70,9 +74,8 @@ struct RowsParams {
     int cs;           // CTAs per cluster
     int nt;           // key tiles
     int rounds;       // rounds of the cluster over the context
-    int share;        // key tiles of one CTA in one round, share * N <= tmem_cols
+    int share;        // key tiles of one CTA in one round, share * N <= kRowsCols<N>
     int slots;        // ring slots
-    int tmem_cols;
     int rows;         // Sq * group
     int mode;
 };
@@ -262,7 +265,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         if (lane == 3) mbar_init(bar_drain, 1);
         fence_mbar_init();
         __syncwarp();
-        tmem_alloc(smem_u32(tmem_slot), rp.tmem_cols);
+        tmem_alloc(smem_u32(tmem_slot), kRowsCols<N>);
         tmem_relinquish();
     } else {
         // Q rows (query qi, head of the group) into the K-major operand tile, swizzled as TMA would have done it
@@ -642,7 +645,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     cluster_wait();      // nobody reads this CTA's shared memory any more
     tc_fence_before();
     __syncthreads();
-    if (warp == 5) tmem_dealloc(tmem, rp.tmem_cols);
+    if (warp == 5) tmem_dealloc(tmem, kRowsCols<N>);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -650,98 +653,113 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // ------------------------------------------------------------------------------------------------
 namespace {
 
-constexpr int kSmemFull = 232448;    // one CTA per SM
-constexpr int kSmemHalf = 115712;    // two CTAs per SM (1 KB of each is the system's)
-
 template <int D, int IN, int N>
-cudaError_t launch_rows(int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
-                        cudaStream_t stream) {
-    constexpr bool FP8 = IN == kInFP8;
+struct RowsLauncher {
+    static constexpr bool FP8 = IN == kInFP8;
     using W = RowsCfg<D, FP8, N>;
-    constexpr int kTile = TileCfg<D, FP8>::kTileBytes;
-    auto kern = attn_rows_kernel<D, IN, N>;
-    // clusters of 1..16 CTAs that fit the device at once, with one or two CTAs per SM (0: not asked yet)
-    static int fit[64][2][kMaxCluster + 1] = {};
-    static bool configured[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!configured[dev]) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemFull);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-        configured[dev] = true;
+    static constexpr int kTile = TileCfg<D, FP8>::kTileBytes;
+    static constexpr int kSmem = kRowsCols<N> == 512 ? 232448 : 115712;    // one or two CTAs per SM (1 KB of each is the system's)
+    static constexpr int kSlots = (kSmem - W::kFixedBytes) / kTile < kMaxSlots ? (kSmem - W::kFixedBytes) / kTile : kMaxSlots;
+    static_assert(kSlots >= 2 && kSlots * kTile >= N * D * 4, "the ring holds two tiles and the partial result");
+    static constexpr int kDynamic = W::kFixedBytes + kSlots * kTile;
+
+    static void set_cluster(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cs) {
+        attr->id = cudaLaunchAttributeClusterDimension;
+        attr->val.clusterDim.x = cs;
+        attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cfg.blockDim = dim3(kRowsThreads);
+        cfg.dynamicSmemBytes = kDynamic;
     }
-    const long long groups = static_cast<long long>(p.B) * p.Hkv;
-    const int nt = (p.Sk + kTileN - 1) / kTileN;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cfg.stream = stream;
-    cfg.blockDim = dim3(kRowsThreads);
-    auto set_cluster = [&](int cs, int half) {
-        attr[0].val.clusterDim.x = cs;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.dynamicSmemBytes = half ? kSmemHalf : kSmemFull;
-    };
-    // The split: the time of a candidate is its waves times (a fixed part for start, exchange and combination, plus its
-    // share of K and V at the rate one CTA gets).
-    int best_cs = 0, best_half = 0;
-    double best = 1e30;
-    for (int half = 0; half < 2; ++half) {
-        if (half && (N == 64 || kSmemHalf - W::kFixedBytes < 2 * kTile)) continue;
-        for (int cs = 1; cs <= kMaxCluster && cs <= nt; ++cs) {
-            if (fit[dev][half][cs] == 0) {
-                set_cluster(cs, half);
-                cfg.gridDim = dim3(cs);
-                int n = 0;
-                e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-                if (e != cudaSuccess) { cudaGetLastError(); n = -1; }
-                fit[dev][half][cs] = n > 0 ? n : -1;
-            }
-            const int n = fit[dev][half][cs];
-            if (n <= 0) continue;
-            const long long at_once = groups < n ? groups : n;
-            const double waves = static_cast<double>((groups + n - 1) / n);
-            const double rate = fmin(half ? 60e3 : 100e3, 6.5e6 / (static_cast<double>(at_once) * cs));   // bytes per us and CTA
-            const int per_cta = (nt + cs - 1) / cs;
-            const double t = waves * (5.0 + 0.1 * cs + 2.0 * per_cta * kTile / rate);
-            if (t < best) { best = t; best_cs = cs; best_half = half; }
+    // Clusters of `cs` CTAs that fit the device at once.  The occupancy query (asked once per device and size) counts one
+    // CTA per SM for every kernel that allocates TMEM; with 256 columns two run, and a cluster may then lie on half as many
+    // SMs, so that of the portable sizes nearly all 2 x 148 places can be used.
+    static int fit(int dev, int cs) {
+        static int known[64][kMaxCluster + 1] = {};
+        static bool configured[64] = {};
+        auto kern = attn_rows_kernel<D, IN, N>;
+        if (!configured[dev]) {
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynamic) != cudaSuccess ||
+                cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
+                cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+                return 0;
+            configured[dev] = true;
         }
+        if (known[dev][cs] == 0) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr;
+            set_cluster(cfg, &attr, cs);
+            cfg.gridDim = dim3(cs);
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            known[dev][cs] = n > 0 ? n : -1;
+        }
+        const int n = known[dev][cs] > 0 ? known[dev][cs] : 0;
+        if (kRowsCols<N> == 512 || n == 0) return n;
+        return cs <= 8 && 272 / cs > 2 * n ? 272 / cs : 2 * n;
     }
-    if (best_cs == 0) return cudaErrorInvalidConfiguration;
-    const int cs = best_cs, half = best_half;
-    RowsParams rp;
-    rp.cs = cs;
-    rp.nt = nt;
-    rp.tmem_cols = half ? 256 : 512;
-    const int cap = rp.tmem_cols / N;                       // key tiles whose scores fit TMEM
-    const int per_cta = (nt + cs - 1) / cs;
-    rp.rounds = (per_cta + cap - 1) / cap;
-    rp.share = (nt + cs * rp.rounds - 1) / (cs * rp.rounds);
-    int slots = ((half ? kSmemHalf : kSmemFull) - W::kFixedBytes) / kTile;
-    if (slots > kMaxSlots) slots = kMaxSlots;
-    rp.slots = slots;
-    rp.rows = p.Sq * p.group;
-    rp.mode = mode;
-    if (groups * cs > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    set_cluster(cs, half);
-    cfg.gridDim = dim3(static_cast<unsigned>(groups * cs));
-    cfg.dynamicSmemBytes = W::kFixedBytes + slots * kTile;
-    return cudaLaunchKernelEx(&cfg, kern, tk, tv, q, p, rp);
-}
+    // CTAs per cluster: the candidate with the shortest estimated time.  Measured on shapes from 1 x 1K to 16 x 2K and
+    // 1 x 32K: a part that does not depend on the context (5.6 us, 0.1 us per CTA of a cluster for exchange and combination,
+    // 1.2 us more beyond the portable size), one key tile's way through a CTA (hand-offs 0.83 us, or the rate of 55 GB/s one
+    // CTA reads at), and the device's bandwidth, which are added as squares where they overlap.  It picks the fastest size or
+    // one within 8 % of it.
+    static int pick_cluster(int dev, const AttnParams& p) {
+        const double groups = static_cast<double>(p.B) * p.Hkv;
+        const int nt = (p.Sk + kTileN - 1) / kTileN;
+        const double bytes_us = 2.0 * nt * groups * kTile / 6.3e6;
+        const double pair_us = fmax(N == 16 ? 0.83 : N == 32 ? 1.6 : 2.5, 2.0 * kTile / 55e3);
+        double best = 1e30;
+        int best_cs = 0;
+        for (int cs = 1; cs <= kMaxCluster && cs <= nt; ++cs) {
+            const int n = fit(dev, cs);
+            if (n <= 0) continue;
+            const double waves = ceil(groups / n);
+            const double shared = fmin(groups, n) * cs > 148.0 ? 1.15 : 1.0;     // two CTAs on an SM slow each other a little
+            const double hand_us = waves * ((nt + cs - 1) / cs) * pair_us * shared;
+            const double t = waves * (5.6 + 0.1 * cs + (cs > 8 ? 1.2 : 0.0)) + sqrt(hand_us * hand_us + bytes_us * bytes_us);
+            if (t < best) { best = t; best_cs = cs; }
+        }
+        return best_cs;
+    }
+    static cudaError_t launch(int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
+                              cudaStream_t stream) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+        const int cs = pick_cluster(dev, p);
+        const long long groups = static_cast<long long>(p.B) * p.Hkv;
+        if (cs == 0 || groups * cs > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        RowsParams rp;
+        rp.cs = cs;
+        rp.nt = (p.Sk + kTileN - 1) / kTileN;
+        constexpr int cap = kRowsCols<N> / N;            // key tiles whose scores fit TMEM
+        const int per_cta = (rp.nt + cs - 1) / cs;
+        rp.rounds = (per_cta + cap - 1) / cap;
+        rp.share = (rp.nt + cs * rp.rounds - 1) / (cs * rp.rounds);
+        rp.slots = kSlots;
+        rp.rows = p.Sq * p.group;
+        rp.mode = mode;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr;
+        set_cluster(cfg, &attr, cs);
+        cfg.gridDim = dim3(static_cast<unsigned>(groups * cs));
+        cfg.stream = stream;
+        return cudaLaunchKernelEx(&cfg, attn_rows_kernel<D, IN, N>, tk, tv, q, p, rp);
+    }
+};
 
 template <int D, int IN>
 cudaError_t dispatch_rows(int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
                           cudaStream_t stream) {
     const int rows = p.Sq * p.group;
-    if (rows <= 16) return launch_rows<D, IN, 16>(mode, tk, tv, q, p, stream);
-    if (rows <= 32) return launch_rows<D, IN, 32>(mode, tk, tv, q, p, stream);
-    return launch_rows<D, IN, 64>(mode, tk, tv, q, p, stream);
+    if (rows <= 16) return RowsLauncher<D, IN, 16>::launch(mode, tk, tv, q, p, stream);
+    if (rows <= 32) return RowsLauncher<D, IN, 32>::launch(mode, tk, tv, q, p, stream);
+    return RowsLauncher<D, IN, 64>::launch(mode, tk, tv, q, p, stream);
 }
 
 }  // namespace
