@@ -1,4 +1,5 @@
-"""Thin ctypes binding over the C-ABI library declared in ``include/attn.h``.
+"""Thin binding over the C-ABI library declared in ``include/attn.h``: ctypes, and for ``attn_fwd`` the native module
+``_host`` (csrc/host_binding.cpp), which does the same work in a quarter of the time.
 
 Argument marshalling only: every step of the attention forward runs in the CUDA kernels of
 ``libattn_b200.so``.  There is no fallback: if the library is missing or fails to load, importing a
@@ -19,6 +20,7 @@ MODES = {"exact": W_EXACT, "pot": W_POT, "h15": W_H15, "h15k2": W_H15K2, "h15k3"
 
 _LIB_PATH = Path(__file__).resolve().parent / "libattn_b200.so"
 _lib = None
+_forward = None      # _host.forward, once the library is loaded
 
 EXPORTS = ("attn_fwd", "attn_fwd_tau", "attn_fwd_pot", "attn_fwd_exact_emulated", "attn_weight_map", "attn_weight_map_pot", "attn_weight_map_fused", "attn_get_schedule", "attn_device_status",
            "attn_device_status_code", "attn_selftest_wait", "attn_device_status_reset", "attn_launch_count", "attn_status_string",
@@ -32,7 +34,7 @@ class AttnError(RuntimeError):
 
 
 def lib() -> ctypes.CDLL:
-    global _lib
+    global _lib, _forward
     if _lib is None:
         if not _LIB_PATH.exists():
             raise RuntimeError(
@@ -66,6 +68,12 @@ def lib() -> ctypes.CDLL:
         L.attn_status_string.argtypes = [i]
         L.attn_last_cuda_error.restype = i
         L.attn_version.restype = ctypes.c_char_p
+        try:
+            from . import _host
+        except ImportError as e:
+            raise RuntimeError("the host module is missing: build it with `python -m paper_2609_33586_b200.build`") from e
+        _host.set_entries(*(ctypes.cast(f, vp).value for f in (L.attn_fwd, L.attn_fwd_tau, L.attn_fwd_pot, L.attn_fwd_exact_emulated)))
+        _forward = _host.forward
         _lib = L
     return _lib
 
@@ -169,27 +177,21 @@ def attn_fwd(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, *, causal: bool,
         raise ValueError("poly_eighths goes with weight_mode = W_EXACT_POLY")
     if pot_tail is not None and weight_mode != W_POT:
         raise ValueError("pot_tail goes with weight_mode = W_POT")
-    for t in (q, k, v):
-        if not t.is_cuda or not t.is_contiguous():
-            raise ValueError("q, k, v must be contiguous CUDA tensors")
-    dt = in_dtype_of(q)
-    if in_dtype_of(k) != dt or in_dtype_of(v) != dt:
-        raise TypeError("q, k, v must share one storage dtype")
-    B, Sq, Hq, D = q.shape
-    Bk, Sk, Hkv, Dk = k.shape
-    if v.shape != k.shape or Bk != B or Dk != D:
-        raise ValueError("shape mismatch between q, k, v")
-    if out is None:
-        out = torch.empty((B, Sq, Hq, D), dtype=torch.bfloat16, device=q.device)
-    if lse is None and return_lse:
-        lse = torch.empty((B, Hq, Sq), dtype=torch.float32, device=q.device)
-    rc = attn_fwd_raw(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(),
-                      lse.data_ptr() if lse is not None else None, B, Hq, Hkv, Sq, Sk, D, causal,
-                      softmax_scale, weight_mode, dt, q_descale, k_descale, v_descale,
-                      _stream_ptr(stream), rescale_tau, pot_tail, poly_eighths)
-    if rc != 0:
-        raise AttnError(rc, "attn_fwd")
-    return out, lse
+    if _lib is None:
+        lib()
+    if poly_eighths is not None:
+        kind, option, option2 = 3, poly_eighths, False
+    elif pot_tail is not None:
+        kind, option, option2 = 2, pot_tail[0], pot_tail[1]
+    elif rescale_tau is not None:
+        kind, option, option2 = 1, rescale_tau, False
+    else:
+        kind, option, option2 = 0, 0, False
+    r = _forward(q, k, v, out, lse, return_lse, causal, softmax_scale, weight_mode, q_descale, k_descale, v_descale,
+                 kind, option, option2, stream if stream is None else int(stream.cuda_stream))
+    if type(r) is int:
+        raise AttnError(r, "attn_fwd")
+    return r
 
 
 def weight_map(x: torch.Tensor, weight_mode: int, out: torch.Tensor | None = None, stream=None):

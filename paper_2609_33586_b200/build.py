@@ -1,18 +1,20 @@
-"""Builds the C-ABI library ``libattn_b200.so`` in-tree with nvcc for sm_100a."""
+"""Builds the C-ABI library ``libattn_b200.so`` (nvcc, sm_100a) and the host module ``_host`` in-tree."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 import tempfile
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libattn_b200.so"
+HOST = PKG / f"_host{sysconfig.get_config_var('EXT_SUFFIX')}"
 SOURCES = ["api.cu", "attn_fwd_sm100.cu", "attn_rows_sm100.cu"]
-HEADERS = ["ptx.cuh", "weight_map.cuh", "attn_kernel_common.cuh", "softmax_math.cuh", "../../include/attn.h"]
+HEADERS = ["ptx.cuh", "attn_fwd_kernel.cuh", "weight_map.cuh", "attn_kernel_common.cuh", "softmax_math.cuh", "../../include/attn.h"]
 
 
 def _nvcc() -> str:
@@ -29,7 +31,28 @@ def needs_build() -> bool:
     return any((CSRC / f).stat().st_mtime > t for f in SOURCES + HEADERS)
 
 
+def build_host(force: bool = False) -> Path:
+    """The CPython module that does the per-call host work (csrc/host_binding.cpp)."""
+    src = CSRC / "host_binding.cpp"
+    if not force and HOST.exists() and HOST.stat().st_mtime >= max(src.stat().st_mtime, (CSRC / "../../include/attn.h").stat().st_mtime):
+        return HOST
+    import torch
+    troot = Path(torch.__file__).resolve().parent
+    cuda = Path(_nvcc()).resolve().parent.parent
+    tmp = HOST.with_suffix(f".so.tmp{os.getpid()}")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-w", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f"-I{sysconfig.get_paths()['include']}", f"-I{troot}/include", f"-I{troot}/include/torch/csrc/api/include",
+           f"-I{cuda}/include", "-o", str(tmp), str(src), f"-L{troot}/lib", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda",
+           "-ltorch_python", f"-Wl,-rpath,{troot}/lib"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("g++ failed on host_binding.cpp:\n" + res.stdout + res.stderr)
+    os.replace(tmp, HOST)
+    return HOST
+
+
 def build(force: bool = False, verbose: bool = False) -> Path:
+    build_host(force)
     if not force and not needs_build():
         return LIB
     tmp = LIB.with_suffix(f".so.tmp{os.getpid()}")
@@ -43,7 +66,7 @@ def build(force: bool = False, verbose: bool = False) -> Path:
         for (f, job), log in zip(jobs, logs):
             if job.returncode != 0:
                 raise RuntimeError(f"nvcc failed on {f}:\n{log}")
-        link = subprocess.run([_nvcc(), "-shared", "-o", str(tmp), *(f"{objs}/{f}.o" for f in SOURCES), "-lcudart"],
+        link = subprocess.run([_nvcc(), *flags[:2], "-shared", "-o", str(tmp), *(f"{objs}/{f}.o" for f in SOURCES), "-lcudart"],
                               capture_output=True, text=True)
         if link.returncode != 0:
             raise RuntimeError("nvcc failed at the link:\n" + link.stdout + link.stderr)

@@ -250,6 +250,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         if (lane == 31) *abort_flag = 0;
         fence_mbar_init();
         __syncwarp();
+        griddep_wait();    // what follows reads the caller's tensors
         if (lane == 0) {
             const int t0 = first_tile(0), n = tile_count(0);
             for (int i = 0; i < 2 * n && i < rp.slots; ++i) load_tile(t0, i, n);
@@ -268,6 +269,13 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         tmem_alloc(smem_u32(tmem_slot), kRowsCols<N>);
         tmem_relinquish();
     } else {
+        for (int e = tid; e < 2 * kTmemBlockCols; e += 128) anchors[e] = 0.f;   // and alphas, which follow: rows beyond R stay finite
+        for (int r = tid; r < N; r += 128) {
+            int lim = p.Sk;
+            if (p.causal && r < R) lim = min(p.Sk, r / p.group + 1 + p.Sk - p.Sq);
+            limits[r] = lim;
+        }
+        griddep_wait();
         // Q rows (query qi, head of the group) into the K-major operand tile, swizzled as TMA would have done it
         constexpr int kChunks = D * C::kElem / 16;              // 16-byte pieces of a row
         constexpr int kBoxChunks = C::kSwizzle / 16;
@@ -283,17 +291,13 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             const int sw = C::kSwizzle == 128 ? (c ^ (r & 7)) : (c ^ ((r >> 1) & 3));
             *reinterpret_cast<uint4*>(fix + W::kQOff + (ch / kBoxChunks) * W::kQBoxBytes + r * C::kSwizzle + sw * 16) = v;
         }
-        for (int e = tid; e < 2 * kTmemBlockCols; e += 128) anchors[e] = 0.f;   // and alphas, which follow: rows beyond R stay finite
-        for (int r = tid; r < N; r += 128) {
-            int lim = p.Sk;
-            if (p.causal && r < R) lim = min(p.Sk, r / p.group + 1 + p.Sk - p.Sq);
-            limits[r] = lim;
-        }
         fence_proxy_async();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    griddep_wait();
+    griddep_launch();
     // The status word is sticky: while it is set every wait returns at once and nothing is stored.  All CTAs of the
     // cluster still take every step, because the others read their shared memory.
     if (tid == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) *abort_flag = 1;
@@ -663,12 +667,16 @@ struct RowsLauncher {
     static_assert(kSlots >= 2 && kSlots * kTile >= N * D * 4, "the ring holds two tiles and the partial result");
     static constexpr int kDynamic = W::kFixedBytes + kSlots * kTile;
 
+    // attr: room for two.  The second one is programmatic dependent launch: the set-up of this kernel overlaps the end of the
+    // kernel before it in the stream.
     static void set_cluster(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cs) {
-        attr->id = cudaLaunchAttributeClusterDimension;
-        attr->val.clusterDim.x = cs;
-        attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = cs;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = 2;
         cfg.blockDim = dim3(kRowsThreads);
         cfg.dynamicSmemBytes = kDynamic;
     }
@@ -688,8 +696,9 @@ struct RowsLauncher {
         }
         if (known[dev][cs] == 0) {
             cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute attr;
-            set_cluster(cfg, &attr, cs);
+            cudaLaunchAttribute attr[2];
+            set_cluster(cfg, attr, cs);
+            cfg.numAttrs = 1;
             cfg.gridDim = dim3(cs);
             int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
@@ -745,8 +754,8 @@ struct RowsLauncher {
         rp.rows = p.Sq * p.group;
         rp.mode = mode;
         cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr;
-        set_cluster(cfg, &attr, cs);
+        cudaLaunchAttribute attr[2];
+        set_cluster(cfg, attr, cs);
         cfg.gridDim = dim3(static_cast<unsigned>(groups * cs));
         cfg.stream = stream;
         return cudaLaunchKernelEx(&cfg, attn_rows_kernel<D, IN, N>, tk, tv, q, p, rp);

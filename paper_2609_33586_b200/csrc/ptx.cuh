@@ -165,6 +165,13 @@ __device__ __forceinline__ void mbar_wait_cluster(uint32_t bar, uint32_t parity,
     }
 }
 
+// ---------------------------------------------------------------- programmatic dependent launch
+// A kernel launched with the stream-serialisation attribute may start while its predecessor in the stream still runs; what
+// comes before griddep_wait must not touch memory that the predecessor writes or reads.  griddep_launch lets the successor
+// start in turn once every CTA has called it.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- warp and block helpers
 __device__ __forceinline__ float redux_max(float v) {
     float d;
