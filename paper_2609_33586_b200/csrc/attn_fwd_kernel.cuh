@@ -16,6 +16,11 @@
 //   warp 12        MMA issuer (one thread): S_t = Q_t K^T and O_t += P_t V on the tensor cores
 //   warp 13        TMA producer (one thread): Q per item, K/V through a ring of shared-memory slots
 // While warpgroup 0 works on S_0(j), the tensor cores compute P_1 V(j-1) and S_1(j), and vice versa.
+// Split form (SPLIT): when there are fewer items than SMs a cluster of CTAs shares an item, each taking a contiguous part
+// of its key tiles.  Every part must start with the anchor the sequential loop would have reached there, so for the rounding
+// maps the cluster first goes over all parts but the last for the row maxima alone (Q K^T and a maximum, a quarter of a
+// full step); exact-like modes need no such pass, their result does not depend on the anchor.  At the end each CTA leaves
+// O, l and its anchor in shared memory and adds up its share of the rows over the cluster.
 // TMEM columns: S_0/P_0 [0,128), S_1/P_1 [128,256), O_0 [256,384), O_1 [384,512).
 #pragma once
 #include "softmax_math.cuh"
@@ -24,7 +29,9 @@ namespace rowmax {
 
 namespace {
 
-template <int D, bool FP8>
+constexpr int kMaxSplit = 8;   // CTAs that share an item (the portable cluster size)
+
+template <int D, bool FP8, bool SPLIT = false>
 struct WsCfg {
     using C = TileCfg<D, FP8>;
     static constexpr int kSlots = FP8 ? 8 : (D == 128 ? 4 : 8);  // K/V ring slots (one tile each)
@@ -32,9 +39,16 @@ struct WsCfg {
     static constexpr int kRingBytes = kSlots * C::kTileBytes;
     static constexpr int kScaleOff = kQBytes + kRingBytes;        // float alpha[2][128]
     static constexpr int kBarOff = kScaleOff + 2 * 128 * 4;
-    static constexpr int kNumBars = 2 * kSlots + 8 * 2 + 1;
+    static constexpr int kNumBars = 2 * kSlots + 8 * 2 + 1 + (SPLIT ? 4 + 2 + 3 : 0);
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
-    static constexpr int kSmemBytes = kMiscOff + 16 + 1024;       // + manual 1024-byte alignment slack
+    // split form: row maxima of the parts before this one, [part][256]; anchor and row sum of this part, [256][2]; weights of
+    // the parts for the rows this CTA adds up, [part][rows]
+    static constexpr int kXmaxOff = kMiscOff + 16;
+    static constexpr int kMlOff = kXmaxOff + (SPLIT ? (kMaxSplit - 1) * 256 * 4 : 0);
+    static constexpr int kPartWOff = kMlOff + (SPLIT ? 256 * 8 : 0);
+    static constexpr int kEndOff = kPartWOff + (SPLIT ? (256 + kMaxSplit) * 4 : 0);
+    static constexpr int kSmemBytes = kEndOff + 1024;             // + manual 1024-byte alignment slack
+    static_assert(!SPLIT || 2 * kTileM * D * 4 <= kQBytes + kRingBytes, "O of both tiles is parked over Q and the ring");
     static_assert(kSmemBytes <= 232448, "exceeds the 227 KB shared memory of an sm_100 CTA");
 };
 
@@ -64,14 +78,18 @@ constexpr bool kStagger = true;
 
 constexpr int kBarSelftest = 0x7F;
 enum BarId : int { kBarQFull = 0, kBarQEmpty = 1, kBarKvFull = 2, kBarKvEmpty = 3, kBarSFull = 4, kBarPFull = 5,
-                   kBarOFull = 6, kBarScale = 7, kBarORescaled = 8, kBarOFree = 9 };
+                   kBarOFull = 6, kBarScale = 7, kBarORescaled = 8, kBarOFree = 9,
+                   kBarSFree = 10, kBarXmax = 11, kBarPart = 12, kBarItem = 13 };
 
 // One work item = two query tiles of 128 rows of one (batch, head).
 struct WorkItem {
     int h, b, hk;
     int q0[2];   // first query row of each tile
-    int n[2];    // key tiles of each tile (0: the tile is out of range or sees no key)
+    int n[2];    // key tiles of each tile (0: the tile is out of range or sees no key), split form: of this CTA's part
     int n_max;
+    int j0;      // first key tile (0 but in the split form)
+    // split form, maxima pass: first key tile, key tiles of each query tile
+    int pre_j0, pre_n[2];
 };
 
 // Items are numbered heaviest first (under a causal mask the last query tiles have the most key
@@ -95,6 +113,25 @@ __device__ __forceinline__ WorkItem decode_item(int w, const AttnParams& p, int 
         it.n[t] = (it.q0[t] < p.Sq && kv_end > 0) ? (kv_end + kTileN - 1) / kTileN : 0;
     }
     it.n_max = max(it.n[0], it.n[1]);
+    it.j0 = it.pre_j0 = it.pre_n[0] = it.pre_n[1] = 0;
+    return it;
+}
+// Part `rank` of `parts` of an item: key tiles [j0, j0 + n[t]) of each query tile, and of the maxima pass key tiles
+// [pre_j0, pre_j0 + pre_n[t]): the CTA's own part unless it is the last, whose maxima nobody needs; with two parts each CTA
+// takes half of the first one.
+__device__ __forceinline__ WorkItem part_of_item(WorkItem it, int rank, int parts) {
+    const int full[2] = {it.n[0], it.n[1]};
+    const int j1 = (rank + 1) * it.n_max / parts;
+    it.j0 = rank * it.n_max / parts;
+    const int half = it.n_max / 2;
+    it.pre_j0 = parts == 2 ? (rank == 0 ? 0 : half / 2) : it.j0;
+    const int pre_j1 = parts == 2 ? (rank == 0 ? half / 2 : half) : (rank == parts - 1 ? it.j0 : j1);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        it.n[t] = max(0, min(full[t], j1) - it.j0);
+        it.pre_n[t] = max(0, min(full[t], pre_j1) - it.pre_j0);
+    }
+    it.n_max = max(it.n[0], it.n[1]);
     return it;
 }
 
@@ -102,15 +139,16 @@ __device__ __forceinline__ WorkItem decode_item(int w, const AttnParams& p, int 
 
 // IN: storage type of q, k, v (kInBF16 / kInFP8 / kInFP16).  P has the type of V at 16 bits (the f16
 // kind wants both MMA operands in one format) and one of the two fp8 formats at 8 bits.
-template <int D, int IN, int MODE>
+template <int D, int IN, int MODE, bool SPLIT = false>
 __global__ void __launch_bounds__(512, 1)
 attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
     constexpr bool FP8 = IN == kInFP8;
     constexpr bool HALF = IN == kInFP16;
     using C = TileCfg<D, FP8>;
-    using W = WsCfg<D, FP8>;
+    using W = WsCfg<D, FP8, SPLIT>;
     constexpr int NS = W::kSlots;
+    constexpr bool kPre = SPLIT && !is_exact_like(MODE);   // row maxima of the part first
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const uint32_t sQ = smem_u32(smem);
@@ -134,6 +172,12 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     auto bar_o_rescaled = [&](int t) { return bar_x(6, t); };  // correction -> MMA: O_t rescaled for tile j
     auto bar_o_free = [&](int t) { return bar_x(7, t); };      // epilogue -> MMA: O_t has been read out
     const uint32_t bar_drain = bar0 + 8u * (2 * NS + 16);      // abort path only: the MMA warp's last commit
+    // split form.  The maxima pass has two score buffers per query tile: S_t and, as O_t is not in use yet, O_t.
+    auto bar_s_free = [&](int t, int b) { return bar0 + 8u * (2 * NS + 17 + 2 * b + t); };   // softmax -> MMA: buffer b of tile t has been read
+    auto bar_s_full2 = [&](int t) { return bar0 + 8u * (2 * NS + 21 + t); };                  // MMA -> softmax: scores in buffer 1 of tile t
+    const uint32_t bar_xmax = bar0 + 8u * (2 * NS + 23);       // the maxima of all parts before this one are here
+    const uint32_t bar_item = bar0 + 8u * (2 * NS + 24);       // MMA -> softmax: all products of the item are complete
+    const uint32_t bar_part = bar0 + 8u * (2 * NS + 25);       // all parts have left O, l and anchor
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
     // The status word is sticky: once a wait has expired (in an earlier launch, or in another CTA of this one) and
@@ -148,7 +192,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const int n_pairs = (p.Sq + 2 * kTileM - 1) / (2 * kTileM);
     const int bh = p.Hq * p.B;
     const int n_items = n_pairs * bh;
-    const int cta = blockIdx.x, n_ctas = gridDim.x;
+    const int parts = SPLIT ? p.split : 1, rank = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+    const int cta = SPLIT ? blockIdx.x / parts : blockIdx.x, n_ctas = SPLIT ? gridDim.x / parts : gridDim.x;
     const int shift = p.Sk - p.Sq;
 
     if (warp == 13) {
@@ -160,13 +205,19 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             mbar_init(bar_q_full(t), 1);
             mbar_init(bar_q_empty(t), 1);
             mbar_init(bar_s_full(t), 1);
-            mbar_init(bar_p_full(t), 4);      // one arrival per softmax warp
+            mbar_init(bar_p_full(t), 8);      // one arrival per softmax warp, one per correction warp
             mbar_init(bar_o_full(t), 1);
             mbar_init(bar_scale(t), 4);
-            mbar_init(bar_o_rescaled(t), 4);  // one arrival per correction warp
             mbar_init(bar_o_free(t), 4);      // one arrival per softmax warp (epilogue)
         } else if (lane == 18) {
             mbar_init(bar_drain, 1);
+        } else if (SPLIT && lane == 19) {
+            for (int i = 0; i < 4; ++i) mbar_init(bar_s_free(i & 1, i >> 1), 4);   // one arrival per softmax warp
+            mbar_init(bar_s_full2(0), 1);
+            mbar_init(bar_s_full2(1), 1);
+            mbar_init(bar_item, 1);
+            mbar_init(bar_xmax, rank > 0 ? 8 * rank : 1);   // one per softmax warp of each part before
+            mbar_init(bar_part, 8 * parts);   // one per softmax warp of every part
         }
         fence_mbar_init();
     }
@@ -183,10 +234,20 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     // stream may still be writing.
     griddep_wait();
     griddep_launch();
-    if (*abort_flag) {
+    if constexpr (SPLIT) {
+        // The others of the cluster reach into this CTA's shared memory: every CTA takes all steps, with waits that return at
+        // once if the flag is set, and leaves with the cluster.
+        cluster_arrive();
+        cluster_wait();
+    } else if (*abort_flag) {
         if (warp == 12) tmem_dealloc(tmem, kTmemCols);
         return;
     }
+    auto get_item = [&](int w) {
+        WorkItem it = decode_item(w, p, n_pairs, bh);
+        if constexpr (SPLIT) it = part_of_item(it, rank, parts);
+        return it;
+    };
     if (tid == 256) ROWMAX_STAMP(2, 63, 1);
     auto tmem_S = [&](int t) { return tmem + 128u * t; };
     auto tmem_O = [&](int t) { return tmem + 256u + 128u * t; };
@@ -207,7 +268,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             for (int round = 0;; ++round) {
                 const int w = item_index(round, cta, n_ctas);
                 if (w >= n_items || *abort_flag) break;
-                const WorkItem it = decode_item(w, p, n_pairs, bh);
+                const WorkItem it = get_item(w);
                 auto load_tile = [&](const CUtensorMap* tm, uint32_t dst, uint32_t bar, int head, int row0) {
                     mbar_arrive_expect_tx(bar, C::kTileBytes);
 #pragma unroll
@@ -217,7 +278,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 // After an expired wait nothing more is loaded: a wait then returns at once, and a copy into a buffer
                 // whose last copy may still be under way would leave more in flight than the waits below account for.
                 auto load_q = [&](int t) {
-                    if (it.n[t] > 0) {
+                    if (it.n[t] > 0 || (kPre && it.pre_n[t] > 0)) {
                         mbar_wait(bar_q_empty(t), (q_use[t] & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarQEmpty);
                         if (*abort_flag) return;
                         load_tile(&tmQ, sQ + t * C::kTileBytes, bar_q_full(t), it.h, it.q0[t]);
@@ -226,6 +287,17 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 };
                 if (round == 0) ROWMAX_STAMP(3, 63, 0);
                 load_q(0);
+                const int pre_max = kPre ? max(it.pre_n[0], it.pre_n[1]) : 0;
+                if constexpr (kPre) {
+                    for (int j = 0; j < pre_max && !*abort_flag; ++j) {
+                        const int slot = kv_idx % NS, use = kv_idx / NS;
+                        mbar_wait_poll(bar_kv_empty(slot), (use & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarKvEmpty);
+                        if (*abort_flag) break;
+                        load_tile(&tmK, sRing + slot * C::kTileBytes, bar_kv_full(slot), it.hk, (it.pre_j0 + j) * kTileN);
+                        ++kv_idx;
+                        if (j == 0) load_q(1);
+                    }
+                }
                 for (int j = 0; j < it.n_max && !*abort_flag; ++j) {
 #pragma unroll
                     for (int kv = 0; kv < 2; ++kv) {
@@ -233,12 +305,12 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         mbar_wait(bar_kv_empty(slot), (use & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarKvEmpty);
                         if (*abort_flag) break;
                         load_tile(kv == 0 ? &tmK : &tmV, sRing + slot * C::kTileBytes, bar_kv_full(slot), it.hk,
-                                  j * kTileN);
+                                  (it.j0 + j) * kTileN);
                         ++kv_idx;
-                        if (j == 0 && kv == 0) load_q(1);
+                        if (pre_max == 0 && j == 0 && kv == 0) load_q(1);
                     }
                 }
-                if (it.n_max == 0) load_q(1);
+                if (it.n_max == 0 && pre_max == 0) load_q(1);
             }
             // Before the CTA ends every load this thread issued must have landed.  Normally the consumers have
             // seen to that and these waits return at once; after an expired wait they may have stopped waiting while
@@ -259,12 +331,12 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             const uint32_t ring_lo_k = umma_desc_lo(sRing, 16);               // K tiles: K-major
             const uint32_t ring_lo_v = umma_desc_lo(sRing, C::kBoxBytes);     // V tiles: MN-major, LBO = next 128-byte column block
             constexpr uint32_t kTileLo = C::kTileBytes >> 4;
-            auto issue_s = [&](int t, uint32_t k_lo) {
+            auto issue_s = [&](int t, uint32_t k_lo, uint32_t dst) {
                 const uint32_t q_lo = q_lo0 + t * kTileLo;
 #pragma unroll
                 for (int ks = 0; ks < C::kQkSteps; ++ks) {
                     const uint32_t off = ((ks / C::kStepsPerBox) * C::kBoxBytes + (ks % C::kStepsPerBox) * 32) >> 4;
-                    umma_ss_lo<FP8>(tmem_S(t), q_lo + off, k_lo + off, desc_hi, idesc_s, ks > 0 ? 1u : 0u);
+                    umma_ss_lo<FP8>(dst, q_lo + off, k_lo + off, desc_hi, idesc_s, ks > 0 ? 1u : 0u);
                 }
             };
             auto issue_pv = [&](int t, uint32_t v_lo, bool accumulate) {
@@ -285,19 +357,47 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             for (int round = 0;; ++round) {
                 const int w = item_index(round, cta, n_ctas);
                 if (w >= n_items) break;
-                const WorkItem it = decode_item(w, p, n_pairs, bh);
+                const WorkItem it = get_item(w);
+                if constexpr (kPre) {
+                    const int pre_max = max(it.pre_n[0], it.pre_n[1]);
+                    for (int j = 0; j < pre_max; ++j) {
+                        mbar_wait_poll(bar_kv_full(kv_base % NS), (kv_base / NS) & 1, wctx, (kRoleMma << 8) | kBarKvFull);
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            if (j < it.pre_n[t]) {
+                                const int buf = j & 1;
+                                if (j == 0) mbar_wait(bar_q_full(t), q_use[t] & 1, wctx, (kRoleMma << 8) | kBarQFull);
+                                if (j >= 2) mbar_wait_poll(bar_s_free(t, buf), (j / 2 - 1) & 1, wctx, (kRoleMma << 8) | kBarSFree);
+                                tc_fence_after();
+                                if (leader) {
+                                    if (!*abort_flag) issue_s(t, ring_lo_k + slot_lo(kv_base), buf == 0 ? tmem_S(t) : tmem_O(t));
+                                    umma_commit(buf == 0 ? bar_s_full(t) : bar_s_full2(t));
+                                }
+                            }
+                        }
+                        if (leader) umma_commit(bar_kv_empty(kv_base % NS));
+                        __syncwarp();
+                        ++kv_base;
+                    }
+                }
                 if (it.n_max > 0) {
                     wait_full(kv_base);
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
                         if (it.n[t] > 0) {
-                            mbar_wait(bar_q_full(t), q_use[t] & 1, wctx, (kRoleMma << 8) | kBarQFull);
+                            if (kPre && it.pre_n[t] > 0) {   // both buffers have been read: their last uses
+                                const int last = it.pre_n[t] - 1;
+                                mbar_wait_poll(bar_s_free(t, last & 1), (last / 2) & 1, wctx, (kRoleMma << 8) | kBarSFree);
+                                if (last > 0) mbar_wait_poll(bar_s_free(t, (last - 1) & 1), ((last - 1) / 2) & 1, wctx, (kRoleMma << 8) | kBarSFree);
+                            } else {
+                                mbar_wait(bar_q_full(t), q_use[t] & 1, wctx, (kRoleMma << 8) | kBarQFull);
+                            }
                             if (kStagger && round == 0 && t == 1 && it.n[0] > 0)
                                 mbar_wait(bar_p_full(0), 0, wctx, (kRoleMma << 8) | kBarPFull);
                             tc_fence_after();
                             if (leader) {
                                 if (round == 0) ROWMAX_STAMP(3, 63, 1 + t);
-                                if (!*abort_flag) issue_s(t, ring_lo_k + slot_lo(kv_base));
+                                if (!*abort_flag) issue_s(t, ring_lo_k + slot_lo(kv_base), tmem_S(t));
                                 umma_commit(bar_s_full(t));
                                 if (it.n[t] == 1) umma_commit(bar_q_empty(t));
                             }
@@ -316,10 +416,9 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         for (int t = 0; t < 2; ++t) {
                             if (j < it.n[t]) {
                                 const uint32_t ph = (tiles[t] + j) & 1;
-                                mbar_wait(bar_o_rescaled(t), ph, wctx, (kRoleMma << 8) | kBarORescaled);
                                 // the accumulator of the previous item must have been read out
                                 if (j == 0) mbar_wait(bar_o_free(t), (q_use[t] & 1) ^ 1, wctx, (kRoleMma << 8) | kBarOFree);
-                                mbar_wait(bar_p_full(t), ph, wctx, (kRoleMma << 8) | kBarPFull);
+                                mbar_wait_poll(bar_p_full(t), ph, wctx, (kRoleMma << 8) | kBarPFull);
                                 if (leader) ROWMAX_STAMP(3, j, t * 4 + 0);
                                 tc_fence_after();
                                 if (leader) {
@@ -327,7 +426,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                                     umma_commit(bar_o_full(t));
                                     ROWMAX_STAMP(3, j, t * 4 + 2);
                                     if (j + 1 < it.n[t]) {
-                                        if (ok) issue_s(t, ring_lo_k + slot_lo(kv_base + 2 * j + 2));
+                                        if (ok) issue_s(t, ring_lo_k + slot_lo(kv_base + 2 * j + 2), tmem_S(t));
                                         umma_commit(bar_s_full(t));
                                         if (j + 2 == it.n[t]) umma_commit(bar_q_empty(t));   // last S of this item
                                         ROWMAX_STAMP(3, j, t * 4 + 3);
@@ -341,6 +440,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         }
                         __syncwarp();
                     }
+                }
+                if constexpr (SPLIT) {
+                    if (leader) umma_commit(bar_item);
+                    __syncwarp();
                 }
                 kv_base += 2 * it.n_max;
 #pragma unroll
@@ -367,7 +470,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         for (int round = 0;; ++round) {
             const int w = item_index(round, cta, n_ctas);
             if (w >= n_items) break;
-            const WorkItem it = decode_item(w, p, n_pairs, bh);
+            const WorkItem it = get_item(w);
             for (int j = 0; j < it.n_max; ++j) {
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
@@ -400,7 +503,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             tc_fence_before();
                         }
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(bar_o_rescaled(t));
+                        if (lane == 0) mbar_arrive(bar_p_full(t));
                         if (r == 0) ROWMAX_STAMP(2, j, t * 4 + 2);
                     }
                 }
@@ -429,13 +532,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         for (int round = 0;; ++round) {
             const int w = item_index(round, cta, n_ctas);
             if (w >= n_items) break;
-            const WorkItem it = decode_item(w, p, n_pairs, bh);
+            const WorkItem it = get_item(w);
             const int q0 = t == 0 ? it.q0[0] : it.q0[1];
             const int nt = t == 0 ? it.n[0] : it.n[1];
             const int row = q0 + r;
             const int row_limit = p.causal ? min(p.Sk, row + shift + 1) : p.Sk;  // visible keys of this row
             // first key index that some row of this tile cannot see (tile-uniform)
             const int tile_limit = p.causal ? min(p.Sk, q0 + shift + 1) : p.Sk;
+            const int j0 = SPLIT ? it.j0 : 0;
             float m_run = -INFINITY, l_run = 0.f;
             // h15 family at fp8: a lower bound of every raw score of this row that costs nothing per score.
             // |q . k| <= (sum_i |q_i|) * max_i |k_i| and an e4m3 key element is at most 448 in magnitude, so
@@ -450,8 +554,46 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     score_floor = -448.0f * 1.02f * abs_sum_e4m3_row<D / 16>(sQ + t * C::kTileBytes + r * D);
                 }
             }
+            const int pre_n = !kPre ? 0 : t == 0 ? it.pre_n[0] : it.pre_n[1];
+            if constexpr (kPre) {
+                // the row's maxima; those over the parts before this one are the anchor to start from
+                float m_part = -INFINITY;
+                for (int j = 0; j < pre_n; ++j) {
+                    const int buf = j & 1;
+                    mbar_wait_poll(buf == 0 ? bar_s_full(t) : bar_s_full2(t), (j / 2) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
+                    __syncwarp();
+                    tc_fence_after();
+                    uint32_t s[4][32];
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) tmem_ld32((buf == 0 ? tS : tO) + cc * 32, s[cc]);
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_s_free(t, buf));
+                    if ((it.pre_j0 + j + 1) * kTileN > tile_limit) {
+                        const int col_limit = row_limit - (it.pre_j0 + j) * kTileN;
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+                            for (int i = 0; i < 32; ++i)
+                                if (cc * 32 + i >= col_limit) s[cc][i] = __float_as_uint(-INFINITY);
+                    }
+                    m_part = fmaxf(m_part, row_max128(s));
+                }
+                const uint32_t xmax = smem_u32(smem + W::kXmaxOff) + (t * 128 + r) * 4;
+                for (int q = rank + 1; q < parts; ++q) st_cluster_f32(mapa(xmax + rank * 1024, q), m_part);
+                __syncwarp();
+                if (lane > rank && lane < parts) mbar_arrive_cluster(mapa(bar_xmax, lane));
+                if (rank > 0) {
+                    if (parts == 2) m_run = m_part;   // of the first part's second half
+                    mbar_wait_cluster(bar_xmax, 0, wctx, (kRoleSoftmax << 8) | kBarXmax);
+                    __syncwarp();
+                    for (int q = 0; q < rank; ++q)
+                        m_run = fmaxf(m_run, *reinterpret_cast<const volatile float*>(smem + W::kXmaxOff + q * 1024 + (t * 128 + r) * 4));
+                }
+            }
             for (int j = 0; j < nt; ++j) {
-                mbar_wait(bar_s_full(t), (tiles + j) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
+                mbar_wait(bar_s_full(t), (tiles + (kPre ? (pre_n + 1) / 2 : 0) + j) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
                 if (r == 0) ROWMAX_STAMP(t, j, 0);
                 __syncwarp();
                 tc_fence_after();
@@ -468,8 +610,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 // exact mode zero the masked weights explicitly (pot's floor 2^-20 is not nothing, and the
                 // polynomial route does not take -inf).  Keeping a masked variant out of the common modes
                 // makes their hot loop markedly faster.
-                const bool masked_tile = (j + 1) * kTileN > tile_limit;
-                const int col_limit = row_limit - j * kTileN;
+                const bool masked_tile = (j0 + j + 1) * kTileN > tile_limit;
+                const int col_limit = row_limit - (j0 + j) * kTileN;
                 if (masked_tile) {
 #pragma unroll
                     for (int cc = 0; cc < 4; ++cc)
@@ -582,6 +724,110 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 l_run = l_run * alpha + l_tile;
             }
 
+            if constexpr (SPLIT) {
+                // O of this part, unscaled, over Q and the ring: [row of 256][D], 16-byte pieces swizzled by the row
+                float2* ml = reinterpret_cast<float2*>(smem + W::kMlOff);
+                ml[t * 128 + r] = make_float2(m_run, l_run);
+                // the products of both query tiles read Q and the ring
+                mbar_wait_poll(bar_item, 0, wctx, (kRoleEpi << 8) | kBarItem);
+                __syncwarp();
+                tc_fence_after();
+                constexpr int kPieces = D / 4;
+                if (nt > 0) {
+                    uint8_t* mine = smem + (t * 128 + r) * (D * 4);
+#pragma unroll
+                    for (int cc = 0; cc < D / 32; ++cc) {
+                        uint32_t o[32];
+                        tmem_ld32(tO + cc * 32, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int v4 = 0; v4 < 8; ++v4)
+                            *reinterpret_cast<uint4*>(mine + (((cc * 8 + v4) ^ (r & (kPieces - 1))) << 4)) =
+                                make_uint4(o[v4 * 4], o[v4 * 4 + 1], o[v4 * 4 + 2], o[v4 * 4 + 3]);
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_o_free(t));
+                }
+                __syncwarp();
+                if (lane < parts) mbar_arrive_cluster(mapa(bar_part, lane));
+                mbar_wait_cluster(bar_part, 0, wctx, (kRoleEpi << 8) | kBarPart);
+                __syncwarp();
+                // this CTA's share of the 256 rows, added up over the parts
+                const int row_lo = rank * 256 / parts, n_rows = (rank + 1) * 256 / parts - row_lo;
+                float* weight = reinterpret_cast<float*>(smem + W::kPartWOff);    // [part][n_rows]
+                const int wt = tid;      // 0..255 over both softmax warpgroups
+                const float flag = lane < parts ? ld_cluster_f32(mapa(smem_u32(const_cast<int*>(abort_flag)), lane)) : 0.0f;
+                const bool alive = __all_sync(0xffffffffu, __float_as_int(flag) == 0);
+                if (wt < n_rows) {
+                    const int prow = row_lo + wt, tt = prow >> 7;
+                    const int out_row = (tt == 0 ? it.q0[0] : it.q0[1]) + (prow & 127);
+                    const uint32_t at = smem_u32(smem + W::kMlOff) + prow * 8;
+                    float m_fin = -INFINITY;
+                    float2 v[kMaxSplit];
+#pragma unroll
+                    for (int q = 0; q < kMaxSplit; ++q) {
+                        v[q] = q < parts ? ld_cluster_f32x2(mapa(at, q)) : make_float2(-INFINITY, 0.f);
+                    }
+#pragma unroll
+                    for (int q = 0; q < kMaxSplit; ++q) v[q].y = v[q].x == -INFINITY ? 0.f : v[q].y;   // no visible key yet
+#pragma unroll
+                    for (int q = 0; q < kMaxSplit; ++q) {
+                        if (v[q].y > 0.f) m_fin = fmaxf(m_fin, v[q].x);
+                    }
+                    float l_fin = 0.f;
+#pragma unroll
+                    for (int q = 0; q < kMaxSplit; ++q) {
+                        v[q].x = v[q].y > 0.f ? ex2_approx((v[q].x - m_fin) * p.c) : 0.f;   // a part without visible keys weighs nothing
+                        l_fin += v[q].x * v[q].y;
+                    }
+                    const bool has_keys = l_fin > 0.f;
+                    const float inv = has_keys ? p.v_descale / l_fin : 0.f;
+#pragma unroll
+                    for (int q = 0; q < kMaxSplit; ++q)
+                        if (q < parts) weight[q * n_rows + wt] = v[q].x * inv;
+                    if (alive && out_row < p.Sq && p.lse != nullptr)
+                        p.lse[(static_cast<size_t>(it.b) * p.Hq + it.h) * p.Sq + out_row] =
+                            has_keys ? 0.6931471805599453f * (m_fin * p.c + log2f(l_fin) - p_off) : -INFINITY;
+                }
+                named_barrier<2>(256);
+                constexpr int kBatch = 8;      // pieces a thread has in flight from one part
+                for (int e0 = wt; e0 < n_rows * kPieces; e0 += 256 * kBatch) {
+                    float4 acc[kBatch] = {};
+                    for (int q = 0; q < parts; ++q) {
+                        float4 v[kBatch];
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u) {
+                            const int e = e0 + 256 * u, prow = row_lo + e / kPieces, piece = e % kPieces;
+                            if (e < n_rows * kPieces)
+                                v[u] = ld_cluster_f32x4(mapa(smem_u32(smem) + prow * (D * 4) + ((piece ^ (prow & (kPieces - 1))) << 4), q));
+                        }
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u) {
+                            const int e = e0 + 256 * u;
+                            const float wq = e < n_rows * kPieces ? weight[q * n_rows + e / kPieces] : 0.f;
+                            if (wq > 0.f) {      // a part that weighs nothing has not written O
+                                acc[u].x = fmaf(wq, v[u].x, acc[u].x);
+                                acc[u].y = fmaf(wq, v[u].y, acc[u].y);
+                                acc[u].z = fmaf(wq, v[u].z, acc[u].z);
+                                acc[u].w = fmaf(wq, v[u].w, acc[u].w);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const int e = e0 + 256 * u, prow = row_lo + e / kPieces, piece = e % kPieces;
+                        const int out_row = (prow < 128 ? it.q0[0] : it.q0[1]) + (prow & 127);
+                        if (alive && e < n_rows * kPieces && out_row < p.Sq) {
+                            uint2 pk;
+                            pk.x = pack_bf16_rn(acc[u].x, acc[u].y);
+                            pk.y = pack_bf16_rn(acc[u].z, acc[u].w);
+                            *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.o) +
+                                                      ((static_cast<size_t>(it.b) * p.Sq + out_row) * p.Hq + it.h) * D + piece * 4) = pk;
+                        }
+                    }
+                }
+            } else
             // epilogue of this tile: O = v_descale * acc / l (the P offset cancels), LSE = ln2 * (m c + log2 l)
             if (q0 < p.Sq) {
                 const bool has_keys = (m_run != -INFINITY) && l_run > 0.f;
@@ -632,6 +878,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     }
 
     if (tid == 256) ROWMAX_STAMP(2, 63, 6);
+    if constexpr (SPLIT) {
+        cluster_arrive();
+        cluster_wait();     // nobody reads this CTA's shared memory any more
+    }
     tc_fence_before();
     __syncthreads();
     if (tid == 256) ROWMAX_STAMP(2, 63, 7);

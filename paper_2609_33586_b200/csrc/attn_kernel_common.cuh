@@ -41,6 +41,7 @@ struct AttnParams {
     // Rowmax-PoT tail (Eq. rowmax-pot and the sentence after it): index cap K_max and what happens beyond it
     float pot_neg_cap;  // lower clamp of the offset: -K_max (clamped tail) or -(K_max + 1) (dropped tail)
     float pot_drop_x;   // dropped tail: offsets below -(K_max + 1/2) weigh zero
+    int split;        // split form: CTAs that share a work item
     int* status;      // device-global sticky status word
 #ifdef ROWMAX_TRACE
     long long* trace;  // optional per-role cycle stamps of one CTA: [role 4][tile 64][slot 8]
