@@ -167,7 +167,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     auto bar_q_empty = [&](int t) { return bar_x(1, t); };     // MMA -> TMA: last S_t MMA of the item done
     auto bar_s_full = [&](int t) { return bar_x(2, t); };      // MMA -> softmax: S_t(j) is in TMEM
     auto bar_p_full = [&](int t) { return bar_x(3, t); };      // softmax -> MMA: P_t(j) is in TMEM
-    auto bar_o_full = [&](int t) { return bar_x(4, t); };      // MMA -> correction / epilogue: P_t V(j) accumulated
+    auto bar_o_full = [&](int t) { return bar_x(4, t); };      // MMA -> epilogue: the last P_t V of the item accumulated
     auto bar_scale = [&](int t) { return bar_x(5, t); };       // softmax -> correction: alpha_t(j) in smem
     auto bar_o_rescaled = [&](int t) { return bar_x(6, t); };  // correction -> MMA: O_t rescaled for tile j
     auto bar_o_free = [&](int t) { return bar_x(7, t); };      // epilogue -> MMA: O_t has been read out
@@ -423,7 +423,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                                 tc_fence_after();
                                 if (leader) {
                                     if (ok) issue_pv(t, ring_lo_v + slot_lo(kv_base + 2 * j + 1), j > 0);
-                                    umma_commit(bar_o_full(t));
+                                    if (j + 1 == it.n[t]) umma_commit(bar_o_full(t));
                                     ROWMAX_STAMP(3, j, t * 4 + 2);
                                     if (j + 1 < it.n[t]) {
                                         if (ok) issue_s(t, ring_lo_k + slot_lo(kv_base + 2 * j + 2), tmem_S(t));
@@ -479,7 +479,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         if (r == 0) ROWMAX_STAMP(2, j, t * 4 + 0);
                         const float alpha = sScale[t * 128 + r];
                         if (j > 0) {
-                            mbar_wait(bar_o_full(t), (tiles[t] + j - 1) & 1, wctx, (kRoleCorr << 8) | kBarOFull);
+                            // P V(j - 1) is complete: the softmax warps post alpha(j) after they have seen S(j), whose commit
+                            // covers everything issued before it
                             if (r == 0) ROWMAX_STAMP(2, j, t * 4 + 1);
                             __syncwarp();
                             tc_fence_after();
@@ -529,6 +530,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         constexpr bool kLattice = kFam > 0 && !FP8;
         const bool sat_form = kLattice && (IN != kInBF16 || !(p.tau > 0.0f));
         int tiles = 0;
+        int o_use = 0;      // items with key tiles so far
         for (int round = 0;; ++round) {
             const int w = item_index(round, cta, n_ctas);
             if (w >= n_items) break;
@@ -838,7 +840,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     p.lse[(static_cast<size_t>(it.b) * p.Hq + it.h) * p.Sq + row] = lse;
                 }
                 if (nt > 0) {
-                    mbar_wait(bar_o_full(t), (tiles + nt - 1) & 1, wctx, (kRoleEpi << 8) | kBarOFull);
+                    mbar_wait(bar_o_full(t), o_use & 1, wctx, (kRoleEpi << 8) | kBarOFull);
+                    ++o_use;
                     __syncwarp();
                     tc_fence_after();
                 }
