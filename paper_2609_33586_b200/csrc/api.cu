@@ -12,7 +12,7 @@
 namespace rowmax {
 cudaError_t launch_attn_fwd(int D, int in_type, int mode, const CUtensorMap& tq, const CUtensorMap& tk,
                             const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream);
-int plan_split(int mode, const AttnParams& p);
+int plan_attn_split(int D, int in_type, int mode, const AttnParams& p);
 cudaError_t launch_attn_fwd_split(int D, int in_type, int mode, int parts, const CUtensorMap& tq, const CUtensorMap& tk,
                                   const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream);
 bool use_rows_kernel(int in_type, int mode, const AttnParams& p);
@@ -201,7 +201,7 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
         e = rowmax::launch_attn_rows(D, in_dtype, kernel_mode, tk, tv, q, p, static_cast<cudaStream_t>(stream));
     } else {
         if ((rc = make_tile_map(&tq, q, fp8, half_in, B, Sq, Hq, D)) != ATTN_OK) return rc;
-        const int parts = rowmax::plan_split(kernel_mode, p);
+        const int parts = rowmax::plan_attn_split(D, in_dtype, kernel_mode, p);
         if (parts > 1) e = rowmax::launch_attn_fwd_split(D, in_dtype, kernel_mode, parts, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
         else e = rowmax::launch_attn_fwd(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
     }

@@ -72,10 +72,6 @@ template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setma
 #define ROWMAX_STAMP(role, j, slot) do { } while (0)
 #endif
 
-// Tile 1 of a CTA's first work item starts once tile 0's first P is done, which spreads the two
-// tiles' softmax phases apart for the first iterations.
-constexpr bool kStagger = true;
-
 constexpr int kBarSelftest = 0x7F;
 enum BarId : int { kBarQFull = 0, kBarQEmpty = 1, kBarKvFull = 2, kBarKvEmpty = 3, kBarSFull = 4, kBarPFull = 5,
                    kBarOFull = 6, kBarScale = 7, kBarORescaled = 8, kBarOFree = 9,
@@ -160,8 +156,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const WaitCtx wctx{abort_flag, p.status, kWaitLimitCycles};
 
     // barrier addresses
-    auto bar_kv_full = [&](int s) { return bar0 + 8u * s; };
-    auto bar_kv_empty = [&](int s) { return bar0 + 8u * (NS + s); };
+    // Ring positions count tiles: K(0), V(0), K(1), V(1), ... over all items.  V(j) and K(j + 1), positions 2i - 1 and 2i, share
+    // their barriers: the MMA warp needs both at once and is done with both at once, and every barrier that it waits for or
+    // commits to is time in which the tensor cores idle.  (The last V of an item goes with the first K of the next.)
+    constexpr int NP = NS / 2;
+    auto bar_kv_full = [&](int idx) { return bar0 + 8u * (((idx + 1) >> 1) % NP); };
+    auto bar_kv_empty = [&](int idx) { return bar0 + 8u * (NS + ((idx + 1) >> 1) % NP); };
+    auto ph_kv_full = [&](int idx) { return (((idx + 1) >> 1) / NP) & 1; };
+    auto ph_kv_empty = [&](int idx) { return ph_kv_full(idx) ^ 1; };
     auto bar_x = [&](int which, int t) { return bar0 + 8u * (2 * NS + 2 * which + t); };
     auto bar_q_full = [&](int t) { return bar_x(0, t); };      // TMA -> MMA: Q_t of the current item landed
     auto bar_q_empty = [&](int t) { return bar_x(1, t); };     // MMA -> TMA: last S_t MMA of the item done
@@ -197,9 +199,9 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const int shift = p.Sk - p.Sq;
 
     if (warp == 13) {
-        if (lane < NS) {
-            mbar_init(bar_kv_full(lane), 1);
-            mbar_init(bar_kv_empty(lane), 1);
+        if (lane < NP) {
+            mbar_init(bar0 + 8u * lane, 2);            // V(j) and K(j + 1)
+            mbar_init(bar0 + 8u * (NS + lane), 1);
         } else if (lane >= 16 && lane < 18) {
             const int t = lane - 16;
             mbar_init(bar_q_full(t), 1);
@@ -264,6 +266,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         if (warp == 13 && lane == 0) {
             // ------------------------------------------------------------ TMA producer
             int kv_idx = 0;             // K/V tiles loaded so far (ring position), over all items
+            mbar_arrive(bar_kv_full(0));   // the first pair has no V
             int q_use[2] = {0, 0};      // items that used Q buffer t so far
             for (int round = 0;; ++round) {
                 const int w = item_index(round, cta, n_ctas);
@@ -286,38 +289,40 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     }
                 };
                 if (round == 0) ROWMAX_STAMP(3, 63, 0);
-                load_q(0);
+                // K first: the last P V of the item before waits for it along with its V; then Q, once its buffers are free
                 const int pre_max = kPre ? max(it.pre_n[0], it.pre_n[1]) : 0;
+                auto load_kv = [&](const CUtensorMap* tm, int tile) {
+                    if constexpr (SPLIT) mbar_wait_poll(bar_kv_empty(kv_idx), ph_kv_empty(kv_idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
+                    else mbar_wait(bar_kv_empty(kv_idx), ph_kv_empty(kv_idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
+                    if (*abort_flag) return;
+                    load_tile(tm, sRing + (kv_idx % NS) * C::kTileBytes, bar_kv_full(kv_idx), it.hk, tile * kTileN);
+                    ++kv_idx;
+                };
                 if constexpr (kPre) {
                     for (int j = 0; j < pre_max && !*abort_flag; ++j) {
-                        const int slot = kv_idx % NS, use = kv_idx / NS;
-                        mbar_wait_poll(bar_kv_empty(slot), (use & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarKvEmpty);
-                        if (*abort_flag) break;
-                        load_tile(&tmK, sRing + slot * C::kTileBytes, bar_kv_full(slot), it.hk, (it.pre_j0 + j) * kTileN);
+                        load_kv(&tmK, it.pre_j0 + j);
+                        if (j == 0) { load_q(0); load_q(1); }
+                    }
+                    if (kv_idx & 1) {     // an odd number of tiles: the position that V would have stays empty
+                        mbar_arrive(bar_kv_full(kv_idx));
                         ++kv_idx;
-                        if (j == 0) load_q(1);
                     }
                 }
                 for (int j = 0; j < it.n_max && !*abort_flag; ++j) {
-#pragma unroll
-                    for (int kv = 0; kv < 2; ++kv) {
-                        const int slot = kv_idx % NS, use = kv_idx / NS;
-                        mbar_wait(bar_kv_empty(slot), (use & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarKvEmpty);
-                        if (*abort_flag) break;
-                        load_tile(kv == 0 ? &tmK : &tmV, sRing + slot * C::kTileBytes, bar_kv_full(slot), it.hk,
-                                  (it.j0 + j) * kTileN);
-                        ++kv_idx;
-                        if (pre_max == 0 && j == 0 && kv == 0) load_q(1);
-                    }
+                    load_kv(&tmK, it.j0 + j);
+                    if (pre_max == 0 && j == 0) { load_q(0); load_q(1); }
+                    if (*abort_flag) break;
+                    load_kv(&tmV, it.j0 + j);
                 }
-                if (it.n_max == 0 && pre_max == 0) load_q(1);
             }
+            // the last pair is complete without a K
+            mbar_arrive(bar_kv_full(kv_idx));
             // Before the CTA ends every load this thread issued must have landed.  Normally the consumers have
             // seen to that and these waits return at once; after an expired wait they may have stopped waiting while
-            // copies were still writing shared memory, so wait (bounded) for the last use of every ring slot and
+            // copies were still writing shared memory, so wait (bounded) for the last use of every pair of ring slots and
             // Q buffer.
-            for (int idx = kv_idx > NS ? kv_idx - NS : 0; idx < kv_idx; ++idx)
-                mbar_wait_quiet(bar_kv_full(idx % NS), (idx / NS) & 1, kDrainLimitCycles);
+            for (int idx = kv_idx >= NS ? kv_idx - NS + 1 : 0; idx < kv_idx; ++idx)
+                mbar_wait_quiet(bar_kv_full(idx), ph_kv_full(idx), kDrainLimitCycles);
 #pragma unroll
             for (int t = 0; t < 2; ++t)
                 if (q_use[t] > 0) mbar_wait_quiet(bar_q_full(t), (q_use[t] - 1) & 1, kDrainLimitCycles);
@@ -349,7 +354,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             };
             auto slot_lo = [&](int idx) { return static_cast<uint32_t>(idx % NS) * kTileLo; };
             auto wait_full = [&](int idx) {
-                mbar_wait(bar_kv_full(idx % NS), (idx / NS) & 1, wctx, (kRoleMma << 8) | kBarKvFull);
+                mbar_wait(bar_kv_full(idx), ph_kv_full(idx), wctx, (kRoleMma << 8) | kBarKvFull);
             };
             int kv_base = 0;            // ring index of K_0 of the current item
             int tiles[2] = {0, 0};      // key tiles of query tile t finished in earlier items (barrier phases)
@@ -361,7 +366,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 if constexpr (kPre) {
                     const int pre_max = max(it.pre_n[0], it.pre_n[1]);
                     for (int j = 0; j < pre_max; ++j) {
-                        mbar_wait_poll(bar_kv_full(kv_base % NS), (kv_base / NS) & 1, wctx, (kRoleMma << 8) | kBarKvFull);
+                        if (kv_base == 0 || (kv_base & 1)) mbar_wait_poll(bar_kv_full(kv_base), ph_kv_full(kv_base), wctx, (kRoleMma << 8) | kBarKvFull);
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
                             if (j < it.pre_n[t]) {
@@ -375,10 +380,11 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                                 }
                             }
                         }
-                        if (leader) umma_commit(bar_kv_empty(kv_base % NS));
+                        if (leader && (kv_base & 1) == 0) umma_commit(bar_kv_empty(kv_base));
                         __syncwarp();
                         ++kv_base;
                     }
+                    kv_base += kv_base & 1;
                 }
                 if (it.n_max > 0) {
                     wait_full(kv_base);
@@ -392,8 +398,6 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             } else {
                                 mbar_wait(bar_q_full(t), q_use[t] & 1, wctx, (kRoleMma << 8) | kBarQFull);
                             }
-                            if (kStagger && round == 0 && t == 1 && it.n[0] > 0)
-                                mbar_wait(bar_p_full(0), 0, wctx, (kRoleMma << 8) | kBarPFull);
                             tc_fence_after();
                             if (leader) {
                                 if (round == 0) ROWMAX_STAMP(3, 63, 1 + t);
@@ -403,15 +407,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             }
                         }
                     }
-                    if (leader) umma_commit(bar_kv_empty(kv_base % NS));
+                    if (leader) umma_commit(bar_kv_empty(kv_base));
                     for (int j = 0; j < it.n_max; ++j) {
                         // Everything the next MMAs need besides P is awaited first (it is normally there long
                         // before), so that once P_t(j) arrives the P V and next-S MMAs go out back to back.  (The flag
                         // is read here, off that path: if one of the waits below expires, this step's MMAs still go
                         // out, on stale operands; nothing is stored after that and the MMAs are awaited at the end.)
                         const bool ok = !*abort_flag;
-                        wait_full(kv_base + 2 * j + 1);
-                        if (j + 1 < it.n_max) wait_full(kv_base + 2 * j + 2);
+                        wait_full(kv_base + 2 * j + 1);      // V(j) and K(j + 1)
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
                             if (j < it.n[t]) {
@@ -434,10 +437,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                                 }
                             }
                         }
-                        if (leader) {
-                            umma_commit(bar_kv_empty((kv_base + 2 * j + 1) % NS));
-                            if (j + 1 < it.n_max) umma_commit(bar_kv_empty((kv_base + 2 * j + 2) % NS));
-                        }
+                        // V(j) and K(j + 1); V of the last tile goes with K(0) of the next item
+                        if (leader && j + 1 < it.n_max) umma_commit(bar_kv_empty(kv_base + 2 * j + 2));
                         __syncwarp();
                     }
                 }
@@ -629,20 +630,12 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
                 const float alpha = ex2_approx((m_run - m_use) * p.c);
                 m_run = m_new;
-                // exact-like modes post the rescale factor after the first 32 weights are under way, so that its
-                // special-function latency, the shared-memory store and the arrival hide behind them (measured +2 %);
-                // their weight phase is long enough for the correction warps to rescale O in what is left of it.  The
-                // rounding maps post it at once: their weight phase is shorter, and posting late put the correction on
-                // the critical path (measured 5 to 8 % slower).
-                constexpr bool kPostLate = is_exact_like(MODE);
-                auto post_alpha_now = [&]() {
-                    sScale[t * 128 + r] = alpha;
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_scale(t));
-                    if (r == 0) ROWMAX_STAMP(t, j, 2);
-                };
-                auto post_alpha = [&]() { if constexpr (kPostLate) post_alpha_now(); };
-                if constexpr (!kPostLate) post_alpha_now();
+                // Posted at once: the correction warps need the whole weight phase.  (Posting it after the first weights, behind
+                // which the special-function latency would hide, cost 3 to 8 %.)
+                sScale[t * 128 + r] = alpha;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_scale(t));
+                if (r == 0) ROWMAX_STAMP(t, j, 2);
 
                 // exact: x = s*c - m*c + P offset;  h15 family: scaled input 2^K x = s*(2^K c) - m*(2^K c);  pot: x = s*c - m*c
                 RowScale rs;
@@ -672,7 +665,6 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         uint32_t pw[16];
                         weights_chunk32<FP8, MODE, false, true, HALF, true>(s[cc], rs, 32, acc, pw);
                         tmem_st16(tS + cc * 16, pw);
-                        if (cc == 0) post_alpha();
                     }
                 } else if (is_pot(MODE) && masked_tile) {
 #pragma unroll
@@ -681,7 +673,6 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         weights_chunk32<FP8, MODE, true, true, HALF>(s[cc], rs, col_limit - cc * 32, acc, pw);
                         if constexpr (FP8) tmem_st8(tS + cc * 8, pw);
                         else tmem_st16(tS + cc * 16, pw);
-                        if (cc == 0) post_alpha();
                     }
                 } else {
                     // h15: the clamp is a no-op unless some score of the warp's rows lies more than 126 octaves
@@ -703,7 +694,6 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             weights_chunk32<FP8, MODE, false, true, HALF>(s[cc], rs, 32, acc, pw);
                             if constexpr (FP8) tmem_st8(tS + cc * 8, pw);
                             else tmem_st16(tS + cc * 16, pw);
-                            if (cc == 0) post_alpha();
                         }
                     } else {
 #pragma unroll
@@ -712,7 +702,6 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             weights_chunk32<FP8, MODE, false, false, HALF>(s[cc], rs, 32, acc, pw);
                             if constexpr (FP8) tmem_st8(tS + cc * 8, pw);
                             else tmem_st16(tS + cc * 16, pw);
-                            if (cc == 0) post_alpha();
                         }
                     }
                 }

@@ -42,63 +42,95 @@ struct SplitLauncher {
         }
         return known[dev][parts] > 0 ? known[dev][parts] : 0;
     }
+    // CTAs per item, 1 for the plain form.  Times are in steps of the loop (one key tile of a pair of query tiles), measured:
+    // a part costs its key tiles, with the rounding maps 0.65 of a step more for each tile of its maxima pass (two parts share
+    // the pass, so it is half as long), and 4.5 steps + 0.5 per part for the exchange and the sum of O; all SMs working slow
+    // each other by a tenth.  512 queries on 16K, 32/8 heads: bf16 h15 198 -> 154 us, exact 226 -> 138, e4m3 178 -> 125
+    // (2 parts); 64 queries on 8K 97 -> 49 (4 parts).  16 x 1K and 16 x 2K gain nothing and stay whole.
+    static int plan(const AttnParams& p) {
+        const int pairs = (p.Sq + 2 * kTileM - 1) / (2 * kTileM);
+        const double items = static_cast<double>(pairs) * p.Hq * p.B;
+        if (items > 148.0) return 1;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+        // key tiles of the last (longest) pair and of the middle one
+        const int shift = p.Sk - p.Sq;
+        const int all = (p.Sk + kTileN - 1) / kTileN;
+        const int first_end = p.causal ? 2 * kTileM + shift : p.Sk;
+        const int first = first_end <= 0 ? 0 : ((first_end < p.Sk ? first_end : p.Sk) + kTileN - 1) / kTileN;
+        const double longest = all, mean = 0.5 * (all + first);
+        double best = 0.93 * (longest + 1.5);      // a gain below that is not worth the risk of being wrong
+        int best_parts = 1;
+        for (int parts = 2; parts <= kMaxSplit && parts <= all; ++parts) {
+            const int n = fit(dev, parts);
+            if (n <= 0) continue;
+            const double per_tile = (is_exact_like(MODE) ? 1.0 : parts == 2 ? 1.325 : 1.65) / parts;
+            const double fixed = 4.5 + 0.5 * parts, busy = items * parts > 100.0 ? 1.1 : 1.0;
+            const double waves = ceil(items / n);
+            const double t = fmax(longest * per_tile + fixed, waves * (mean * per_tile + fixed)) * busy;
+            if (t < best) { best = t; best_parts = parts; }
+        }
+        return best_parts;
+    }
     static cudaError_t launch(int parts, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, AttnParams p,
                               cudaStream_t stream) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        const int n = fit(dev, parts);
-        if (n <= 0) return cudaErrorInvalidConfiguration;
         const long long items = static_cast<long long>((p.Sq + 2 * kTileM - 1) / (2 * kTileM)) * p.Hq * p.B;
+        if (items * parts > 0x7fffffffLL) return cudaErrorInvalidValue;
         p.split = parts;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[2];
         configure(cfg, attr, parts);
-        if (items * parts > 0x7fffffffLL) return cudaErrorInvalidValue;
         cfg.gridDim = dim3(static_cast<unsigned>(items * parts));     // one item per cluster, heaviest first
         cfg.stream = stream;
         return cudaLaunchKernelEx(&cfg, attn_fwd_ws_kernel<D, IN, MODE, true>, tq, tk, tv, p);
     }
 };
 
-template <int D, int IN>
-cudaError_t split_mode(int mode, int parts, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                       const AttnParams& p, cudaStream_t stream) {
+// Calls f with the launcher of a combination; false for one that has no split form.
+template <int D, int IN, typename F>
+bool with_mode(int mode, F f) {
     switch (mode) {
-        case kExact: return SplitLauncher<D, IN, kExact>::launch(parts, tq, tk, tv, p, stream);
-        case kPot: return SplitLauncher<D, IN, kPot>::launch(parts, tq, tk, tv, p, stream);
-        case kPotDrop: return SplitLauncher<D, IN, kPotDrop>::launch(parts, tq, tk, tv, p, stream);
-        case kH15: return SplitLauncher<D, IN, kH15>::launch(parts, tq, tk, tv, p, stream);
+        case kExact: f(SplitLauncher<D, IN, kExact>{}); return true;
+        case kPot: f(SplitLauncher<D, IN, kPot>{}); return true;
+        case kPotDrop: f(SplitLauncher<D, IN, kPotDrop>{}); return true;
+        case kH15: f(SplitLauncher<D, IN, kH15>{}); return true;
         default: break;
     }
     if constexpr (IN != kInFP16) {
         switch (mode) {
-            case kH15K2: return SplitLauncher<D, IN, kH15K2>::launch(parts, tq, tk, tv, p, stream);
-            case kH15K3: return SplitLauncher<D, IN, kH15K3>::launch(parts, tq, tk, tv, p, stream);
+            case kH15K2: f(SplitLauncher<D, IN, kH15K2>{}); return true;
+            case kH15K3: f(SplitLauncher<D, IN, kH15K3>{}); return true;
             default: break;
         }
     }
-    return cudaErrorInvalidValue;
+    return false;
+}
+template <typename F>
+bool with_launcher(int D, int in_type, int mode, F f) {
+    if (D == 128) {
+        if (in_type == kInBF16) return with_mode<128, kInBF16>(mode, f);
+        if (in_type == kInFP16) return with_mode<128, kInFP16>(mode, f);
+        return with_mode<128, kInFP8>(mode, f);
+    }
+    if (in_type == kInBF16) return with_mode<64, kInBF16>(mode, f);
+    if (in_type == kInFP16) return with_mode<64, kInFP16>(mode, f);
+    return with_mode<64, kInFP8>(mode, f);
 }
 
 }  // namespace
 
-int plan_split(int mode, const AttnParams& p) {
-    (void)mode; (void)p;
-    return 1;
+// CTAs that should share a work item (1: the plain form).  A deferred rescale stays whole: its anchor depends on the order.
+int plan_attn_split(int D, int in_type, int mode, const AttnParams& p) {
+    int parts = 1;
+    if (!(p.tau > 0.0f)) with_launcher(D, in_type, mode, [&](auto l) { parts = decltype(l)::plan(p); });
+    return parts;
 }
 
 cudaError_t launch_attn_fwd_split(int D, int in_type, int mode, int parts, const CUtensorMap& tq, const CUtensorMap& tk,
                                   const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream) {
-    if (D == 128) {
-        if (in_type == kInBF16) return split_mode<128, kInBF16>(mode, parts, tq, tk, tv, p, stream);
-        if (in_type == kInFP16) return split_mode<128, kInFP16>(mode, parts, tq, tk, tv, p, stream);
-        return split_mode<128, kInFP8>(mode, parts, tq, tk, tv, p, stream);
-    }
-    if (in_type == kInBF16) return split_mode<64, kInBF16>(mode, parts, tq, tk, tv, p, stream);
-    if (in_type == kInFP16) return split_mode<64, kInFP16>(mode, parts, tq, tk, tv, p, stream);
-    return split_mode<64, kInFP8>(mode, parts, tq, tk, tv, p, stream);
+    cudaError_t e = cudaErrorInvalidValue;
+    with_launcher(D, in_type, mode, [&](auto l) { e = decltype(l)::launch(parts, tq, tk, tv, p, stream); });
+    return e;
 }
 
 }  // namespace rowmax
