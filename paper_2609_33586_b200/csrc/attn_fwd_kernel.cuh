@@ -145,15 +145,16 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     using W = WsCfg<D, FP8, SPLIT>;
     constexpr int NS = W::kSlots;
     constexpr bool kPre = SPLIT && !is_exact_like(MODE);   // row maxima of the part first
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    // Declared with the alignment that the swizzled tiles need: all shared-memory addresses are then constants, not
+    // registers, of which the softmax warps have none to spare (checked below).
+    extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t sQ = smem_u32(smem);
     const uint32_t sRing = sQ + W::kQBytes;
-    float* sScale = reinterpret_cast<float*>(smem + W::kScaleOff);
+    const uint32_t sScale = smem_u32(smem + W::kScaleOff);
     const uint32_t bar0 = smem_u32(smem + W::kBarOff);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + W::kMiscOff);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + W::kMiscOff + 4);
-    const WaitCtx wctx{abort_flag, p.status, kWaitLimitCycles};
+    const uint32_t abort_at = smem_u32(smem + W::kMiscOff + 4);
+    const WaitCtx wctx{abort_at, p.status, kWaitLimitCycles};
 
     // barrier addresses
     // Ring positions count tiles: K(0), V(0), K(1), V(1), ... over all items.  V(j) and K(j + 1), positions 2i - 1 and 2i, share
@@ -182,10 +183,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const uint32_t bar_part = bar0 + 8u * (2 * NS + 25);       // all parts have left O, l and anchor
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
+    if ((smem_u32(smem) & 1023u) != 0) {
+        if (tid == 0) atomicCAS(p.status, 0, (kRoleSerial << 8) | kBarSelftest);
+        return;
+    }
     // The status word is sticky: once a wait has expired (in an earlier launch, or in another CTA of this one) and
     // until the host clears it, a CTA that starts is a no-op: it touches neither its outputs nor TMEM nor TMA.
     // One thread reads the word so that the whole CTA takes the same way.
-    if (tid == 0) *abort_flag = (*reinterpret_cast<volatile int*>(p.status) != 0);
+    if (tid == 0) write_flag(abort_at, *reinterpret_cast<volatile int*>(p.status) != 0 ? 1 : 0);
 #ifdef ROWMAX_TRACE
     const long long trace_t0 = clock64();
 #endif
@@ -241,7 +246,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // once if the flag is set, and leaves with the cluster.
         cluster_arrive();
         cluster_wait();
-    } else if (*abort_flag) {
+    } else if (flag_is_set(abort_at)) {
         if (warp == 12) tmem_dealloc(tmem, kTmemCols);
         return;
     }
@@ -270,7 +275,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             int q_use[2] = {0, 0};      // items that used Q buffer t so far
             for (int round = 0;; ++round) {
                 const int w = item_index(round, cta, n_ctas);
-                if (w >= n_items || *abort_flag) break;
+                if (w >= n_items || flag_is_set(abort_at)) break;
                 const WorkItem it = get_item(w);
                 auto load_tile = [&](const CUtensorMap* tm, uint32_t dst, uint32_t bar, int head, int row0) {
                     mbar_arrive_expect_tx(bar, C::kTileBytes);
@@ -283,7 +288,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 auto load_q = [&](int t) {
                     if (it.n[t] > 0 || (kPre && it.pre_n[t] > 0)) {
                         mbar_wait(bar_q_empty(t), (q_use[t] & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarQEmpty);
-                        if (*abort_flag) return;
+                        if (flag_is_set(abort_at)) return;
                         load_tile(&tmQ, sQ + t * C::kTileBytes, bar_q_full(t), it.h, it.q0[t]);
                         ++q_use[t];
                     }
@@ -294,12 +299,12 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 auto load_kv = [&](const CUtensorMap* tm, int tile) {
                     if constexpr (SPLIT) mbar_wait_poll(bar_kv_empty(kv_idx), ph_kv_empty(kv_idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
                     else mbar_wait(bar_kv_empty(kv_idx), ph_kv_empty(kv_idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
-                    if (*abort_flag) return;
+                    if (flag_is_set(abort_at)) return;
                     load_tile(tm, sRing + (kv_idx % NS) * C::kTileBytes, bar_kv_full(kv_idx), it.hk, tile * kTileN);
                     ++kv_idx;
                 };
                 if constexpr (kPre) {
-                    for (int j = 0; j < pre_max && !*abort_flag; ++j) {
+                    for (int j = 0; j < pre_max && !flag_is_set(abort_at); ++j) {
                         load_kv(&tmK, it.pre_j0 + j);
                         if (j == 0) { load_q(0); load_q(1); }
                     }
@@ -308,10 +313,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         ++kv_idx;
                     }
                 }
-                for (int j = 0; j < it.n_max && !*abort_flag; ++j) {
+                for (int j = 0; j < it.n_max && !flag_is_set(abort_at); ++j) {
                     load_kv(&tmK, it.j0 + j);
                     if (pre_max == 0 && j == 0) { load_q(0); load_q(1); }
-                    if (*abort_flag) break;
+                    if (flag_is_set(abort_at)) break;
                     load_kv(&tmV, it.j0 + j);
                 }
             }
@@ -375,7 +380,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                                 if (j >= 2) mbar_wait_poll(bar_s_free(t, buf), (j / 2 - 1) & 1, wctx, (kRoleMma << 8) | kBarSFree);
                                 tc_fence_after();
                                 if (leader) {
-                                    if (!*abort_flag) issue_s(t, ring_lo_k + slot_lo(kv_base), buf == 0 ? tmem_S(t) : tmem_O(t));
+                                    if (!flag_is_set(abort_at)) issue_s(t, ring_lo_k + slot_lo(kv_base), buf == 0 ? tmem_S(t) : tmem_O(t));
                                     umma_commit(buf == 0 ? bar_s_full(t) : bar_s_full2(t));
                                 }
                             }
@@ -401,7 +406,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             tc_fence_after();
                             if (leader) {
                                 if (round == 0) ROWMAX_STAMP(3, 63, 1 + t);
-                                if (!*abort_flag) issue_s(t, ring_lo_k + slot_lo(kv_base), tmem_S(t));
+                                if (!flag_is_set(abort_at)) issue_s(t, ring_lo_k + slot_lo(kv_base), tmem_S(t));
                                 umma_commit(bar_s_full(t));
                                 if (it.n[t] == 1) umma_commit(bar_q_empty(t));
                             }
@@ -413,7 +418,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         // before), so that once P_t(j) arrives the P V and next-S MMAs go out back to back.  (The flag
                         // is read here, off that path: if one of the waits below expires, this step's MMAs still go
                         // out, on stale operands; nothing is stored after that and the MMAs are awaited at the end.)
-                        const bool ok = !*abort_flag;
+                        const bool ok = !flag_is_set(abort_at);
                         wait_full(kv_base + 2 * j + 1);      // V(j) and K(j + 1)
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
@@ -463,7 +468,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         reg_dec<kRegCorr>();
         // The kernel before this one may have set the status word after the check above; no P V, and so no epilogue, is
         // reached before this warp's first arrival.
-        if (warp == 8 && lane == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) *abort_flag = 1;
+        if (warp == 8 && lane == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) write_flag(abort_at, 1);
         __syncwarp();
         const int r = tid & 127;
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
@@ -478,7 +483,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     if (j < it.n[t]) {
                         mbar_wait(bar_scale(t), (tiles[t] + j) & 1, wctx, (kRoleCorr << 8) | kBarScale);
                         if (r == 0) ROWMAX_STAMP(2, j, t * 4 + 0);
-                        const float alpha = sScale[t * 128 + r];
+                        const float alpha = ld_shared_f32(sScale + (t * 128 + r) * 4);
                         if (j > 0) {
                             // P V(j - 1) is complete: the softmax warps post alpha(j) after they have seen S(j), whose commit
                             // covers everything issued before it
@@ -632,7 +637,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 m_run = m_new;
                 // Posted at once: the correction warps need the whole weight phase.  (Posting it after the first weights, behind
                 // which the special-function latency would hide, cost 3 to 8 %.)
-                sScale[t * 128 + r] = alpha;
+                st_shared_f32(sScale + (t * 128 + r) * 4, alpha);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_scale(t));
                 if (r == 0) ROWMAX_STAMP(t, j, 2);
@@ -748,7 +753,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 const int row_lo = rank * 256 / parts, n_rows = (rank + 1) * 256 / parts - row_lo;
                 float* weight = reinterpret_cast<float*>(smem + W::kPartWOff);    // [part][n_rows]
                 const int wt = tid;      // 0..255 over both softmax warpgroups
-                const float flag = lane < parts ? ld_cluster_f32(mapa(smem_u32(const_cast<int*>(abort_flag)), lane)) : 0.0f;
+                const float flag = lane < parts ? ld_cluster_f32(mapa(abort_at, lane)) : 0.0f;
                 const bool alive = __all_sync(0xffffffffu, __float_as_int(flag) == 0);
                 if (wt < n_rows) {
                     const int prow = row_lo + wt, tt = prow >> 7;
@@ -823,7 +828,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             if (q0 < p.Sq) {
                 const bool has_keys = (m_run != -INFINITY) && l_run > 0.f;
                 const float inv = has_keys ? p.v_descale / l_run : 0.f;
-                const bool alive = !*abort_flag;      // after an expired wait the accumulators are not to be trusted: store nothing
+                const bool alive = !flag_is_set(abort_at);      // after an expired wait the accumulators are not to be trusted: store nothing
                 if (alive && row < p.Sq && p.lse != nullptr) {
                     const float lse = has_keys ? 0.6931471805599453f * (m_run * p.c + log2f(l_run) - p_off) : -INFINITY;
                     p.lse[(static_cast<size_t>(it.b) * p.Hq + it.h) * p.Sq + row] = lse;

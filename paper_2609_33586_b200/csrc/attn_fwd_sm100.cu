@@ -251,7 +251,7 @@ __global__ void selftest_wait_kernel(int* status, long long limit_cycles) {
         fence_mbar_init();
     }
     __syncthreads();
-    const WaitCtx ctx{&cta_abort, status, limit_cycles};
+    const WaitCtx ctx{smem_u32(&cta_abort), status, limit_cycles};
     mbar_wait(smem_u32(&bar), 0, ctx, (kRoleSelftest << 8) | kBarSelftest);
 }
 

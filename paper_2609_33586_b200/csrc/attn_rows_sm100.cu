@@ -207,8 +207,8 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     float* mfin = reinterpret_cast<float*>(fix + W::kMfinOff);
     float* lw = reinterpret_cast<float*>(fix + W::kLwOff);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fix + W::kMiscOff);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(fix + W::kMiscOff + 4);
-    const WaitCtx wctx{abort_flag, p.status, kWaitLimitCycles};
+    const uint32_t abort_at = smem_u32(fix + W::kMiscOff + 4);
+    const WaitCtx wctx{abort_at, p.status, kWaitLimitCycles};
     const uint32_t bar0 = sFix + W::kBarOff;
     auto bar_full = [&](int s) { return bar0 + 8u * s; };                      // TMA -> MMA: slot landed
     auto bar_empty = [&](int s) { return bar0 + 8u * (kMaxSlots + s); };       // MMA -> TMA: slot read
@@ -247,7 +247,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             mbar_init(bar_full(lane), 1);
             mbar_init(bar_empty(lane), 1);
         }
-        if (lane == 31) *abort_flag = 0;
+        if (lane == 31) write_flag(abort_at, 0);
         fence_mbar_init();
         __syncwarp();
         griddep_wait();    // what follows reads the caller's tensors
@@ -300,7 +300,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     griddep_launch();
     // The status word is sticky: while it is set every wait returns at once and nothing is stored.  All CTAs of the
     // cluster still take every step, because the others read their shared memory.
-    if (tid == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) *abort_flag = 1;
+    if (tid == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) write_flag(abort_at, 1);
     cluster_arrive();       // barriers are initialised; waited for before the first remote access and at the end
     const uint32_t tmem = *tmem_slot;
 
@@ -313,10 +313,10 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             int at = 0;           // tiles of the stream passed so far
             for (int c = 0; c < rp.rounds; ++c) {
                 const int t0 = first_tile(c), n = tile_count(c);
-                for (int i = 0; i < 2 * n && !*abort_flag; ++i, ++at) {
+                for (int i = 0; i < 2 * n && !flag_is_set(abort_at); ++i, ++at) {
                     if (at < filled) continue;
                     mbar_wait_poll(bar_empty(loaded % rp.slots), ((loaded / rp.slots) & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarSlot);
-                    if (*abort_flag) break;
+                    if (flag_is_set(abort_at)) break;
                     load_tile(t0, i, n);
                 }
             }
@@ -351,7 +351,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 mbar_wait_poll(bar_full(slot), (idx / rp.slots) & 1, wctx, (kRoleMma << 8) | kBarFull);
                 tc_fence_after();
                 if (leader) {
-                    if (!*abort_flag) {
+                    if (!flag_is_set(abort_at)) {
                         const uint32_t k_lo = k_lo0 + slot * kTileLo;
 #pragma unroll
                         for (int ks = 0; ks < C::kQkSteps; ++ks) {
@@ -371,7 +371,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 mbar_wait_poll(bar_p(buf), (np >> 1) & 1, wctx, (kRoleMma << 8) | kBarP);
                 tc_fence_after();
                 if (leader) {
-                    if (!*abort_flag) {
+                    if (!flag_is_set(abort_at)) {
                         const uint32_t v_lo = v_lo0 + slot * kTileLo;
                         const uint32_t pb_lo = p_lo + buf * (W::kPBytes >> 4);
 #pragma unroll

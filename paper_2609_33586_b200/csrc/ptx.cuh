@@ -50,11 +50,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 
 
+__device__ __forceinline__ bool flag_is_set(uint32_t saddr) {
+    int v;
+    asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(saddr) : "memory");
+    return v != 0;
+}
+__device__ __forceinline__ void write_flag(uint32_t saddr, int v) {
+    asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(saddr), "r"(v) : "memory");
+}
+
 // Sticky status: a CTA-local word in shared memory plus a device-global word.  Once either is
 // non-zero every wait returns at once, so all roles run their (finite) loops to the end and the
 // CTA tears down normally.
 struct WaitCtx {
-    volatile int* cta_abort;  // shared memory
+    uint32_t cta_abort;       // shared-memory address of an int (32 bits: it stays live over the whole loop)
     int* global_status;       // global memory
     long long limit_cycles;   // how long one wait may last
 };
@@ -67,12 +76,12 @@ constexpr long long kWaitLimitCycles = 2000000000LL;  // about one second at B20
 // reads); a quick-polling variant for single hand-offs changed nothing.
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& ctx, int code) {
     if (mbar_try_wait(bar, parity)) return;
-    if (*ctx.cta_abort) return;
+    if (flag_is_set(ctx.cta_abort)) return;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
-        if (*ctx.cta_abort) return;
+        if (flag_is_set(ctx.cta_abort)) return;
         if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
-            *ctx.cta_abort = 1;
+            write_flag(ctx.cta_abort, 1);
             atomicCAS(ctx.global_status, 0, code);
             return;
         }
@@ -89,9 +98,9 @@ __device__ __forceinline__ void mbar_wait_poll(uint32_t bar, uint32_t parity, co
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
             if (mbar_try_wait(bar, parity)) return;
-        if (*ctx.cta_abort) return;
+        if (flag_is_set(ctx.cta_abort)) return;
         if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
-            *ctx.cta_abort = 1;
+            write_flag(ctx.cta_abort, 1);
             atomicCAS(ctx.global_status, 0, code);
             return;
         }
@@ -161,9 +170,9 @@ __device__ __forceinline__ void mbar_wait_cluster(uint32_t bar, uint32_t parity,
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
             if (mbar_try_wait_cluster(bar, parity)) return;
-        if (*ctx.cta_abort) return;
+        if (flag_is_set(ctx.cta_abort)) return;
         if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
-            *ctx.cta_abort = 1;
+            write_flag(ctx.cta_abort, 1);
             atomicCAS(ctx.global_status, 0, code);
             return;
         }
@@ -178,6 +187,14 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------- warp and block helpers
+__device__ __forceinline__ float ld_shared_f32(uint32_t saddr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(saddr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_shared_f32(uint32_t saddr, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(saddr), "f"(v) : "memory");
+}
 __device__ __forceinline__ float redux_max(float v) {
     float d;
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(v));

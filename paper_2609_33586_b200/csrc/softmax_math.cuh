@@ -112,21 +112,20 @@ __device__ __forceinline__ uint32_t pack_e5m2x4_exact(float b0, float b1, float 
     return d;
 }
 
-// Row maximum of 128 scores held as 4 x 32 registers.
+// Row maximum of 128 scores held as 4 x 32 registers (four accumulators: the scores leave few registers).
 __device__ __forceinline__ float row_max128(const uint32_t (&s)[4][32]) {
-    float m[8];
+    float m[4];
 #pragma unroll
-    for (int a = 0; a < 8; ++a) m[a] = -INFINITY;
+    for (int a = 0; a < 4; ++a) m[a] = max3(__uint_as_float(s[0][3 * a]), __uint_as_float(s[0][3 * a + 1]), __uint_as_float(s[0][3 * a + 2]));
 #pragma unroll
-    for (int cc = 0; cc < 4; ++cc) {
+    for (int i = 12; i < 128; i += 8) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 16) {
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-                m[a] = max3(m[a], __uint_as_float(s[cc][i + 2 * a]), __uint_as_float(s[cc][i + 2 * a + 1]));
+        for (int a = 0; a < 4; ++a) {
+            const int k = i + 2 * a;
+            if (k < 128) m[a] = max3(m[a], __uint_as_float(s[k >> 5][k & 31]), __uint_as_float(s[(k + 1) >> 5][(k + 1) & 31]));
         }
     }
-    return fmaxf(max3(m[0], m[1], m[2]), max3(m[3], m[4], max3(m[5], m[6], m[7])));
+    return fmaxf(max3(m[0], m[1], m[2]), m[3]);
 }
 
 // Row minimum of the same 128 scores (decides whether the h15 clamp can be skipped for a tile).
