@@ -12,6 +12,8 @@
 namespace rowmax {
 cudaError_t launch_attn_fwd(int D, int in_type, int mode, const CUtensorMap& tq, const CUtensorMap& tk,
                             const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream);
+cudaError_t launch_attn_fwd_tau(int D, int mode, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                                const AttnParams& p, cudaStream_t stream);
 int plan_attn_split(int D, int in_type, int mode, const AttnParams& p);
 cudaError_t launch_attn_fwd_split(int D, int in_type, int mode, int parts, const CUtensorMap& tq, const CUtensorMap& tk,
                                   const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream);
@@ -202,7 +204,8 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     } else {
         if ((rc = make_tile_map(&tq, q, fp8, half_in, B, Sq, Hq, D)) != ATTN_OK) return rc;
         const int parts = rowmax::plan_attn_split(D, in_dtype, kernel_mode, p);
-        if (parts > 1) e = rowmax::launch_attn_fwd_split(D, in_dtype, kernel_mode, parts, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
+        if (p.tau > 0.0f) e = rowmax::launch_attn_fwd_tau(D, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
+        else if (parts > 1) e = rowmax::launch_attn_fwd_split(D, in_dtype, kernel_mode, parts, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
         else e = rowmax::launch_attn_fwd(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
     }
     if (e != cudaSuccess) {

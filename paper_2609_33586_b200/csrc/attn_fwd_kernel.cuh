@@ -135,7 +135,9 @@ __device__ __forceinline__ WorkItem part_of_item(WorkItem it, int rank, int part
 
 // IN: storage type of q, k, v (kInBF16 / kInFP8 / kInFP16).  P has the type of V at 16 bits (the f16
 // kind wants both MMA operands in one format) and one of the two fp8 formats at 8 bits.
-template <int D, int IN, int MODE, bool SPLIT = false>
+// TAU: deferred rescale (attn_fwd_tau, bf16 only), an instance of its own: the adoption rule in the common instances cost
+// them 1.5 to 3.5 % (bf16 8K h15 251.0 -> 244.3 us without).
+template <int D, int IN, int MODE, bool SPLIT = false, bool TAU = false>
 __global__ void __launch_bounds__(512, 1)
 attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -538,7 +540,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // packed form: there a bound on the key magnitude already removes the row-minimum pass, and the
         // scalar multiply-adds of the saturating form cost more issue slots than they save (measured 4 to 6 %).
         constexpr bool kLattice = kFam > 0 && !FP8;
-        const bool sat_form = kLattice && (IN != kInBF16 || !(p.tau > 0.0f));
+        constexpr bool kSatForm = kLattice && !TAU;
         int tiles = 0;
         int o_use = 0;      // items with key tiles so far
         for (int round = 0;; ++round) {
@@ -634,8 +636,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 const float m_t = row_max128(s);
                 // The tile maximum becomes the new anchor when there is none yet or when it exceeds the
                 // anchor by more than tau octaves (tau = 0: always, so the anchor is the running maximum).
-                const bool adopt = (m_run == -INFINITY) || ((m_t - m_run) * p.c > p.tau);
-                const float m_new = adopt ? fmaxf(m_run, m_t) : m_run;
+                float m_new = fmaxf(m_run, m_t);
+                if constexpr (TAU) {
+                    if (!((m_run == -INFINITY) || ((m_t - m_run) * p.c > p.tau))) m_new = m_run;
+                }
                 const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
                 const float alpha = ex2_approx((m_run - m_use) * p.c);
                 m_run = m_new;
@@ -663,7 +667,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 rs.clamp_lo = 0.f;
                 if constexpr (kFam > 0) rs.clamp_lo = masked_tile ? h15_clamp_zero<kFam>() : h15_clamp_floor<kFam>();
                 float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                if (kLattice && sat_form) {
+                if constexpr (kSatForm) {
                     // distance below the anchor as a fraction of the clamp distance R, which is also where a masked
                     // score (-inf) ends up: 2^K * 126 (weight floor 2^-126, Eq. h15), in a tile with masked scores
                     // 2^K * 127 (pattern of +0)
@@ -898,6 +902,48 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     if (tid == 0 && p.trace != nullptr && p.trace_block < 0) p.trace[blockIdx.x] = clock64() - trace_t0;   // per-CTA busy time
 #endif
     if (warp == 12) tmem_dealloc(tmem, kTmemCols);
+}
+
+// Launches the plain form.
+template <int D, int IN, int MODE, bool TAU = false>
+static cudaError_t launch_ws(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                             const AttnParams& p, cudaStream_t stream) {
+    using W = WsCfg<D, IN == kInFP8>;
+    auto kern = attn_fwd_ws_kernel<D, IN, MODE, false, TAU>;
+    // per-device launch set-up: the shared-memory opt-in of this instance and the SM count
+    static bool configured[64] = {};
+    static int sm_counts[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!configured[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmemBytes);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_counts[dev], cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+    }
+    const int sm_count = sm_counts[dev];
+    const long long n_pairs = (p.Sq + 2 * kTileM - 1) / (2 * kTileM);
+    const long long items = n_pairs * p.Hq * p.B;
+    if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
+    // persistent CTAs: one per SM (shared memory and TMEM allow no more), each walking its share of the items
+    const unsigned blocks = static_cast<unsigned>(items < sm_count ? items : sm_count);
+    // Programmatic dependent launch: the set-up of this kernel (barriers, TMEM, first instructions) overlaps the end of the
+    // kernel before it in the stream, 1.1 us (2 heads x 256 keys 8.6 -> 7.4 us, 16 x 1K e4m3 20.3 -> 19.4).  Not where a CTA
+    // takes more than one item: CTAs that become resident in the order in which SMs fall free, instead of all at once, run
+    // longer there than the overlap saves (48 heads x 2K bf16 60.5 -> 62.6 us).
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = W::kSmemBytes;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = items <= sm_count ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, tq, tk, tv, p);
 }
 
 }  // namespace rowmax

@@ -6,47 +6,6 @@ namespace rowmax {
 // ------------------------------------------------------------------------------------------------
 // Host launcher
 // ------------------------------------------------------------------------------------------------
-template <int D, int IN, int MODE>
-static cudaError_t launch_ws(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                             const AttnParams& p, cudaStream_t stream) {
-    using W = WsCfg<D, IN == kInFP8>;
-    auto kern = attn_fwd_ws_kernel<D, IN, MODE>;
-    // per-device launch set-up: the shared-memory opt-in of this instance and the SM count
-    static bool configured[64] = {};
-    static int sm_counts[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!configured[dev]) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmemBytes);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_counts[dev], cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        configured[dev] = true;
-    }
-    const int sm_count = sm_counts[dev];
-    const long long n_pairs = (p.Sq + 2 * kTileM - 1) / (2 * kTileM);
-    const long long items = n_pairs * p.Hq * p.B;
-    if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
-    // persistent CTAs: one per SM (shared memory and TMEM allow no more), each walking its share of the items
-    const unsigned blocks = static_cast<unsigned>(items < sm_count ? items : sm_count);
-    // Programmatic dependent launch: the set-up of this kernel (barriers, TMEM, first instructions) overlaps the end of the
-    // kernel before it in the stream, 1.1 us (2 heads x 256 keys 8.6 -> 7.4 us, 16 x 1K e4m3 20.3 -> 19.4).  Not where a CTA
-    // takes more than one item: CTAs that become resident in the order in which SMs fall free, instead of all at once, run
-    // longer there than the overlap saves (48 heads x 2K bf16 60.5 -> 62.6 us).
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(512);
-    cfg.dynamicSmemBytes = W::kSmemBytes;
-    cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = items <= sm_count ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, tq, tk, tv, p);
-}
-
 template <int D, int IN>
 static cudaError_t dispatch_mode(int mode, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                  const AttnParams& p, cudaStream_t stream) {
