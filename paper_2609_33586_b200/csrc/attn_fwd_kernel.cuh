@@ -18,8 +18,9 @@
 // While warpgroup 0 works on S_0(j), the tensor cores compute P_1 V(j-1) and S_1(j), and vice versa.
 // Split form (SPLIT): when there are fewer items than SMs a cluster of CTAs shares an item, each taking a contiguous part
 // of its key tiles.  Every part must start with the anchor the sequential loop would have reached there, so for the rounding
-// maps the cluster first goes over all parts but the last for the row maxima alone (Q K^T and a maximum, a quarter of a
-// full step); exact-like modes need no such pass, their result does not depend on the anchor.  At the end each CTA leaves
+// maps the cluster first goes over all parts but the last for the row maxima alone (Q K^T and a maximum, two thirds of a
+// full step).  Exact-like modes on 16-bit inputs need no such pass; on fp8 inputs the rounding of P to e4m3 depends on the
+// anchor, and the result should not depend on the split.  At the end each CTA leaves
 // O, l and its anchor in shared memory and adds up its share of the rows over the cluster.
 // TMEM columns: S_0/P_0 [0,128), S_1/P_1 [128,256), O_0 [256,384), O_1 [384,512).
 #pragma once
@@ -29,6 +30,8 @@ namespace rowmax {
 
 namespace {
 
+// Whether the parts of a split item need the row maxima of the parts before them.
+__host__ __device__ constexpr bool split_takes_maxima(int mode, bool fp8) { return fp8 || !is_exact_like(mode); }
 constexpr int kMaxSplit = 8;   // CTAs that share an item (the portable cluster size)
 
 template <int D, bool FP8, bool SPLIT = false>
@@ -147,7 +150,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     using W = WsCfg<D, FP8, SPLIT>;
     constexpr int NS = W::kSlots;
     constexpr bool kOutOfStep = FP8 && is_exact_like(MODE);   // keep the softmax warpgroups apart (see below)
-    constexpr bool kPre = SPLIT && !is_exact_like(MODE);   // row maxima of the part first
+    constexpr bool kPre = SPLIT && split_takes_maxima(MODE, FP8);   // row maxima of the part first
     // Declared with the alignment that the swizzled tiles need: all shared-memory addresses are then constants, not
     // registers, of which the softmax warps have none to spare (checked below).
     extern __shared__ __align__(1024) uint8_t smem[];

@@ -43,7 +43,7 @@ struct SplitLauncher {
         return known[dev][parts] > 0 ? known[dev][parts] : 0;
     }
     // CTAs per item, 1 for the plain form.  Times are in steps of the loop (one key tile of a pair of query tiles), measured:
-    // a part costs its key tiles, with the rounding maps 0.65 of a step more for each tile of its maxima pass (two parts share
+    // a part costs its key tiles, with a maxima pass 0.65 of a step more for each tile of its maxima pass (two parts share
     // the pass, so it is half as long), and 4.5 steps + 0.5 per part for the exchange and the sum of O; all SMs working slow
     // each other by a tenth.  512 queries on 16K, 32/8 heads: bf16 h15 198 -> 154 us, exact 226 -> 138, e4m3 178 -> 125
     // (2 parts); 64 queries on 8K 97 -> 49 (4 parts).  16 x 1K and 16 x 2K gain nothing and stay whole.
@@ -64,7 +64,7 @@ struct SplitLauncher {
         for (int parts = 2; parts <= kMaxSplit && parts <= all; ++parts) {
             const int n = fit(dev, parts);
             if (n <= 0) continue;
-            const double per_tile = (is_exact_like(MODE) ? 1.0 : parts == 2 ? 1.325 : 1.65) / parts;
+            const double per_tile = (!split_takes_maxima(MODE, IN == kInFP8) ? 1.0 : parts == 2 ? 1.325 : 1.65) / parts;
             const double fixed = 4.5 + 0.5 * parts, busy = items * parts > 100.0 ? 1.1 : 1.0;
             const double waves = ceil(items / n);
             const double t = fmax(longest * per_tile + fixed, waves * (mean * per_tile + fixed)) * busy;
