@@ -16,6 +16,12 @@
 //   warp 12        MMA issuer (one thread): S_t = Q_t K^T and O_t += P_t V on the tensor cores
 //   warp 13        TMA producer (one thread): Q per item, K/V through a ring of shared-memory slots
 // While warpgroup 0 works on S_0(j), the tensor cores compute P_1 V(j-1) and S_1(j), and vice versa.
+//
+// What bounds it: at 16 bits the MMA warp.  Issuing blocks until the tensor cores take the instruction (eight bf16 MMAs of
+// 128 x 128 x 16: 520 clocks), and every barrier it waits for costs 100 to 150 clocks even when it is ready, in which the tensor
+// cores idle; so P and the rescaled O share a barrier, V(j) and K(j + 1) share theirs, and O is committed once per item
+// (bf16 8K h15 267 -> 247 us).  At fp8 the chain of one softmax warpgroup (about 1500 clocks of work, 1000 until its next
+// scores are there).
 // Split form (SPLIT): when there are fewer items than SMs a cluster of CTAs shares an item, each taking a contiguous part
 // of its key tiles.  Every part must start with the anchor the sequential loop would have reached there, so for the rounding
 // maps the cluster first goes over all parts but the last for the row maxima alone (Q K^T and a maximum, two thirds of a
@@ -42,7 +48,7 @@ struct WsCfg {
     static constexpr int kRingBytes = kSlots * C::kTileBytes;
     static constexpr int kScaleOff = kQBytes + kRingBytes;        // float alpha[2][128]
     static constexpr int kBarOff = kScaleOff + 2 * 128 * 4;
-    static constexpr int kNumBars = 2 * kSlots + 8 * 2 + 1 + (SPLIT ? 4 + 2 + 3 : 0);
+    static constexpr int kNumBars = 2 * kSlots + 7 * 2 + 1 + (SPLIT ? 4 + 2 + 3 : 0);
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     // split form: row maxima of the parts before this one, [part][256]; anchor and row sum of this part, [256][2]; weights of
     // the parts for the rows this CTA adds up, [part][rows]
@@ -76,8 +82,9 @@ template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setma
 #endif
 
 constexpr int kBarSelftest = 0x7F;
+constexpr int kBarAlign = 0x7E;      // not a barrier: the shared memory of the launch is not aligned as declared
 enum BarId : int { kBarQFull = 0, kBarQEmpty = 1, kBarKvFull = 2, kBarKvEmpty = 3, kBarSFull = 4, kBarPFull = 5,
-                   kBarOFull = 6, kBarScale = 7, kBarORescaled = 8, kBarOFree = 9,
+                   kBarOFull = 6, kBarScale = 7, kBarOFree = 9,
                    kBarSFree = 10, kBarXmax = 11, kBarPart = 12, kBarItem = 13 };
 
 // One work item = two query tiles of 128 rows of one (batch, head).
@@ -175,22 +182,21 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     auto bar_q_full = [&](int t) { return bar_x(0, t); };      // TMA -> MMA: Q_t of the current item landed
     auto bar_q_empty = [&](int t) { return bar_x(1, t); };     // MMA -> TMA: last S_t MMA of the item done
     auto bar_s_full = [&](int t) { return bar_x(2, t); };      // MMA -> softmax: S_t(j) is in TMEM
-    auto bar_p_full = [&](int t) { return bar_x(3, t); };      // softmax -> MMA: P_t(j) is in TMEM
+    auto bar_p_full = [&](int t) { return bar_x(3, t); };      // softmax and correction -> MMA: P_t(j) is in TMEM, O_t rescaled
     auto bar_o_full = [&](int t) { return bar_x(4, t); };      // MMA -> epilogue: the last P_t V of the item accumulated
     auto bar_scale = [&](int t) { return bar_x(5, t); };       // softmax -> correction: alpha_t(j) in smem
-    auto bar_o_rescaled = [&](int t) { return bar_x(6, t); };  // correction -> MMA: O_t rescaled for tile j
-    auto bar_o_free = [&](int t) { return bar_x(7, t); };      // epilogue -> MMA: O_t has been read out
-    const uint32_t bar_drain = bar0 + 8u * (2 * NS + 16);      // abort path only: the MMA warp's last commit
+    auto bar_o_free = [&](int t) { return bar_x(6, t); };      // epilogue -> MMA: O_t has been read out
+    const uint32_t bar_drain = bar0 + 8u * (2 * NS + 14);      // abort path only: the MMA warp's last commit
     // split form.  The maxima pass has two score buffers per query tile: S_t and, as O_t is not in use yet, O_t.
-    auto bar_s_free = [&](int t, int b) { return bar0 + 8u * (2 * NS + 17 + 2 * b + t); };   // softmax -> MMA: buffer b of tile t has been read
-    auto bar_s_full2 = [&](int t) { return bar0 + 8u * (2 * NS + 21 + t); };                  // MMA -> softmax: scores in buffer 1 of tile t
-    const uint32_t bar_xmax = bar0 + 8u * (2 * NS + 23);       // the maxima of all parts before this one are here
-    const uint32_t bar_item = bar0 + 8u * (2 * NS + 24);       // MMA -> softmax: all products of the item are complete
-    const uint32_t bar_part = bar0 + 8u * (2 * NS + 25);       // all parts have left O, l and anchor
+    auto bar_s_free = [&](int t, int b) { return bar0 + 8u * (2 * NS + 15 + 2 * b + t); };   // softmax -> MMA: buffer b of tile t has been read
+    auto bar_s_full2 = [&](int t) { return bar0 + 8u * (2 * NS + 19 + t); };                  // MMA -> softmax: scores in buffer 1 of tile t
+    const uint32_t bar_xmax = bar0 + 8u * (2 * NS + 21);       // the maxima of all parts before this one are here
+    const uint32_t bar_item = bar0 + 8u * (2 * NS + 22);       // MMA -> softmax: all products of the item are complete
+    const uint32_t bar_part = bar0 + 8u * (2 * NS + 23);       // all parts have left O, l and anchor
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
     if ((smem_u32(smem) & 1023u) != 0) {
-        if (tid == 0) atomicCAS(p.status, 0, (kRoleSerial << 8) | kBarSelftest);
+        if (tid == 0) atomicCAS(p.status, 0, (kRoleSetup << 8) | kBarAlign);
         return;
     }
     // The status word is sticky: once a wait has expired (in an earlier launch, or in another CTA of this one) and
@@ -814,13 +820,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 #pragma unroll
                         for (int u = 0; u < kBatch; ++u) {
                             const int e = e0 + 256 * u, prow = row_lo + e / kPieces, piece = e % kPieces;
-                            if (e < n_rows * kPieces)
+                            if (e < n_rows * kPieces && (prow < 128 ? it.q0[0] : it.q0[1]) + (prow & 127) < p.Sq)
                                 v[u] = ld_cluster_f32x4(mapa(smem_u32(smem) + prow * (D * 4) + ((piece ^ (prow & (kPieces - 1))) << 4), q));
                         }
 #pragma unroll
                         for (int u = 0; u < kBatch; ++u) {
-                            const int e = e0 + 256 * u;
-                            const float wq = e < n_rows * kPieces ? weight[q * n_rows + e / kPieces] : 0.f;
+                            const int e = e0 + 256 * u, prow = row_lo + e / kPieces;
+                            const bool wanted = e < n_rows * kPieces && (prow < 128 ? it.q0[0] : it.q0[1]) + (prow & 127) < p.Sq;
+                            const float wq = wanted ? weight[q * n_rows + e / kPieces] : 0.f;
                             if (wq > 0.f) {      // a part that weighs nothing has not written O
                                 acc[u].x = fmaf(wq, v[u].x, acc[u].x);
                                 acc[u].y = fmaf(wq, v[u].y, acc[u].y);
