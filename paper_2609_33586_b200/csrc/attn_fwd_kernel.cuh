@@ -63,8 +63,10 @@ struct WsCfg {
 
 // Register split of the 512 threads x 128 registers the CTA is launched with (setmaxnreg can only
 // redistribute that allocation; a larger total would make the increase wait for ever): softmax /
-// correction / MMA+TMA warpgroups.
-constexpr int kRegSoftmax = 192, kRegCorr = 80, kRegMma = 48;
+// correction / MMA+TMA warpgroups.  The softmax warps hold a row of 128 scores; what decides is that no role spills: with
+// 192 / 80 / 48 and a correction that took 32 columns at a time the 16-bit instances spilled in the MMA and correction
+// warps (bf16 8K exact 277.6 against 267.5 us, full-attention fp8 exact 420 against 410); 208 / 48 / 48 spills again (287).
+constexpr int kRegSoftmax = 200, kRegCorr = 56, kRegMma = 56;
 static_assert(256 * kRegSoftmax + 128 * kRegCorr + 128 * kRegMma <= 512 * 128, "setmaxnreg targets exceed the launch allocation");
 template <int N> __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
@@ -507,18 +509,17 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             tc_fence_after();
                             if (__any_sync(0xffffffffu, alpha != 1.0f)) {
 #pragma unroll
-                                for (int cc = 0; cc < D / 32; ++cc) {
-                                    uint32_t o[32];
-                                    tmem_ld32(tmem_O(t) + lane_base + cc * 32, o);
+                                for (int cc = 0; cc < D / 16; ++cc) {
+                                    uint32_t o[16];
+                                    tmem_ld16(tmem_O(t) + lane_base + cc * 16, o);
                                     tmem_wait_ld();
 #pragma unroll
-                                    for (int i = 0; i < 32; i += 2) {
-                                        const float2 v = fmul2(make_float2(__uint_as_float(o[i]), __uint_as_float(o[i + 1])),
-                                                               make_float2(alpha, alpha));
+                                    for (int i = 0; i < 16; i += 2) {
+                                        const float2 v = fmul2(make_float2(__uint_as_float(o[i]), __uint_as_float(o[i + 1])), make_float2(alpha, alpha));
                                         o[i] = __float_as_uint(v.x);
                                         o[i + 1] = __float_as_uint(v.y);
                                     }
-                                    tmem_st32(tmem_O(t) + lane_base + cc * 32, o);
+                                    tmem_st16(tmem_O(t) + lane_base + cc * 16, o);
                                 }
                                 tmem_wait_st();
                             }
