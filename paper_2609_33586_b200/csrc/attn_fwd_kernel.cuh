@@ -287,7 +287,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             int kv_idx = 0;             // K/V tiles loaded so far (ring position), over all items
             mbar_arrive(bar_kv_full(0));   // the first pair has no V
             int q_use[2] = {0, 0};      // items that used Q buffer t so far
-            for (int round = 0;; ++round) {
+            for (int round = 0; !SPLIT || round < 1; ++round) {   // split form: one item per cluster
                 const int w = item_index(round, cta, n_ctas);
                 if (w >= n_items || flag_is_set(abort_at)) break;
                 const WorkItem it = get_item(w);
@@ -378,7 +378,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             int kv_base = 0;            // ring index of K_0 of the current item
             int tiles[2] = {0, 0};      // key tiles of query tile t finished in earlier items (barrier phases)
             int q_use[2] = {0, 0};      // items that used Q buffer / O accumulator t so far
-            for (int round = 0;; ++round) {
+            for (int round = 0; !SPLIT || round < 1; ++round) {   // split form: one item per cluster
                 const int w = item_index(round, cta, n_ctas);
                 if (w >= n_items) break;
                 const WorkItem it = get_item(w);
@@ -490,7 +490,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const int r = tid & 127;
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
         int tiles[2] = {0, 0};
-        for (int round = 0;; ++round) {
+        for (int round = 0; !SPLIT || round < 1; ++round) {   // split form: one item per cluster
             const int w = item_index(round, cta, n_ctas);
             if (w >= n_items) break;
             const WorkItem it = get_item(w);
@@ -553,7 +553,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         constexpr bool kSatForm = kLattice && !TAU;
         int tiles = 0;
         int o_use = 0;      // items with key tiles so far
-        for (int round = 0;; ++round) {
+        for (int round = 0; !SPLIT || round < 1; ++round) {   // split form: one item per cluster
             const int w = item_index(round, cta, n_ctas);
             if (w >= n_items) break;
             const WorkItem it = get_item(w);
