@@ -48,7 +48,7 @@ struct WsCfg {
     static constexpr int kRingBytes = kSlots * C::kTileBytes;
     static constexpr int kScaleOff = kQBytes + kRingBytes;        // float alpha[2][128]
     static constexpr int kBarOff = kScaleOff + 2 * 128 * 4;
-    static constexpr int kNumBars = 2 * kSlots + 7 * 2 + 1 + (SPLIT ? 4 + 2 + 3 : 0);
+    static constexpr int kNumBars = 2 * kSlots + 7 * 2 + 1 + (SPLIT ? 2 + 2 + 3 : 0);
     static constexpr int kMiscOff = kBarOff + kNumBars * 8;
     // split form: row maxima of the parts before this one, [part][256]; anchor and row sum of this part, [256][2]; weights of
     // the parts for the rows this CTA adds up, [part][rows]
@@ -189,12 +189,13 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     auto bar_scale = [&](int t) { return bar_x(5, t); };       // softmax -> correction: alpha_t(j) in smem
     auto bar_o_free = [&](int t) { return bar_x(6, t); };      // epilogue -> MMA: O_t has been read out
     const uint32_t bar_drain = bar0 + 8u * (2 * NS + 14);      // abort path only: the MMA warp's last commit
-    // split form.  The maxima pass has two score buffers per query tile: S_t and, as O_t is not in use yet, O_t.
-    auto bar_s_free = [&](int t, int b) { return bar0 + 8u * (2 * NS + 15 + 2 * b + t); };   // softmax -> MMA: buffer b of tile t has been read
-    auto bar_s_full2 = [&](int t) { return bar0 + 8u * (2 * NS + 19 + t); };                  // MMA -> softmax: scores in buffer 1 of tile t
-    const uint32_t bar_xmax = bar0 + 8u * (2 * NS + 21);       // the maxima of all parts before this one are here
-    const uint32_t bar_item = bar0 + 8u * (2 * NS + 22);       // MMA -> softmax: all products of the item are complete
-    const uint32_t bar_part = bar0 + 8u * (2 * NS + 23);       // all parts have left O, l and anchor
+    // split form.  The maxima pass has two score buffers per query tile: S_t and, as O_t is not in use yet, O_t; the two tiles
+    // go through it together (one wait and one commit for both; 512 queries on 16K, bf16 h15: 147 -> 142 us).
+    auto bar_pre_free = [&](int b) { return bar0 + 8u * (2 * NS + 15 + b); };   // softmax -> MMA: buffer b of both tiles has been read
+    auto bar_pre_full = [&](int b) { return bar0 + 8u * (2 * NS + 17 + b); };   // MMA -> softmax: scores of both tiles in buffer b
+    const uint32_t bar_xmax = bar0 + 8u * (2 * NS + 19);       // the maxima of all parts before this one are here
+    const uint32_t bar_item = bar0 + 8u * (2 * NS + 20);       // MMA -> softmax: all products of the item are complete
+    const uint32_t bar_part = bar0 + 8u * (2 * NS + 21);       // all parts have left O, l and anchor
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
     if ((smem_u32(smem) & 1023u) != 0) {
@@ -233,9 +234,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         } else if (lane == 18) {
             mbar_init(bar_drain, 1);
         } else if (SPLIT && lane == 19) {
-            for (int i = 0; i < 4; ++i) mbar_init(bar_s_free(i & 1, i >> 1), 4);   // one arrival per softmax warp
-            mbar_init(bar_s_full2(0), 1);
-            mbar_init(bar_s_full2(1), 1);
+            for (int i = 0; i < 2; ++i) {
+                mbar_init(bar_pre_free(i), 8);      // one arrival per softmax warp of both tiles
+                mbar_init(bar_pre_full(i), 1);
+            }
             mbar_init(bar_item, 1);
             mbar_init(bar_xmax, rank > 0 ? 8 * rank : 1);   // one per softmax warp of each part before
             mbar_init(bar_part, 8 * parts);   // one per softmax warp of every part
@@ -386,37 +388,40 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     const int pre_max = max(it.pre_n[0], it.pre_n[1]);
                     for (int j = 0; j < pre_max; ++j) {
                         if (kv_base == 0 || (kv_base & 1)) mbar_wait_poll(bar_kv_full(kv_base), ph_kv_full(kv_base), wctx, (kRoleMma << 8) | kBarKvFull);
+                        const int buf = j & 1;
+                        if (j == 0) {
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {
-                            if (j < it.pre_n[t]) {
-                                const int buf = j & 1;
-                                if (j == 0) mbar_wait(bar_q_full(t), q_use[t] & 1, wctx, (kRoleMma << 8) | kBarQFull);
-                                if (j >= 2) mbar_wait_poll(bar_s_free(t, buf), (j / 2 - 1) & 1, wctx, (kRoleMma << 8) | kBarSFree);
-                                tc_fence_after();
-                                if (leader) {
-                                    if (!flag_is_set(abort_at)) issue_s(t, ring_lo_k + slot_lo(kv_base), buf == 0 ? tmem_S(t) : tmem_O(t));
-                                    umma_commit(buf == 0 ? bar_s_full(t) : bar_s_full2(t));
-                                }
+                            for (int t = 0; t < 2; ++t)
+                                if (it.pre_n[t] > 0) mbar_wait(bar_q_full(t), q_use[t] & 1, wctx, (kRoleMma << 8) | kBarQFull);
+                        }
+                        if (j >= 2) mbar_wait_poll(bar_pre_free(buf), (j / 2 - 1) & 1, wctx, (kRoleMma << 8) | kBarSFree);
+                        tc_fence_after();
+                        if (leader) {
+                            if (!flag_is_set(abort_at)) {
+#pragma unroll
+                                for (int t = 0; t < 2; ++t)
+                                    if (j < it.pre_n[t]) issue_s(t, ring_lo_k + slot_lo(kv_base), buf == 0 ? tmem_S(t) : tmem_O(t));
                             }
+                            umma_commit(bar_pre_full(buf));
                         }
                         if (leader && (kv_base & 1) == 0) umma_commit(bar_kv_empty(kv_base));
                         __syncwarp();
                         ++kv_base;
                     }
                     kv_base += kv_base & 1;
+                    if (pre_max > 0) {     // both buffers have been read: their last uses
+                        const int last = pre_max - 1;
+                        mbar_wait_poll(bar_pre_free(last & 1), (last / 2) & 1, wctx, (kRoleMma << 8) | kBarSFree);
+                        if (last > 0) mbar_wait_poll(bar_pre_free((last - 1) & 1), ((last - 1) / 2) & 1, wctx, (kRoleMma << 8) | kBarSFree);
+                    }
                 }
                 if (it.n_max > 0) {
                     wait_full(kv_base);
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
                         if (it.n[t] > 0) {
-                            if (kPre && it.pre_n[t] > 0) {   // both buffers have been read: their last uses
-                                const int last = it.pre_n[t] - 1;
-                                mbar_wait_poll(bar_s_free(t, last & 1), (last / 2) & 1, wctx, (kRoleMma << 8) | kBarSFree);
-                                if (last > 0) mbar_wait_poll(bar_s_free(t, (last - 1) & 1), ((last - 1) / 2) & 1, wctx, (kRoleMma << 8) | kBarSFree);
-                            } else {
+                            if (!kPre || it.pre_n[t] == 0)
                                 mbar_wait(bar_q_full(t), q_use[t] & 1, wctx, (kRoleMma << 8) | kBarQFull);
-                            }
                             // spread the two tiles' weight phases apart from the start (D = 64: 199 -> 190 us at 8K)
                             if (kOutOfStep && round == 0 && t == 1 && it.n[0] > 0)
                                 mbar_wait(bar_p_full(0), 0, wctx, (kRoleMma << 8) | kBarPFull);
@@ -565,44 +570,35 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             const int tile_limit = p.causal ? min(p.Sk, q0 + shift + 1) : p.Sk;
             const int j0 = SPLIT ? it.j0 : 0;
             float m_run = -INFINITY, l_run = 0.f;
-            // h15 family at fp8: a lower bound of every raw score of this row that costs nothing per score.
-            // |q . k| <= (sum_i |q_i|) * max_i |k_i| and an e4m3 key element is at most 448 in magnitude, so
-            // s >= -448 * sum_i |q_i|.  When that bound already keeps the scaled offsets of a tile above the
-            // clamp, the tile needs neither the row-minimum pass nor the clamped variant.  The row of Q is
-            // read from shared memory (a sum does not care about the swizzle, which stays within the row), which
-            // is safe while S_t(1) has not been issued, i.e. for items with at least two key tiles (used from four on).
-            float score_floor = -INFINITY;
-            if constexpr (FP8 && kFam > 0) {
-                if (nt >= 4) {   // the sum costs about three row-minimum passes
-                    mbar_wait(bar_s_full(t), tiles & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);   // Q_t has landed
-                    score_floor = -448.0f * 1.02f * abs_sum_e4m3_row<D / 16>(sQ + t * C::kTileBytes + r * D);
-                }
-            }
-            const int pre_n = !kPre ? 0 : t == 0 ? it.pre_n[0] : it.pre_n[1];
             if constexpr (kPre) {
                 // the row's maxima; those over the parts before this one are the anchor to start from
+                const int pre_n = t == 0 ? it.pre_n[0] : it.pre_n[1], pre_max = max(it.pre_n[0], it.pre_n[1]);
                 float m_part = -INFINITY;
-                for (int j = 0; j < pre_n; ++j) {
+                for (int j = 0; j < pre_max; ++j) {
                     const int buf = j & 1;
-                    mbar_wait_poll(buf == 0 ? bar_s_full(t) : bar_s_full2(t), (j / 2) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
+                    mbar_wait_poll(bar_pre_full(buf), (j / 2) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
                     __syncwarp();
                     tc_fence_after();
                     uint32_t s[4][32];
+                    if (j < pre_n) {
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) tmem_ld32((buf == 0 ? tS : tO) + cc * 32, s[cc]);
-                    tmem_wait_ld();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_s_free(t, buf));
-                    if ((it.pre_j0 + j + 1) * kTileN > tile_limit) {
-                        const int col_limit = row_limit - (it.pre_j0 + j) * kTileN;
-#pragma unroll
-                        for (int cc = 0; cc < 4; ++cc)
-#pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                if (cc * 32 + i >= col_limit) s[cc][i] = __float_as_uint(-INFINITY);
+                        for (int cc = 0; cc < 4; ++cc) tmem_ld32((buf == 0 ? tS : tO) + cc * 32, s[cc]);
+                        tmem_wait_ld();
+                        tc_fence_before();
                     }
-                    m_part = fmaxf(m_part, row_max128(s));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_pre_free(buf));
+                    if (j < pre_n) {
+                        if ((it.pre_j0 + j + 1) * kTileN > tile_limit) {
+                            const int col_limit = row_limit - (it.pre_j0 + j) * kTileN;
+#pragma unroll
+                            for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+                                for (int i = 0; i < 32; ++i)
+                                    if (cc * 32 + i >= col_limit) s[cc][i] = __float_as_uint(-INFINITY);
+                        }
+                        m_part = fmaxf(m_part, row_max128(s));
+                    }
                 }
                 const uint32_t xmax = smem_u32(smem + W::kXmaxOff) + (t * 128 + r) * 4;
                 for (int q = rank + 1; q < parts; ++q) st_cluster_f32(mapa(xmax + rank * 1024, q), m_part);
@@ -616,8 +612,21 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         m_run = fmaxf(m_run, *reinterpret_cast<const volatile float*>(smem + W::kXmaxOff + q * 1024 + (t * 128 + r) * 4));
                 }
             }
+            // h15 family at fp8: a lower bound of every raw score of this row that costs nothing per score.
+            // |q . k| <= (sum_i |q_i|) * max_i |k_i| and an e4m3 key element is at most 448 in magnitude, so
+            // s >= -448 * sum_i |q_i|.  When that bound already keeps the scaled offsets of a tile above the
+            // clamp, the tile needs neither the row-minimum pass nor the clamped variant.  The row of Q is
+            // read from shared memory (a sum does not care about the swizzle, which stays within the row), which
+            // is safe while S_t(1) has not been issued, i.e. for items with at least two key tiles (used from four on).
+            float score_floor = -INFINITY;
+            if constexpr (FP8 && kFam > 0) {
+                if (nt >= 4) {   // the sum costs about three row-minimum passes
+                    mbar_wait(bar_s_full(t), tiles & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);   // Q_t has landed
+                    score_floor = -448.0f * 1.02f * abs_sum_e4m3_row<D / 16>(sQ + t * C::kTileBytes + r * D);
+                }
+            }
             for (int j = 0; j < nt; ++j) {
-                mbar_wait(bar_s_full(t), (tiles + (kPre ? (pre_n + 1) / 2 : 0) + j) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
+                mbar_wait(bar_s_full(t), (tiles + j) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
                 if (r == 0) ROWMAX_STAMP(t, j, 0);
                 __syncwarp();
                 tc_fence_after();
