@@ -921,7 +921,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
 #ifdef ROWMAX_TRACE
     if (tid == 0 && p.trace != nullptr && p.trace_block < 0) p.trace[blockIdx.x] = clock64() - trace_t0;   // per-CTA busy time
 #endif
-    if (warp == 12) tmem_dealloc(tmem, kTmemCols);
+    if (warp == 12) {
+        __syncwarp();      // the lanes leave the bounded wait on bar_drain each by itself, and this wants the whole warp
+        tmem_dealloc(tmem, kTmemCols);
+    }
 }
 
 // Launches the plain form.
