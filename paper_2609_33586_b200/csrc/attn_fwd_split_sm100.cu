@@ -15,10 +15,11 @@ struct SplitLauncher {
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = parts;
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_ws
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        // No programmatic dependent launch, as a precaution: its gain is small if any (512 queries on 16K, bf16 h15, stream of 300
+        // calls: 161.9 us with it and 159.9 without in one call; 166.5 without on another machine, where graph replays were
+        // 3 % slower too).
         cfg.attrs = attr;
-        cfg.numAttrs = 2;
+        cfg.numAttrs = 1;
         cfg.blockDim = dim3(512);
         cfg.dynamicSmemBytes = W::kSmemBytes;
     }
@@ -28,9 +29,8 @@ struct SplitLauncher {
         if (known[dev][parts] == 0) {
             auto kern = attn_fwd_ws_kernel<D, IN, MODE, true>;
             cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute attr[2];
+            cudaLaunchAttribute attr[1];
             configure(cfg, attr, parts);
-            cfg.numAttrs = 1;
             cfg.gridDim = dim3(parts);
             int n = 0;
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmemBytes) != cudaSuccess ||
@@ -78,7 +78,7 @@ struct SplitLauncher {
         if (items * parts > 0x7fffffffLL) return cudaErrorInvalidValue;
         p.split = parts;
         cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[2];
+        cudaLaunchAttribute attr[1];
         configure(cfg, attr, parts);
         cfg.gridDim = dim3(static_cast<unsigned>(items * parts));     // one item per cluster, heaviest first
         cfg.stream = stream;
