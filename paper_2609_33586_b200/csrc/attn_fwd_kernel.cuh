@@ -30,6 +30,7 @@
 // O, l and its anchor in shared memory and adds up its share of the rows over the cluster.
 // TMEM columns: S_0/P_0 [0,128), S_1/P_1 [128,256), O_0 [256,384), O_1 [384,512).
 #pragma once
+#include "kv_ring.cuh"
 #include "softmax_math.cuh"
 
 namespace rowmax {
@@ -172,14 +173,13 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const WaitCtx wctx{abort_at, p.status, kWaitLimitCycles};
 
     // barrier addresses
-    // Ring positions count tiles: K(0), V(0), K(1), V(1), ... over all items.  V(j) and K(j + 1), positions 2i - 1 and 2i, share
-    // their barriers: the MMA warp needs both at once and is done with both at once, and every barrier that it waits for or
-    // commits to is time in which the tensor cores idle.  (The last V of an item goes with the first K of the next.)
-    constexpr int NP = NS / 2;
-    auto bar_kv_full = [&](int idx) { return bar0 + 8u * (((idx + 1) >> 1) % NP); };
-    auto bar_kv_empty = [&](int idx) { return bar0 + 8u * (NS + ((idx + 1) >> 1) % NP); };
-    auto ph_kv_full = [&](int idx) { return (((idx + 1) >> 1) / NP) & 1; };
-    auto ph_kv_empty = [&](int idx) { return ph_kv_full(idx) ^ 1; };
+    // ring positions, pairs of them and the order of waits and arrivals: kv_ring.cuh
+    using Ring = KvRing<NS>;
+    constexpr int NP = Ring::kPairs;
+    auto bar_kv_full = [&](int idx) { return bar0 + 8u * Ring::bar(idx); };
+    auto bar_kv_empty = [&](int idx) { return bar0 + 8u * (NS + Ring::bar(idx)); };
+    auto ph_kv_full = [&](int idx) { return Ring::ph_full(idx); };
+    auto ph_kv_empty = [&](int idx) { return Ring::ph_empty(idx); };
     auto bar_x = [&](int which, int t) { return bar0 + 8u * (2 * NS + 2 * which + t); };
     auto bar_q_full = [&](int t) { return bar_x(0, t); };      // TMA -> MMA: Q_t of the current item landed
     auto bar_q_empty = [&](int t) { return bar_x(1, t); };     // MMA -> TMA: last S_t MMA of the item done
@@ -286,63 +286,53 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         reg_dec<kRegMma>();
         if (warp == 13 && lane == 0) {
             // ------------------------------------------------------------ TMA producer
-            int kv_idx = 0;             // K/V tiles loaded so far (ring position), over all items
-            mbar_arrive(bar_kv_full(0));   // the first pair has no V
+            int kv_idx = 0;             // ring position: K/V tiles loaded so far, over all items
             int q_use[2] = {0, 0};      // items that used Q buffer t so far
+            WorkItem it;
+            auto load_tile = [&](const CUtensorMap* tm, uint32_t dst, uint32_t bar, int head, int row0) {
+                mbar_arrive_expect_tx(bar, C::kTileBytes);
+#pragma unroll
+                for (int bx = 0; bx < C::kBoxes; ++bx)
+                    tma_load_4d(dst + bx * C::kBoxBytes, tm, bar, bx * C::kBoxElems, head, row0, it.b);
+            };
+            auto load_kv = [&](const CUtensorMap* tm, int idx, int tile) {
+                load_tile(tm, sRing + (idx % NS) * C::kTileBytes, bar_kv_full(idx), it.hk, tile * kTileN);
+            };
+            // After an expired wait nothing more is loaded: a wait then returns at once, and a copy into a buffer
+            // whose last copy may still be under way would leave more in flight than the waits below account for.
+            auto load_q = [&](int t) {
+                if (it.n[t] > 0 || (kPre && it.pre_n[t] > 0)) {
+                    mbar_wait(bar_q_empty(t), (q_use[t] & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarQEmpty);
+                    if (flag_is_set(abort_at)) return false;
+                    load_tile(&tmQ, sQ + t * C::kTileBytes, bar_q_full(t), it.h, it.q0[t]);
+                    ++q_use[t];
+                }
+                return true;
+            };
+            KvOps ops{[&](int idx) { mbar_arrive(bar_kv_full(idx)); },
+                      [&](int idx) {
+                          if constexpr (SPLIT) mbar_wait_poll(bar_kv_empty(idx), ph_kv_empty(idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
+                          else mbar_wait(bar_kv_empty(idx), ph_kv_empty(idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
+                          return !flag_is_set(abort_at);
+                      },
+                      [&](int idx, int j) { load_kv(&tmK, idx, it.j0 + j); },
+                      [&](int idx, int j) { load_kv(&tmV, idx, it.j0 + j); },
+                      [&](int idx, int j) { load_kv(&tmK, idx, it.pre_j0 + j); },
+                      [&]() { return load_q(0) && load_q(1); }};
+            kv_begin(ops);
             for (int round = 0; !SPLIT || round < 1; ++round) {   // split form: one item per cluster
                 const int w = item_index(round, cta, n_ctas);
-                if (w >= n_items || flag_is_set(abort_at)) break;
-                const WorkItem it = get_item(w);
-                auto load_tile = [&](const CUtensorMap* tm, uint32_t dst, uint32_t bar, int head, int row0) {
-                    mbar_arrive_expect_tx(bar, C::kTileBytes);
-#pragma unroll
-                    for (int bx = 0; bx < C::kBoxes; ++bx)
-                        tma_load_4d(dst + bx * C::kBoxBytes, tm, bar, bx * C::kBoxElems, head, row0, it.b);
-                };
-                // After an expired wait nothing more is loaded: a wait then returns at once, and a copy into a buffer
-                // whose last copy may still be under way would leave more in flight than the waits below account for.
-                auto load_q = [&](int t) {
-                    if (it.n[t] > 0 || (kPre && it.pre_n[t] > 0)) {
-                        mbar_wait(bar_q_empty(t), (q_use[t] & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarQEmpty);
-                        if (flag_is_set(abort_at)) return;
-                        load_tile(&tmQ, sQ + t * C::kTileBytes, bar_q_full(t), it.h, it.q0[t]);
-                        ++q_use[t];
-                    }
-                };
+                if (w >= n_items) break;
+                it = get_item(w);
                 if (round == 0) ROWMAX_STAMP(3, 63, 0);
-                // K first: the last P V of the item before waits for it along with its V; then Q, once its buffers are free
-                const int pre_max = kPre ? max(it.pre_n[0], it.pre_n[1]) : 0;
-                auto load_kv = [&](const CUtensorMap* tm, int tile) {
-                    if constexpr (SPLIT) mbar_wait_poll(bar_kv_empty(kv_idx), ph_kv_empty(kv_idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
-                    else mbar_wait(bar_kv_empty(kv_idx), ph_kv_empty(kv_idx), wctx, (kRoleLoad << 8) | kBarKvEmpty);
-                    if (flag_is_set(abort_at)) return;
-                    load_tile(tm, sRing + (kv_idx % NS) * C::kTileBytes, bar_kv_full(kv_idx), it.hk, tile * kTileN);
-                    ++kv_idx;
-                };
-                if constexpr (kPre) {
-                    for (int j = 0; j < pre_max && !flag_is_set(abort_at); ++j) {
-                        load_kv(&tmK, it.pre_j0 + j);
-                        if (j == 0) { load_q(0); load_q(1); }
-                    }
-                    if (kv_idx & 1) {     // an odd number of tiles: the position that V would have stays empty
-                        mbar_arrive(bar_kv_full(kv_idx));
-                        ++kv_idx;
-                    }
-                }
-                for (int j = 0; j < it.n_max && !flag_is_set(abort_at); ++j) {
-                    load_kv(&tmK, it.j0 + j);
-                    if (pre_max == 0 && j == 0) { load_q(0); load_q(1); }
-                    if (flag_is_set(abort_at)) break;
-                    load_kv(&tmV, it.j0 + j);
-                }
+                if (!kv_item<kPre>(ops, kv_idx, kPre ? max(it.pre_n[0], it.pre_n[1]) : 0, it.n_max)) break;
             }
-            // the last pair is complete without a K
-            mbar_arrive(bar_kv_full(kv_idx));
+            kv_end(ops, kv_idx);
             // Before the CTA ends every load this thread issued must have landed.  Normally the consumers have
             // seen to that and these waits return at once; after an expired wait they may have stopped waiting while
             // copies were still writing shared memory, so wait (bounded) for the last use of every pair of ring slots and
             // Q buffer.
-            for (int idx = kv_idx >= NS ? kv_idx - NS + 1 : 0; idx < kv_idx; ++idx)
+            for (int idx = kv_drain_from<NS>(kv_idx); idx < kv_idx; ++idx)
                 mbar_wait_quiet(bar_kv_full(idx), ph_kv_full(idx), kDrainLimitCycles);
 #pragma unroll
             for (int t = 0; t < 2; ++t)
