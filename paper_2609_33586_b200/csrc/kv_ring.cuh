@@ -62,9 +62,12 @@ ROWMAX_HD bool kv_item(Ops& ops, int& idx, int pre_max, int n_max) {
     return true;
 }
 
-// After the last item: the last pair is complete without a K.
+// After the last item: the last pair is complete without a K.  At an odd position the producer gave up between K and V: the
+// pair of that position has not been waited for and nothing is loaded into it.
 template <class Ops>
-ROWMAX_HD void kv_end(Ops& ops, int idx) { ops.arrive(idx); }
+ROWMAX_HD void kv_end(Ops& ops, int idx) {
+    if ((idx & 1) == 0) ops.arrive(idx);
+}
 
 // First position of those that may still have copies under way when the producer ends at idx.
 template <int NS>

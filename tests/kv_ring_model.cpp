@@ -43,9 +43,10 @@ struct World {
     std::vector<int> landing;         // positions whose copies are under way
     size_t at = 0;
     std::mt19937 rng;
-    bool late;
+    bool late, abort_now = false;
+    int waits_until_abort;            // the producer gives up at this wait (< 0: never)
 
-    World(const std::vector<Item>& items, unsigned seed, bool late_) : rng(seed), late(late_) {
+    World(const std::vector<Item>& items, unsigned seed, bool late_, int abort_at) : rng(seed), late(late_), waits_until_abort(abort_at) {
         for (auto& b : full) b.init(2);
         int base = 0;
         for (const Item& it : items) {
@@ -89,6 +90,7 @@ struct World {
     void arrive(int idx) { some(); full[R::bar(idx)].arrive(0, "the producer", idx); }
     bool wait_empty(int idx) {
         some();
+        if (abort_now || waits_until_abort-- == 0) { abort_now = true; return false; }
         while (!empty[R::bar(idx)].done(R::ph_empty(idx)))
             if (!consume() && !land()) throw Failure{"deadlock at position " + std::to_string(idx)};
         return true;
@@ -97,32 +99,49 @@ struct World {
     void load_k(int idx, int) { load(idx); }
     void load_v(int idx, int) { load(idx); }
     void pre_k(int idx, int) { load(idx); }
-    bool load_q() { return true; }
+    bool load_q() { return !abort_now; }
 };
 
 template <int NS, bool PRE>
-void walk(const std::vector<Item>& items, unsigned seed, bool late) {
-    World<NS> w(items, seed, late);
+void walk(const std::vector<Item>& items, unsigned seed, bool late, int abort_at) {
+    World<NS> w(items, seed, late, abort_at);
     int idx = 0;
     rowmax::kv_begin(w);
-    for (const Item& it : items) rowmax::kv_item<PRE>(w, idx, it.pre, it.n);
+    bool ok = true;
+    for (const Item& it : items)
+        if (ok) ok = rowmax::kv_item<PRE>(w, idx, it.pre, it.n);
     rowmax::kv_end(w, idx);
-    while (w.consume() || w.land()) {}
-    if (w.at != w.mma.size() || !w.landing.empty()) throw Failure{"the MMA warp does not get to the end"};
+    if (ok) {
+        while (w.consume() || w.land()) {}
+        if (w.at != w.mma.size() || !w.landing.empty()) throw Failure{"the MMA warp does not get to the end"};
+    } else {
+        // The waits at the end: every copy under way belongs to a position that is waited for, and landing ends the phase.
+        for (int l : w.landing) {
+            bool covered = false;
+            for (int i = rowmax::kv_drain_from<NS>(idx); i < idx; ++i) covered = covered || ((i + 1) >> 1) == ((l + 1) >> 1);
+            if (!covered) throw Failure{"a copy under way at position " + std::to_string(l) + " is not waited for at the end"};
+        }
+        while (w.land()) {}
+        for (int i = rowmax::kv_drain_from<NS>(idx); i < idx; ++i)
+            if (!w.full[KvRing<NS>::bar(i)].done(KvRing<NS>::ph_full(i))) throw Failure{"the wait at the end for position " + std::to_string(i) + " runs out"};
+    }
 }
 
 template <int NS, bool PRE>
 void all(const std::vector<Item>& items, int seeds) {
-    for (int s = 0; s <= seeds; ++s) {
-        try {
-            walk<NS, PRE>(items, s, s == 0);
-        } catch (const Failure& f) {
-            std::string list;
-            for (const Item& it : items) list += " " + std::to_string(it.pre) + "+" + std::to_string(it.n);
-            std::printf("%d slots, items (maxima pass + tiles)%s, seed %d: %s\n", NS, list.c_str(), s, f.what.c_str());
-            std::exit(1);
+    int steps = 0;
+    for (const Item& it : items) steps += it.pre + 2 * it.n;
+    for (int abort_at = -1; abort_at < steps; ++abort_at)
+        for (int s = 0; s <= seeds; ++s) {
+            try {
+                walk<NS, PRE>(items, s, s == 0, abort_at);
+            } catch (const Failure& f) {
+                std::string list;
+                for (const Item& it : items) list += " " + std::to_string(it.pre) + "+" + std::to_string(it.n);
+                std::printf("%d slots, items (maxima pass + tiles)%s, gives up at wait %d, seed %d: %s\n", NS, list.c_str(), abort_at, s, f.what.c_str());
+                std::exit(1);
+            }
         }
-    }
 }
 
 }  // namespace
