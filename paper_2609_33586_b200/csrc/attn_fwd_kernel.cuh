@@ -169,7 +169,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     const uint32_t sScale = smem_u32(smem + W::kScaleOff);
     const uint32_t bar0 = smem_u32(smem + W::kBarOff);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + W::kMiscOff);
-    const uint32_t abort_at = smem_u32(smem + W::kMiscOff + 4);
+    const uint32_t abort_at = smem_u32(smem + W::kMiscOff + 4), leave_at = smem_u32(smem + W::kMiscOff + 8);
     const WaitCtx wctx{abort_at, p.status, kWaitLimitCycles};
 
     // barrier addresses
@@ -204,8 +204,13 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     }
     // The status word is sticky: once a wait has expired (in an earlier launch, or in another CTA of this one) and
     // until the host clears it, a CTA that starts is a no-op: it touches neither its outputs nor TMEM nor TMA.
-    // One thread reads the word so that the whole CTA takes the same way.
-    if (tid == 0) write_flag(abort_at, *reinterpret_cast<volatile int*>(p.status) != 0 ? 1 : 0);
+    // One thread reads the word, and what it read is kept in a place of its own (leave_at), so that the whole CTA takes the
+    // same way: abort_at may be set by a role while slower warps are still on their way to theirs.
+    if (tid == 0) {
+        const int set = *reinterpret_cast<volatile int*>(p.status) != 0 ? 1 : 0;
+        write_flag(abort_at, set);
+        write_flag(leave_at, set);
+    }
 #ifdef ROWMAX_TRACE
     const long long trace_t0 = clock64();
 #endif
@@ -262,7 +267,7 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         // once if the flag is set, and leaves with the cluster.
         cluster_arrive();
         cluster_wait();
-    } else if (flag_is_set(abort_at)) {
+    } else if (flag_is_set(leave_at)) {
         if (warp == 12) tmem_dealloc(tmem, kTmemCols);
         return;
     }
@@ -478,10 +483,6 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     } else if (wg == 2) {
         // ---------------------------------------------------------------- correction
         reg_dec<kRegCorr>();
-        // The kernel before this one may have set the status word after the check above; no P V, and so no epilogue, is
-        // reached before this warp's first arrival.
-        if (warp == 8 && lane == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) write_flag(abort_at, 1);
-        __syncwarp();
         const int r = tid & 127;
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
         int tiles[2] = {0, 0};
@@ -532,6 +533,10 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     } else {
         // ---------------------------------------------------------------- softmax + epilogue of query tile t
         reg_inc<kRegSoftmax>();
+        // The kernel before this one may have set the status word after the check above.  Each of the warps that store looks
+        // again for itself, while it would wait for its first scores.
+        if (lane == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) write_flag(abort_at, 1);
+        __syncwarp();
         const int t = wg;
         const int r = tid & 127;
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;

@@ -48,6 +48,32 @@ def test_an_expired_wait_sets_the_sticky_word_and_later_launches_store_nothing_u
     assert binding.device_status() == 0
 
 
+@pytest.mark.parametrize("wl", [
+    Workload("one_key_tile", 1, 2, 2, 300, 100, 128, False, "bf16", 83),
+    Workload("rows_without_keys", 1, 2, 2, 300, 20, 64, True, "bf16", 84),
+    Workload("several_key_tiles", 1, 2, 2, 600, 600, 128, True, "fp8_e4m3", 85)], ids=lambda w: w.name)
+def test_launches_queued_behind_the_expiring_one_store_nothing(wl):
+    """No synchronisation in between: the forwards may start (programmatic launch) before the word is set, and warps of one
+    block may see it at different times."""
+    binding.device_status_reset()
+    inp = make_inputs(wl)
+    q, k, v = inp.q.cuda(), inp.k.cuda(), inp.v.cuda()
+    out = torch.full((wl.B, wl.Sq, wl.Hq, wl.D), 7.0, dtype=torch.bfloat16, device="cuda")
+    lse = torch.full((wl.B, wl.Hq, wl.Sq), -3.0, dtype=torch.float32, device="cuda")
+    try:
+        binding.selftest_wait(200_000)
+        for _ in range(8):
+            binding.attn_fwd(q, k, v, causal=wl.causal, softmax_scale=wl.softmax_scale, weight_mode=orc.W_H15,
+                             q_descale=inp.q_descale, k_descale=inp.k_descale, v_descale=inp.v_descale, out=out, lse=lse)
+        torch.cuda.synchronize()
+        assert torch.all(out == 7.0) and torch.all(lse == -3.0)
+        assert binding.device_status_code() == SELFTEST_CODE
+    finally:
+        binding.device_status_reset()
+    st = compare(wl, orc.W_H15, inp)
+    assert st["ok"], st
+
+
 def test_selftest_limits_are_checked():
     assert binding.lib().attn_selftest_wait(0, None) == -9
     assert binding.lib().attn_selftest_wait(3_000_000_000, None) == -9
