@@ -48,7 +48,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-
+// One look that does not park the thread.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 
 __device__ __forceinline__ bool flag_is_set(uint32_t saddr) {
     int v;
@@ -90,15 +101,15 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const W
 
 // The same bound with a loop that polls the barrier (its hint parks the warp until the phase completes) and looks at
 // the status word only now and then: for kernels whose hand-offs are on the critical path and whose tensor-core operand
-// traffic is light.
+// traffic is light.  The CTA's flag is looked at before the warp is parked and after each turn: with the flag set, a wait for
+// a phase that will not complete returns at once (a turn may park for the whole hint, a millisecond).
 __device__ __forceinline__ void mbar_wait_poll(uint32_t bar, uint32_t parity, const WaitCtx& ctx, int code) {
-    if (mbar_try_wait(bar, parity)) return;
+    if (mbar_test_wait(bar, parity) || flag_is_set(ctx.cta_abort)) return;
     const long long t0 = clock64();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait(bar, parity)) return;
-        if (flag_is_set(ctx.cta_abort)) return;
+            if (mbar_try_wait(bar, parity) || flag_is_set(ctx.cta_abort)) return;
         if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
             write_flag(ctx.cta_abort, 1);
             atomicCAS(ctx.global_status, 0, code);
@@ -163,14 +174,25 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
         : "memory");
     return ok != 0;
 }
+__device__ __forceinline__ bool mbar_test_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// mbar_wait_poll for phases that other CTAs of the cluster complete.
 __device__ __forceinline__ void mbar_wait_cluster(uint32_t bar, uint32_t parity, const WaitCtx& ctx, int code) {
-    if (mbar_try_wait_cluster(bar, parity)) return;
+    if (mbar_test_wait_cluster(bar, parity) || flag_is_set(ctx.cta_abort)) return;
     const long long t0 = clock64();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait_cluster(bar, parity)) return;
-        if (flag_is_set(ctx.cta_abort)) return;
+            if (mbar_try_wait_cluster(bar, parity) || flag_is_set(ctx.cta_abort)) return;
         if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
             write_flag(ctx.cta_abort, 1);
             atomicCAS(ctx.global_status, 0, code);

@@ -74,6 +74,35 @@ def test_launches_queued_behind_the_expiring_one_store_nothing(wl):
     assert st["ok"], st
 
 
+@pytest.mark.parametrize("wl", [
+    Workload("few_rows", 1, 8, 1, 1, 70001, 128, True, "bf16", 86),
+    Workload("shared_items", 1, 2, 2, 300, 16384, 128, True, "bf16", 87)], ids=lambda w: w.name)
+def test_cluster_kernels_store_nothing_and_do_not_linger_while_the_word_is_set(wl):
+    """They take all their steps whatever the word says, and no wait of theirs may last: the limit is fifty turns of a parked
+    wait (a millisecond each at most), the steps number hundreds."""
+    q = torch.randn(wl.B, wl.Sq, wl.Hq, wl.D, device="cuda").to(torch.bfloat16)
+    k = torch.randn(wl.B, wl.Sk, wl.Hkv, wl.D, device="cuda").to(torch.bfloat16)
+    kw = dict(causal=True, softmax_scale=wl.softmax_scale, weight_mode=orc.W_H15)
+    binding.device_status_reset()
+    want, want_lse = binding.attn_fwd(q, k, k, **kw)
+    assert binding.device_status() == 0
+    out, lse = torch.full_like(want, 7.0), torch.full_like(want_lse, -3.0)
+    try:
+        binding.selftest_wait(1000)
+        assert binding.device_status() == TIMEOUT
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        binding.attn_fwd(q, k, k, out=out, lse=lse, **kw)
+        end.record()
+        torch.cuda.synchronize()
+        assert torch.all(out == 7.0) and torch.all(lse == -3.0)
+        assert start.elapsed_time(end) < 50.0
+    finally:
+        binding.device_status_reset()
+    binding.attn_fwd(q, k, k, out=out, lse=lse, **kw)
+    assert torch.equal(out, want) and torch.equal(lse, want_lse) and binding.device_status() == 0
+
+
 def test_selftest_limits_are_checked():
     assert binding.lib().attn_selftest_wait(0, None) == -9
     assert binding.lib().attn_selftest_wait(3_000_000_000, None) == -9
