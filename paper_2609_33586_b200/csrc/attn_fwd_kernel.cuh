@@ -751,9 +751,12 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
             }
 
             if constexpr (SPLIT) {
-                // O of this part, unscaled, over Q and the ring: [row of 256][D], 16-byte pieces swizzled by the row
+                // O of this part, unscaled, over Q and the ring: [row of 256][D], 16-byte pieces swizzled by the row.  A part
+                // without key tiles leaves no O and says so by its row sum; every other part is added, also where it weighs
+                // nothing: as in the loop over all tiles, 0 times an infinity or a NaN shows in O.
+                constexpr float kNoPart = -1.0f;
                 float2* ml = reinterpret_cast<float2*>(smem + W::kMlOff);
-                ml[t * 128 + r] = make_float2(m_run, l_run);
+                ml[t * 128 + r] = make_float2(m_run, nt > 0 ? l_run : kNoPart);
                 // the products of both query tiles read Q and the ring
                 mbar_wait_poll(bar_item, 0, wctx, (kRoleEpi << 8) | kBarItem);
                 __syncwarp();
@@ -793,25 +796,26 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     float2 v[kMaxSplit];
 #pragma unroll
                     for (int q = 0; q < kMaxSplit; ++q) {
-                        v[q] = q < parts ? ld_cluster_f32x2(mapa(at, q)) : make_float2(-INFINITY, 0.f);
+                        v[q] = q < parts ? ld_cluster_f32x2(mapa(at, q)) : make_float2(-INFINITY, kNoPart);
                     }
 #pragma unroll
-                    for (int q = 0; q < kMaxSplit; ++q) v[q].y = v[q].x == -INFINITY ? 0.f : v[q].y;   // no visible key yet
-#pragma unroll
                     for (int q = 0; q < kMaxSplit; ++q) {
-                        if (v[q].y > 0.f) m_fin = fmaxf(m_fin, v[q].x);
+                        if (v[q].y > 0.f || v[q].y != v[q].y) m_fin = fmaxf(m_fin, v[q].x);
                     }
                     float l_fin = 0.f;
 #pragma unroll
                     for (int q = 0; q < kMaxSplit; ++q) {
-                        v[q].x = v[q].y > 0.f ? ex2_approx((v[q].x - m_fin) * p.c) : 0.f;   // a part without visible keys weighs nothing
-                        l_fin += v[q].x * v[q].y;
+                        // a part without visible keys (no anchor) or with a row sum of zero weighs nothing; a row sum that is no
+                        // number makes the row's one
+                        const bool weighs = v[q].x != -INFINITY && !(v[q].y <= 0.f);
+                        v[q].x = weighs ? ex2_approx((v[q].x - m_fin) * p.c) : 0.f;
+                        if (weighs || v[q].y != v[q].y) l_fin += v[q].x * v[q].y;
                     }
                     const bool has_keys = l_fin > 0.f;
                     const float inv = has_keys ? p.v_descale / l_fin : 0.f;
 #pragma unroll
                     for (int q = 0; q < kMaxSplit; ++q)
-                        if (q < parts) weight[q * n_rows + wt] = v[q].x * inv;
+                        if (q < parts) weight[q * n_rows + wt] = v[q].y == kNoPart ? kNoPart : v[q].x * inv;
                     if (alive && out_row < p.Sq && p.lse != nullptr)
                         p.lse[(static_cast<size_t>(it.b) * p.Hq + it.h) * p.Sq + out_row] =
                             has_keys ? 0.6931471805599453f * (m_fin * p.c + log2f(l_fin) - p_off) : -INFINITY;
@@ -832,8 +836,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                         for (int u = 0; u < kBatch; ++u) {
                             const int e = e0 + 256 * u, prow = row_lo + e / kPieces;
                             const bool wanted = e < n_rows * kPieces && (prow < 128 ? it.q0[0] : it.q0[1]) + (prow & 127) < p.Sq;
-                            const float wq = wanted ? weight[q * n_rows + e / kPieces] : 0.f;
-                            if (wq > 0.f) {      // a part that weighs nothing has not written O
+                            const float wq = wanted ? weight[q * n_rows + e / kPieces] : kNoPart;
+                            if (!(wq < 0.f)) {
                                 acc[u].x = fmaf(wq, v[u].x, acc[u].x);
                                 acc[u].y = fmaf(wq, v[u].y, acc[u].y);
                                 acc[u].z = fmaf(wq, v[u].z, acc[u].z);
