@@ -60,10 +60,34 @@ const at::Tensor* as_tensor(PyObject* o) {
     return &THPVariable_Unpack(o);
 }
 
+// As ctypes takes an int argument: an integer (anything with __index__), of which the low bits count.  With `convert`
+// whatever int() takes.
+int as_int(PyObject* o, bool convert = false) {
+    if (PyErr_Occurred()) return 0;
+    PyObject* i = convert ? PyNumber_Long(o) : PyNumber_Index(o);
+    if (i == nullptr) return 0;
+    const unsigned long bits = PyLong_AsUnsignedLongMask(i);
+    Py_DECREF(i);
+    return static_cast<int>(static_cast<unsigned int>(bits));
+}
+
+float as_float(PyObject* o) { return PyErr_Occurred() ? 0.0f : static_cast<float>(PyFloat_AsDouble(o)); }
+
+// Address of a tensor's data, or of whatever else has a data_ptr().
+void* data_of(PyObject* o) {
+    if (THPVariable_Check(o)) return THPVariable_Unpack(o).data_ptr();
+    PyObject* address = PyObject_CallMethod(o, "data_ptr", nullptr);
+    if (address == nullptr) return nullptr;
+    void* p = PyLong_AsVoidPtr(address);
+    Py_DECREF(address);
+    return p;
+}
+
 // forward(q, k, v, out | None, lse | None, return_lse, causal, softmax_scale, weight_mode, q_descale, k_descale, v_descale,
 //         kind, option, option2, stream | None) -> (out, lse | None), or the status code of a call that failed.
 // kind: 0 attn_fwd, 1 attn_fwd_tau (option = threshold), 2 attn_fwd_pot (option = K_max, option2 = drop_tail),
-// 3 attn_fwd_exact_emulated (option = share in eighths).
+// 3 attn_fwd_exact_emulated (option = share in eighths).  `causal`, K_max and the share go through int(), weight_mode must be an
+// integer, truth decides return_lse and drop_tail.
 PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     HANDLE_TH_ERRORS
     if (n != 16) {
@@ -102,13 +126,14 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
             return nullptr;
         }
     }
-    const int return_lse = PyObject_IsTrue(a[5]), causal = PyObject_IsTrue(a[6]);
-    const float scale = static_cast<float>(PyFloat_AsDouble(a[7]));
-    const int mode = static_cast<int>(PyLong_AsLong(a[8]));
-    const float dq = static_cast<float>(PyFloat_AsDouble(a[9])), dk = static_cast<float>(PyFloat_AsDouble(a[10])),
-                dv = static_cast<float>(PyFloat_AsDouble(a[11]));
-    const int kind = static_cast<int>(PyLong_AsLong(a[12]));
-    const double option = PyFloat_AsDouble(a[13]);
+    const int return_lse = PyObject_IsTrue(a[5]);
+    const int causal = a[6] == Py_True ? 1 : a[6] == Py_False ? 0 : as_int(a[6], true);
+    const float scale = as_float(a[7]);
+    const int mode = as_int(a[8]);
+    const float dq = as_float(a[9]), dk = as_float(a[10]), dv = as_float(a[11]);
+    const int kind = as_int(a[12]);
+    const float tau = kind == 1 ? as_float(a[13]) : 0.0f;
+    const int option = kind >= 2 ? as_int(a[13], true) : 0;
     const int option2 = PyObject_IsTrue(a[14]);
     if (PyErr_Occurred()) return nullptr;
     void* stream;
@@ -120,35 +145,31 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     }
 
     at::Tensor out, lse;
-    void* lse_ptr = nullptr;
+    void *op, *lp = nullptr;
     if (a[3] == Py_None) {
         out = at::detail::empty_cuda({B, Sq, Hq, D}, at::kBFloat16, q.device(), std::nullopt);
+        op = out.data_ptr();
     } else {
-        const at::Tensor* x = as_tensor(a[3]);
-        if (x == nullptr) return nullptr;
-        out = *x;
+        op = data_of(a[3]);
     }
     if (a[4] != Py_None) {
-        const at::Tensor* x = as_tensor(a[4]);
-        if (x == nullptr) return nullptr;
-        lse = *x;
-        lse_ptr = lse.data_ptr();
+        lp = data_of(a[4]);
     } else if (return_lse) {
         lse = at::detail::empty_cuda({B, Hq, Sq}, at::kFloat, q.device(), std::nullopt);
-        lse_ptr = lse.data_ptr();
+        lp = lse.data_ptr();
     }
+    if (PyErr_Occurred()) return nullptr;
     const void *qp = q.data_ptr(), *kp = k.data_ptr(), *vp = v.data_ptr();
-    void* op = out.data_ptr();
-    float* lp = static_cast<float*>(lse_ptr);
+    float* lsep = static_cast<float*>(lp);
     const int b = static_cast<int>(B), hq = static_cast<int>(Hq), hkv = static_cast<int>(Hkv), sq = static_cast<int>(Sq),
               sk = static_cast<int>(Sk), d = static_cast<int>(D);
     int rc;
     Py_BEGIN_ALLOW_THREADS
     switch (kind) {
-        case 1: rc = g_entries.tau(qp, kp, vp, op, lp, b, hq, hkv, sq, sk, d, causal, scale, mode, dt, dq, dk, dv, static_cast<float>(option), stream); break;
-        case 2: rc = g_entries.pot(qp, kp, vp, op, lp, b, hq, hkv, sq, sk, d, causal, scale, dt, dq, dk, dv, static_cast<int>(option), option2, stream); break;
-        case 3: rc = g_entries.emulated(qp, kp, vp, op, lp, b, hq, hkv, sq, sk, d, causal, scale, dt, dq, dk, dv, static_cast<int>(option), stream); break;
-        default: rc = g_entries.fwd(qp, kp, vp, op, lp, b, hq, hkv, sq, sk, d, causal, scale, mode, dt, dq, dk, dv, stream); break;
+        case 1: rc = g_entries.tau(qp, kp, vp, op, lsep, b, hq, hkv, sq, sk, d, causal, scale, mode, dt, dq, dk, dv, tau, stream); break;
+        case 2: rc = g_entries.pot(qp, kp, vp, op, lsep, b, hq, hkv, sq, sk, d, causal, scale, dt, dq, dk, dv, option, option2, stream); break;
+        case 3: rc = g_entries.emulated(qp, kp, vp, op, lsep, b, hq, hkv, sq, sk, d, causal, scale, dt, dq, dk, dv, option, stream); break;
+        default: rc = g_entries.fwd(qp, kp, vp, op, lsep, b, hq, hkv, sq, sk, d, causal, scale, mode, dt, dq, dk, dv, stream); break;
     }
     Py_END_ALLOW_THREADS
     if (rc != 0) return PyLong_FromLong(rc);

@@ -382,3 +382,41 @@ def test_argument_errors_are_reported_without_launching():
                               128, 1, -1.0, 0, 0, 1.0, 1.0, 1.0, None)
     assert rc == -9
     assert binding.launch_count() == before
+
+
+def test_arguments_convert_as_they_would_for_ctypes():
+    """`causal` and the options go through int(), weight_mode has to be an integer, scales are whatever float() takes."""
+    wl = Workload("arguments", 1, 2, 2, 70, 70, 64, True, "bf16", 61)
+    inp = make_inputs(wl)
+    q, k, v = inp.q.cuda(), inp.k.cuda(), inp.v.cuda()
+
+    def call(causal=True, mode=orc.W_H15, scale=0.125, **kw):
+        return binding.attn_fwd(q, k, v, causal=causal, softmax_scale=scale, weight_mode=mode, **kw)[0]
+
+    want, full = call(True), call(False)
+    for causal in (1, "1", np.True_, np.int64(3), 1.5):
+        assert torch.equal(call(causal), want), causal
+    for causal in (0, 0.5, "0"):
+        assert torch.equal(call(causal), full), causal
+    for causal in (None, "yes", [], torch.ones(2)):
+        with pytest.raises((TypeError, ValueError, RuntimeError)):
+            call(causal)
+    assert torch.equal(call(mode=np.int64(orc.W_H15), scale=np.float32(0.125)), want)
+    for bad in (2.0, None, "2"):
+        with pytest.raises(TypeError):
+            call(mode=bad)
+    for bad in (None, "1"):
+        with pytest.raises(TypeError):
+            call(scale=bad)
+    tail = call(mode=orc.W_POT, pot_tail=(8, True))
+    assert torch.equal(call(mode=orc.W_POT, pot_tail=("8", 1)), tail) and torch.equal(call(mode=orc.W_POT, pot_tail=(8.9, "x")), tail)
+    with pytest.raises(ValueError):
+        call(mode=orc.W_POT, pot_tail=(float("nan"), True))
+    with pytest.raises(TypeError):
+        call(mode=EXACT_POLY, poly_eighths=[2])
+    out = torch.zeros_like(want)
+    assert binding.attn_fwd(q, k, v, causal=True, softmax_scale=0.125, weight_mode=orc.W_H15, out=out.untyped_storage(), return_lse=False)[1] is None
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    with pytest.raises((TypeError, AttributeError)):
+        call(out=3)
