@@ -20,7 +20,7 @@ MODES = {"exact": W_EXACT, "pot": W_POT, "h15": W_H15, "h15k2": W_H15K2, "h15k3"
 
 _LIB_PATH = Path(__file__).resolve().parent / "libattn_b200.so"
 _lib = None
-_forward = None      # _host.forward, once the library is loaded
+_forward = None      # _host.forward, once attn_fwd has been called
 
 EXPORTS = ("attn_fwd", "attn_fwd_tau", "attn_fwd_pot", "attn_fwd_exact_emulated", "attn_weight_map", "attn_weight_map_pot", "attn_weight_map_fused", "attn_get_schedule", "attn_device_status",
            "attn_device_status_code", "attn_selftest_wait", "attn_device_status_reset", "attn_launch_count", "attn_status_string",
@@ -34,7 +34,7 @@ class AttnError(RuntimeError):
 
 
 def lib() -> ctypes.CDLL:
-    global _lib, _forward
+    global _lib
     if _lib is None:
         if not _LIB_PATH.exists():
             raise RuntimeError(
@@ -68,14 +68,26 @@ def lib() -> ctypes.CDLL:
         L.attn_status_string.argtypes = [i]
         L.attn_last_cuda_error.restype = i
         L.attn_version.restype = ctypes.c_char_p
+        _lib = L
+    return _lib
+
+
+def host_forward():
+    """The native call path of attn_fwd.  Loaded on its first use: nothing else here needs it."""
+    global _forward
+    if _forward is None:
+        L = lib()
         try:
             from . import _host
         except ImportError as e:
-            raise RuntimeError("the host module is missing: build it with `python -m paper_2609_33586_b200.build`") from e
-        _host.set_entries(*(ctypes.cast(f, vp).value for f in (L.attn_fwd, L.attn_fwd_tau, L.attn_fwd_pot, L.attn_fwd_exact_emulated)))
+            raise RuntimeError("the host module does not load: build it with `python -m paper_2609_33586_b200.build`") from e
+        if _host.torch_version != torch.__version__:
+            raise RuntimeError(f"the host module was built for torch {_host.torch_version}, this is {torch.__version__}: build it "
+                               "again with `python -m paper_2609_33586_b200.build`")
+        _host.set_entries(*(ctypes.cast(f, ctypes.c_void_p).value
+                            for f in (L.attn_fwd, L.attn_fwd_tau, L.attn_fwd_pot, L.attn_fwd_exact_emulated)))
         _forward = _host.forward
-        _lib = L
-    return _lib
+    return _forward
 
 
 def status_string(code: int) -> str:
@@ -177,8 +189,7 @@ def attn_fwd(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, *, causal: bool,
         raise ValueError("poly_eighths goes with weight_mode = W_EXACT_POLY")
     if pot_tail is not None and weight_mode != W_POT:
         raise ValueError("pot_tail goes with weight_mode = W_POT")
-    if _lib is None:
-        lib()
+    forward = _forward or host_forward()
     if poly_eighths is not None:
         kind, option, option2 = 3, poly_eighths, False
     elif pot_tail is not None:
@@ -187,7 +198,7 @@ def attn_fwd(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, *, causal: bool,
         kind, option, option2 = 1, rescale_tau, False
     else:
         kind, option, option2 = 0, 0, False
-    r = _forward(q, k, v, out, lse, return_lse, causal, softmax_scale, weight_mode, q_descale, k_descale, v_descale,
+    r = forward(q, k, v, out, lse, return_lse, causal, softmax_scale, weight_mode, q_descale, k_descale, v_descale,
                  kind, option, option2, stream if stream is None else int(stream.cuda_stream))
     if type(r) is int:
         raise AttnError(r, "attn_fwd")

@@ -31,16 +31,23 @@ def needs_build() -> bool:
     return any((CSRC / f).stat().st_mtime > t for f in SOURCES + HEADERS)
 
 
+def host_is_current(path: Path, torch_version: str) -> bool:
+    """Whether the host module at `path` is newer than its sources and was built for this torch (its text says which)."""
+    if not path.exists() or path.stat().st_mtime < max((CSRC / f).stat().st_mtime for f in ("host_binding.cpp", "../../include/attn.h")):
+        return False
+    return f"host module for torch {torch_version}\0".encode() in path.read_bytes()
+
+
 def build_host(force: bool = False) -> Path:
     """The CPython module that does the per-call host work (csrc/host_binding.cpp)."""
     src = CSRC / "host_binding.cpp"
-    if not force and HOST.exists() and HOST.stat().st_mtime >= max(src.stat().st_mtime, (CSRC / "../../include/attn.h").stat().st_mtime):
-        return HOST
     import torch
+    if not force and host_is_current(HOST, torch.__version__):
+        return HOST
     troot = Path(torch.__file__).resolve().parent
     cuda = Path(_nvcc()).resolve().parent.parent
     tmp = HOST.with_suffix(f".so.tmp{os.getpid()}")
-    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-w", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-w", f'-DROWMAX_TORCH="{torch.__version__}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            f"-I{sysconfig.get_paths()['include']}", f"-I{troot}/include", f"-I{troot}/include/torch/csrc/api/include",
            f"-I{cuda}/include", "-o", str(tmp), str(src), f"-L{troot}/lib", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda",
            "-ltorch_python", f"-Wl,-rpath,{troot}/lib"]

@@ -196,8 +196,17 @@ PyMethodDef methods[] = {
     {"set_entries", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(set_entries)), METH_FASTCALL, nullptr},
     {"forward", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(forward)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
-PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_host", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+// build.py looks for this text to tell which torch the module was built for
+constexpr char kBuiltFor[] = "host module for torch " ROWMAX_TORCH;
+PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_host", kBuiltFor, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__host() { return PyModule_Create(&module_def); }
+PyMODINIT_FUNC PyInit__host() {
+    PyObject* m = PyModule_Create(&module_def);
+    if (m != nullptr && PyModule_AddStringConstant(m, "torch_version", ROWMAX_TORCH) != 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

@@ -1,7 +1,12 @@
 """The C-ABI library loads and exports every symbol that include/attn.h declares (no GPU needed)."""
 import ctypes
+import os
 import re
+import subprocess
+import sys
 from pathlib import Path
+
+import torch
 
 from paper_2609_33586_b200 import binding, build
 
@@ -36,3 +41,29 @@ def test_host_only_entry_points_work_without_a_gpu():
     assert binding.attn_fwd_raw(None, None, None, None, None, 1, 1, 1, 1, 1, 64, 0, 1.0, 0, 0, 1, 1, 1, None) == -1
     assert binding.lib().attn_weight_map(None, None, 0, 2, None) == 0
     assert binding.lib().attn_weight_map(None, None, 4, 2, None) == -1
+
+
+def test_only_attn_fwd_needs_the_host_module():
+    code = """
+import sys
+sys.modules["paper_2609_33586_b200._host"] = None      # its import fails
+from paper_2609_33586_b200 import binding
+import torch
+assert binding.version() and binding.launch_count() == 0 and binding.get_schedule(64, 0, 0, True)["tile_n"] == 128
+x = torch.zeros(1, 1, 1, 64, dtype=torch.bfloat16)
+try:
+    binding.attn_fwd(x, x, x, causal=True, softmax_scale=1.0, weight_mode=0)
+except RuntimeError as e:
+    assert "host module" in str(e)
+else:
+    raise SystemExit("no error")
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT, env=dict(os.environ, PYTHONPATH=str(ROOT)))
+
+
+def test_a_host_module_built_for_another_torch_is_not_current(tmp_path):
+    built = build.build_host()
+    assert build.host_is_current(built, torch.__version__)
+    assert not build.host_is_current(built, torch.__version__ + "1") and not build.host_is_current(built, torch.__version__[:-1])
+    assert not build.host_is_current(tmp_path / "absent.so", torch.__version__)
+    binding.host_forward()
