@@ -6,7 +6,7 @@
 #include <Python.h>
 
 #include <ATen/core/Tensor.h>
-#include <ATen/cuda/EmptyTensor.h>
+#include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -147,7 +147,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor out, lse;
     void *op, *lp = nullptr;
     if (a[3] == Py_None) {
-        out = at::detail::empty_cuda({B, Sq, Hq, D}, at::kBFloat16, q.device(), std::nullopt);
+        out = at::empty({B, Sq, Hq, D}, q.options().dtype(at::kBFloat16));
         op = out.data_ptr();
     } else {
         op = data_of(a[3]);
@@ -155,7 +155,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (a[4] != Py_None) {
         lp = data_of(a[4]);
     } else if (return_lse) {
-        lse = at::detail::empty_cuda({B, Hq, Sq}, at::kFloat, q.device(), std::nullopt);
+        lse = at::empty({B, Hq, Sq}, q.options().dtype(at::kFloat));
         lp = lse.data_ptr();
     }
     if (PyErr_Occurred()) return nullptr;

@@ -420,3 +420,32 @@ def test_arguments_convert_as_they_would_for_ctypes():
     assert torch.equal(out, want)
     with pytest.raises((TypeError, AttributeError)):
         call(out=3)
+
+
+def test_output_allocations_go_through_the_dispatcher():
+    """A dispatch mode sees them, and deterministic mode fills them as it does every torch.empty."""
+    from torch.utils._python_dispatch import TorchDispatchMode
+    seen = []
+
+    class Log(TorchDispatchMode):
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            seen.append(func)
+            return func(*args, **(kwargs or {}))
+
+    q = torch.zeros(1, 70, 2, 64, device="cuda", dtype=torch.bfloat16)
+    kw = dict(causal=True, softmax_scale=0.125, weight_mode=orc.W_H15)
+    with Log():
+        o, lse = binding.attn_fwd(q, q, q, **kw)
+    assert seen.count(torch.ops.aten.empty.memory_format) == 2
+    assert o.dtype == torch.bfloat16 and lse.dtype == torch.float32 and o.shape == q.shape and lse.shape == (1, 2, 70)
+    torch.cuda.synchronize()
+    torch.use_deterministic_algorithms(True)
+    try:
+        binding.selftest_wait(1000)      # with the status word set nothing is stored, which shows what was allocated
+        torch.cuda.synchronize()
+        o, lse = binding.attn_fwd(q, q, q, **kw)
+        torch.cuda.synchronize()
+        assert torch.isnan(o).all() and torch.isnan(lse).all()
+    finally:
+        torch.use_deterministic_algorithms(False)
+        binding.device_status_reset()
