@@ -14,7 +14,7 @@ CSRC = PKG / "csrc"
 LIB = PKG / "libattn_b200.so"
 HOST = PKG / f"_host{sysconfig.get_config_var('EXT_SUFFIX')}"
 SOURCES = ["api.cu", "attn_fwd_sm100.cu", "attn_fwd_split_sm100.cu", "attn_fwd_tau_sm100.cu", "attn_rows_sm100.cu"]
-HEADERS = ["ptx.cuh", "kv_ring.cuh", "attn_fwd_kernel.cuh", "weight_map.cuh", "attn_kernel_common.cuh", "softmax_math.cuh", "../../include/attn.h"]
+HEADERS = ["ptx.cuh", "kv_ring.cuh", "plan.h", "attn_fwd_kernel.cuh", "weight_map.cuh", "attn_kernel_common.cuh", "softmax_math.cuh", "../../include/attn.h"]
 
 
 def _nvcc() -> str:

@@ -31,6 +31,7 @@
 // TMEM columns: S_0/P_0 [0,128), S_1/P_1 [128,256), O_0 [256,384), O_1 [384,512).
 #pragma once
 #include "kv_ring.cuh"
+#include "plan.h"
 #include "softmax_math.cuh"
 
 namespace rowmax {
@@ -39,7 +40,6 @@ namespace {
 
 // Whether the parts of a split item need the row maxima of the parts before them.
 __host__ __device__ constexpr bool split_takes_maxima(int mode, bool fp8) { return fp8 || !is_exact_like(mode); }
-constexpr int kMaxSplit = 8;   // CTAs that share an item (the portable cluster size)
 
 template <int D, bool FP8, bool SPLIT = false>
 struct WsCfg {
@@ -932,20 +932,15 @@ static cudaError_t launch_ws(const CUtensorMap& tq, const CUtensorMap& tk, const
                              const AttnParams& p, cudaStream_t stream) {
     using W = WsCfg<D, IN == kInFP8>;
     auto kern = attn_fwd_ws_kernel<D, IN, MODE, false, TAU>;
-    // per-device launch set-up: the shared-memory opt-in of this instance and the SM count
-    static bool configured[64] = {};
-    static int sm_counts[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static bool configured[64] = {};   // per device: the shared-memory opt-in of this instance
+    int dev = 0, sm_count = 0;
+    cudaError_t e = device_and_sms(&dev, &sm_count);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!configured[dev]) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmemBytes);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_counts[dev], cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    const int sm_count = sm_counts[dev];
     const long long n_pairs = (p.Sq + 2 * kTileM - 1) / (2 * kTileM);
     const long long items = n_pairs * p.Hq * p.B;
     if (items > 0x7fffffffLL) return cudaErrorInvalidValue;

@@ -219,6 +219,19 @@ cudaError_t launch_selftest_wait(int* status, long long limit_cycles, cudaStream
     return cudaGetLastError();
 }
 
+cudaError_t device_and_sms(int* dev, int* sms) {
+    static int known[64] = {};
+    cudaError_t e = cudaGetDevice(dev);
+    if (e != cudaSuccess) return e;
+    if (*dev < 0 || *dev >= 64) return cudaErrorInvalidDevice;
+    if (known[*dev] == 0) {
+        e = cudaDeviceGetAttribute(&known[*dev], cudaDevAttrMultiProcessorCount, *dev);
+        if (e != cudaSuccess) return e;
+    }
+    *sms = known[*dev];
+    return cudaSuccess;
+}
+
 __device__ int g_attn_status = 0;
 
 cudaError_t status_word_address(int** out) {

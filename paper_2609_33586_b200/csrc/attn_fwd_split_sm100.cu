@@ -1,8 +1,6 @@
 // Launcher of the split form of the attention forward (attn_fwd_kernel.cuh): a cluster of CTAs shares each work item.
 #include "attn_fwd_kernel.cuh"
 
-#include <cmath>
-
 namespace rowmax {
 
 namespace {
@@ -42,35 +40,16 @@ struct SplitLauncher {
         }
         return known[dev][parts] > 0 ? known[dev][parts] : 0;
     }
-    // CTAs per item, 1 for the plain form.  Times are in steps of the loop (one key tile of a pair of query tiles), measured:
-    // a part costs its key tiles, with a maxima pass 0.65 of a step more for each tile of its maxima pass (two parts share
-    // the pass, so it is half as long), and 4.5 steps + 0.5 per part for the exchange and the sum of O; all SMs working slow
-    // each other by a tenth.  512 queries on 16K, 32/8 heads: bf16 h15 198 -> 154 us, exact 226 -> 138, e4m3 178 -> 125
-    // (2 parts); 64 queries on 8K 97 -> 49 (4 parts).  16 x 1K and 16 x 2K gain nothing and stay whole.
+    // CTAs per item (plan.h), 1 for the plain form.
     static int plan(const AttnParams& p) {
+        int dev = 0, sms = 0;
+        if (device_and_sms(&dev, &sms) != cudaSuccess) return 1;
         const int pairs = (p.Sq + 2 * kTileM - 1) / (2 * kTileM);
-        const double items = static_cast<double>(pairs) * p.Hq * p.B;
-        if (items > 148.0) return 1;
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-        // key tiles of the last (longest) pair and of the middle one
-        const int shift = p.Sk - p.Sq;
         const int all = (p.Sk + kTileN - 1) / kTileN;
-        const int first_end = p.causal ? 2 * kTileM + shift : p.Sk;
+        const int first_end = p.causal ? 2 * kTileM + p.Sk - p.Sq : p.Sk;
         const int first = first_end <= 0 ? 0 : ((first_end < p.Sk ? first_end : p.Sk) + kTileN - 1) / kTileN;
-        const double longest = all, mean = 0.5 * (all + first);
-        double best = 0.93 * (longest + 1.5);      // a gain below that is not worth the risk of being wrong
-        int best_parts = 1;
-        for (int parts = 2; parts <= kMaxSplit && parts <= all; ++parts) {
-            const int n = fit(dev, parts);
-            if (n <= 0) continue;
-            const double per_tile = (!split_takes_maxima(MODE, IN == kInFP8) ? 1.0 : parts == 2 ? 1.325 : 1.65) / parts;
-            const double fixed = 4.5 + 0.5 * parts, busy = items * parts > 100.0 ? 1.1 : 1.0;
-            const double waves = ceil(items / n);
-            const double t = fmax(longest * per_tile + fixed, waves * (mean * per_tile + fixed)) * busy;
-            if (t < best) { best = t; best_parts = parts; }
-        }
-        return best_parts;
+        const SplitShape s{static_cast<double>(pairs) * p.Hq * p.B, all, first, split_takes_maxima(MODE, IN == kInFP8)};
+        return split_parts(s, sms, [&](int parts) { return fit(dev, parts); });
     }
     static cudaError_t launch(int parts, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, AttnParams p,
                               cudaStream_t stream) {

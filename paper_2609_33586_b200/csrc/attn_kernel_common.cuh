@@ -1,6 +1,7 @@
 // Parameters and small helpers shared by the attention kernels and the host launcher.
 #pragma once
 #include <cuda.h>
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace rowmax {
@@ -48,6 +49,9 @@ struct AttnParams {
     int trace_block;
 #endif
 };
+
+// The current device, below 64, and its SM count (asked once per device).
+cudaError_t device_and_sms(int* dev, int* sms);
 
 // Status codes written by expired waits: role << 8 | barrier id.
 enum : int {

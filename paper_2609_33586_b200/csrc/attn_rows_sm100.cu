@@ -16,16 +16,14 @@
 // Per CTA: warps 0-3 softmax (thread = key on the way in, = output dimension on the way out), warp 4 TMA producer,
 // warp 5 MMA issuer.  O is accumulated in registers: P V of a tile overwrites the TMEM columns of that tile's scores,
 // and each thread adds it to its running sum scaled by the tile's rescale factor.
+#include "plan.h"
 #include "softmax_math.cuh"
-
-#include <cmath>
 
 namespace rowmax {
 
 namespace {
 
 constexpr int kRowsThreads = 192;
-constexpr int kMaxCluster = 16;
 constexpr int kMaxSlots = 24;
 constexpr int kTmemBlockCols = 512;      // floats of the per-(tile, row) arrays: tiles x N <= 512
 
@@ -680,9 +678,7 @@ struct RowsLauncher {
         cfg.blockDim = dim3(kRowsThreads);
         cfg.dynamicSmemBytes = kDynamic;
     }
-    // Clusters of `cs` CTAs that fit the device at once.  The occupancy query (asked once per device and size) counts one
-    // CTA per SM for every kernel that allocates TMEM; with 256 columns two run, and a cluster may then lie on half as many
-    // SMs, so that of the portable sizes nearly all 2 x 148 places can be used.
+    // Clusters of `cs` CTAs that the occupancy query says fit the device at once (asked once per device and size).
     static int fit(int dev, int cs) {
         static int known[64][kMaxCluster + 1] = {};
         static bool configured[64] = {};
@@ -707,40 +703,18 @@ struct RowsLauncher {
             }
             known[dev][cs] = n > 0 ? n : -1;
         }
-        const int n = known[dev][cs] > 0 ? known[dev][cs] : 0;
-        if (kRowsCols<N> == 512 || n == 0) return n;
-        return cs <= 8 && 272 / cs > 2 * n ? 272 / cs : 2 * n;
+        return known[dev][cs] > 0 ? known[dev][cs] : 0;
     }
-    // CTAs per cluster: the candidate with the shortest estimated time.  Measured on shapes from 1 x 1K to 16 x 2K and
-    // 1 x 32K: a part that does not depend on the context (5.6 us, 0.1 us per CTA of a cluster for exchange and combination,
-    // 1.2 us more beyond the portable size), one key tile's way through a CTA (hand-offs 0.83 us, or the rate of 55 GB/s one
-    // CTA reads at), and the device's bandwidth, which are added as squares where they overlap.  It picks the fastest size or
-    // one within 8 % of it.
-    static int pick_cluster(int dev, const AttnParams& p) {
-        const double groups = static_cast<double>(p.B) * p.Hkv;
-        const int nt = (p.Sk + kTileN - 1) / kTileN;
-        const double bytes_us = 2.0 * nt * groups * kTile / 6.3e6;
-        const double pair_us = fmax(N == 16 ? 0.83 : N == 32 ? 1.6 : 2.5, 2.0 * kTile / 55e3);
-        double best = 1e30;
-        int best_cs = 0;
-        for (int cs = 1; cs <= kMaxCluster && cs <= nt; ++cs) {
-            const int n = fit(dev, cs);
-            if (n <= 0) continue;
-            const double waves = ceil(groups / n);
-            const double shared = fmin(groups, n) * cs > 148.0 ? 1.15 : 1.0;     // two CTAs on an SM slow each other a little
-            const double hand_us = waves * ((nt + cs - 1) / cs) * pair_us * shared;
-            const double t = waves * (5.6 + 0.1 * cs + (cs > 8 ? 1.2 : 0.0)) + sqrt(hand_us * hand_us + bytes_us * bytes_us);
-            if (t < best) { best = t; best_cs = cs; }
-        }
-        return best_cs;
+    static int pick_cluster(int dev, int sms, const AttnParams& p) {
+        const RowsShape s{static_cast<double>(p.B) * p.Hkv, (p.Sk + kTileN - 1) / kTileN, N, kTile};
+        return rows_cluster_size(s, sms, [&](int cs) { return fit(dev, cs); });
     }
     static cudaError_t launch(int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
                               cudaStream_t stream) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
+        int dev = 0, sms = 0;
+        const cudaError_t e = device_and_sms(&dev, &sms);
         if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        const int cs = pick_cluster(dev, p);
+        const int cs = pick_cluster(dev, sms, p);
         const long long groups = static_cast<long long>(p.B) * p.Hkv;
         if (cs == 0 || groups * cs > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         RowsParams rp;

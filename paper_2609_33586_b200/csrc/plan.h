@@ -1,0 +1,83 @@
+// How many CTAs share a work item of the attention forward: cost models fitted to measured times, as plain functions of the
+// shape, the SM count and what fits the device, so that they can be tested without one (tests/plan_model.cpp).
+#pragma once
+#include <algorithm>
+#include <cmath>
+
+namespace rowmax {
+
+constexpr int kMaxSplit = 8;     // CTAs that share an item in the split form (the portable cluster size)
+constexpr int kMaxCluster = 16;  // CTAs that share a (batch, key/value head) in the few-row kernel
+
+// The machine that the figures were measured on.  Counts of SMs below are shares of it.
+constexpr int kMeasuredSms = 148;
+
+struct SplitShape {
+    double items;       // pairs of query tiles of all (batch, head)
+    int all, first;     // key tiles of the longest pair and of the first one
+    bool takes_maxima;  // the parts need the row maxima of the parts before them
+};
+
+// CTAs per item, 1 for the plain form.  fit(parts): clusters of that size that fit the device at once.  Times are in steps of the
+// loop (one key tile of a pair of query tiles), measured: a part costs its key tiles, with a maxima pass 0.65 of a step more for
+// each tile of its maxima pass (two parts share the pass, so it is half as long), and 4.5 steps + 0.5 per part for the exchange
+// and the sum of O; from two thirds of the SMs on they slow each other by a tenth.  512 queries on 16K, 32/8 heads: bf16 h15
+// 198 -> 154 us, exact 226 -> 138, e4m3 178 -> 125 (2 parts); 64 queries on 8K 97 -> 49 (4 parts).  16 x 1K and 16 x 2K gain
+// nothing and stay whole.
+template <class Fit>
+int split_parts(const SplitShape& s, int sms, Fit fit) {
+    if (s.items > sms) return 1;
+    const double longest = s.all, mean = 0.5 * (s.all + s.first);
+    double best = 0.93 * (longest + 1.5);      // a gain below that is not worth the risk of being wrong
+    int best_parts = 1;
+    for (int parts = 2; parts <= kMaxSplit && parts <= s.all; ++parts) {
+        const int n = fit(parts);
+        if (n <= 0) continue;
+        const double per_tile = (!s.takes_maxima ? 1.0 : parts == 2 ? 1.325 : 1.65) / parts;
+        const double fixed = 4.5 + 0.5 * parts, busy = s.items * parts * kMeasuredSms > 100.0 * sms ? 1.1 : 1.0;
+        const double waves = std::ceil(s.items / n);
+        const double t = std::fmax(longest * per_tile + fixed, waves * (mean * per_tile + fixed)) * busy;
+        if (t < best) { best = t; best_parts = parts; }
+    }
+    return best_parts;
+}
+
+struct RowsShape {
+    double groups;      // (batch, key/value head) pairs
+    int nt;             // key tiles
+    int n;              // rows of the tile: 16, 32 or 64
+    int tile_bytes;     // of K or V
+};
+
+// Clusters of cs CTAs that the few-row kernel can have on the device, given what the occupancy query says.  The query counts one
+// CTA per SM for every kernel that allocates TMEM; tiles of 16 and 32 rows run two, and a cluster may then lie on half as many
+// SMs, so that of the portable sizes 272 of the 2 x 148 places can be used.
+inline int rows_clusters(int n_rows, int cs, int queried, int sms) {
+    if (n_rows == 64 || queried <= 0) return queried;
+    return cs <= 8 ? std::max(272 * sms / kMeasuredSms / cs, 2 * queried) : 2 * queried;
+}
+
+// CTAs per cluster of the few-row kernel, 0 if none fits: the candidate with the shortest estimated time.  Measured on shapes
+// from 1 x 1K to 16 x 2K and 1 x 32K: a part that does not depend on the context (5.6 us, 0.1 us per CTA of a cluster for exchange
+// and combination, 1.2 us more beyond the portable size), one key tile's way through a CTA (hand-offs 0.83 us, or the rate of
+// 55 GB/s one CTA reads at), and the device's bandwidth, which are added as squares where they overlap.  It picks the fastest
+// size or one within 8 % of it.  fit(cs): what the occupancy query says.
+template <class Fit>
+int rows_cluster_size(const RowsShape& s, int sms, Fit fit) {
+    const double bytes_us = 2.0 * s.nt * s.groups * s.tile_bytes / 6.3e6;
+    const double pair_us = std::fmax(s.n == 16 ? 0.83 : s.n == 32 ? 1.6 : 2.5, 2.0 * s.tile_bytes / 55e3);
+    double best = 1e30;
+    int best_cs = 0;
+    for (int cs = 1; cs <= kMaxCluster && cs <= s.nt; ++cs) {
+        const int n = rows_clusters(s.n, cs, fit(cs), sms);
+        if (n <= 0) continue;
+        const double waves = std::ceil(s.groups / n);
+        const double shared = std::fmin(s.groups, n) * cs > sms ? 1.15 : 1.0;     // two CTAs on an SM slow each other a little
+        const double hand_us = waves * ((s.nt + cs - 1) / cs) * pair_us * shared;
+        const double t = waves * (5.6 + 0.1 * cs + (cs > 8 ? 1.2 : 0.0)) + std::sqrt(hand_us * hand_us + bytes_us * bytes_us);
+        if (t < best) { best = t; best_cs = cs; }
+    }
+    return best_cs;
+}
+
+}  // namespace rowmax
