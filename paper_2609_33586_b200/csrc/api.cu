@@ -17,8 +17,8 @@ cudaError_t launch_attn_fwd_tau(int D, int mode, const CUtensorMap& tq, const CU
 int plan_attn_split(int D, int in_type, int mode, const AttnParams& p);
 cudaError_t launch_attn_fwd_split(int D, int in_type, int mode, int parts, const CUtensorMap& tq, const CUtensorMap& tk,
                                   const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream);
-bool use_rows_kernel(int in_type, int mode, const AttnParams& p);
-cudaError_t launch_attn_rows(int D, int in_type, int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q,
+int plan_attn_rows(int D, int in_type, int mode, const AttnParams& p);
+cudaError_t launch_attn_rows(int D, int in_type, int mode, int cs, const CUtensorMap& tk, const CUtensorMap& tv, const void* q,
                              const AttnParams& p, cudaStream_t stream);
 cudaError_t launch_weight_map(const float* x, float* w, size_t n, int mode, cudaStream_t stream);
 cudaError_t launch_weight_map_pot(const float* x, float* w, size_t n, int kmax, int drop, cudaStream_t stream);
@@ -199,8 +199,8 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     if ((rc = make_tile_map(&tk, k, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
     if ((rc = make_tile_map(&tv, v, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
     cudaError_t e;
-    if (rowmax::use_rows_kernel(in_dtype, kernel_mode, p)) {
-        e = rowmax::launch_attn_rows(D, in_dtype, kernel_mode, tk, tv, q, p, static_cast<cudaStream_t>(stream));
+    if (const int cs = rowmax::plan_attn_rows(D, in_dtype, kernel_mode, p)) {
+        e = rowmax::launch_attn_rows(D, in_dtype, kernel_mode, cs, tk, tv, q, p, static_cast<cudaStream_t>(stream));
     } else {
         if ((rc = make_tile_map(&tq, q, fp8, half_in, B, Sq, Hq, D)) != ATTN_OK) return rc;
         const int parts = rowmax::plan_attn_split(D, in_dtype, kernel_mode, p);

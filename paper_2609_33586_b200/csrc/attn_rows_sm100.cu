@@ -705,18 +705,16 @@ struct RowsLauncher {
         }
         return known[dev][cs] > 0 ? known[dev][cs] : 0;
     }
-    static int pick_cluster(int dev, int sms, const AttnParams& p) {
-        const RowsShape s{static_cast<double>(p.B) * p.Hkv, (p.Sk + kTileN - 1) / kTileN, N, kTile};
-        return rows_cluster_size(s, sms, [&](int cs) { return fit(dev, cs); });
-    }
-    static cudaError_t launch(int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
-                              cudaStream_t stream) {
+    static int plan(const AttnParams& p) {
         int dev = 0, sms = 0;
-        const cudaError_t e = device_and_sms(&dev, &sms);
-        if (e != cudaSuccess) return e;
-        const int cs = pick_cluster(dev, sms, p);
+        if (device_and_sms(&dev, &sms) != cudaSuccess) return 0;
+        const RowsShape s{static_cast<double>(p.B) * p.Hkv, (p.Sk + kTileN - 1) / kTileN, N, kTile};
+        const int cs = rows_cluster_size(s, sms, [&](int c) { return fit(dev, c); });
+        return static_cast<long long>(p.B) * p.Hkv * cs > 0x7fffffffLL ? 0 : cs;
+    }
+    static cudaError_t launch(int mode, int cs, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
+                              cudaStream_t stream) {
         const long long groups = static_cast<long long>(p.B) * p.Hkv;
-        if (cs == 0 || groups * cs > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
         RowsParams rp;
         rp.cs = cs;
         rp.nt = (p.Sk + kTileN - 1) / kTileN;
@@ -736,34 +734,42 @@ struct RowsLauncher {
     }
 };
 
-template <int D, int IN>
-cudaError_t dispatch_rows(int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
-                          cudaStream_t stream) {
-    const int rows = p.Sq * p.group;
-    if (rows <= 16) return RowsLauncher<D, IN, 16>::launch(mode, tk, tv, q, p, stream);
-    if (rows <= 32) return RowsLauncher<D, IN, 32>::launch(mode, tk, tv, q, p, stream);
-    return RowsLauncher<D, IN, 64>::launch(mode, tk, tv, q, p, stream);
+// Calls f with the launcher of a combination.
+template <int D, int IN, typename F>
+void with_rows(int rows, F f) {
+    if (rows <= 16) f(RowsLauncher<D, IN, 16>{});
+    else if (rows <= 32) f(RowsLauncher<D, IN, 32>{});
+    else f(RowsLauncher<D, IN, 64>{});
+}
+template <typename F>
+void with_rows_launcher(int D, int in_type, int rows, F f) {
+    if (D == 128) {
+        if (in_type == kInBF16) with_rows<128, kInBF16>(rows, f);
+        else if (in_type == kInFP16) with_rows<128, kInFP16>(rows, f);
+        else with_rows<128, kInFP8>(rows, f);
+    } else {
+        if (in_type == kInBF16) with_rows<64, kInBF16>(rows, f);
+        else if (in_type == kInFP16) with_rows<64, kInFP16>(rows, f);
+        else with_rows<64, kInFP8>(rows, f);
+    }
 }
 
 }  // namespace
 
-// Whether a forward goes to attn_rows_kernel.
-bool use_rows_kernel(int in_type, int mode, const AttnParams& p) {
-    (void)in_type;
-    if (exact_poly_eighths(mode) > 0 || p.tau > 0.0f) return false;
-    return static_cast<long long>(p.Sq) * p.group <= 64;
+// CTAs per (batch, key/value head) for a forward that goes to attn_rows_kernel, 0 for one that does not: it has too many rows,
+// a mode the kernel is not built for, or no cluster fits the device.
+int plan_attn_rows(int D, int in_type, int mode, const AttnParams& p) {
+    if (exact_poly_eighths(mode) > 0 || p.tau > 0.0f || static_cast<long long>(p.Sq) * p.group > 64) return 0;
+    int cs = 0;
+    with_rows_launcher(D, in_type, p.Sq * p.group, [&](auto l) { cs = decltype(l)::plan(p); });
+    return cs;
 }
 
-cudaError_t launch_attn_rows(int D, int in_type, int mode, const CUtensorMap& tk, const CUtensorMap& tv, const void* q,
+cudaError_t launch_attn_rows(int D, int in_type, int mode, int cs, const CUtensorMap& tk, const CUtensorMap& tv, const void* q,
                              const AttnParams& p, cudaStream_t stream) {
-    if (D == 128) {
-        if (in_type == kInBF16) return dispatch_rows<128, kInBF16>(mode, tk, tv, q, p, stream);
-        if (in_type == kInFP16) return dispatch_rows<128, kInFP16>(mode, tk, tv, q, p, stream);
-        return dispatch_rows<128, kInFP8>(mode, tk, tv, q, p, stream);
-    }
-    if (in_type == kInBF16) return dispatch_rows<64, kInBF16>(mode, tk, tv, q, p, stream);
-    if (in_type == kInFP16) return dispatch_rows<64, kInFP16>(mode, tk, tv, q, p, stream);
-    return dispatch_rows<64, kInFP8>(mode, tk, tv, q, p, stream);
+    cudaError_t e = cudaErrorInvalidValue;
+    with_rows_launcher(D, in_type, p.Sq * p.group, [&](auto l) { e = decltype(l)::launch(mode, cs, tk, tv, q, p, stream); });
+    return e;
 }
 
 }  // namespace rowmax
