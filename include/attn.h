@@ -190,13 +190,26 @@ int attn_get_schedule(int D, int in_dtype, int weight_mode, int causal,
                       int* pot_kmax, int* p_format, int* p_offset_log2);
 
 /*
+ * attn_get_plan — which kernel attn_fwd (or attn_fwd_pot) would take for a shape on the current device, and how many CTAs
+ * would share a piece of its work.  The order in which fp32 sums are added follows from it, so O and LSE may differ in their
+ * last bits between devices with other SM counts.
+ *   kernel  ATTN_KERNEL_PLAIN: one CTA takes a pair of query tiles (ctas = 1); ATTN_KERNEL_SHARED: fewer such pairs than SMs,
+ *           ctas CTAs share one; ATTN_KERNEL_FEW_ROWS: few query rows per key/value head, ctas CTAs share a head
+ */
+#define ATTN_KERNEL_PLAIN 0
+#define ATTN_KERNEL_SHARED 1
+#define ATTN_KERNEL_FEW_ROWS 2
+int attn_get_plan(int B, int Hq, int Hkv, int Sq, int Sk, int D, int causal, int weight_mode, int in_dtype,
+                  int* kernel, int* ctas);
+
+/*
  * Device-side waits and the status word.  (No counterpart in the paper: safety net of the mbarrier / TMEM pipeline.)
  * Every wait inside the kernels is bounded (about one second).  A wait that runs out writes a code, role << 8 |
  * barrier id, into one status word per device, and the kernel winds down: the roles leave their loops, copies and
  * MMAs in flight are awaited with a bound, nothing more is stored, TMEM is released.  No trap, no hang.
  * The word is STICKY: it stays set across launches until attn_device_status_reset.  While it is set, attn_fwd,
  * attn_fwd_tau and attn_fwd_pot still return ATTN_OK (they are asynchronous and do not read the word), but their
- * kernels return at once WITHOUT writing o or lse.  So: after a batch of launches call attn_device_status; on
+ * kernels end WITHOUT writing o or lse, and without waiting for anything.  So: after a batch of launches call attn_device_status; on
  * ATTN_ERR_TIMEOUT treat every output since the last clean check as invalid, reset, and launch again.
  *   attn_device_status        synchronises the current device; ATTN_OK, ATTN_ERR_TIMEOUT (the word is set), or
  *                             ATTN_ERR_CUDA

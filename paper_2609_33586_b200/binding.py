@@ -15,6 +15,7 @@ import torch
 W_EXACT, W_POT, W_H15, W_H15K2, W_H15K3, W_EXACT_POLY = 0, 1, 2, 3, 4, 5
 IN_BF16, IN_FP8_E4M3, IN_FP16 = 0, 1, 2
 P_BF16, P_E4M3, P_E5M2, P_FP16 = 0, 1, 2, 3
+KERNEL_PLAIN, KERNEL_SHARED, KERNEL_FEW_ROWS = 0, 1, 2
 MODES = {"exact": W_EXACT, "pot": W_POT, "h15": W_H15, "h15k2": W_H15K2, "h15k3": W_H15K3,
          "exact_poly": W_EXACT_POLY}
 
@@ -22,7 +23,7 @@ _LIB_PATH = Path(__file__).resolve().parent / "libattn_b200.so"
 _lib = None
 _forward = None      # _host.forward, once attn_fwd has been called
 
-EXPORTS = ("attn_fwd", "attn_fwd_tau", "attn_fwd_pot", "attn_fwd_exact_emulated", "attn_weight_map", "attn_weight_map_pot", "attn_weight_map_fused", "attn_get_schedule", "attn_device_status",
+EXPORTS = ("attn_fwd", "attn_fwd_tau", "attn_fwd_pot", "attn_fwd_exact_emulated", "attn_weight_map", "attn_weight_map_pot", "attn_weight_map_fused", "attn_get_schedule", "attn_get_plan", "attn_device_status",
            "attn_device_status_code", "attn_selftest_wait", "attn_device_status_reset", "attn_launch_count", "attn_status_string",
            "attn_last_cuda_error", "attn_version")
 
@@ -58,6 +59,8 @@ def lib() -> ctypes.CDLL:
         L.attn_weight_map_fused.argtypes = [vp, vp, ctypes.c_size_t, i, i, i, i, vp]
         L.attn_get_schedule.restype = i
         L.attn_get_schedule.argtypes = [i, i, i, i] + [vp] * 7
+        L.attn_get_plan.restype = i
+        L.attn_get_plan.argtypes = [i] * 9 + [vp] * 2
         L.attn_device_status.restype = i
         L.attn_device_status_code.restype = i
         L.attn_selftest_wait.restype = i
@@ -136,6 +139,15 @@ def get_schedule(D: int, in_dtype: int, weight_mode: int, causal: bool) -> dict:
     return {"tile_m": ints[0].value, "tile_n": ints[1].value, "kv_order": ints[2].value,
             "rescale_tau": tau.value, "pot_kmax": ints[3].value, "p_format": ints[4].value,
             "p_offset_log2": ints[5].value}
+
+
+def get_plan(B: int, Hq: int, Hkv: int, Sq: int, Sk: int, D: int, causal: bool, weight_mode: int, in_dtype: int) -> tuple[int, int]:
+    """(kernel, CTAs that share a piece of work) of attn_fwd for a shape on the current device: KERNEL_PLAIN, _SHARED, _FEW_ROWS."""
+    kernel, ctas = ctypes.c_int(), ctypes.c_int()
+    rc = lib().attn_get_plan(B, Hq, Hkv, Sq, Sk, D, int(causal), weight_mode, in_dtype, ctypes.addressof(kernel), ctypes.addressof(ctas))
+    if rc != 0:
+        raise AttnError(rc, "attn_get_plan")
+    return kernel.value, ctas.value
 
 
 def _stream_ptr(stream) -> int:

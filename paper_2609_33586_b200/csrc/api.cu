@@ -132,6 +132,23 @@ void attn_set_trace(long long* device_buffer, int block) {
 
 namespace {
 
+struct Plan {
+    int kernel, ctas;
+};
+// Which kernel a forward takes; `mode` is the kernel's.
+Plan make_plan(int D, int in_dtype, int mode, const rowmax::AttnParams& p) {
+    if (const int cs = rowmax::plan_attn_rows(D, in_dtype, mode, p)) return {ATTN_KERNEL_FEW_ROWS, cs};
+    const int parts = rowmax::plan_attn_split(D, in_dtype, mode, p);
+    return {parts > 1 ? ATTN_KERNEL_SHARED : ATTN_KERNEL_PLAIN, parts};
+}
+
+int check_shape(int B, int Hq, int Hkv, int Sq, int Sk, int D) {
+    if (B <= 0 || Hq <= 0 || Hkv <= 0 || Sq <= 0 || Sk <= 0 || Hq % Hkv != 0) return ATTN_ERR_BAD_SHAPE;
+    if (D != 64 && D != 128) return ATTN_ERR_BAD_SHAPE;
+    if (B > 65535 || Hq > 65535) return ATTN_ERR_BAD_SHAPE;  // grid y/z limits
+    return static_cast<long long>(Sq) + Sk >= (1ll << 30) ? ATTN_ERR_BAD_SHAPE : ATTN_OK;
+}
+
 // Every forward entry point ends here.  pot_kmax / pot_drop_tail matter in ATTN_W_POT mode only.
 int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, int B, int Hq, int Hkv, int Sq,
              int Sk, int D, int causal, float softmax_scale, int weight_mode, int in_dtype, float q_descale,
@@ -140,10 +157,7 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     if (!q || !k || !v || !o) return ATTN_ERR_NULLPTR;
     if (weight_mode < ATTN_W_EXACT || weight_mode > ATTN_W_EXACT_POLY) return ATTN_ERR_BAD_ENUM;
     if (in_dtype != ATTN_IN_BF16 && in_dtype != ATTN_IN_FP8_E4M3 && in_dtype != ATTN_IN_FP16) return ATTN_ERR_BAD_ENUM;
-    if (B <= 0 || Hq <= 0 || Hkv <= 0 || Sq <= 0 || Sk <= 0 || Hq % Hkv != 0) return ATTN_ERR_BAD_SHAPE;
-    if (D != 64 && D != 128) return ATTN_ERR_BAD_SHAPE;
-    if (B > 65535 || Hq > 65535) return ATTN_ERR_BAD_SHAPE;  // grid y/z limits
-    if (static_cast<long long>(Sq) + Sk >= (1ll << 30)) return ATTN_ERR_BAD_SHAPE;
+    if (const int bad = check_shape(B, Hq, Hkv, Sq, Sk, D)) return bad;
     const bool fp8 = in_dtype == ATTN_IN_FP8_E4M3;
     if (!(softmax_scale > 0.f) || !std::isfinite(softmax_scale)) return ATTN_ERR_BAD_VALUE;
     if (fp8 && (!(q_descale > 0.f) || !(k_descale > 0.f) || !(v_descale > 0.f) || !std::isfinite(q_descale) ||
@@ -199,13 +213,13 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     if ((rc = make_tile_map(&tk, k, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
     if ((rc = make_tile_map(&tv, v, fp8, half_in, B, Sk, Hkv, D)) != ATTN_OK) return rc;
     cudaError_t e;
-    if (const int cs = rowmax::plan_attn_rows(D, in_dtype, kernel_mode, p)) {
-        e = rowmax::launch_attn_rows(D, in_dtype, kernel_mode, cs, tk, tv, q, p, static_cast<cudaStream_t>(stream));
+    const Plan plan = make_plan(D, in_dtype, kernel_mode, p);
+    if (plan.kernel == ATTN_KERNEL_FEW_ROWS) {
+        e = rowmax::launch_attn_rows(D, in_dtype, kernel_mode, plan.ctas, tk, tv, q, p, static_cast<cudaStream_t>(stream));
     } else {
         if ((rc = make_tile_map(&tq, q, fp8, half_in, B, Sq, Hq, D)) != ATTN_OK) return rc;
-        const int parts = rowmax::plan_attn_split(D, in_dtype, kernel_mode, p);
         if (p.tau > 0.0f) e = rowmax::launch_attn_fwd_tau(D, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
-        else if (parts > 1) e = rowmax::launch_attn_fwd_split(D, in_dtype, kernel_mode, parts, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
+        else if (plan.kernel == ATTN_KERNEL_SHARED) e = rowmax::launch_attn_fwd_split(D, in_dtype, kernel_mode, plan.ctas, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
         else e = rowmax::launch_attn_fwd(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
     }
     if (e != cudaSuccess) {
@@ -309,6 +323,22 @@ int attn_get_schedule(int D, int in_dtype, int weight_mode, int causal, int* til
     const bool e4m3 = weight_mode == ATTN_W_EXACT || weight_mode == ATTN_W_EXACT_POLY || weight_mode == ATTN_W_H15K3;
     if (p_format) *p_format = in_dtype == ATTN_IN_FP16 ? ATTN_P_FP16 : !fp8 ? ATTN_P_BF16 : (e4m3 ? ATTN_P_E4M3 : ATTN_P_E5M2);
     if (p_offset_log2) *p_offset_log2 = !fp8 ? 0 : (e4m3 ? 8 : 15);
+    return ATTN_OK;
+}
+
+int attn_get_plan(int B, int Hq, int Hkv, int Sq, int Sk, int D, int causal, int weight_mode, int in_dtype, int* kernel, int* ctas) {
+    if (weight_mode < ATTN_W_EXACT || weight_mode > ATTN_W_EXACT_POLY) return ATTN_ERR_BAD_ENUM;
+    if (in_dtype != ATTN_IN_BF16 && in_dtype != ATTN_IN_FP8_E4M3 && in_dtype != ATTN_IN_FP16) return ATTN_ERR_BAD_ENUM;
+    if (const int bad = check_shape(B, Hq, Hkv, Sq, Sk, D)) return bad;
+    const int rc = check_arch();
+    if (rc != ATTN_OK) return rc;
+    rowmax::AttnParams p{};
+    p.B = B; p.Hq = Hq; p.Hkv = Hkv; p.Sq = Sq; p.Sk = Sk;
+    p.causal = causal != 0;
+    p.group = Hq / Hkv;
+    const Plan plan = make_plan(D, in_dtype, weight_mode, p);
+    if (kernel) *kernel = plan.kernel;
+    if (ctas) *ctas = plan.ctas;
     return ATTN_OK;
 }
 

@@ -39,6 +39,7 @@ def test_host_only_entry_points_work_without_a_gpu():
     assert binding.lib().attn_get_schedule(96, 0, 0, 0, *([None] * 7)) == -2
     # argument validation happens before any CUDA call
     assert binding.attn_fwd_raw(None, None, None, None, None, 1, 1, 1, 1, 1, 64, 0, 1.0, 0, 0, 1, 1, 1, None) == -1
+    assert binding.lib().attn_get_plan(1, 3, 2, 64, 64, 64, 0, 0, 0, None, None) == -2
     assert binding.lib().attn_weight_map(None, None, 0, 2, None) == 0
     assert binding.lib().attn_weight_map(None, None, 4, 2, None) == -1
 

@@ -449,3 +449,66 @@ def test_output_allocations_go_through_the_dispatcher():
     finally:
         torch.use_deterministic_algorithms(False)
         binding.device_status_reset()
+
+
+def test_captured_with_copies_and_joins_around_it():
+    """The three kernels in one graph behind a copy, a fill and a join of two streams, replayed on new inputs."""
+    shapes = [(1, 2, 256, 256), (1, 2, 1, 4000), (1, 2, 300, 8192)]      # plain, few rows, shared items
+
+    def inputs(seed):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        return [[torch.randn(B, s, H, 64, device="cuda", generator=g).to(torch.bfloat16) for s in (Sq, Sk, Sk)] for B, H, Sq, Sk in shapes]
+
+    kw = dict(causal=True, softmax_scale=0.125, weight_mode=orc.W_H15)
+    staged, bufs = inputs(1), [[torch.empty_like(x) for x in qkv] for qkv in inputs(1)]
+    outs = [(torch.empty_like(qkv[0]), torch.empty(1, 2, qkv[0].shape[1], device="cuda")) for qkv in bufs]
+    for qkv in staged:      # set-up of the kernels outside the capture, as a program's first step does it
+        binding.attn_fwd(*qkv, **kw)
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        main = torch.cuda.current_stream()
+        side.wait_stream(main)
+        with torch.cuda.stream(side):
+            for dst, src in zip(bufs[1], staged[1]):
+                dst.copy_(src)
+        for dst, src in zip(bufs[0], staged[0]):
+            dst.copy_(src)
+        outs[0][0].zero_()
+        binding.attn_fwd(*bufs[0], out=outs[0][0], lse=outs[0][1], **kw)
+        main.wait_stream(side)
+        binding.attn_fwd(*bufs[1], out=outs[1][0], lse=outs[1][1], **kw)
+        for dst, src in zip(bufs[2], staged[2]):
+            dst.copy_(src)
+        binding.attn_fwd(*bufs[2], out=outs[2][0], lse=outs[2][1], **kw)
+        binding.attn_fwd(*bufs[0], out=outs[0][0], lse=outs[0][1], **kw)
+    for seed in (2, 3):
+        fresh = inputs(seed)
+        for a, b in zip(staged, fresh):
+            for dst, src in zip(a, b):
+                dst.copy_(src)
+        graph.replay()
+        torch.cuda.synchronize()
+        for qkv, (o, lse) in zip(fresh, outs):
+            want, want_lse = binding.attn_fwd(*qkv, **kw)
+            assert torch.equal(o, want) and torch.equal(lse, want_lse)
+    del graph
+
+
+def test_drawn_sizes_match_the_oracle():
+    """A fixed sample of the ranges that the measured workloads stand for, as far as the oracle is quick on it."""
+    import random
+    from perf import cases
+    rng = random.Random(20)
+    kernels = set()
+    for n in range(24):
+        c = cases.draw(rng)
+        while cases.work(c)["flops"] > 6e9:
+            c = cases.draw(rng)
+        wl = Workload(f"drawn_{n}", c["B"], c["Hq"], c["Hkv"], c["Sq"], c["Sk"], c["D"], c["causal"], c["dtype"], 200 + n, peaked_keys=c["peaked"])
+        mode = binding.MODES[c["mode"]]
+        rows = sorted({0, 1, wl.Sq // 3, wl.Sq // 2, max(0, wl.Sq - 129), wl.Sq - 1} & set(range(wl.Sq)))
+        st = compare(wl, mode, rows=rows, allow_output_rounding=True, model_p_storage=True)
+        assert st["ok"], (c, st)
+        dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
+        kernels.add(binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)[0])
+    assert kernels == {binding.KERNEL_PLAIN, binding.KERNEL_SHARED, binding.KERNEL_FEW_ROWS}

@@ -41,6 +41,8 @@ def _device_status_is_clean():
 @pytest.mark.parametrize("mode", ALL)
 @pytest.mark.parametrize("wl", SHAPES, ids=lambda w: w.name)
 def test_few_rows_match_the_oracle(wl, mode):
+    dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
+    assert binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)[0] == binding.KERNEL_FEW_ROWS
     st = compare(wl, mode, model_p_storage=True)
     assert st["ok"], st
 
@@ -74,3 +76,15 @@ def test_few_rows_nothing_is_stored_while_the_status_word_is_set():
     binding.attn_fwd(q, k, k, causal=True, softmax_scale=0.1, weight_mode=orc.W_H15, out=out, lse=lse)
     torch.cuda.synchronize()
     assert torch.all(out != 7.0)
+
+
+@pytest.mark.parametrize("key", [100, 4000, 8190])
+@pytest.mark.parametrize("rows", [1, 20, 50])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16, torch.float8_e4m3fn])
+def test_few_rows_show_a_score_that_is_no_number(dtype, rows, key):
+    g = torch.Generator(device="cuda").manual_seed(6)
+    q, k, v = (torch.randn(1, s, 2, 128, device="cuda", generator=g) for s in (rows, 8192, 8192))
+    k[0, key, 0, 3] = float("nan")
+    o, lse = binding.attn_fwd(q.to(dtype), k.to(dtype), v.to(dtype), causal=False, softmax_scale=0.0625, weight_mode=orc.W_EXACT)
+    assert torch.isnan(o[0, :, 0]).all() and torch.isneginf(lse[0, 0]).all()
+    assert torch.isfinite(o[0, :, 1]).all() and torch.isfinite(lse[0, 1]).all()
