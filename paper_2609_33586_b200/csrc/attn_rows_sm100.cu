@@ -708,9 +708,10 @@ struct RowsLauncher {
     static int plan(const AttnParams& p) {
         int dev = 0, sms = 0;
         if (device_and_sms(&dev, &sms) != cudaSuccess) return 0;
-        const RowsShape s{static_cast<double>(p.B) * p.Hkv, (p.Sk + kTileN - 1) / kTileN, N, kTile};
+        const RowsShape s{static_cast<double>(p.B) * p.Hkv, (p.Sk + kTileN - 1) / kTileN, N, kTile, static_cast<double>(p.B) * p.Hq, p.Sq * p.group, D};
         const int cs = rows_cluster_size(s, sms, [&](int c) { return fit(dev, c); });
-        return static_cast<long long>(p.B) * p.Hkv * cs > 0x7fffffffLL ? 0 : cs;
+        if (cs == 0 || static_cast<long long>(p.B) * p.Hkv * cs > 0x7fffffffLL) return 0;
+        return rows_pay(s, cs, sms) ? cs : 0;
     }
     static cudaError_t launch(int mode, int cs, const CUtensorMap& tk, const CUtensorMap& tv, const void* q, const AttnParams& p,
                               cudaStream_t stream) {
@@ -757,7 +758,7 @@ void with_rows_launcher(int D, int in_type, int rows, F f) {
 }  // namespace
 
 // CTAs per (batch, key/value head) for a forward that goes to attn_rows_kernel, 0 for one that does not: it has too many rows,
-// a mode the kernel is not built for, or no cluster fits the device.
+// a mode the kernel is not built for, no cluster fits the device, or the general path is the faster one (plan.h).
 int plan_attn_rows(int D, int in_type, int mode, const AttnParams& p) {
     if (exact_poly_eighths(mode) > 0 || p.tau > 0.0f || static_cast<long long>(p.Sq) * p.group > 64) return 0;
     int cs = 0;

@@ -27,10 +27,39 @@ int main() {
             CHECK(rows_clusters(n, cs, 0, 148) == 0, "cluster of %d", cs);
             CHECK(rows_clusters(n, cs, 296, 148) == (n == 64 ? 296 : 592), "cluster of %d", cs);
             if (n < 64 && 136 % cs == 0 && cs <= 8) CHECK(rows_clusters(n, cs, 2, 148) == 2 * rows_clusters(n, cs, 1, 74), "cluster of %d", cs);
-            CHECK(rows_cluster_size({8, 64, n, 32768}, 148, [](int) { return 0; }) == 0, "nothing fits");
-            const int got = rows_cluster_size({8, 3, n, 32768}, 148, [](int c) { return 148 / c; });
+            CHECK(rows_cluster_size({8, 64, n, 32768, 8, n, 128}, 148, [](int) { return 0; }) == 0, "nothing fits");
+            const int got = rows_cluster_size({8, 3, n, 32768, 8, n, 128}, 148, [](int c) { return 148 / c; });
             CHECK(got >= 1 && got <= 3, "%d CTAs for 3 key tiles", got);
         }
+    // Measured (us, few-row kernel with that cluster size and plain form): the faster one is taken.
+    const struct { RowsShape s; int cs; double rows_us, plain_us; } measured[] = {
+        {{32, 1, 16, 32768, 32, 16, 128}, 1, 10.7, 5.2},
+        {{4, 1, 16, 16384, 16, 4, 128}, 1, 7.1, 4.4},
+        {{64, 1, 16, 8192, 64, 4, 64}, 1, 6.7, 4.6},
+        {{2048, 1, 16, 8192, 2048, 11, 64}, 1, 62.6, 48.0},
+        {{8, 1, 32, 16384, 8, 32, 128}, 1, 12.7, 4.5},
+        {{1, 1, 32, 16384, 8, 24, 64}, 1, 9.3, 4.3},
+        {{128, 2, 32, 32768, 128, 24, 128}, 2, 12.4, 7.5},
+        {{256, 1, 32, 16384, 256, 24, 128}, 1, 12.9, 9.8},
+        {{1024, 1, 64, 32768, 1024, 64, 128}, 1, 173.7, 33.2},
+        {{96, 1, 64, 16384, 96, 40, 64}, 1, 14.5, 4.8},
+        {{128, 3, 64, 16384, 128, 33, 128}, 1, 19.6, 9.0},
+        {{256, 1, 64, 16384, 1024, 44, 128}, 1, 35.9, 27.2},
+        {{32, 95, 16, 16384, 256, 8, 128}, 8, 20.4, 228.6},
+        {{256, 1, 16, 8192, 1024, 12, 64}, 1, 9.3, 25.2},
+        {{512, 10, 16, 16384, 512, 1, 128}, 1, 38.0, 62.6},
+        {{8, 6, 16, 16384, 32, 12, 128}, 6, 8.7, 11.3},
+        {{256, 30, 32, 8192, 1024, 32, 64}, 1, 66.9, 236.9},
+        {{64, 25, 32, 32768, 256, 32, 128}, 4, 28.2, 76.3},
+        {{128, 1, 32, 32768, 768, 24, 128}, 1, 12.4, 21.6},
+        {{16, 8, 32, 16384, 16, 24, 128}, 8, 10.1, 13.7},
+        {{64, 63, 64, 32768, 4096, 64, 128}, 2, 99.9, 2769.4},
+        {{4, 35, 64, 16384, 256, 64, 128}, 12, 18.7, 89.9},
+        {{16, 2, 64, 16384, 1024, 64, 64}, 2, 14.4, 25.4},
+        {{128, 2, 64, 16384, 768, 48, 64}, 1, 16.7, 25.4},
+    };
+    for (const auto& m : measured)
+        CHECK(rows_pay(m.s, m.cs, 148) == (m.rows_us < m.plain_us), "%g groups of %d rows, %d key tiles: %.1f us, plain %.1f us", m.s.groups, m.s.rows, m.s.nt, m.rows_us, m.plain_us);
     std::puts("ok");
     return 0;
 }

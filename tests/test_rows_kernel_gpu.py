@@ -25,10 +25,16 @@ SHAPES = [
     Workload("rows_64", 1, 32, 8, 16, 1500, 128, True, "fp8_e4m3", 88),
     Workload("rows_without_keys", 1, 2, 1, 20, 9, 64, True, "fp16", 89),
     Workload("many_groups", 10, 32, 32, 2, 300, 64, True, "bf16", 90),   # more (batch, head) pairs than SMs
+    Workload("one_tile_many_heads", 32, 32, 8, 3, 100, 64, True, "fp8_e4m3", 96),
+    Workload("no_keys_many_heads", 32, 32, 8, 3, 2, 64, True, "bf16", 97),
+    Workload("rows_33_of_many", 40, 66, 2, 1, 260, 128, True, "fp16", 98),
     Workload("rounds_n16", 1, 1, 1, 1, 70001, 64, True, "bf16", 91),     # more than 16 x 32 key tiles
     Workload("rounds_n64", 1, 4, 1, 15, 17000, 128, True, "bf16", 92),   # more than 16 x 8
     Workload("rounds_n32_fp8", 1, 8, 1, 4, 40000, 128, True, "fp8_e4m3", 93),
 ]
+
+# Shapes that the few-row kernel could take, of so few keys that the plain form is faster.
+PLAIN = {"one_key", "one_tile", "tile_plus_one", "rows_32_full", "rows_without_keys"}
 
 
 @pytest.fixture(autouse=True)
@@ -42,7 +48,8 @@ def _device_status_is_clean():
 @pytest.mark.parametrize("wl", SHAPES, ids=lambda w: w.name)
 def test_few_rows_match_the_oracle(wl, mode):
     dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
-    assert binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)[0] == binding.KERNEL_FEW_ROWS
+    kernel, _ = binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)
+    assert kernel == (binding.KERNEL_PLAIN if wl.name in PLAIN else binding.KERNEL_FEW_ROWS), wl.name
     st = compare(wl, mode, model_p_storage=True)
     assert st["ok"], st
 
