@@ -13,6 +13,9 @@ resident in HBM for `value`; the `e2e` figure repeats the step from pinned host 
 copies inside the timed region.  With N > 1 (one process per GPU under torchrun) every rank runs an
 independent replica of the workload: the operator has no exchange step.
 
+The result is one short JSON line on stdout; the figures of the other workloads and modes and the energy leg
+are one long line on stderr before it ("bench detail {...}").
+
     python bench.py --workload NAME --modes exact,h15 --launches 2
 
 runs one workload of the matrix a few times and prints its device time (for profilers).
@@ -258,6 +261,20 @@ def workload_config(wl: Workload):
             "l2": "Q+K+V+O = 168 MB per step exceeds the 126 MB L2; no explicit flush"}
 
 
+# What the result line leaves to the detail line: tens of kilobytes, of which a reader of the last lines would see a piece.
+DETAIL_KEYS = ("modes", "energy")
+
+
+def print_result(line: dict) -> None:
+    """The detail (every mode of every workload, energy) as one JSON line on stderr, then the result on stdout, short."""
+    detail = {k: line[k] for k in DETAIL_KEYS if k in line}
+    print("bench detail " + json.dumps(detail), file=sys.stderr, flush=True)
+    short = {k: v for k, v in line.items() if k not in DETAIL_KEYS}
+    short["speedup_over_exact_pct"] = {name: entry["modes"]["h15"]["speedup_over_exact_pct"]
+                                       for name, entry in line.get("modes", {}).items() if name in (HEADLINE.name, TWIN.name)}
+    print(json.dumps(short), flush=True)
+
+
 class DeviceRun:
     def __init__(self, wl: Workload, inp, device):
         from paper_2609_33586_b200 import binding
@@ -500,7 +517,7 @@ def run_ours(args):
     if rank == 0:
         if world == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_baseline_leg(wl, inp)
-        print(json.dumps(line), flush=True)
+        print_result(line)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()

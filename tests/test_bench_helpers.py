@@ -1,4 +1,5 @@
 """Host-side helpers of bench.py that need no GPU: the timing matrix and the roofline arithmetic."""
+import json
 import sys
 from pathlib import Path
 
@@ -44,3 +45,21 @@ def test_roofline_fractions():
     assert out["exact"]["frac_mufu"] == pytest.approx(bound_ms / ms, rel=1e-6)
     assert out["exact"]["roofline_frac"] == max(out["exact"]["frac_tensor_burst"], out["exact"]["frac_mufu"])
     assert out["exact_poly_25"]["mufu_bound_ms"] == pytest.approx(0.75 * bound_ms, rel=1e-6)
+
+
+def test_the_result_line_is_short_and_comes_last(capsys):
+    mode = {"ms": 0.123456789012345, "tflops": 1234.56789012345, "speedup_over_exact_pct": 7.25, "frac": 0.4567890123456789}
+    entry = {"modes": {m: dict(mode, ms_windows=[0.1] * 21) for m in bench.MODE_IDS}}
+    contract = {"metric": bench.METRIC, "value": 1583.0123456789, "unit": "TFLOP/s", "n_gpus": 1, "steps": 20, "warmup": 5,
+                "ms_per_step": 0.34721234567, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "fp8_e4m3",
+                "data": "synthetic", "config": bench.workload_config(bench.HEADLINE), "clocks": {"sm_mhz": 1815.0, "sm_max_mhz": 1965.0, "reasons": []},
+                "gpu_launches": 20, "cpu_baseline": {"rows": 3}, "e2e": {"value": 160.123456789, "unit": "TFLOP/s", "ms_per_step": 3.43512345, "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 2}}
+    names = [bench.HEADLINE.name, bench.TWIN.name] + [n for n, _, _ in bench.matrix_workloads()]
+    bench.print_result(dict(contract, modes={n: entry for n in names}, energy={"h15": mode}))
+    got = capsys.readouterr()
+    assert got.out.count("\n") == 1 and len(got.out) < 2000
+    line = json.loads(got.out)
+    assert {k: line[k] for k in contract} == contract and "modes" not in line
+    assert line["speedup_over_exact_pct"] == {bench.HEADLINE.name: 7.25, bench.TWIN.name: 7.25}
+    detail = json.loads(got.err.split("bench detail ", 1)[1])
+    assert set(detail) == {"modes", "energy"} and set(detail["modes"]) == set(names)
