@@ -263,8 +263,8 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
     griddep_wait();
     griddep_launch();
     if constexpr (SPLIT) {
-        // The others of the cluster reach into this CTA's shared memory: every CTA takes all steps, with waits that return at
-        // once if the flag is set, and leaves with the cluster.
+        // The others of the cluster reach into this CTA's shared memory: every CTA takes all steps, with waits that end soon
+        // if the flag is set, and leaves with the cluster.
         cluster_arrive();
         cluster_wait();
     } else if (flag_is_set(leave_at)) {

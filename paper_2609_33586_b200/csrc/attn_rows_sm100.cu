@@ -296,7 +296,7 @@ attn_rows_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     tc_fence_after();
     griddep_wait();
     griddep_launch();
-    // The status word is sticky: while it is set every wait returns at once and nothing is stored.  All CTAs of the
+    // The status word is sticky: while it is set every wait ends soon and nothing is stored.  All CTAs of the
     // cluster still take every step, because the others read their shared memory.
     if (tid == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) write_flag(abort_at, 1);
     cluster_arrive();       // barriers are initialised; waited for before the first remote access and at the end

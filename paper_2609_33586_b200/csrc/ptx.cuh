@@ -37,6 +37,7 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 // One try_wait with a suspend-time hint: the hardware parks the thread until the phase completes or
 // the hint (in nanoseconds) runs out, so a waiting warp does not burn issue slots polling.
 constexpr uint32_t kSuspendHintNs = 1000000u;
+template <uint32_t kHintNs = kSuspendHintNs>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -44,19 +45,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
-        : "memory");
-    return ok != 0;
-}
-// One look that does not park the thread.
-__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
+        : "r"(bar), "r"(parity), "r"(kHintNs)
         : "memory");
     return ok != 0;
 }
@@ -101,15 +90,17 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const W
 
 // The same bound with a loop that polls the barrier (its hint parks the warp until the phase completes) and looks at
 // the status word only now and then: for kernels whose hand-offs are on the critical path and whose tensor-core operand
-// traffic is light.  The CTA's flag is looked at before the warp is parked and after each turn: with the flag set, a wait for
-// a phase that will not complete returns at once (a turn may park for the whole hint, a millisecond).
+// traffic is light.  The CTA's flag is looked at after each turn, and a turn parks for 20 us at most: so long lasts a wait for
+// a phase that will not complete once the flag is set.  (A look at the barrier and the flag before the first turn cost 512 queries on
+// 16K 4 us of 167.)
+constexpr uint32_t kPollHintNs = 20000u;
 __device__ __forceinline__ void mbar_wait_poll(uint32_t bar, uint32_t parity, const WaitCtx& ctx, int code) {
-    if (mbar_test_wait(bar, parity) || flag_is_set(ctx.cta_abort)) return;
+    if (mbar_try_wait<kPollHintNs>(bar, parity)) return;
     const long long t0 = clock64();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait(bar, parity) || flag_is_set(ctx.cta_abort)) return;
+            if (flag_is_set(ctx.cta_abort) || mbar_try_wait<kPollHintNs>(bar, parity)) return;
         if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
             write_flag(ctx.cta_abort, 1);
             atomicCAS(ctx.global_status, 0, code);
@@ -170,29 +161,18 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
         "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(kSuspendHintNs)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ bool mbar_test_wait_cluster(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
+        : "r"(bar), "r"(parity), "r"(kPollHintNs)
         : "memory");
     return ok != 0;
 }
 // mbar_wait_poll for phases that other CTAs of the cluster complete.
 __device__ __forceinline__ void mbar_wait_cluster(uint32_t bar, uint32_t parity, const WaitCtx& ctx, int code) {
-    if (mbar_test_wait_cluster(bar, parity) || flag_is_set(ctx.cta_abort)) return;
+    if (mbar_try_wait_cluster(bar, parity)) return;
     const long long t0 = clock64();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait_cluster(bar, parity) || flag_is_set(ctx.cta_abort)) return;
+            if (flag_is_set(ctx.cta_abort) || mbar_try_wait_cluster(bar, parity)) return;
         if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
             write_flag(ctx.cta_abort, 1);
             atomicCAS(ctx.global_status, 0, code);

@@ -78,8 +78,8 @@ def test_launches_queued_behind_the_expiring_one_store_nothing(wl):
     Workload("few_rows", 1, 8, 1, 1, 70001, 128, True, "bf16", 86),
     Workload("shared_items", 1, 2, 2, 300, 16384, 128, True, "bf16", 87)], ids=lambda w: w.name)
 def test_cluster_kernels_store_nothing_and_do_not_linger_while_the_word_is_set(wl):
-    """They take all their steps whatever the word says, and no wait of theirs may last: the limit is fifty turns of a parked
-    wait (a millisecond each at most), the steps number hundreds."""
+    """They take all their steps whatever the word says, and no wait of theirs may last: a few hundred waits one after the
+    other, each of which parks for 20 us at most."""
     q = torch.randn(wl.B, wl.Sq, wl.Hq, wl.D, device="cuda").to(torch.bfloat16)
     k = torch.randn(wl.B, wl.Sk, wl.Hkv, wl.D, device="cuda").to(torch.bfloat16)
     kw = dict(causal=True, softmax_scale=wl.softmax_scale, weight_mode=orc.W_H15)
