@@ -6,7 +6,10 @@
 #include <Python.h>
 
 #include <ATen/core/Tensor.h>
+#include <ATen/Context.h>
+#include <ATen/cuda/EmptyTensor.h>
 #include <ATen/ops/empty.h>
+#include <c10/core/impl/TorchDispatchModeTLS.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -83,6 +86,14 @@ void* data_of(PyObject* o) {
     return p;
 }
 
+// An output tensor.  The allocation goes past the dispatcher (0.25 us a tensor) unless somebody there would see or change it: a
+// dispatch mode, or the fill of deterministic mode.
+at::Tensor new_output(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& q) {
+    if (c10::impl::TorchDispatchModeTLS::any_modes_set() || at::globalContext().deterministicAlgorithms())
+        return at::empty(sizes, q.options().dtype(type));
+    return at::detail::empty_cuda(sizes, type, q.device(), std::nullopt);
+}
+
 // forward(q, k, v, out | None, lse | None, return_lse, causal, softmax_scale, weight_mode, q_descale, k_descale, v_descale,
 //         kind, option, option2, stream | None) -> (out, lse | None), or the status code of a call that failed.
 // kind: 0 attn_fwd, 1 attn_fwd_tau (option = threshold), 2 attn_fwd_pot (option = K_max, option2 = drop_tail),
@@ -147,7 +158,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor out, lse;
     void *op, *lp = nullptr;
     if (a[3] == Py_None) {
-        out = at::empty({B, Sq, Hq, D}, q.options().dtype(at::kBFloat16));
+        out = new_output({B, Sq, Hq, D}, at::kBFloat16, q);
         op = out.data_ptr();
     } else {
         op = data_of(a[3]);
@@ -155,7 +166,7 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (a[4] != Py_None) {
         lp = data_of(a[4]);
     } else if (return_lse) {
-        lse = at::empty({B, Hq, Sq}, q.options().dtype(at::kFloat));
+        lse = new_output({B, Hq, Sq}, at::kFloat, q);
         lp = lse.data_ptr();
     }
     if (PyErr_Occurred()) return nullptr;

@@ -83,29 +83,28 @@ int rows_cluster_size(const RowsShape& s, int sms, Fit fit) {
 }
 
 // Estimated times (us) of the two kernels that a forward with few rows can take, fitted to 700 measured shapes (1 to 64 rows, 1 to
-// 140 key tiles, 1 to 4096 heads; graph replays): off by 8 % (rms).  The kernels' own work and the reading of K and V overlap, the
-// less the more alike they are; how much is the exponent.
-inline double overlapped(double work_us, double read_us, double e) { return std::pow(std::pow(work_us, e) + std::pow(read_us, e), 1.0 / e); }
+// 140 key tiles, 1 to 4096 heads; graph replays): off by 8 % (rms).  The kernels' own work and the reading of K and V overlap and
+// are added as squares.
 inline double rows_us(const RowsShape& s, int cs, int sms) {
-    struct Fit { double fixed, per_row, per_tile, per_cta, start, rate, e; };
-    const Fit f = s.n == 16 ? Fit{5.41, 0.279, 0.608, 0.220, 1.0, 0.83, 1.5} :
-                  s.n == 32 ? Fit{5.03, 0.204, 1.691, 0.123, 8.0, 1.28, 5.8} : Fit{7.12, 0.200, 2.178, 0.171, 8.0, 1.11, 2.64};
-    const double read_us = 2.0 * s.nt * s.groups * s.tile_bytes / 6.3e6;
+    struct Fit { double fixed, per_row, per_tile, per_cta, start, rate; };
+    const Fit f = s.n == 16 ? Fit{5.35, 0.286, 0.699, 0.213, 1.93, 0.927} :
+                  s.n == 32 ? Fit{5.42, 0.181, 1.393, 0.150, 3.88, 1.118} : Fit{7.05, 0.197, 2.146, 0.161, 6.32, 0.876};
+    const double read_us = f.start + f.rate * 2.0 * s.nt * s.groups * s.tile_bytes / 6.3e6;
     const double places = s.n == 64 ? sms : 2.0 * sms, waves = std::ceil(s.groups * cs / places);
     const double shared = std::fmin(s.groups, std::floor(places / cs)) * cs > sms ? 1.15 : 1.0;
     const double work_us = waves * (f.fixed + f.per_row * s.rows * s.D / 128.0 / cs + f.per_cta * cs + (cs > 8 ? 1.2 : 0.0) +
                                     (s.nt + cs - 1) / cs * f.per_tile * shared);
-    return overlapped(work_us, f.start + f.rate * read_us, f.e);
+    return std::sqrt(work_us * work_us + read_us * read_us);
 }
 inline double plain_us(const RowsShape& s, int sms) {      // one pair of query tiles per head: at most 64 rows
-    const double rounds = std::ceil(s.items / sms);
-    const double work_us = 1.73 + rounds * (1.85 + s.nt * (s.D == 64 ? 1.07 : 1.33)) + (rounds > 1.0 ? 1.49 : 0.0);
-    return overlapped(work_us, 2.32 + 2.0 * s.nt * s.groups * s.tile_bytes / 6.3e6, 2.48);
+    const double rounds = std::ceil(s.items / sms), read_us = 1.49 + 2.0 * s.nt * s.groups * s.tile_bytes / 6.3e6;
+    const double work_us = 1.85 + rounds * (1.83 + s.nt * (s.D == 64 ? 1.05 : 1.30)) + (rounds > 1.0 ? 1.41 : 0.0);
+    return std::sqrt(work_us * work_us + read_us * read_us);
 }
 // Whether the few-row kernel with clusters of cs CTAs is the faster one.  Its epilogue costs 0.2 to 0.28 us for each row of a
 // CTA, which many short heads do not earn back: 1024 heads x 64 rows x 1 key tile 174 us against 33 in the plain form, 32 x 48
 // rows x 1 tile 18.2 against 4.8.  It wins once the keys are read for long enough: 32 groups of 8 rows x 95 tiles 20 against 229.
-// Over the shapes measured the choice costs 0.5 % against always taking the better one, 29 % at most.
-inline bool rows_pay(const RowsShape& s, int cs, int sms) { return plain_us(s, sms) >= 0.97 * rows_us(s, cs, sms); }
+// Over the shapes measured the choice costs 0.6 % against always taking the better one, 29 % at most.
+inline bool rows_pay(const RowsShape& s, int cs, int sms) { return plain_us(s, sms) >= rows_us(s, cs, sms); }
 
 }  // namespace rowmax
