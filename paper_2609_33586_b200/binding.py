@@ -142,7 +142,8 @@ def get_schedule(D: int, in_dtype: int, weight_mode: int, causal: bool) -> dict:
 
 
 def get_plan(B: int, Hq: int, Hkv: int, Sq: int, Sk: int, D: int, causal: bool, weight_mode: int, in_dtype: int) -> tuple[int, int]:
-    """(kernel, CTAs that share a piece of work) of attn_fwd for a shape on the current device: KERNEL_PLAIN, _SHARED, _FEW_ROWS."""
+    """(kernel, CTAs that share a piece of work) of attn_fwd for a shape on the current device: KERNEL_PLAIN, _SHARED, _FEW_ROWS.
+    `in_dtype` is in_dtype_of(q)."""
     kernel, ctas = ctypes.c_int(), ctypes.c_int()
     rc = lib().attn_get_plan(B, Hq, Hkv, Sq, Sk, D, int(causal), weight_mode, in_dtype, ctypes.addressof(kernel), ctypes.addressof(ctas))
     if rc != 0:
