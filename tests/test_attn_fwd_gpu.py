@@ -509,6 +509,38 @@ def test_drawn_sizes_match_the_oracle():
         rows = sorted({0, 1, wl.Sq // 3, wl.Sq // 2, max(0, wl.Sq - 129), wl.Sq - 1} & set(range(wl.Sq)))
         st = compare(wl, mode, rows=rows, allow_output_rounding=True, model_p_storage=True)
         assert st["ok"], (c, st)
-        dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
+        dt = binding.in_dtype_of(torch.empty(0, dtype=cases.DTYPES[wl.in_dtype]))
         kernels.add(binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)[0])
     assert kernels == {binding.KERNEL_PLAIN, binding.KERNEL_SHARED, binding.KERNEL_FEW_ROWS}
+
+
+def test_threads_with_streams_of_their_own():
+    """Four threads, each with its stream and its mix of the three kernels, get what one thread gets."""
+    import threading
+    shapes = [(1, 2, 256, 256), (2, 4, 1, 4000), (1, 2, 300, 8192), (8, 16, 40, 600), (1, 16, 700, 700)]
+    kw = dict(causal=True, softmax_scale=0.125, weight_mode=orc.W_H15)
+    g = torch.Generator(device="cuda").manual_seed(9)
+    inputs = [[torch.randn(B, s, H, 64, device="cuda", generator=g).to(torch.bfloat16) for s in (Sq, Sk, Sk)] for B, H, Sq, Sk in shapes]
+    want = [binding.attn_fwd(*qkv, **kw) for qkv in inputs]
+    torch.cuda.synchronize()
+    wrong = []
+
+    def work(first):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                for n in range(60):
+                    i = (first + n) % len(shapes)
+                    o, lse = binding.attn_fwd(*inputs[i], **kw)
+                    if not (torch.equal(o, want[i][0]) and torch.equal(lse, want[i][1])):
+                        wrong.append((first, n))
+            stream.synchronize()
+        except Exception as e:      # noqa: BLE001  (reported below, in the main thread)
+            wrong.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
