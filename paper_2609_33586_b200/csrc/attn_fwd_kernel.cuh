@@ -66,7 +66,8 @@ struct WsCfg {
 // redistribute that allocation; a larger total would make the increase wait for ever): softmax /
 // correction / MMA+TMA warpgroups.  The softmax warps hold a row of 128 scores; what decides is that no role spills: with
 // 192 / 80 / 48 and a correction that took 32 columns at a time the 16-bit instances spilled in the MMA and correction
-// warps (bf16 8K exact 277.6 against 267.5 us, full-attention fp8 exact 420 against 410); 208 / 48 / 48 spills again (287).
+// warps and were 2 to 4 % slower (bf16 8K exact, full-attention fp8 exact; both in turn on one machine, SM clock not recorded);
+// 208 / 48 / 48 spills again (7 % slower).
 constexpr int kRegSoftmax = 200, kRegCorr = 56, kRegMma = 56;
 static_assert(256 * kRegSoftmax + 128 * kRegCorr + 128 * kRegMma <= 512 * 128, "setmaxnreg targets exceed the launch allocation");
 template <int N> __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }

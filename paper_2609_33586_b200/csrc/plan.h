@@ -21,9 +21,9 @@ struct SplitShape {
 // CTAs per item, 1 for the plain form.  fit(parts): clusters of that size that fit the device at once.  Times are in steps of the
 // loop (one key tile of a pair of query tiles), measured: a part costs its key tiles, with a maxima pass 0.65 of a step more for
 // each tile of its maxima pass (two parts share the pass, so it is half as long), and 4.5 steps + 0.5 per part for the exchange
-// and the sum of O; from two thirds of the SMs on they slow each other by a tenth.  512 queries on 16K, 32/8 heads: bf16 h15
-// 198 -> 154 us, exact 226 -> 138, e4m3 178 -> 125 (2 parts); 64 queries on 8K 97 -> 49 (4 parts).  16 x 1K and 16 x 2K gain
-// nothing and stay whole.
+// and the sum of O; from two thirds of the SMs on they slow each other by a tenth.  512 queries on 16K, 32/8 heads, streams of 40
+// calls: bf16 h15 218 -> 143 us, exact 256 -> 134, e4m3 h15 203 -> 132 (2 parts); 64 queries on 8K e4m3 90 -> 45 (4 parts).
+// 16 x 1K and 16 x 2K gain nothing and stay whole.
 template <class Fit>
 int split_parts(const SplitShape& s, int sms, Fit fit) {
     if (s.items > sms) return 1;
@@ -101,7 +101,7 @@ inline double plain_us(const RowsShape& s, int sms) {      // one pair of query 
     const double work_us = 1.85 + rounds * (1.83 + s.nt * (s.D == 64 ? 1.05 : 1.30)) + (rounds > 1.0 ? 1.41 : 0.0);
     return std::sqrt(work_us * work_us + read_us * read_us);
 }
-// Whether the few-row kernel with clusters of cs CTAs is the faster one.  Its epilogue costs 0.2 to 0.28 us for each row of a
+// Whether the few-row kernel with clusters of cs CTAs is the faster one.  Its epilogue costs 0.18 to 0.29 us for each row of a
 // CTA, which many short heads do not earn back: 1024 heads x 64 rows x 1 key tile 174 us against 33 in the plain form, 32 x 48
 // rows x 1 tile 18.2 against 4.8.  It wins once the keys are read for long enough: 32 groups of 8 rows x 95 tiles 20 against 229.
 // Over the shapes measured the choice costs 0.6 % against always taking the better one, 29 % at most.
