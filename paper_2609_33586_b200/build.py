@@ -13,8 +13,8 @@ PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libattn_b200.so"
 HOST = PKG / f"_host{sysconfig.get_config_var('EXT_SUFFIX')}"
-SOURCES = ["api.cu", "attn_fwd_sm100.cu", "attn_fwd_split_sm100.cu", "attn_fwd_tau_sm100.cu", "attn_rows_sm100.cu"]
-HEADERS = ["ptx.cuh", "kv_ring.cuh", "plan.h", "attn_fwd_kernel.cuh", "weight_map.cuh", "attn_kernel_common.cuh", "softmax_math.cuh", "../../include/attn.h"]
+SOURCES = ["api.cu", "attn_fwd_sm100.cu", "attn_fwd_split_sm100.cu", "attn_fwd_streams_sm100.cu", "attn_fwd_tau_sm100.cu", "attn_rows_sm100.cu"]
+HEADERS = ["ptx.cuh", "kv_ring.cuh", "plan.h", "attn_fwd_kernel.cuh", "attn_streams_kernel.cuh", "weight_map.cuh", "attn_kernel_common.cuh", "softmax_math.cuh", "../../include/attn.h"]
 
 
 def _nvcc() -> str:

@@ -1,0 +1,609 @@
+// Attention forward with one query tile per CTA and two streams of key tiles.
+//
+// The plain form (attn_fwd_kernel.cuh) keeps its two softmax warpgroups busy with two query tiles that share the staged K/V
+// tiles.  Here both work on ONE query tile: key tiles take turns, tile G of the CTA's walk (counted over all its items) belongs
+// to stream G mod 2, which has a softmax warpgroup, a score buffer and an O accumulator of its own.
+//
+// PAIR = false: a work item is one query tile, half as large as an item of the plain form.
+// PAIR = true: two CTAs on neighbouring SMs take a pair of query tiles, one each, and one MMA (cta_group::2, M = 256) works for
+// both.  Of every K tile a CTA holds 64 keys, of every V tile 64 columns: half the K/V traffic into shared memory and half the
+// operand reads of K and V, which are what bounds PAIR = false at 16 bits and D = 128.
+//
+// Semantics are those of the sequential loop: the anchor that tile g starts from is the one tile g - 1 left, handed from
+// warpgroup to warpgroup through shared memory as soon as a tile's row maximum is known, half a period before the other needs it
+// (exact modes on 16-bit inputs need no such hand-over: each stream keeps its own anchor).  Only the sums are kept per stream and
+// joined at the end: O = (a_0 O_0 + a_1 O_1) dv / l with a_t = 2^((m_t - m) c).
+//   warpgroup 0/1  softmax of stream 0/1: one thread per row
+//   warpgroup 2    correction (rescales the accumulators) and epilogue (joins them and stores O)
+//   warp 12        MMA issuer (PAIR: of the first CTA): P V of tile G, then S of tile G + 2, which may be the next item's
+//   warp 13        TMA producer: V(G - 2) and K(G) arrive as one pair of ring slots
+// TMEM columns: S_0/P_0 [0,128), S_1/P_1 [128,256), O_0 [256,384), O_1 [384,512).
+#pragma once
+#include "attn_fwd_kernel.cuh"
+
+namespace rowmax {
+
+namespace {
+
+template <int D, bool FP8, bool PAIR>
+struct StreamsCfg {
+    using C = TileCfg<D, FP8>;
+    static_assert(!PAIR || D == 128, "half a V tile has 64 columns");
+    static constexpr int kPartBytes = C::kTileBytes / (PAIR ? 2 : 1);    // of a K or V tile: what this CTA holds
+    static constexpr int kKeys = PAIR ? kTileN / 2 : kTileN;             // keys of a K tile in this CTA
+    static constexpr int kKBoxBytes = kKeys * C::kSwizzle;
+    static constexpr int kVSwizzle = PAIR ? 64 * C::kElem : C::kSwizzle; // swizzle span of a V row
+    static constexpr int kVBoxes = PAIR ? 1 : C::kBoxes;
+    static constexpr int kQBufs = C::kTileBytes <= 16384 ? 2 : 1;        // query tiles staged
+    static constexpr int kPairs = PAIR ? (FP8 ? 8 : 6) : (C::kTileBytes <= 16384 ? 4 : 3);   // pairs of K/V ring slots
+    static constexpr int kQBytes = kQBufs * C::kTileBytes;
+    static constexpr int kRingBytes = 2 * kPairs * kPartBytes;
+    static constexpr int kScaleOff = kQBytes + kRingBytes;       // float alpha[2][128]
+    static constexpr int kAnchorOff = kScaleOff + 2 * 128 * 4;   // float anchor[128]: of the last tile that has its maximum
+    static constexpr int kFinOff = kAnchorOff + 128 * 4;         // float factor[2][128] of the accumulators (before: m and l of a stream)
+    static constexpr int kBarOff = kFinOff + 2 * 128 * 4;
+    static constexpr int kNumBars = 2 * kPairs + 16;
+    static constexpr int kMiscOff = kBarOff + kNumBars * 8;
+    static constexpr int kCountOff = kMiscOff + 16;              // int done[4], left[4]: per warp of rows
+    static constexpr int kSmemBytes = kCountOff + 32;
+    static_assert(kSmemBytes <= 232448, "exceeds the 227 KB shared memory of an sm_100 CTA");
+};
+
+// Register split (see the plain form).  The softmax warps have no epilogue here, the MMA warp looks two tiles ahead and the
+// correction warps join two accumulators: 200 / 56 / 56 spills in these, 192 / 64 / 64 does not.
+constexpr int kStreamRegSoftmax = 192, kStreamRegOther = 64;
+static_assert(256 * kStreamRegSoftmax + 256 * kStreamRegOther <= 512 * 128, "setmaxnreg targets exceed the launch allocation");
+
+// One work item: this CTA's query tile of one (batch, head), and the key tiles that it goes over (PAIR: the longer walk of both
+// query tiles; a tile beyond a row's keys is masked as a whole).  n = 0: no row sees a key.  Heaviest first, as in the plain form.
+struct StreamItem {
+    int h, b, hk, q0, n;
+};
+template <bool PAIR>
+__device__ __forceinline__ StreamItem decode_stream_item(int w, const AttnParams& p, int n_groups, int bh, int rank) {
+    constexpr int kRows = (PAIR ? 2 : 1) * kTileM;
+    StreamItem it;
+    const int rem = w % bh, first = (n_groups - 1 - w / bh) * kRows;
+    it.h = rem % p.Hq;
+    it.b = rem / p.Hq;
+    it.hk = it.h / p.group;
+    it.q0 = first + rank * kTileM;
+    const int last = PAIR && first + kTileM < p.Sq ? first + kTileM : first;      // the later query tile that exists
+    const int kv_end = p.causal ? min(p.Sk, last + kTileM + p.Sk - p.Sq) : p.Sk;
+    it.n = kv_end > 0 ? (kv_end + kTileN - 1) / kTileN : 0;
+    return it;
+}
+
+// Waits (bounded) until a counter in shared memory has come to `want`.  Counters only grow, so unlike a barrier's phases they
+// can be looked at by whoever needs them, however many steps apart.
+__device__ __forceinline__ void wait_count(uint32_t at, int want, const WaitCtx& ctx, int code) {
+    if (ld_acquire_shared(at) >= want) return;
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i)
+            if (ld_acquire_shared(at) >= want || flag_is_set(ctx.cta_abort)) return;
+        if (*reinterpret_cast<volatile int*>(ctx.global_status) != 0 || clock64() - t0 > ctx.limit_cycles) {
+            write_flag(ctx.cta_abort, 1);
+            atomicCAS(ctx.global_status, 0, code);
+            return;
+        }
+    }
+}
+
+// Stores 16 rows x 32 columns of O as bf16.  `v` is laid out as tcgen05.ld.16x256b.x4 gives it: of each 8 columns lane i has
+// columns 2 (i mod 4) and the next of row i / 4 (v[4k], v[4k + 1]) and of row i / 4 + 8 (v[4k + 2], v[4k + 3]).  The four lanes of
+// a row exchange their words so that each has 16 bytes in a row: a store then takes 8 rows x 64 bytes, whole sectors, where one
+// row per thread takes 32 rows x 16 bytes.  (In the plain form, cross attention of 1337 x 2803: 93.9 -> 90.2 us.)
+__device__ __forceinline__ void store_rows16(const uint32_t (&v)[16], __nv_bfloat16* base, size_t row_stride, int rows, int lane) {
+    const bool odd = lane & 1, upper = lane & 2;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        const int row = (lane >> 2) + 8 * half;
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = pack_bf16_rn(__uint_as_float(v[4 * k + 2 * half]), __uint_as_float(v[4 * k + 2 * half + 1]));
+        // word k of lane j becomes word j of lane k
+        const uint32_t x01 = __shfl_xor_sync(0xffffffffu, odd ? w[0] : w[1], 1), x23 = __shfl_xor_sync(0xffffffffu, odd ? w[2] : w[3], 1);
+        if (odd) { w[0] = x01; w[2] = x23; }
+        else { w[1] = x01; w[3] = x23; }
+        const uint32_t y0 = __shfl_xor_sync(0xffffffffu, upper ? w[0] : w[2], 2), y1 = __shfl_xor_sync(0xffffffffu, upper ? w[1] : w[3], 2);
+        const uint4 pk = upper ? make_uint4(y0, y1, w[2], w[3]) : make_uint4(w[0], w[1], y0, y1);
+        if (row < rows) *reinterpret_cast<uint4*>(base + row * row_stride + 8 * (lane & 3)) = pk;
+    }
+}
+
+}  // namespace
+
+template <int D, int IN, int MODE, bool PAIR>
+__global__ void __launch_bounds__(512, 1)
+attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                        const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
+    constexpr bool FP8 = IN == kInFP8;
+    constexpr bool HALF = IN == kInFP16;
+    using C = TileCfg<D, FP8>;
+    using W = StreamsCfg<D, FP8, PAIR>;
+    constexpr int NP = W::kPairs;
+    constexpr int kCtas = PAIR ? 2 : 1;
+    constexpr bool kOneAnchor = split_takes_maxima(MODE, FP8);     // the streams hand the anchor on
+    constexpr bool kOutOfStep = FP8 && is_exact_like(MODE);
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const uint32_t sQ = smem_u32(smem);
+    const uint32_t sRing = sQ + W::kQBytes;
+    const uint32_t sScale = smem_u32(smem + W::kScaleOff);
+    const uint32_t sAnchor = smem_u32(smem + W::kAnchorOff);
+    const uint32_t sFin = smem_u32(smem + W::kFinOff);
+    const uint32_t bar0 = smem_u32(smem + W::kBarOff);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + W::kMiscOff);
+    const uint32_t abort_at = smem_u32(smem + W::kMiscOff + 4), leave_at = smem_u32(smem + W::kMiscOff + 8);
+    const uint32_t count_done = smem_u32(smem + W::kCountOff), count_left = count_done + 16;
+    const WaitCtx wctx{abort_at, p.status, kWaitLimitCycles};
+
+    // PAIR: the barriers that the MMA warp waits for count the arrivals of both CTAs in the first one's shared memory; what it
+    // commits arrives in both.
+    using Ring = StreamRing<NP>;
+    auto bar_kv_full = [&](int pair) { return bar0 + 8u * Ring::bar(pair); };              // TMA -> MMA: V(G - 2) and K(G)
+    auto bar_kv_empty = [&](int pair) { return bar0 + 8u * (NP + Ring::bar(pair)); };      // MMA -> TMA
+    auto bar_x = [&](int which, int t) { return bar0 + 8u * (2 * NP + 2 * which + t); };
+    auto bar_q_full = [&](int b) { return bar_x(0, b); };      // TMA -> MMA: Q of the item landed
+    auto bar_q_empty = [&](int b) { return bar_x(1, b); };     // MMA -> TMA: last S MMA of the item done
+    auto bar_s_full = [&](int t) { return bar_x(2, t); };      // MMA -> softmax: S(G) is in TMEM
+    auto bar_p_full = [&](int t) { return bar_x(3, t); };      // softmax and correction -> MMA: P(G) is in TMEM, O_t rescaled
+    auto bar_scale = [&](int t) { return bar_x(4, t); };       // softmax -> correction: alpha(G) in shared memory
+    auto bar_anchor = [&](int t) { return bar_x(5, t); };      // softmax -> the other softmax: anchor after tile G
+    const uint32_t bar_o_full = bar_x(6, 0);                   // MMA -> epilogue: the last P V of the item accumulated
+    const uint32_t bar_o_free = bar_x(6, 1);                   // epilogue -> MMA: both accumulators have been read out
+    const uint32_t bar_fin = bar_x(7, 0);                      // softmax -> epilogue: factors of the accumulators
+    const uint32_t bar_drain = bar_x(7, 1);                    // the MMA warp's last commit
+    auto arrive_at_mma = [&](uint32_t bar) {
+        if constexpr (PAIR) mbar_arrive_peer(mapa(bar, 0));
+        else mbar_arrive(bar);
+    };
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
+    if ((smem_u32(smem) & 1023u) != 0) {
+        if (tid == 0) atomicCAS(p.status, 0, (kRoleSetup << 8) | kBarAlign);
+        return;
+    }
+    // As in the plain form one thread (PAIR: of both CTAs) reads the sticky status word, and the CTA or the pair leaves as a whole
+    // if it is set.
+    const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
+    if (tid == 0) {
+        write_flag(abort_at, 0);
+        write_flag(leave_at, rank == 0 ? *reinterpret_cast<volatile int*>(p.status) : 0);
+    }
+    const int n_groups = (p.Sq + kCtas * kTileM - 1) / (kCtas * kTileM);
+    const int bh = p.Hq * p.B;
+    const int n_items = n_groups * bh;
+    const int cta = blockIdx.x / kCtas, n_ctas = gridDim.x / kCtas;      // PAIR: of pairs
+    const int shift = p.Sk - p.Sq;
+
+    if (warp == 13) {
+        if (lane < NP) {
+            mbar_init(bar0 + 8u * lane, 2);            // V(G - 2) and K(G)
+            mbar_init(bar0 + 8u * (NP + lane), 1);
+        } else if (lane >= 16 && lane < 18) {
+            const int t = lane - 16;
+            mbar_init(bar_q_full(t), 1);
+            mbar_init(bar_q_empty(t), 1);
+            mbar_init(bar_s_full(t), 1);
+            mbar_init(bar_p_full(t), 8 * kCtas);      // one arrival per softmax warp, one per correction warp
+            mbar_init(bar_scale(t), 4);
+            mbar_init(bar_anchor(t), 4);
+        } else if (lane == 18) {
+            mbar_init(bar_o_full, 1);
+            mbar_init(bar_o_free, 4 * kCtas);
+            mbar_init(bar_fin, 4);
+            mbar_init(bar_drain, 1);
+        } else if (lane >= 20 && lane < 28) {
+            write_flag(count_done + 4 * (lane - 20), 0);
+        }
+        fence_mbar_init();
+    }
+    constexpr uint32_t kTmemCols = 512;
+    if (warp == 12) tmem_take<PAIR>(smem_u32(tmem_slot), kTmemCols);
+    tc_fence_before();
+    __syncthreads();
+    if constexpr (PAIR) {      // the barriers of both CTAs are there
+        cluster_arrive();
+        cluster_wait();
+    }
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    griddep_wait();        // what follows reads the caller's tensors
+    griddep_launch();
+    if (PAIR ? __float_as_int(ld_cluster_f32(mapa(leave_at, 0))) != 0 : flag_is_set(leave_at)) {
+        if constexpr (PAIR) {
+            cluster_arrive();
+            cluster_wait();
+        }
+        if (warp == 12) tmem_give<PAIR>(tmem, kTmemCols);
+        return;
+    }
+    auto get_item = [&](int w) { return decode_stream_item<PAIR>(w, p, n_groups, bh, rank); };
+    auto tmem_S = [&](int t) { return tmem + 128u * t; };
+    auto tmem_O = [&](int t) { return tmem + 256u + 128u * t; };
+
+    constexpr uint32_t fmt_16 = HALF ? kFmtF16 : kFmtBF16;
+    constexpr uint32_t fmt_ab = FP8 ? kFmtE4M3 : fmt_16;
+    constexpr uint32_t fmt_p = FP8 ? (PFormat<FP8, MODE>::kE4M3 ? kFmtE4M3 : kFmtE5M2) : fmt_16;
+    constexpr uint32_t idesc_s = umma_idesc(fmt_ab, fmt_ab, false, false, kCtas * kTileM, kTileN);
+    constexpr uint32_t idesc_pv = umma_idesc(fmt_p, fmt_ab, false, true, kCtas * kTileM, D);
+    constexpr float p_off = static_cast<float>(PFormat<FP8, MODE>::kOffLog2);
+
+    if (wg == 3) {
+        reg_dec<kStreamRegOther>();
+        if (warp == 13 && lane == 0) {
+            // ------------------------------------------------------------ TMA producer
+            int walked = 0;       // tiles of the walk so far
+            int items = 0;        // items with tiles so far
+            StreamItem it;
+            int v_b[2] = {0, 0}, v_hk[2] = {0, 0}, v_tile[2] = {0, 0};     // the last two tiles, whose V comes with the K of two tiles later
+            // The arrival for copies of `bytes` (PAIR: of both CTAs, by the first one's producer) and the barrier they count on.
+            auto expect = [&](uint32_t bar, uint32_t bytes) {
+                if (rank == 0) mbar_arrive_expect_tx(bar, kCtas * bytes);
+                return PAIR ? mapa(bar, 0) : bar;
+            };
+            int j = 0;
+            // After an expired wait nothing more is loaded (see the plain form).
+            StreamOps ops{[&](int pair) { if (rank == 0) mbar_arrive(bar_kv_full(pair)); },
+                          [&](int pair) {
+                              mbar_wait(bar_kv_empty(pair), Ring::ph_empty(pair), wctx, (kRoleLoad << 8) | kBarKvEmpty);
+                              return !flag_is_set(abort_at);
+                          },
+                          [&](int pair) {      // PAIR: keys 64 * rank .. of the tile
+                              const uint32_t dst = sRing + Ring::slot_k(pair) * W::kPartBytes, bar = expect(bar_kv_full(pair), W::kPartBytes);
+#pragma unroll
+                              for (int bx = 0; bx < C::kBoxes; ++bx)
+                                  group_load_4d<PAIR>(dst + bx * W::kKBoxBytes, &tmK, bar, bx * C::kBoxElems, it.hk, j * kTileN + W::kKeys * rank, it.b);
+                          },
+                          [&](int pair) {      // PAIR: columns 64 * rank .. of the tile
+                              const uint32_t dst = sRing + Ring::slot_v(pair) * W::kPartBytes, bar = expect(bar_kv_full(pair), W::kPartBytes);
+#pragma unroll
+                              for (int bx = 0; bx < W::kVBoxes; ++bx)
+                                  group_load_4d<PAIR>(dst + bx * C::kBoxBytes, &tmV, bar, PAIR ? 64 * rank : bx * C::kBoxElems, v_hk[0], v_tile[0] * kTileN, v_b[0]);
+                          }};
+            bool ok = true;
+            for (int round = 0; ok; ++round) {
+                const int w = item_index(round, cta, n_ctas);
+                if (w >= n_items) break;
+                it = get_item(w);
+                for (j = 0; j < it.n; ++j) {
+                    ok = stream_tile(ops, walked);
+                    if (!ok) break;
+                    ++walked;
+                    v_b[0] = v_b[1]; v_hk[0] = v_hk[1]; v_tile[0] = v_tile[1];
+                    v_b[1] = it.b; v_hk[1] = it.hk; v_tile[1] = j;
+                    if (j == 0) {
+                        const int buf = items % W::kQBufs;
+                        mbar_wait(bar_q_empty(buf), ((items / W::kQBufs) & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarQEmpty);
+                        ok = !flag_is_set(abort_at);
+                        if (!ok) break;
+                        const uint32_t bar = expect(bar_q_full(buf), C::kTileBytes);
+#pragma unroll
+                        for (int bx = 0; bx < C::kBoxes; ++bx)
+                            group_load_4d<PAIR>(sQ + buf * C::kTileBytes + bx * C::kBoxBytes, &tmQ, bar, bx * C::kBoxElems, it.h, it.q0, it.b);
+                        ++items;
+                    }
+                }
+            }
+            // the last two tiles' V
+            int pairs = walked;
+            for (int e = walked; ok && e < walked + 2; ++e) {
+                ok = stream_tail(ops, e);
+                if (ok) pairs = e + 1;
+                v_b[0] = v_b[1]; v_hk[0] = v_hk[1]; v_tile[0] = v_tile[1];
+            }
+            // Every load this thread issued has to land before the CTA ends (see the plain form).  PAIR: the first CTA's barriers
+            // count the copies of both; a second CTA that gave up leaves its copies time to land.
+            if (rank == 0) {
+                for (int pair = pairs > NP ? pairs - NP : 0; pair < pairs; ++pair)
+                    if (stream_pair_is_used(pair, walked)) mbar_wait_quiet(bar_kv_full(pair), Ring::ph_full(pair), kDrainLimitCycles);
+                for (int i = items > W::kQBufs ? items - W::kQBufs : 0; i < items; ++i)
+                    mbar_wait_quiet(bar_q_full(i % W::kQBufs), (i / W::kQBufs) & 1, kDrainLimitCycles);
+            } else if (!ok) {
+                const long long t0 = clock64();
+                while (clock64() - t0 < kDrainLimitCycles / 50) {}
+            }
+        } else if (warp == 12 && rank == 0) {
+            // ------------------------------------------------------------ MMA issuer
+            const bool leader = elect_one();
+            constexpr uint32_t desc_hi = umma_desc_hi_sw(C::kSwizzle), desc_hi_v = umma_desc_hi_sw(W::kVSwizzle);
+            const uint32_t q_lo0 = umma_desc_lo(sQ, 16);
+            const uint32_t ring_lo_k = umma_desc_lo(sRing, 16);               // K tiles: K-major
+            const uint32_t ring_lo_v = umma_desc_lo(sRing, C::kBoxBytes);     // V tiles: MN-major, LBO = next block of columns
+            constexpr uint32_t kTileLo = C::kTileBytes >> 4, kPartLo = W::kPartBytes >> 4;
+            auto issue_s = [&](int t, uint32_t q_lo, uint32_t k_lo) {
+#pragma unroll
+                for (int ks = 0; ks < C::kQkSteps; ++ks) {
+                    const uint32_t box = ks / C::kStepsPerBox, in_row = (ks % C::kStepsPerBox) * 32;
+                    group_mma_ss<PAIR, FP8>(tmem_S(t), q_lo + ((box * C::kBoxBytes + in_row) >> 4), k_lo + ((box * W::kKBoxBytes + in_row) >> 4), desc_hi,
+                                            idesc_s, ks > 0 ? 1u : 0u);
+                }
+            };
+            auto issue_pv = [&](int t, uint32_t v_lo, bool accumulate) {
+#pragma unroll
+                for (int ks = 0; ks < C::kPvSteps; ++ks) {
+                    const uint32_t off = (ks * C::kUmmaK * W::kVSwizzle) >> 4;
+                    group_mma_ts<PAIR, FP8>(tmem_O(t), tmem_S(t) + ks * 8, v_lo + off, desc_hi_v, idesc_pv, (accumulate || ks > 0) ? 1u : 0u);
+                }
+            };
+            auto tiles_of = [&](int round) {       // of the item of a round, 0 beyond the last
+                const int w = item_index(round, cta, n_ctas);
+                return w < n_items ? get_item(w).n : 0;
+            };
+            // The scores run two tiles ahead of the products: tile s_j of s_n of the item whose Q is in buffer s_buf.
+            int s_round = 0, s_n = tiles_of(0), s_j = 0, s_buf = 0;
+            uint32_t q_phase = 0;
+            int pos = 0;              // ring position of the pair that is used next, and its phase
+            uint32_t kv_phase = 0;
+            auto wait_pair = [&]() {   // the pair and, for an item's first scores, its Q
+                mbar_wait(bar0 + 8u * pos, kv_phase, wctx, (kRoleMma << 8) | kBarKvFull);
+                if (s_j == 0 && s_n > 0) mbar_wait(bar_q_full(s_buf), q_phase, wctx, (kRoleMma << 8) | kBarQFull);
+            };
+            auto next_s = [&](int t, bool ok) {
+                if (s_n == 0) return;
+                if (leader) {
+                    if (ok) issue_s(t, q_lo0 + s_buf * kTileLo, ring_lo_k + (2 * pos + 1) * kPartLo);
+                    group_commit<PAIR>(bar_s_full(t));
+                    if (s_j + 1 == s_n) group_commit<PAIR>(bar_q_empty(s_buf));
+                    group_commit<PAIR>(bar0 + 8u * (NP + pos));       // V(G - 2), whose product was issued before, and K(G)
+                }
+                __syncwarp();
+                if (++s_j == s_n) {
+                    s_n = tiles_of(++s_round);
+                    s_j = 0;
+                    if (W::kQBufs == 1 || s_buf == 1) q_phase ^= 1;
+                    if (W::kQBufs == 2) s_buf ^= 1;
+                }
+            };
+            auto step = [&]() {
+                if (++pos == NP) {
+                    pos = 0;
+                    kv_phase ^= 1;
+                }
+            };
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (s_n > 0) {
+                    wait_pair();
+                    tc_fence_after();
+                    next_s(t, !flag_is_set(abort_at));
+                }
+                step();
+            }
+            int round = 0, n = tiles_of(0), g = 0;
+            uint32_t odd_item = 0;
+            for (uint32_t phase = 0; n > 0; phase ^= 1) {         // items without key tiles come last
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {                     // a stream each: unrolled, so that its addresses are constants
+                    if (n == 0) break;
+                    const bool ok = !flag_is_set(abort_at);
+                    wait_pair();
+                    if (g == 0) mbar_wait_poll(bar_o_free, odd_item ^ 1, wctx, (kRoleMma << 8) | kBarOFree);
+                    mbar_wait_poll(bar_p_full(t), phase, wctx, (kRoleMma << 8) | kBarPFull);
+                    tc_fence_after();
+                    if (leader) {
+                        if (ok) issue_pv(t, ring_lo_v + 2 * pos * kPartLo, g >= 2);
+                        if (g + 1 == n) group_commit<PAIR>(bar_o_full);
+                    }
+                    __syncwarp();
+                    next_s(t, ok);
+                    step();
+                    if (++g == n) {
+                        n = tiles_of(++round);
+                        g = 0;
+                        odd_item ^= 1;
+                    }
+                }
+            }
+            // No MMA or commit of this thread may still be under way when the CTA ends (see the plain form): awaited below.
+            if (leader) group_commit<PAIR>(bar_drain);
+        }
+    } else if (wg == 2) {
+        // ---------------------------------------------------------------- correction and epilogue
+        reg_dec<kStreamRegOther>();
+        // The kernel before this one may have set the status word after the check above: whoever stores looks again, and stores
+        // nothing if it is set (the hand-offs go on).
+        const bool mute = *reinterpret_cast<volatile int*>(p.status) != 0;
+        const int r = tid & 127;
+        const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
+        int G = 0, items = 0;
+        int due = -1, due_first = 0;     // an item whose O waits for its epilogue; the stream of its first tile
+        for (int round = 0;; ++round) {
+            const int w = item_index(round, cta, n_ctas);
+            StreamItem it;
+            it.n = 0;
+            if (w < n_items) it = get_item(w);
+            if (due >= 0) {
+                const StreamItem e = get_item(due);
+                const int first = due_first;
+                float f_first = 0.f, f_second = 0.f;
+                if (e.n > 0) {
+                    mbar_wait(bar_fin, items & 1, wctx, (kRoleEpi << 8) | kBarFin);
+                    f_first = ld_shared_f32(sFin + (first * 128 + r) * 4);
+                    if (e.n > 1) f_second = ld_shared_f32(sFin + ((first ^ 1) * 128 + r) * 4);
+                    ++items;
+                    __syncwarp();
+                    if (lane == 0) st_release_shared(count_done + 4 * (warp & 3), items);
+                    mbar_wait(bar_o_full, (items - 1) & 1, wctx, (kRoleEpi << 8) | kBarOFull);
+                    __syncwarp();
+                    tc_fence_after();
+                }
+                const bool alive = !mute && !flag_is_set(abort_at);      // after an expired wait the accumulators are not to be trusted
+                const int warp_row = e.q0 + (warp & 3) * 32;
+                const size_t row_stride = static_cast<size_t>(p.Hq) * D;
+                __nv_bfloat16* obase = reinterpret_cast<__nv_bfloat16*>(p.o) + ((static_cast<size_t>(e.b) * p.Sq + warp_row) * p.Hq + e.h) * D;
+                const int rows = alive ? p.Sq - warp_row : 0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int lo = 16 * h + (lane >> 2);
+                    const float a_lo = __shfl_sync(0xffffffffu, f_first, lo), a_hi = __shfl_sync(0xffffffffu, f_first, lo + 8);
+                    const float b_lo = __shfl_sync(0xffffffffu, f_second, lo), b_hi = __shfl_sync(0xffffffffu, f_second, lo + 8);
+#pragma unroll
+                    for (int cb = 0; cb < D / 32; ++cb) {
+                        uint32_t o[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) o[i] = 0;
+                        if (e.n > 0) {
+                            uint32_t o2[16];
+                            const uint32_t at = lane_base + (static_cast<uint32_t>(16 * h) << 16) + cb * 32;
+                            tmem_ld_16x256b_x4(tmem_O(first) + at, o);
+                            if (e.n > 1) tmem_ld_16x256b_x4(tmem_O(first ^ 1) + at, o2);
+                            tmem_wait_ld();
+                            if (h == 1 && cb == D / 32 - 1) {   // the accumulators are in registers: the next item may overwrite them
+                                tc_fence_before();
+                                __syncwarp();
+                                if (lane == 0) arrive_at_mma(bar_o_free);
+                            }
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                float v = __uint_as_float(o[i]) * ((i & 2) ? a_hi : a_lo);
+                                if (e.n > 1) v = fmaf(__uint_as_float(o2[i]), (i & 2) ? b_hi : b_lo, v);
+                                o[i] = __float_as_uint(v);
+                            }
+                        }
+                        store_rows16(o, obase + 16 * h * row_stride + cb * 32, row_stride, rows - 16 * h, lane);
+                    }
+                }
+                if (alive && e.q0 + r < p.Sq && e.n == 0 && p.lse != nullptr)
+                    p.lse[(static_cast<size_t>(e.b) * p.Hq + e.h) * p.Sq + e.q0 + r] = -INFINITY;
+            }
+            if (w >= n_items) break;
+            due = w;
+            due_first = G & 1;
+            for (int g = 0; g < it.n; ++g, ++G) {
+                const int t = G & 1;
+                mbar_wait(bar_scale(t), (G >> 1) & 1, wctx, (kRoleCorr << 8) | kBarScale);
+                const float alpha = ld_shared_f32(sScale + (t * 128 + r) * 4);
+                if (g >= 2) rescale_o<D>(tmem_O(t) + lane_base, alpha);     // P V(G - 2) is complete: alpha(G) was posted after S(G) was seen
+                __syncwarp();
+                if (lane == 0) arrive_at_mma(bar_p_full(t));
+            }
+        }
+    } else {
+        // ---------------------------------------------------------------- softmax of stream t
+        reg_inc<kStreamRegSoftmax>();
+        const bool mute = *reinterpret_cast<volatile int*>(p.status) != 0;
+        const int t = wg;
+        const int r = tid & 127;
+        const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
+        const uint32_t tS = tmem_S(t) + lane_base;
+        constexpr int kFam = h15_family_k(MODE);
+        int base = 0;       // tiles of earlier items
+        int items = 0;      // items with key tiles so far
+        for (int round = 0;; ++round) {
+            const int w = item_index(round, cta, n_ctas);
+            if (w >= n_items) break;
+            const StreamItem it = get_item(w);
+            if (it.n == 0) break;       // these come last and are the epilogue's alone
+            const int n = it.n;
+            const int row = it.q0 + r;
+            const int row_limit = p.causal ? min(p.Sk, row + shift + 1) : p.Sk;          // visible keys of this row
+            const int tile_limit = p.causal ? min(p.Sk, it.q0 + shift + 1) : p.Sk;       // first key that some row of the tile cannot see
+            const int first = (t ^ base) & 1;       // this stream's first tile of the item
+            float m_run = -INFINITY, l_run = 0.f;
+            float score_floor = -INFINITY;
+            if constexpr (FP8 && kFam > 0) {     // lower bound of the row's scores, as in the plain form
+                if (n >= first + 7) {
+                    mbar_wait(bar_s_full(t), ((base + first) >> 1) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
+                    score_floor = -448.0f * 1.02f * abs_sum_e4m3_row<D / 16>(sQ + (items % W::kQBufs) * C::kTileBytes + r * D);
+                }
+            }
+            for (int g = first; g < n; g += 2) {
+                const int G = base + g;
+                float m_prev = m_run;
+                if constexpr (kOneAnchor) {
+                    // The anchor after tile G - 1.  Every tile waits for the one before and posts its own, over item boundaries
+                    // too, so that neither side of the hand-over can get two steps ahead of the other.
+                    if (G > 0) {
+                        mbar_wait(bar_anchor(t ^ 1), ((G - 1) >> 1) & 1, wctx, (kRoleSoftmax << 8) | kBarXmax);
+                        if (g > 0) m_prev = ld_shared_f32(sAnchor + r * 4);
+                    }
+                }
+                mbar_wait(bar_s_full(t), (G >> 1) & 1, wctx, (kRoleSoftmax << 8) | kBarSFull);
+                __syncwarp();
+                tc_fence_after();
+                uint32_t s[4][32];
+#pragma unroll
+                for (int cc = 0; cc < 4; ++cc) tmem_ld32(tS + cc * 32, s[cc]);
+                tmem_wait_ld();
+                const bool masked_tile = (g + 1) * kTileN > tile_limit;
+                const int col_limit = row_limit - g * kTileN;
+                if (masked_tile) mask_scores(s, col_limit);
+                const float m_new = fmaxf(m_prev, row_max128(s));
+                if constexpr (kOneAnchor) {
+                    st_shared_f32(sAnchor + r * 4, m_new);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_anchor(t));
+                }
+                const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
+                const float alpha = ex2_approx((m_run - m_use) * p.c);
+                m_run = m_new;
+                auto post_alpha = [&]() {
+                    st_shared_f32(sScale + (t * 128 + r) * 4, alpha);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_scale(t));
+                };
+                if constexpr (!kOutOfStep) post_alpha();
+                const float l_tile = tile_weights<FP8, HALF, MODE, false, kOutOfStep>(s, masked_tile, col_limit, m_use, score_floor, p, tS, post_alpha);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_at_mma(bar_p_full(t));
+                l_run = l_run * alpha + l_tile;
+            }
+            // The streams meet: the one that does not have the last tile leaves its anchor and row sum, the other joins them,
+            // stores LSE and leaves the factors of the two accumulators for the epilogue.  A row's threads are in the same warp
+            // of each warpgroup, so each warp deals with its counterparts alone.
+            const bool has_last = ((base + n - 1) & 1) == t;
+            if (has_last ? n == 1 : n > 1)
+                wait_count(count_done + 4 * (warp & 3), items, wctx, (kRoleSoftmax << 8) | kBarOFree);    // the factors before have been read
+            if (!has_last && n > 1) {
+                st_shared_f32(sFin + r * 4, m_run);
+                st_shared_f32(sFin + (128 + r) * 4, l_run);
+                __syncwarp();
+                if (lane == 0) st_release_shared(count_left + 4 * (warp & 3), items + 1);
+            }
+            if (has_last) {
+                float m_other = -INFINITY, l_other = 0.f;
+                if (n > 1) {
+                    wait_count(count_left + 4 * (warp & 3), items + 1, wctx, (kRoleSoftmax << 8) | kBarPart);
+                    m_other = ld_shared_f32(sFin + r * 4);
+                    l_other = ld_shared_f32(sFin + (128 + r) * 4);
+                }
+                const float m = fmaxf(m_run, m_other), m_use = m == -INFINITY ? 0.f : m;
+                const float a_own = ex2_approx((m_run - m_use) * p.c), a_other = ex2_approx((m_other - m_use) * p.c);
+                const float l = n > 1 ? a_own * l_run + a_other * l_other : l_run;
+                const bool has_keys = m != -INFINITY && l > 0.f;
+                const float inv = has_keys ? p.v_descale / l : 0.f;
+                st_shared_f32(sFin + (t * 128 + r) * 4, a_own * inv);
+                if (n > 1) st_shared_f32(sFin + ((t ^ 1) * 128 + r) * 4, a_other * inv);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_fin);
+                if (row < p.Sq && p.lse != nullptr && !mute && !flag_is_set(abort_at))
+                    p.lse[(static_cast<size_t>(it.b) * p.Hq + it.h) * p.Sq + row] =
+                        has_keys ? 0.6931471805599453f * (m * p.c + log2f(l) - p_off) : -INFINITY;
+            }
+            ++items;
+            base += n;
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 12) {      // every role is through, so this arrives at once unless a wait expired
+        mbar_wait_quiet(bar_drain, 0, kDrainLimitCycles);
+        __syncwarp();
+    }
+    if constexpr (PAIR) {
+        cluster_arrive();      // nobody reaches into the other CTA any more
+        cluster_wait();
+    }
+    if (warp == 12) {
+        __syncwarp();
+        tmem_give<PAIR>(tmem, kTmemCols);
+    }
+}
+
+}  // namespace rowmax

@@ -73,6 +73,47 @@ ROWMAX_HD void kv_end(Ops& ops, int idx) {
 template <int NS>
 ROWMAX_HD constexpr int kv_drain_from(int idx) { return idx >= NS ? idx - NS + 1 : 0; }
 
+// ---- The ring of the two-stream form (attn_streams_kernel.cuh).  Tiles G = 0, 1, ... are counted over all items.  The MMA warp
+// needs V(G - 2) and K(G) at once and is done with both at once: they are pair G, whose two slots share a full and an empty
+// barrier.  The first two pairs have no V, the two after the last tile no K.
+template <int NP>
+struct StreamRing {
+    static ROWMAX_HD constexpr int bar(int pair) { return pair % NP; }
+    static ROWMAX_HD constexpr int ph_full(int pair) { return (pair / NP) & 1; }
+    static ROWMAX_HD constexpr int ph_empty(int pair) { return ph_full(pair) ^ 1; }
+    static ROWMAX_HD constexpr int slot_v(int pair) { return 2 * (pair % NP); }
+    static ROWMAX_HD constexpr int slot_k(int pair) { return 2 * (pair % NP) + 1; }
+};
+// Ops: arrive(pair), wait_empty(pair), load_k(pair), load_v(pair), with the meaning they have above.  False: the producer gave up.
+template <class Ops>
+ROWMAX_HD bool stream_tile(Ops& ops, int pair) {
+    if (!ops.wait_empty(pair)) return false;
+    if (pair >= 2) ops.load_v(pair);
+    else ops.arrive(pair);
+    ops.load_k(pair);
+    return true;
+}
+template <class Ops>
+ROWMAX_HD bool stream_tail(Ops& ops, int pair) {
+    if (pair < 2) return true;
+    if (!ops.wait_empty(pair)) return false;
+    ops.load_v(pair);
+    ops.arrive(pair);
+    return true;
+}
+// Whether anything arrives for a pair up to the second one after the last of `tiles` tiles.
+ROWMAX_HD constexpr bool stream_pair_is_used(int pair, int tiles) { return pair < tiles || pair >= 2; }
+
+template <class Arrive, class WaitEmpty, class LoadK, class LoadV>
+struct StreamOps {
+    Arrive arrive;
+    WaitEmpty wait_empty;
+    LoadK load_k;
+    LoadV load_v;
+};
+template <class A, class W, class K, class V>
+StreamOps(A, W, K, V) -> StreamOps<A, W, K, V>;
+
 // Ops out of callables.
 template <class Arrive, class WaitEmpty, class LoadK, class LoadV, class PreK, class LoadQ>
 struct KvOps {
