@@ -22,3 +22,7 @@ def test_ring_protocol_holds_for_all_lengths_and_landing_orders(tmp_path):
 
 def test_plans_follow_the_device(tmp_path):
     _run(tmp_path, "plan_model")
+
+
+def test_stream_ring_protocol_holds_for_all_lengths_and_landing_orders(tmp_path):
+    _run(tmp_path, "stream_ring_model", "12")
