@@ -193,8 +193,8 @@ int attn_get_schedule(int D, int in_dtype, int weight_mode, int causal,
  * attn_get_plan — which kernel attn_fwd (or attn_fwd_pot) would take for a shape on the current device, and how many CTAs
  * would share a piece of its work.  The order in which fp32 sums are added follows from it, so O and LSE may differ in their
  * last bits between devices with other SM counts.
- *   kernel  ATTN_KERNEL_PLAIN: one CTA takes a pair of query tiles (ctas = 1); ATTN_KERNEL_SHARED: fewer such pairs than SMs,
- *           ctas CTAs share one; ATTN_KERNEL_FEW_ROWS: few query rows per key/value head, ctas CTAs share a head
+ *   kernel  ATTN_KERNEL_PLAIN: one CTA takes a pair of query tiles (ctas = 1); ATTN_KERNEL_SHARED: ctas CTAs share one,
+ *           each with some of its keys or (2) each with one of its query tiles; ATTN_KERNEL_FEW_ROWS: few query rows per key/value head, ctas CTAs share a head
  */
 #define ATTN_KERNEL_PLAIN 0
 #define ATTN_KERNEL_SHARED 1

@@ -41,7 +41,7 @@ struct SplitLauncher {
         return known[dev][parts] > 0 ? known[dev][parts] : 0;
     }
     // CTAs per item (plan.h), 1 for the plain form.
-    static int plan(const AttnParams& p) {
+    static int plan(const AttnParams& p, double* steps) {
         int dev = 0, sms = 0;
         if (device_and_sms(&dev, &sms) != cudaSuccess) return 1;
         const int pairs = (p.Sq + 2 * kTileM - 1) / (2 * kTileM);
@@ -49,7 +49,7 @@ struct SplitLauncher {
         const int first_end = p.causal ? 2 * kTileM + p.Sk - p.Sq : p.Sk;
         const int first = first_end <= 0 ? 0 : ((first_end < p.Sk ? first_end : p.Sk) + kTileN - 1) / kTileN;
         const SplitShape s{static_cast<double>(pairs) * p.Hq * p.B, all, first, split_takes_maxima(MODE, IN == kInFP8)};
-        return split_parts(s, sms, [&](int parts) { return fit(dev, parts); });
+        return split_parts(s, sms, [&](int parts) { return fit(dev, parts); }, steps);
     }
     static cudaError_t launch(int parts, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, AttnParams p,
                               cudaStream_t stream) {
@@ -98,10 +98,10 @@ bool with_launcher(int D, int in_type, int mode, F f) {
 
 }  // namespace
 
-// CTAs that should share a work item (1: the plain form).  A deferred rescale stays whole: its anchor depends on the order.
-int plan_attn_split(int D, int in_type, int mode, const AttnParams& p) {
+// CTAs that should share a work item (1: the plain form), and the estimated time.  A deferred rescale stays whole: its anchor depends on the order.
+int plan_attn_split(int D, int in_type, int mode, const AttnParams& p, double* steps) {
     int parts = 1;
-    if (!(p.tau > 0.0f)) with_launcher(D, in_type, mode, [&](auto l) { parts = decltype(l)::plan(p); });
+    if (!(p.tau > 0.0f)) with_launcher(D, in_type, mode, [&](auto l) { parts = decltype(l)::plan(p, steps); });
     return parts;
 }
 

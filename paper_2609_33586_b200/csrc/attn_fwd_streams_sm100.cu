@@ -5,108 +5,77 @@ namespace rowmax {
 
 namespace {
 
-template <int D, int IN, int MODE, bool PAIR>
-struct StreamsLauncher {
-    using W = StreamsCfg<D, IN == kInFP8, PAIR>;
-    static constexpr int kCtas = PAIR ? 2 : 1;
+template <int D, int IN, int MODE>
+cudaError_t launch_streams(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream) {
+    using W = StreamsCfg<D, IN == kInFP8>;
+    auto kern = attn_fwd_streams_kernel<D, IN, MODE>;
+    static bool configured[64] = {};   // per device: the shared-memory opt-in of this instance
+    int dev = 0, sm_count = 0;
+    cudaError_t e = device_and_sms(&dev, &sm_count);
+    if (e != cudaSuccess) return e;
+    if (!configured[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmemBytes);
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+    }
+    const long long items = static_cast<long long>((p.Sq + kTileM - 1) / kTileM) * p.Hq * p.B;
+    if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
+    cudaLaunchAttribute attr;      // programmatic dependent launch where every CTA has one item, as in the plain form
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(items < sm_count ? items : sm_count));
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = W::kSmemBytes;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = items <= sm_count ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, tq, tk, tv, p);
+}
 
-    static void configure(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
-        // Programmatic dependent launch as in the plain form; used where every CTA has one item.
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = kCtas;
-        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.blockDim = dim3(512);
-        cfg.dynamicSmemBytes = W::kSmemBytes;
-    }
-    // CTAs, or pairs of them, that fit the device at once (asked once per device; 0: none).
-    static int fit() {
-        static int known[64] = {};
-        int dev = 0, sms = 0;
-        if (device_and_sms(&dev, &sms) != cudaSuccess) return 0;
-        if (known[dev] == 0) {
-            auto kern = attn_fwd_streams_kernel<D, IN, MODE, PAIR>;
-            int n = sms;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, W::kSmemBytes);
-            if (PAIR && e == cudaSuccess) {
-                cudaLaunchConfig_t cfg = {};
-                cudaLaunchAttribute attr[2];
-                configure(cfg, attr);
-                cfg.attrs = attr + 1;
-                cfg.numAttrs = 1;
-                cfg.gridDim = dim3(kCtas);
-                e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-            }
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                n = 0;
-            }
-            known[dev] = n > 0 ? n : -1;
-        }
-        return known[dev] > 0 ? known[dev] : 0;
-    }
-    static cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream) {
-        const int places = fit();
-        const long long items = static_cast<long long>((p.Sq + kCtas * kTileM - 1) / (kCtas * kTileM)) * p.Hq * p.B;
-        if (places == 0 || items > 0x3fffffffLL) return cudaErrorInvalidValue;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[2];
-        configure(cfg, attr);
-        cfg.gridDim = dim3(kCtas * static_cast<unsigned>(items < places ? items : places));
-        cfg.stream = stream;
-        const bool early = items <= places;
-        cfg.attrs = early ? attr : attr + 1;
-        cfg.numAttrs = (early ? 1 : 0) + (PAIR ? 1 : 0);
-        return cudaLaunchKernelEx(&cfg, attn_fwd_streams_kernel<D, IN, MODE, PAIR>, tq, tk, tv, p);
-    }
-};
-
-// Calls f with the launcher of a combination; false for one that has no two-stream form.
-template <int D, int IN, bool PAIR, typename F>
-bool with_mode(int mode, F f) {
+template <int D, int IN>
+cudaError_t dispatch_mode(int mode, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& p,
+                          cudaStream_t stream) {
     switch (mode) {
-        case kExact: f(StreamsLauncher<D, IN, kExact, PAIR>{}); return true;
-        case kPot: f(StreamsLauncher<D, IN, kPot, PAIR>{}); return true;
-        case kPotDrop: f(StreamsLauncher<D, IN, kPotDrop, PAIR>{}); return true;
-        case kH15: f(StreamsLauncher<D, IN, kH15, PAIR>{}); return true;
+        case kExact: return launch_streams<D, IN, kExact>(tq, tk, tv, p, stream);
+        case kPot: return launch_streams<D, IN, kPot>(tq, tk, tv, p, stream);
+        case kPotDrop: return launch_streams<D, IN, kPotDrop>(tq, tk, tv, p, stream);
+        case kH15: return launch_streams<D, IN, kH15>(tq, tk, tv, p, stream);
         default: break;
     }
     if constexpr (IN != kInFP16) {
         switch (mode) {
-            case kH15K2: f(StreamsLauncher<D, IN, kH15K2, PAIR>{}); return true;
-            case kH15K3: f(StreamsLauncher<D, IN, kH15K3, PAIR>{}); return true;
+            case kH15K2: return launch_streams<D, IN, kH15K2>(tq, tk, tv, p, stream);
+            case kH15K3: return launch_streams<D, IN, kH15K3>(tq, tk, tv, p, stream);
             default: break;
         }
     }
-    return false;
-}
-template <typename F>
-bool with_launcher(int D, int in_type, int mode, bool pair, F f) {
-    if (D == 128 && pair) {
-        if (in_type == kInBF16) return with_mode<128, kInBF16, true>(mode, f);
-        if (in_type == kInFP16) return with_mode<128, kInFP16, true>(mode, f);
-        return with_mode<128, kInFP8, true>(mode, f);
-    }
-    if (D == 128) {
-        if (in_type == kInBF16) return with_mode<128, kInBF16, false>(mode, f);
-        if (in_type == kInFP16) return with_mode<128, kInFP16, false>(mode, f);
-        return with_mode<128, kInFP8, false>(mode, f);
-    }
-    if (pair) return false;
-    if (in_type == kInBF16) return with_mode<64, kInBF16, false>(mode, f);
-    if (in_type == kInFP16) return with_mode<64, kInFP16, false>(mode, f);
-    return with_mode<64, kInFP8, false>(mode, f);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t launch_attn_fwd_streams(int D, int in_type, int mode, bool pair, const CUtensorMap& tq, const CUtensorMap& tk,
-                                    const CUtensorMap& tv, const AttnParams& p, cudaStream_t stream) {
-    cudaError_t e = cudaErrorInvalidValue;
-    with_launcher(D, in_type, mode, pair, [&](auto l) { e = decltype(l)::launch(tq, tk, tv, p, stream); });
-    return e;
+// Whether a forward takes this form; parts and split_steps: what the split form would make of it (1: the plain form).  The
+// emulated controls and a deferred rescale have no instances here.
+bool plan_attn_streams(int D, int in_type, int mode, int parts, double split_steps, const AttnParams& p) {
+    if (p.tau > 0.0f || exact_poly_eighths(mode) > 0) return false;
+    int dev = 0, sms = 0;
+    if (device_and_sms(&dev, &sms) != cudaSuccess) return false;
+    const long long heads = static_cast<long long>(p.Hq) * p.B, per_head = (p.Sq + kTileM - 1) / kTileM;
+    const StreamShape s{static_cast<double>(heads * per_head), static_cast<double>(heads * ((per_head + 1) / 2)), static_cast<int>(per_head),
+                        (p.Sk + kTileN - 1) / kTileN, D, p.causal != 0, split_takes_maxima(mode, in_type == kInFP8)};
+    return streams_pay(s, parts, split_steps, sms);
+}
+
+cudaError_t launch_attn_fwd_streams(int D, int in_type, int mode, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                                    const AttnParams& p, cudaStream_t stream) {
+    if (in_type == kInBF16 && D == 128) return dispatch_mode<128, kInBF16>(mode, tq, tk, tv, p, stream);
+    if (in_type == kInBF16 && D == 64) return dispatch_mode<64, kInBF16>(mode, tq, tk, tv, p, stream);
+    if (in_type == kInFP16 && D == 128) return dispatch_mode<128, kInFP16>(mode, tq, tk, tv, p, stream);
+    if (in_type == kInFP16 && D == 64) return dispatch_mode<64, kInFP16>(mode, tq, tk, tv, p, stream);
+    if (in_type == kInFP8 && D == 128) return dispatch_mode<128, kInFP8>(mode, tq, tk, tv, p, stream);
+    if (in_type == kInFP8 && D == 64) return dispatch_mode<64, kInFP8>(mode, tq, tk, tv, p, stream);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace rowmax

@@ -4,10 +4,12 @@
 // tiles.  Here both work on ONE query tile: key tiles take turns, tile G of the CTA's walk (counted over all its items) belongs
 // to stream G mod 2, which has a softmax warpgroup, a score buffer and an O accumulator of its own.
 //
-// PAIR = false: a work item is one query tile, half as large as an item of the plain form.
-// PAIR = true: two CTAs on neighbouring SMs take a pair of query tiles, one each, and one MMA (cta_group::2, M = 256) works for
-// both.  Of every K tile a CTA holds 64 keys, of every V tile 64 columns: half the K/V traffic into shared memory and half the
-// operand reads of K and V, which are what bounds PAIR = false at 16 bits and D = 128.
+// What bounds it: at 16 bits and D = 128 shared memory (64 KB of K and V come in for every tile and 96 KB of operands are read,
+// 1700 to 2000 clocks a tile where the tensor cores need 1024), elsewhere the chain of one warpgroup, as in the plain form.  A tile
+// takes 0.56 to 0.64 of a step of the plain form, which is a tile of two query tiles; so it pays where the plain form's coarser
+// items leave SMs idle (streams_pay in plan.h).  16 x 1K e4m3 h15 17.7 -> 14.1 us, 512 queries on 16K (32/8 heads, bf16 h15)
+// 168 -> 143, cross attention 36 heads x 1337 x 2803 bf16 exact 94 -> 76.  Pairs of CTAs with cta_group::2 and half a K/V tile
+// each were no faster (16.0, 144 and 78 us): their hand-offs take longer than the operand reads that they save.
 //
 // Semantics are those of the sequential loop: the anchor that tile g starts from is the one tile g - 1 left, handed from
 // warpgroup to warpgroup through shared memory as soon as a tile's row maximum is known, half a period before the other needs it
@@ -15,7 +17,7 @@
 // joined at the end: O = (a_0 O_0 + a_1 O_1) dv / l with a_t = 2^((m_t - m) c).
 //   warpgroup 0/1  softmax of stream 0/1: one thread per row
 //   warpgroup 2    correction (rescales the accumulators) and epilogue (joins them and stores O)
-//   warp 12        MMA issuer (PAIR: of the first CTA): P V of tile G, then S of tile G + 2, which may be the next item's
+//   warp 12        MMA issuer: P V of tile G, then S of tile G + 2, which may be the next item's
 //   warp 13        TMA producer: V(G - 2) and K(G) arrive as one pair of ring slots
 // TMEM columns: S_0/P_0 [0,128), S_1/P_1 [128,256), O_0 [256,384), O_1 [384,512).
 #pragma once
@@ -25,19 +27,13 @@ namespace rowmax {
 
 namespace {
 
-template <int D, bool FP8, bool PAIR>
+template <int D, bool FP8>
 struct StreamsCfg {
     using C = TileCfg<D, FP8>;
-    static_assert(!PAIR || D == 128, "half a V tile has 64 columns");
-    static constexpr int kPartBytes = C::kTileBytes / (PAIR ? 2 : 1);    // of a K or V tile: what this CTA holds
-    static constexpr int kKeys = PAIR ? kTileN / 2 : kTileN;             // keys of a K tile in this CTA
-    static constexpr int kKBoxBytes = kKeys * C::kSwizzle;
-    static constexpr int kVSwizzle = PAIR ? 64 * C::kElem : C::kSwizzle; // swizzle span of a V row
-    static constexpr int kVBoxes = PAIR ? 1 : C::kBoxes;
     static constexpr int kQBufs = C::kTileBytes <= 16384 ? 2 : 1;        // query tiles staged
-    static constexpr int kPairs = PAIR ? (FP8 ? 8 : 6) : (C::kTileBytes <= 16384 ? 4 : 3);   // pairs of K/V ring slots
+    static constexpr int kPairs = C::kTileBytes <= 16384 ? 4 : 3;        // pairs of K/V ring slots
     static constexpr int kQBytes = kQBufs * C::kTileBytes;
-    static constexpr int kRingBytes = 2 * kPairs * kPartBytes;
+    static constexpr int kRingBytes = 2 * kPairs * C::kTileBytes;
     static constexpr int kScaleOff = kQBytes + kRingBytes;       // float alpha[2][128]
     static constexpr int kAnchorOff = kScaleOff + 2 * 128 * 4;   // float anchor[128]: of the last tile that has its maximum
     static constexpr int kFinOff = kAnchorOff + 128 * 4;         // float factor[2][128] of the accumulators (before: m and l of a stream)
@@ -54,22 +50,18 @@ struct StreamsCfg {
 constexpr int kStreamRegSoftmax = 192, kStreamRegOther = 64;
 static_assert(256 * kStreamRegSoftmax + 256 * kStreamRegOther <= 512 * 128, "setmaxnreg targets exceed the launch allocation");
 
-// One work item: this CTA's query tile of one (batch, head), and the key tiles that it goes over (PAIR: the longer walk of both
-// query tiles; a tile beyond a row's keys is masked as a whole).  n = 0: no row sees a key.  Heaviest first, as in the plain form.
+// One work item: a query tile of one (batch, head) and its key tiles (0: no row sees a key).  Heaviest first, as in the plain form.
 struct StreamItem {
     int h, b, hk, q0, n;
 };
-template <bool PAIR>
-__device__ __forceinline__ StreamItem decode_stream_item(int w, const AttnParams& p, int n_groups, int bh, int rank) {
-    constexpr int kRows = (PAIR ? 2 : 1) * kTileM;
+__device__ __forceinline__ StreamItem decode_stream_item(int w, const AttnParams& p, int n_tiles, int bh) {
     StreamItem it;
-    const int rem = w % bh, first = (n_groups - 1 - w / bh) * kRows;
+    const int rem = w % bh;
+    it.q0 = (n_tiles - 1 - w / bh) * kTileM;
     it.h = rem % p.Hq;
     it.b = rem / p.Hq;
     it.hk = it.h / p.group;
-    it.q0 = first + rank * kTileM;
-    const int last = PAIR && first + kTileM < p.Sq ? first + kTileM : first;      // the later query tile that exists
-    const int kv_end = p.causal ? min(p.Sk, last + kTileM + p.Sk - p.Sq) : p.Sk;
+    const int kv_end = p.causal ? min(p.Sk, it.q0 + kTileM + p.Sk - p.Sq) : p.Sk;
     it.n = kv_end > 0 ? (kv_end + kTileN - 1) / kTileN : 0;
     return it;
 }
@@ -115,16 +107,15 @@ __device__ __forceinline__ void store_rows16(const uint32_t (&v)[16], __nv_bfloa
 
 }  // namespace
 
-template <int D, int IN, int MODE, bool PAIR>
+template <int D, int IN, int MODE>
 __global__ void __launch_bounds__(512, 1)
 attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
     constexpr bool FP8 = IN == kInFP8;
     constexpr bool HALF = IN == kInFP16;
     using C = TileCfg<D, FP8>;
-    using W = StreamsCfg<D, FP8, PAIR>;
+    using W = StreamsCfg<D, FP8>;
     constexpr int NP = W::kPairs;
-    constexpr int kCtas = PAIR ? 2 : 1;
     constexpr bool kOneAnchor = split_takes_maxima(MODE, FP8);     // the streams hand the anchor on
     constexpr bool kOutOfStep = FP8 && is_exact_like(MODE);
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -139,8 +130,6 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const uint32_t count_done = smem_u32(smem + W::kCountOff), count_left = count_done + 16;
     const WaitCtx wctx{abort_at, p.status, kWaitLimitCycles};
 
-    // PAIR: the barriers that the MMA warp waits for count the arrivals of both CTAs in the first one's shared memory; what it
-    // commits arrives in both.
     using Ring = StreamRing<NP>;
     auto bar_kv_full = [&](int pair) { return bar0 + 8u * Ring::bar(pair); };              // TMA -> MMA: V(G - 2) and K(G)
     auto bar_kv_empty = [&](int pair) { return bar0 + 8u * (NP + Ring::bar(pair)); };      // MMA -> TMA
@@ -155,27 +144,22 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const uint32_t bar_o_free = bar_x(6, 1);                   // epilogue -> MMA: both accumulators have been read out
     const uint32_t bar_fin = bar_x(7, 0);                      // softmax -> epilogue: factors of the accumulators
     const uint32_t bar_drain = bar_x(7, 1);                    // the MMA warp's last commit
-    auto arrive_at_mma = [&](uint32_t bar) {
-        if constexpr (PAIR) mbar_arrive_peer(mapa(bar, 0));
-        else mbar_arrive(bar);
-    };
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wg = warp >> 2;
     if ((smem_u32(smem) & 1023u) != 0) {
         if (tid == 0) atomicCAS(p.status, 0, (kRoleSetup << 8) | kBarAlign);
         return;
     }
-    // As in the plain form one thread (PAIR: of both CTAs) reads the sticky status word, and the CTA or the pair leaves as a whole
-    // if it is set.
-    const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
+    // As in the plain form one thread reads the sticky status word, and the CTA leaves as a whole if it is set.
     if (tid == 0) {
-        write_flag(abort_at, 0);
-        write_flag(leave_at, rank == 0 ? *reinterpret_cast<volatile int*>(p.status) : 0);
+        const int set = *reinterpret_cast<volatile int*>(p.status) != 0 ? 1 : 0;
+        write_flag(abort_at, set);
+        write_flag(leave_at, set);
     }
-    const int n_groups = (p.Sq + kCtas * kTileM - 1) / (kCtas * kTileM);
+    const int n_tiles = (p.Sq + kTileM - 1) / kTileM;
     const int bh = p.Hq * p.B;
-    const int n_items = n_groups * bh;
-    const int cta = blockIdx.x / kCtas, n_ctas = gridDim.x / kCtas;      // PAIR: of pairs
+    const int n_items = n_tiles * bh;
+    const int cta = blockIdx.x, n_ctas = gridDim.x;
     const int shift = p.Sk - p.Sq;
 
     if (warp == 13) {
@@ -187,12 +171,12 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             mbar_init(bar_q_full(t), 1);
             mbar_init(bar_q_empty(t), 1);
             mbar_init(bar_s_full(t), 1);
-            mbar_init(bar_p_full(t), 8 * kCtas);      // one arrival per softmax warp, one per correction warp
+            mbar_init(bar_p_full(t), 8);      // one arrival per softmax warp, one per correction warp
             mbar_init(bar_scale(t), 4);
             mbar_init(bar_anchor(t), 4);
         } else if (lane == 18) {
             mbar_init(bar_o_full, 1);
-            mbar_init(bar_o_free, 4 * kCtas);
+            mbar_init(bar_o_free, 4);
             mbar_init(bar_fin, 4);
             mbar_init(bar_drain, 1);
         } else if (lane >= 20 && lane < 28) {
@@ -201,34 +185,29 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         fence_mbar_init();
     }
     constexpr uint32_t kTmemCols = 512;
-    if (warp == 12) tmem_take<PAIR>(smem_u32(tmem_slot), kTmemCols);
+    if (warp == 12) {
+        tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+        tmem_relinquish();
+    }
     tc_fence_before();
     __syncthreads();
-    if constexpr (PAIR) {      // the barriers of both CTAs are there
-        cluster_arrive();
-        cluster_wait();
-    }
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     griddep_wait();        // what follows reads the caller's tensors
     griddep_launch();
-    if (PAIR ? __float_as_int(ld_cluster_f32(mapa(leave_at, 0))) != 0 : flag_is_set(leave_at)) {
-        if constexpr (PAIR) {
-            cluster_arrive();
-            cluster_wait();
-        }
-        if (warp == 12) tmem_give<PAIR>(tmem, kTmemCols);
+    if (flag_is_set(leave_at)) {
+        if (warp == 12) tmem_dealloc(tmem, kTmemCols);
         return;
     }
-    auto get_item = [&](int w) { return decode_stream_item<PAIR>(w, p, n_groups, bh, rank); };
+    auto get_item = [&](int w) { return decode_stream_item(w, p, n_tiles, bh); };
     auto tmem_S = [&](int t) { return tmem + 128u * t; };
     auto tmem_O = [&](int t) { return tmem + 256u + 128u * t; };
 
     constexpr uint32_t fmt_16 = HALF ? kFmtF16 : kFmtBF16;
     constexpr uint32_t fmt_ab = FP8 ? kFmtE4M3 : fmt_16;
     constexpr uint32_t fmt_p = FP8 ? (PFormat<FP8, MODE>::kE4M3 ? kFmtE4M3 : kFmtE5M2) : fmt_16;
-    constexpr uint32_t idesc_s = umma_idesc(fmt_ab, fmt_ab, false, false, kCtas * kTileM, kTileN);
-    constexpr uint32_t idesc_pv = umma_idesc(fmt_p, fmt_ab, false, true, kCtas * kTileM, D);
+    constexpr uint32_t idesc_s = umma_idesc(fmt_ab, fmt_ab, false, false, kTileM, kTileN);
+    constexpr uint32_t idesc_pv = umma_idesc(fmt_p, fmt_ab, false, true, kTileM, D);
     constexpr float p_off = static_cast<float>(PFormat<FP8, MODE>::kOffLog2);
 
     if (wg == 3) {
@@ -239,30 +218,20 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             int items = 0;        // items with tiles so far
             StreamItem it;
             int v_b[2] = {0, 0}, v_hk[2] = {0, 0}, v_tile[2] = {0, 0};     // the last two tiles, whose V comes with the K of two tiles later
-            // The arrival for copies of `bytes` (PAIR: of both CTAs, by the first one's producer) and the barrier they count on.
-            auto expect = [&](uint32_t bar, uint32_t bytes) {
-                if (rank == 0) mbar_arrive_expect_tx(bar, kCtas * bytes);
-                return PAIR ? mapa(bar, 0) : bar;
+            auto load_tile = [&](const CUtensorMap* tm, uint32_t dst, uint32_t bar, int head, int row0, int b) {
+                mbar_arrive_expect_tx(bar, C::kTileBytes);
+#pragma unroll
+                for (int bx = 0; bx < C::kBoxes; ++bx) tma_load_4d(dst + bx * C::kBoxBytes, tm, bar, bx * C::kBoxElems, head, row0, b);
             };
             int j = 0;
             // After an expired wait nothing more is loaded (see the plain form).
-            StreamOps ops{[&](int pair) { if (rank == 0) mbar_arrive(bar_kv_full(pair)); },
+            StreamOps ops{[&](int pair) { mbar_arrive(bar_kv_full(pair)); },
                           [&](int pair) {
                               mbar_wait(bar_kv_empty(pair), Ring::ph_empty(pair), wctx, (kRoleLoad << 8) | kBarKvEmpty);
                               return !flag_is_set(abort_at);
                           },
-                          [&](int pair) {      // PAIR: keys 64 * rank .. of the tile
-                              const uint32_t dst = sRing + Ring::slot_k(pair) * W::kPartBytes, bar = expect(bar_kv_full(pair), W::kPartBytes);
-#pragma unroll
-                              for (int bx = 0; bx < C::kBoxes; ++bx)
-                                  group_load_4d<PAIR>(dst + bx * W::kKBoxBytes, &tmK, bar, bx * C::kBoxElems, it.hk, j * kTileN + W::kKeys * rank, it.b);
-                          },
-                          [&](int pair) {      // PAIR: columns 64 * rank .. of the tile
-                              const uint32_t dst = sRing + Ring::slot_v(pair) * W::kPartBytes, bar = expect(bar_kv_full(pair), W::kPartBytes);
-#pragma unroll
-                              for (int bx = 0; bx < W::kVBoxes; ++bx)
-                                  group_load_4d<PAIR>(dst + bx * C::kBoxBytes, &tmV, bar, PAIR ? 64 * rank : bx * C::kBoxElems, v_hk[0], v_tile[0] * kTileN, v_b[0]);
-                          }};
+                          [&](int pair) { load_tile(&tmK, sRing + Ring::slot_k(pair) * C::kTileBytes, bar_kv_full(pair), it.hk, j * kTileN, it.b); },
+                          [&](int pair) { load_tile(&tmV, sRing + Ring::slot_v(pair) * C::kTileBytes, bar_kv_full(pair), v_hk[0], v_tile[0] * kTileN, v_b[0]); }};
             bool ok = true;
             for (int round = 0; ok; ++round) {
                 const int w = item_index(round, cta, n_ctas);
@@ -279,10 +248,7 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         mbar_wait(bar_q_empty(buf), ((items / W::kQBufs) & 1) ^ 1, wctx, (kRoleLoad << 8) | kBarQEmpty);
                         ok = !flag_is_set(abort_at);
                         if (!ok) break;
-                        const uint32_t bar = expect(bar_q_full(buf), C::kTileBytes);
-#pragma unroll
-                        for (int bx = 0; bx < C::kBoxes; ++bx)
-                            group_load_4d<PAIR>(sQ + buf * C::kTileBytes + bx * C::kBoxBytes, &tmQ, bar, bx * C::kBoxElems, it.h, it.q0, it.b);
+                        load_tile(&tmQ, sQ + buf * C::kTileBytes, bar_q_full(buf), it.h, it.q0, it.b);
                         ++items;
                     }
                 }
@@ -294,111 +260,90 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (ok) pairs = e + 1;
                 v_b[0] = v_b[1]; v_hk[0] = v_hk[1]; v_tile[0] = v_tile[1];
             }
-            // Every load this thread issued has to land before the CTA ends (see the plain form).  PAIR: the first CTA's barriers
-            // count the copies of both; a second CTA that gave up leaves its copies time to land.
-            if (rank == 0) {
-                for (int pair = pairs > NP ? pairs - NP : 0; pair < pairs; ++pair)
-                    if (stream_pair_is_used(pair, walked)) mbar_wait_quiet(bar_kv_full(pair), Ring::ph_full(pair), kDrainLimitCycles);
-                for (int i = items > W::kQBufs ? items - W::kQBufs : 0; i < items; ++i)
-                    mbar_wait_quiet(bar_q_full(i % W::kQBufs), (i / W::kQBufs) & 1, kDrainLimitCycles);
-            } else if (!ok) {
-                const long long t0 = clock64();
-                while (clock64() - t0 < kDrainLimitCycles / 50) {}
-            }
-        } else if (warp == 12 && rank == 0) {
+            // Every load this thread issued has to land before the CTA ends (see the plain form).
+            for (int pair = pairs > NP ? pairs - NP : 0; pair < pairs; ++pair)
+                if (stream_pair_is_used(pair, walked)) mbar_wait_quiet(bar_kv_full(pair), Ring::ph_full(pair), kDrainLimitCycles);
+            for (int i = items > W::kQBufs ? items - W::kQBufs : 0; i < items; ++i)
+                mbar_wait_quiet(bar_q_full(i % W::kQBufs), (i / W::kQBufs) & 1, kDrainLimitCycles);
+        } else if (warp == 12) {
             // ------------------------------------------------------------ MMA issuer
             const bool leader = elect_one();
-            constexpr uint32_t desc_hi = umma_desc_hi_sw(C::kSwizzle), desc_hi_v = umma_desc_hi_sw(W::kVSwizzle);
+            constexpr uint32_t desc_hi = umma_desc_hi_sw(C::kSwizzle);
             const uint32_t q_lo0 = umma_desc_lo(sQ, 16);
             const uint32_t ring_lo_k = umma_desc_lo(sRing, 16);               // K tiles: K-major
             const uint32_t ring_lo_v = umma_desc_lo(sRing, C::kBoxBytes);     // V tiles: MN-major, LBO = next block of columns
-            constexpr uint32_t kTileLo = C::kTileBytes >> 4, kPartLo = W::kPartBytes >> 4;
+            constexpr uint32_t kTileLo = C::kTileBytes >> 4;
             auto issue_s = [&](int t, uint32_t q_lo, uint32_t k_lo) {
 #pragma unroll
                 for (int ks = 0; ks < C::kQkSteps; ++ks) {
-                    const uint32_t box = ks / C::kStepsPerBox, in_row = (ks % C::kStepsPerBox) * 32;
-                    group_mma_ss<PAIR, FP8>(tmem_S(t), q_lo + ((box * C::kBoxBytes + in_row) >> 4), k_lo + ((box * W::kKBoxBytes + in_row) >> 4), desc_hi,
-                                            idesc_s, ks > 0 ? 1u : 0u);
+                    const uint32_t off = ((ks / C::kStepsPerBox) * C::kBoxBytes + (ks % C::kStepsPerBox) * 32) >> 4;
+                    umma_ss_lo<FP8>(tmem_S(t), q_lo + off, k_lo + off, desc_hi, idesc_s, ks > 0 ? 1u : 0u);
                 }
             };
             auto issue_pv = [&](int t, uint32_t v_lo, bool accumulate) {
 #pragma unroll
                 for (int ks = 0; ks < C::kPvSteps; ++ks) {
-                    const uint32_t off = (ks * C::kUmmaK * W::kVSwizzle) >> 4;
-                    group_mma_ts<PAIR, FP8>(tmem_O(t), tmem_S(t) + ks * 8, v_lo + off, desc_hi_v, idesc_pv, (accumulate || ks > 0) ? 1u : 0u);
+                    const uint32_t off = (ks * C::kUmmaK * C::kSwizzle) >> 4;
+                    umma_ts_lo<FP8>(tmem_O(t), tmem_S(t) + ks * 8, v_lo + off, desc_hi, idesc_pv, (accumulate || ks > 0) ? 1u : 0u);
                 }
             };
             auto tiles_of = [&](int round) {       // of the item of a round, 0 beyond the last
                 const int w = item_index(round, cta, n_ctas);
                 return w < n_items ? get_item(w).n : 0;
             };
-            // The scores run two tiles ahead of the products: tile s_j of s_n of the item whose Q is in buffer s_buf.
-            int s_round = 0, s_n = tiles_of(0), s_j = 0, s_buf = 0;
-            uint32_t q_phase = 0;
-            int pos = 0;              // ring position of the pair that is used next, and its phase
-            uint32_t kv_phase = 0;
-            auto wait_pair = [&]() {   // the pair and, for an item's first scores, its Q
-                mbar_wait(bar0 + 8u * pos, kv_phase, wctx, (kRoleMma << 8) | kBarKvFull);
-                if (s_j == 0 && s_n > 0) mbar_wait(bar_q_full(s_buf), q_phase, wctx, (kRoleMma << 8) | kBarQFull);
+            // The scores run two tiles ahead of the products: tile s_j of s_n of the item that uses Q for the s_item-th time.
+            int s_round = 0, s_n = tiles_of(0), s_j = 0, s_item = 0;
+            auto wait_pair = [&](int pair) { mbar_wait(bar_kv_full(pair), Ring::ph_full(pair), wctx, (kRoleMma << 8) | kBarKvFull); };
+            auto wait_q = [&]() {       // for an item's first scores
+                if (s_j == 0 && s_n > 0) mbar_wait(bar_q_full(s_item % W::kQBufs), (s_item / W::kQBufs) & 1, wctx, (kRoleMma << 8) | kBarQFull);
             };
-            auto next_s = [&](int t, bool ok) {
+            auto next_s = [&](int G, bool ok) {    // scores of tile G: its K is there, its Q has been waited for
                 if (s_n == 0) return;
+                const int t = G & 1, buf = s_item % W::kQBufs;
                 if (leader) {
-                    if (ok) issue_s(t, q_lo0 + s_buf * kTileLo, ring_lo_k + (2 * pos + 1) * kPartLo);
-                    group_commit<PAIR>(bar_s_full(t));
-                    if (s_j + 1 == s_n) group_commit<PAIR>(bar_q_empty(s_buf));
-                    group_commit<PAIR>(bar0 + 8u * (NP + pos));       // V(G - 2), whose product was issued before, and K(G)
+                    if (ok) issue_s(t, q_lo0 + buf * kTileLo, ring_lo_k + Ring::slot_k(G) * kTileLo);
+                    umma_commit(bar_s_full(t));
+                    if (s_j + 1 == s_n) umma_commit(bar_q_empty(buf));
+                    umma_commit(bar_kv_empty(G));       // V(G - 2), whose product was issued before, and K(G)
                 }
                 __syncwarp();
                 if (++s_j == s_n) {
                     s_n = tiles_of(++s_round);
                     s_j = 0;
-                    if (W::kQBufs == 1 || s_buf == 1) q_phase ^= 1;
-                    if (W::kQBufs == 2) s_buf ^= 1;
+                    ++s_item;
                 }
             };
-            auto step = [&]() {
-                if (++pos == NP) {
-                    pos = 0;
-                    kv_phase ^= 1;
-                }
-            };
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
+            for (int G = 0; G < 2; ++G)
                 if (s_n > 0) {
-                    wait_pair();
+                    wait_pair(G);
+                    wait_q();
                     tc_fence_after();
-                    next_s(t, !flag_is_set(abort_at));
+                    next_s(G, !flag_is_set(abort_at));
                 }
-                step();
-            }
-            int round = 0, n = tiles_of(0), g = 0;
-            uint32_t odd_item = 0;
-            for (uint32_t phase = 0; n > 0; phase ^= 1) {         // items without key tiles come last
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {                     // a stream each: unrolled, so that its addresses are constants
-                    if (n == 0) break;
+            int G = 0, items = 0;
+            for (int round = 0;; ++round) {
+                const int n = tiles_of(round);
+                if (n == 0) break;         // items without key tiles come last
+                for (int g = 0; g < n; ++g, ++G) {
+                    const int t = G & 1;
                     const bool ok = !flag_is_set(abort_at);
-                    wait_pair();
-                    if (g == 0) mbar_wait_poll(bar_o_free, odd_item ^ 1, wctx, (kRoleMma << 8) | kBarOFree);
-                    mbar_wait_poll(bar_p_full(t), phase, wctx, (kRoleMma << 8) | kBarPFull);
+                    wait_pair(G + 2);
+                    wait_q();
+                    if (g == 0) mbar_wait_poll(bar_o_free, (items & 1) ^ 1, wctx, (kRoleMma << 8) | kBarOFree);
+                    mbar_wait_poll(bar_p_full(t), (G >> 1) & 1, wctx, (kRoleMma << 8) | kBarPFull);
                     tc_fence_after();
                     if (leader) {
-                        if (ok) issue_pv(t, ring_lo_v + 2 * pos * kPartLo, g >= 2);
-                        if (g + 1 == n) group_commit<PAIR>(bar_o_full);
+                        if (ok) issue_pv(t, ring_lo_v + Ring::slot_v(G + 2) * kTileLo, g >= 2);
+                        if (g + 1 == n) umma_commit(bar_o_full);
                     }
                     __syncwarp();
-                    next_s(t, ok);
-                    step();
-                    if (++g == n) {
-                        n = tiles_of(++round);
-                        g = 0;
-                        odd_item ^= 1;
-                    }
+                    next_s(G + 2, ok);
                 }
+                ++items;
             }
-            // No MMA or commit of this thread may still be under way when the CTA ends (see the plain form): awaited below.
-            if (leader) group_commit<PAIR>(bar_drain);
+            // No MMA of this thread may still be running when TMEM is handed back (see the plain form).
+            if (leader) umma_commit(bar_drain);
+            mbar_wait_quiet(bar_drain, 0, kDrainLimitCycles);
         }
     } else if (wg == 2) {
         // ---------------------------------------------------------------- correction and epilogue
@@ -454,7 +399,7 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             if (h == 1 && cb == D / 32 - 1) {   // the accumulators are in registers: the next item may overwrite them
                                 tc_fence_before();
                                 __syncwarp();
-                                if (lane == 0) arrive_at_mma(bar_o_free);
+                                if (lane == 0) mbar_arrive(bar_o_free);
                             }
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
@@ -478,7 +423,7 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const float alpha = ld_shared_f32(sScale + (t * 128 + r) * 4);
                 if (g >= 2) rescale_o<D>(tmem_O(t) + lane_base, alpha);     // P V(G - 2) is complete: alpha(G) was posted after S(G) was seen
                 __syncwarp();
-                if (lane == 0) arrive_at_mma(bar_p_full(t));
+                if (lane == 0) mbar_arrive(bar_p_full(t));
             }
         }
     } else {
@@ -550,7 +495,7 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) arrive_at_mma(bar_p_full(t));
+                if (lane == 0) mbar_arrive(bar_p_full(t));
                 l_run = l_run * alpha + l_tile;
             }
             // The streams meet: the one that does not have the last tile leaves its anchor and row sum, the other joins them,
@@ -592,17 +537,9 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 12) {      // every role is through, so this arrives at once unless a wait expired
-        mbar_wait_quiet(bar_drain, 0, kDrainLimitCycles);
-        __syncwarp();
-    }
-    if constexpr (PAIR) {
-        cluster_arrive();      // nobody reaches into the other CTA any more
-        cluster_wait();
-    }
     if (warp == 12) {
         __syncwarp();
-        tmem_give<PAIR>(tmem, kTmemCols);
+        tmem_dealloc(tmem, kTmemCols);
     }
 }
 

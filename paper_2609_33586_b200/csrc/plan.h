@@ -24,8 +24,9 @@ struct SplitShape {
 // and the sum of O; from two thirds of the SMs on they slow each other by a tenth.  512 queries on 16K, 32/8 heads, streams of 40
 // calls: bf16 h15 218 -> 143 us, exact 256 -> 134, e4m3 h15 203 -> 132 (2 parts); 64 queries on 8K e4m3 90 -> 45 (4 parts).
 // 16 x 1K and 16 x 2K gain nothing and stay whole.
+// *steps gets the estimated time.
 template <class Fit>
-int split_parts(const SplitShape& s, int sms, Fit fit) {
+int split_parts(const SplitShape& s, int sms, Fit fit, double* steps = nullptr) {
     if (s.items > sms) return 1;
     const double longest = s.all, mean = 0.5 * (s.all + s.first);
     double best = 0.93 * (longest + 1.5);      // a gain below that is not worth the risk of being wrong
@@ -39,7 +40,35 @@ int split_parts(const SplitShape& s, int sms, Fit fit) {
         const double t = std::fmax(longest * per_tile + fixed, waves * (mean * per_tile + fixed)) * busy;
         if (t < best) { best = t; best_parts = parts; }
     }
+    if (steps != nullptr) *steps = best;
     return best_parts;
+}
+
+struct StreamShape {
+    double tiles, pairs;   // query tiles, and pairs of them, of all (batch, head)
+    int per_head;          // query tiles of a head
+    int nt;                // key tiles of the longest
+    int D;
+    bool causal;
+    bool one_anchor;       // the two streams hand the anchor on (all but the exact modes on 16-bit inputs)
+};
+
+// Whether the two-stream form (one query tile per CTA) is faster than the plain form, or than the split form where that would
+// give an item `parts` CTAs in `split_steps`.  In steps of the plain form, measured over 60 shapes: a key tile of one query tile
+// takes 0.64 (0.56 without the hand-over), an item boundary 3.0 against the plain form's 3.6.
+//   One tile per CTA: the plain form has as many steps in a row, each of a whole step.  Lost only to the longer set-up and joining of
+//   a few key tiles (D = 128: 3 tiles 8.9 -> 9.4 us, 5 to 12 tiles 21.9 -> 15.9 and 22.7 -> 16.2; D = 64: 2 tiles 8.3 -> 6.1).
+//   Causal, one pair but more than one tile per CTA: long and short tiles even out over two rounds (16 heads x 1408 23.8 -> 19.6 us,
+//   x 2304 36.2 -> 31.3), from 12 key tiles on (8 tiles 32.9 -> 40.1, which have three rounds).
+//   Full attention, all items equal: whole rounds decide (36 heads x 1337 x 2803 exact: 2 rounds of pairs 94 us, 3 of tiles 76).
+//   Other shapes have enough pairs: 48 heads x 2K 57.8 us in the plain form, 68.2 in this one.
+inline bool streams_pay(const StreamShape& s, int parts, double split_steps, int sms) {
+    const double tile = s.one_anchor ? 0.64 : 0.56, boundary = 3.0;
+    if (s.nt < (s.D == 64 ? 2 : 4)) return false;
+    if (parts > 1) return s.per_head > 1 && s.tiles <= sms && s.nt * tile + boundary < split_steps;
+    if (s.tiles <= sms) return true;
+    if (s.causal) return s.pairs <= sms && s.tiles <= 2.0 * sms && s.nt >= 12;
+    return 1.08 * std::ceil(s.tiles / sms) * (s.nt * tile + boundary) < std::ceil(s.pairs / sms) * (s.nt + 3.6);
 }
 
 struct RowsShape {

@@ -163,11 +163,6 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-// The same where nothing but TMEM is handed over, which the tcgen05 fences order: no release at cluster scope, which takes about
-// 1000 clocks.
-__device__ __forceinline__ void mbar_arrive_peer(uint32_t addr) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -387,85 +382,6 @@ __device__ __forceinline__ void umma_ts_lo(uint32_t d_tmem, uint32_t a_tmem, uin
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
-}
-
-// ---------------------------------------------------------------- cta_group::1 or, PAIR, cta_group::2
-// With cta_group::2 one MMA works on the tiles of a pair of CTAs: 256 rows, of which each CTA has its own 128 (its A operand and
-// its TMEM); of the B operand each CTA holds one half along N.  The first CTA issues; addresses are its own and hold in both.  All
-// of a kernel's tcgen05 instructions have to name the same group.
-template <bool PAIR>
-__device__ __forceinline__ void tmem_take(uint32_t smem_slot, uint32_t ncols) {
-    if constexpr (PAIR) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_slot), "r"(ncols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-        tmem_alloc(smem_slot, ncols);
-        tmem_relinquish();
-    }
-}
-template <bool PAIR>
-__device__ __forceinline__ void tmem_give(uint32_t taddr, uint32_t ncols) {
-    if constexpr (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-    else tmem_dealloc(taddr, ncols);
-}
-template <bool PAIR, bool kFp8>
-__device__ __forceinline__ void group_mma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
-    if constexpr (!PAIR) {
-        umma_ss_lo<kFp8>(d_tmem, a_lo, b_lo, desc_hi, idesc, accumulate);
-    } else if constexpr (kFp8) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-            "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %4, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-            "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-            "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
-            : "memory");
-    }
-}
-template <bool PAIR, bool kFp8>
-__device__ __forceinline__ void group_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate) {
-    if constexpr (!PAIR) {
-        umma_ts_lo<kFp8>(d_tmem, a_tmem, b_lo, desc_hi, idesc, accumulate);
-    } else if constexpr (kFp8) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-            "mov.b64 db, {%2, %3};\n\t"
-            "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], [%1], db, %4, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-            "mov.b64 db, {%2, %3};\n\t"
-            "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], db, %4, p;\n\t}"
-            ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
-            : "memory");
-    }
-}
-// Arrives, once every MMA issued so far by this thread has completed, on the barrier at this address: PAIR: in both CTAs.
-template <bool PAIR>
-__device__ __forceinline__ void group_commit(uint32_t bar) {
-    if constexpr (PAIR)
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                     ::"r"(bar), "h"(static_cast<uint16_t>(3)) : "memory");
-    else umma_commit(bar);
-}
-// A load into this CTA's shared memory; PAIR: its bytes may be counted on a barrier of the other CTA (no multicast).
-template <bool PAIR>
-__device__ __forceinline__ void group_load_4d(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2, int c3) {
-    if constexpr (PAIR)
-        asm volatile(
-            "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-            "[%0], [%1, {%3, %4, %5, %6}], [%2];"
-            ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-            : "memory");
-    else tma_load_4d(dst, m, bar, c0, c1, c2, c3);
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {

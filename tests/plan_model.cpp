@@ -60,6 +60,19 @@ int main() {
     };
     for (const auto& m : measured)
         CHECK(rows_pay(m.s, m.cs, 148) == (m.rows_us < m.plain_us), "%g groups of %d rows, %d key tiles: %.1f us, plain %.1f us", m.s.groups, m.s.rows, m.s.nt, m.rows_us, m.plain_us);
+    // Two streams or the plain form, measured (us): the faster one is taken.
+    const struct { StreamShape s; bool streams; } forms[] = {
+        {{4, 2, 2, 2, 64, true, true}, true},            // 8.3 against 6.1
+        {{128, 64, 8, 8, 128, true, true}, true},        // 17.7, 14.1
+        {{396, 216, 11, 22, 128, false, false}, true},   // 94, 76
+        {{396, 216, 11, 22, 128, false, true}, false},
+        {{288, 144, 18, 18, 128, true, true}, true},     // 36.2, 31.3
+        {{768, 384, 16, 16, 128, true, true}, false},    // 57.8, 68.2
+        {{768, 384, 24, 24, 64, true, true}, false},     // 66.2, 79.9
+        {{48, 32, 3, 3, 128, true, false}, false},       // 8.9, 9.4
+        {{280, 144, 35, 35, 128, false, true}, false},   // 61.3, 72.6
+    };
+    for (const auto& f : forms) CHECK(streams_pay(f.s, 1, 0.0, 148) == f.streams, "%g query tiles, %d key tiles", f.s.tiles, f.s.nt);
     std::puts("ok");
     return 0;
 }
