@@ -46,7 +46,8 @@ struct StreamsCfg {
 };
 
 // Register split (see the plain form).  The softmax warps have no epilogue here, the MMA warp looks two tiles ahead and the
-// correction warps join two accumulators: 200 / 56 / 56 spills in these, 192 / 64 / 64 does not.
+// correction warps join two accumulators: with 200 / 56 / 56 the MMA warp spills in its loop, with 192 / 64 / 64 only the epilogue
+// does (32 bytes, once an item).
 constexpr int kStreamRegSoftmax = 192, kStreamRegOther = 64;
 static_assert(256 * kStreamRegSoftmax + 256 * kStreamRegOther <= 512 * 128, "setmaxnreg targets exceed the launch allocation");
 
