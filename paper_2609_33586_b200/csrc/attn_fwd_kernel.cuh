@@ -145,127 +145,6 @@ __device__ __forceinline__ WorkItem part_of_item(WorkItem it, int rank, int part
     return it;
 }
 
-// Multiplies a row of an O accumulator (one row per thread, at the warp's lanes of `tO`) by alpha, unless no row of the warp moves.
-template <int D>
-__device__ __forceinline__ void rescale_o(uint32_t tO, float alpha) {
-    __syncwarp();
-    tc_fence_after();
-    if (__any_sync(0xffffffffu, alpha != 1.0f)) {
-#pragma unroll
-        for (int cc = 0; cc < D / 16; ++cc) {
-            uint32_t o[16];
-            tmem_ld16(tO + cc * 16, o);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 16; i += 2) {
-                const float2 v = fmul2(make_float2(__uint_as_float(o[i]), __uint_as_float(o[i + 1])), make_float2(alpha, alpha));
-                o[i] = __float_as_uint(v.x);
-                o[i + 1] = __float_as_uint(v.y);
-            }
-            tmem_st16(tO + cc * 16, o);
-        }
-        tmem_wait_st();
-    }
-    tc_fence_before();
-}
-
-// Scores at columns >= limit become -inf.
-__device__ __forceinline__ void mask_scores(uint32_t (&s)[4][32], int limit) {
-#pragma unroll
-    for (int cc = 0; cc < 4; ++cc)
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (cc * 32 + i >= limit) s[cc][i] = __float_as_uint(-INFINITY);
-}
-
-// The weights of one row of a key tile, its scores in s and its anchor m_use: P goes to TMEM at tP, the row sum is returned.
-// LATE: post_alpha is called after the first 32 weights (else not at all).  score_floor bounds the row's scores from below
-// (h15 family on fp8 inputs).
-template <bool FP8, bool HALF, int MODE, bool TAU, bool LATE, typename PostAlpha>
-__device__ __forceinline__ float tile_weights(uint32_t (&s)[4][32], bool masked_tile, int col_limit, float m_use, float score_floor,
-                                              const AttnParams& p, uint32_t tP, PostAlpha post_alpha) {
-    constexpr int kFam = h15_family_k(MODE);   // h15 family: the map takes the offset times 2^kFam
-    const float c_eff = static_cast<float>(1 << kFam) * p.c;
-    constexpr float p_off = static_cast<float>(PFormat<FP8, MODE>::kOffLog2);  // log2 of the P / row-sum scale
-    // 16-bit inputs: the h15 family uses the saturating form of weights_chunk32 (no row-minimum pass, no
-    // clamped or masked variants) whenever the anchor is always current (offsets <= 0); the deferred rescale,
-    // where a score may lie above its anchor, keeps the form with explicit clamps.  fp8 inputs keep the
-    // packed form: there a bound on the key magnitude already removes the row-minimum pass, and the
-    // scalar multiply-adds of the saturating form cost more issue slots than they save (measured 4 to 6 %).
-    constexpr bool kSatForm = kFam > 0 && !FP8 && !TAU;
-    // exact: x = s*c - m*c + P offset;  h15 family: scaled input 2^K x = s*(2^K c) - m*(2^K c);  pot: x = s*c - m*c
-    RowScale rs;
-    const float nmc = (is_exact_like(MODE) ? p_off : 0.0f) - m_use * c_eff;
-    rs.c = make_float2(c_eff, c_eff);
-    rs.nmc = make_float2(nmc, nmc);
-    rs.two22 = p.two22;
-    rs.pot_neg_cap = p.pot_neg_cap;
-    rs.pot_drop_x = p.pot_drop_x;
-    rs.clamp_lo = 0.f;
-    if constexpr (kFam > 0) rs.clamp_lo = masked_tile ? h15_clamp_zero<kFam>() : h15_clamp_floor<kFam>();
-    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    if constexpr (kSatForm) {
-        // distance below the anchor as a fraction of the clamp distance R, which is also where a masked
-        // score (-inf) ends up: 2^K * 126 (weight floor 2^-126, Eq. h15), in a tile with masked scores
-        // 2^K * 127 (pattern of +0)
-        constexpr float kR = 126.0f * (1 << kFam), kRm = 127.0f * (1 << kFam);
-        const float big_r = masked_tile ? kRm : kR;
-        const float inv_r = masked_tile ? 1.0f / kRm : 1.0f / kR;
-        rs.su = -c_eff * inv_r;
-        const float ou = (m_use * c_eff) * inv_r;
-        rs.ou = make_float2(ou, ou);
-        rs.sat_mul = -big_r;
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-            uint32_t pw[16];
-            weights_chunk32<FP8, MODE, false, true, HALF, true>(s[cc], rs, 32, acc, pw);
-            tmem_st16(tP + cc * 16, pw);
-        }
-    } else if (is_pot(MODE) && masked_tile) {
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-            uint32_t pw[16];
-            weights_chunk32<FP8, MODE, true, true, HALF>(s[cc], rs, col_limit - cc * 32, acc, pw);
-            if constexpr (FP8) tmem_st8(tP + cc * 8, pw);
-            else tmem_st16(tP + cc * 16, pw);
-            if (LATE && cc == 0) post_alpha();
-        }
-    } else {
-        // h15: the clamp is a no-op unless some score of the warp's rows lies more than 126 octaves
-        // below its anchor; the row minimum (one more three-input pass) tells, and the common case
-        // runs without the per-score clamp.  A tile with masked scores always takes the clamp.
-        bool clamp = false;
-        if constexpr (kFam > 0) {
-            if (masked_tile) {
-                clamp = true;
-            } else if (!__all_sync(0xffffffffu, (score_floor - m_use) * c_eff >= -125.0f * (1 << kFam))) {
-                const float lowest = (row_min128(s) - m_use) * c_eff;   // smallest scaled offset of the row
-                clamp = __any_sync(0xffffffffu, !(lowest >= -125.0f * (1 << kFam)));
-            }
-        }
-        if (clamp) {
-#pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-                uint32_t pw[16];
-                weights_chunk32<FP8, MODE, false, true, HALF>(s[cc], rs, 32, acc, pw);
-                if constexpr (FP8) tmem_st8(tP + cc * 8, pw);
-                else tmem_st16(tP + cc * 16, pw);
-                if (LATE && cc == 0) post_alpha();
-            }
-        } else {
-#pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-                uint32_t pw[16];
-                weights_chunk32<FP8, MODE, false, false, HALF>(s[cc], rs, 32, acc, pw);
-                if constexpr (FP8) tmem_st8(tP + cc * 8, pw);
-                else tmem_st16(tP + cc * 16, pw);
-                if (LATE && cc == 0) post_alpha();
-            }
-        }
-    }
-    return (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
-}
-
 }  // namespace
 
 // IN: storage type of q, k, v (kInBF16 / kInFP8 / kInFP16).  P has the type of V at 16 bits (the f16
@@ -623,7 +502,25 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                             // P V(j - 1) is complete: the softmax warps post alpha(j) after they have seen S(j), whose commit
                             // covers everything issued before it
                             if (r == 0) ROWMAX_STAMP(2, j, t * 4 + 1);
-                            rescale_o<D>(tmem_O(t) + lane_base, alpha);
+                            __syncwarp();
+                            tc_fence_after();
+                            if (__any_sync(0xffffffffu, alpha != 1.0f)) {
+#pragma unroll
+                                for (int cc = 0; cc < D / 16; ++cc) {
+                                    uint32_t o[16];
+                                    tmem_ld16(tmem_O(t) + lane_base + cc * 16, o);
+                                    tmem_wait_ld();
+#pragma unroll
+                                    for (int i = 0; i < 16; i += 2) {
+                                        const float2 v = fmul2(make_float2(__uint_as_float(o[i]), __uint_as_float(o[i + 1])), make_float2(alpha, alpha));
+                                        o[i] = __float_as_uint(v.x);
+                                        o[i + 1] = __float_as_uint(v.y);
+                                    }
+                                    tmem_st16(tmem_O(t) + lane_base + cc * 16, o);
+                                }
+                                tmem_wait_st();
+                            }
+                            tc_fence_before();
                         }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar_p_full(t));
@@ -647,6 +544,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
         const uint32_t tS = tmem_S(t) + lane_base;
         const uint32_t tO = tmem_O(t) + lane_base;
         constexpr int kFam = h15_family_k(MODE);   // h15 family: the map takes the offset times 2^kFam
+        const float c_eff = static_cast<float>(1 << kFam) * p.c;
+        // 16-bit inputs: the h15 family uses the saturating form of weights_chunk32 (no row-minimum pass, no
+        // clamped or masked variants) whenever the anchor is always current (offsets <= 0); the deferred rescale,
+        // where a score may lie above its anchor, keeps the form with explicit clamps.  fp8 inputs keep the
+        // packed form: there a bound on the key magnitude already removes the row-minimum pass, and the
+        // scalar multiply-adds of the saturating form cost more issue slots than they save (measured 4 to 6 %).
+        constexpr bool kLattice = kFam > 0 && !FP8;
+        constexpr bool kSatForm = kLattice && !TAU;
         int tiles = 0;
         int o_use = 0;      // items with key tiles so far
         for (int round = 0; !SPLIT || round < 1; ++round) {   // split form: one item per cluster
@@ -680,7 +585,14 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_pre_free(buf));
                     if (j < pre_n) {
-                        if ((it.pre_j0 + j + 1) * kTileN > tile_limit) mask_scores(s, row_limit - (it.pre_j0 + j) * kTileN);
+                        if ((it.pre_j0 + j + 1) * kTileN > tile_limit) {
+                            const int col_limit = row_limit - (it.pre_j0 + j) * kTileN;
+#pragma unroll
+                            for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+                                for (int i = 0; i < 32; ++i)
+                                    if (cc * 32 + i >= col_limit) s[cc][i] = __float_as_uint(-INFINITY);
+                        }
                         m_part = fmaxf(m_part, row_max128(s));
                     }
                 }
@@ -729,7 +641,13 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 // makes their hot loop markedly faster.
                 const bool masked_tile = (j0 + j + 1) * kTileN > tile_limit;
                 const int col_limit = row_limit - (j0 + j) * kTileN;
-                if (masked_tile) mask_scores(s, col_limit);
+                if (masked_tile) {
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if (cc * 32 + i >= col_limit) s[cc][i] = __float_as_uint(-INFINITY);
+                }
                 const float m_t = row_max128(s);
                 // The tile maximum becomes the new anchor when there is none yet or when it exceeds the
                 // anchor by more than tau octaves (tau = 0: always, so the anchor is the running maximum).
@@ -752,7 +670,78 @@ attn_fwd_ws_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constan
                 };
                 if constexpr (!kOutOfStep) post_alpha();
 
-                const float l_tile = tile_weights<FP8, HALF, MODE, TAU, kOutOfStep>(s, masked_tile, col_limit, m_use, score_floor, p, tS, post_alpha);
+                // exact: x = s*c - m*c + P offset;  h15 family: scaled input 2^K x = s*(2^K c) - m*(2^K c);  pot: x = s*c - m*c
+                RowScale rs;
+                float nmc = (is_exact_like(MODE) ? p_off : 0.0f) - m_use * c_eff;
+                float c_row = c_eff;
+                rs.c = make_float2(c_row, c_row);
+                rs.nmc = make_float2(nmc, nmc);
+                rs.two22 = p.two22;
+                rs.pot_neg_cap = p.pot_neg_cap;
+                rs.pot_drop_x = p.pot_drop_x;
+                rs.clamp_lo = 0.f;
+                if constexpr (kFam > 0) rs.clamp_lo = masked_tile ? h15_clamp_zero<kFam>() : h15_clamp_floor<kFam>();
+                float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                if constexpr (kSatForm) {
+                    // distance below the anchor as a fraction of the clamp distance R, which is also where a masked
+                    // score (-inf) ends up: 2^K * 126 (weight floor 2^-126, Eq. h15), in a tile with masked scores
+                    // 2^K * 127 (pattern of +0)
+                    constexpr float kR = 126.0f * (1 << kFam), kRm = 127.0f * (1 << kFam);
+                    const float big_r = masked_tile ? kRm : kR;
+                    const float inv_r = masked_tile ? 1.0f / kRm : 1.0f / kR;
+                    rs.su = -c_eff * inv_r;
+                    const float ou = (m_use * c_eff) * inv_r;
+                    rs.ou = make_float2(ou, ou);
+                    rs.sat_mul = -big_r;
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) {
+                        uint32_t pw[16];
+                        weights_chunk32<FP8, MODE, false, true, HALF, true>(s[cc], rs, 32, acc, pw);
+                        tmem_st16(tS + cc * 16, pw);
+                    }
+                } else if (is_pot(MODE) && masked_tile) {
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) {
+                        uint32_t pw[16];
+                        weights_chunk32<FP8, MODE, true, true, HALF>(s[cc], rs, col_limit - cc * 32, acc, pw);
+                        if constexpr (FP8) tmem_st8(tS + cc * 8, pw);
+                        else tmem_st16(tS + cc * 16, pw);
+                        if (kOutOfStep && cc == 0) post_alpha();
+                    }
+                } else {
+                    // h15: the clamp is a no-op unless some score of the warp's rows lies more than 126 octaves
+                    // below its anchor; the row minimum (one more three-input pass) tells, and the common case
+                    // runs without the per-score clamp.  A tile with masked scores always takes the clamp.
+                    bool clamp = false;
+                    if constexpr (kFam > 0) {
+                        if (masked_tile) {
+                            clamp = true;
+                        } else if (!__all_sync(0xffffffffu, (score_floor - m_use) * c_eff >= -125.0f * (1 << kFam))) {
+                            const float lowest = (row_min128(s) - m_use) * c_eff;   // smallest scaled offset of the row
+                            clamp = __any_sync(0xffffffffu, !(lowest >= -125.0f * (1 << kFam)));
+                        }
+                    }
+                    if (clamp) {
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) {
+                            uint32_t pw[16];
+                            weights_chunk32<FP8, MODE, false, true, HALF>(s[cc], rs, 32, acc, pw);
+                            if constexpr (FP8) tmem_st8(tS + cc * 8, pw);
+                            else tmem_st16(tS + cc * 16, pw);
+                            if (kOutOfStep && cc == 0) post_alpha();
+                        }
+                    } else {
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) {
+                            uint32_t pw[16];
+                            weights_chunk32<FP8, MODE, false, false, HALF>(s[cc], rs, 32, acc, pw);
+                            if constexpr (FP8) tmem_st8(tS + cc * 8, pw);
+                            else tmem_st16(tS + cc * 16, pw);
+                            if (kOutOfStep && cc == 0) post_alpha();
+                        }
+                    }
+                }
+                const float l_tile = (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
                 if (r == 0) ROWMAX_STAMP(t, j, 3);
                 tmem_wait_st();
                 tc_fence_before();

@@ -84,6 +84,130 @@ __device__ __forceinline__ void wait_count(uint32_t at, int want, const WaitCtx&
     }
 }
 
+// Rescaling, masking and weights as in the roles of the plain form, where the same code stands inline: as calls of these functions
+// it ran slower there (16K, 32/8 heads, bf16 h15: 1834 -> 1861 us; 48 heads x 2K 64.9 -> 65.4).
+
+// Multiplies a row of an O accumulator (one row per thread, at the warp's lanes of `tO`) by alpha, unless no row of the warp moves.
+template <int D>
+__device__ __forceinline__ void rescale_o(uint32_t tO, float alpha) {
+    __syncwarp();
+    tc_fence_after();
+    if (__any_sync(0xffffffffu, alpha != 1.0f)) {
+#pragma unroll
+        for (int cc = 0; cc < D / 16; ++cc) {
+            uint32_t o[16];
+            tmem_ld16(tO + cc * 16, o);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+                const float2 v = fmul2(make_float2(__uint_as_float(o[i]), __uint_as_float(o[i + 1])), make_float2(alpha, alpha));
+                o[i] = __float_as_uint(v.x);
+                o[i + 1] = __float_as_uint(v.y);
+            }
+            tmem_st16(tO + cc * 16, o);
+        }
+        tmem_wait_st();
+    }
+    tc_fence_before();
+}
+
+// Scores at columns >= limit become -inf.
+__device__ __forceinline__ void mask_scores(uint32_t (&s)[4][32], int limit) {
+#pragma unroll
+    for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (cc * 32 + i >= limit) s[cc][i] = __float_as_uint(-INFINITY);
+}
+
+// The weights of one row of a key tile, its scores in s and its anchor m_use: P goes to TMEM at tP, the row sum is returned.
+// LATE: post_alpha is called after the first 32 weights (else not at all).  score_floor bounds the row's scores from below
+// (h15 family on fp8 inputs).
+template <bool FP8, bool HALF, int MODE, bool TAU, bool LATE, typename PostAlpha>
+__device__ __forceinline__ float tile_weights(uint32_t (&s)[4][32], bool masked_tile, int col_limit, float m_use, float score_floor,
+                                              const AttnParams& p, uint32_t tP, PostAlpha post_alpha) {
+    constexpr int kFam = h15_family_k(MODE);   // h15 family: the map takes the offset times 2^kFam
+    const float c_eff = static_cast<float>(1 << kFam) * p.c;
+    constexpr float p_off = static_cast<float>(PFormat<FP8, MODE>::kOffLog2);  // log2 of the P / row-sum scale
+    // 16-bit inputs: the h15 family uses the saturating form of weights_chunk32 (no row-minimum pass, no
+    // clamped or masked variants) whenever the anchor is always current (offsets <= 0); the deferred rescale,
+    // where a score may lie above its anchor, keeps the form with explicit clamps.  fp8 inputs keep the
+    // packed form: there a bound on the key magnitude already removes the row-minimum pass, and the
+    // scalar multiply-adds of the saturating form cost more issue slots than they save (measured 4 to 6 %).
+    constexpr bool kSatForm = kFam > 0 && !FP8 && !TAU;
+    // exact: x = s*c - m*c + P offset;  h15 family: scaled input 2^K x = s*(2^K c) - m*(2^K c);  pot: x = s*c - m*c
+    RowScale rs;
+    const float nmc = (is_exact_like(MODE) ? p_off : 0.0f) - m_use * c_eff;
+    rs.c = make_float2(c_eff, c_eff);
+    rs.nmc = make_float2(nmc, nmc);
+    rs.two22 = p.two22;
+    rs.pot_neg_cap = p.pot_neg_cap;
+    rs.pot_drop_x = p.pot_drop_x;
+    rs.clamp_lo = 0.f;
+    if constexpr (kFam > 0) rs.clamp_lo = masked_tile ? h15_clamp_zero<kFam>() : h15_clamp_floor<kFam>();
+    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    if constexpr (kSatForm) {
+        // distance below the anchor as a fraction of the clamp distance R, which is also where a masked
+        // score (-inf) ends up: 2^K * 126 (weight floor 2^-126, Eq. h15), in a tile with masked scores
+        // 2^K * 127 (pattern of +0)
+        constexpr float kR = 126.0f * (1 << kFam), kRm = 127.0f * (1 << kFam);
+        const float big_r = masked_tile ? kRm : kR;
+        const float inv_r = masked_tile ? 1.0f / kRm : 1.0f / kR;
+        rs.su = -c_eff * inv_r;
+        const float ou = (m_use * c_eff) * inv_r;
+        rs.ou = make_float2(ou, ou);
+        rs.sat_mul = -big_r;
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+            uint32_t pw[16];
+            weights_chunk32<FP8, MODE, false, true, HALF, true>(s[cc], rs, 32, acc, pw);
+            tmem_st16(tP + cc * 16, pw);
+        }
+    } else if (is_pot(MODE) && masked_tile) {
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+            uint32_t pw[16];
+            weights_chunk32<FP8, MODE, true, true, HALF>(s[cc], rs, col_limit - cc * 32, acc, pw);
+            if constexpr (FP8) tmem_st8(tP + cc * 8, pw);
+            else tmem_st16(tP + cc * 16, pw);
+            if (LATE && cc == 0) post_alpha();
+        }
+    } else {
+        // h15: the clamp is a no-op unless some score of the warp's rows lies more than 126 octaves
+        // below its anchor; the row minimum (one more three-input pass) tells, and the common case
+        // runs without the per-score clamp.  A tile with masked scores always takes the clamp.
+        bool clamp = false;
+        if constexpr (kFam > 0) {
+            if (masked_tile) {
+                clamp = true;
+            } else if (!__all_sync(0xffffffffu, (score_floor - m_use) * c_eff >= -125.0f * (1 << kFam))) {
+                const float lowest = (row_min128(s) - m_use) * c_eff;   // smallest scaled offset of the row
+                clamp = __any_sync(0xffffffffu, !(lowest >= -125.0f * (1 << kFam)));
+            }
+        }
+        if (clamp) {
+#pragma unroll
+            for (int cc = 0; cc < 4; ++cc) {
+                uint32_t pw[16];
+                weights_chunk32<FP8, MODE, false, true, HALF>(s[cc], rs, 32, acc, pw);
+                if constexpr (FP8) tmem_st8(tP + cc * 8, pw);
+                else tmem_st16(tP + cc * 16, pw);
+                if (LATE && cc == 0) post_alpha();
+            }
+        } else {
+#pragma unroll
+            for (int cc = 0; cc < 4; ++cc) {
+                uint32_t pw[16];
+                weights_chunk32<FP8, MODE, false, false, HALF>(s[cc], rs, 32, acc, pw);
+                if constexpr (FP8) tmem_st8(tP + cc * 8, pw);
+                else tmem_st16(tP + cc * 16, pw);
+                if (LATE && cc == 0) post_alpha();
+            }
+        }
+    }
+    return (acc[0].x + acc[0].y) + (acc[1].x + acc[1].y);
+}
+
 // Stores 16 rows x 32 columns of O as bf16.  `v` is laid out as tcgen05.ld.16x256b.x4 gives it: of each 8 columns lane i has
 // columns 2 (i mod 4) and the next of row i / 4 (v[4k], v[4k + 1]) and of row i / 4 + 8 (v[4k + 2], v[4k + 3]).  The four lanes of
 // a row exchange their words so that each has 16 bytes in a row: a store then takes 8 rows x 64 bytes, whole sectors, where one
