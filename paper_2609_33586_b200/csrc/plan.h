@@ -50,12 +50,12 @@ struct StreamShape {
     int nt;                // key tiles of the longest
     int D;
     bool causal;
-    bool one_anchor;       // the two streams hand the anchor on (all but the exact modes on 16-bit inputs)
+    bool one_anchor;       // all but the exact modes on 16-bit inputs
 };
 
 // Whether the two-stream form (one query tile per CTA) is faster than the plain form, or than the split form where that would
 // give an item `parts` CTAs in `split_steps`.  In steps of the plain form, measured over 60 shapes: a key tile of one query tile
-// takes 0.64 (0.56 without the hand-over), an item boundary 3.0 against the plain form's 3.6.
+// takes 0.64 (0.56 in the exact modes on 16-bit inputs), an item boundary 3.0 against the plain form's 3.6.
 //   One tile per CTA: the plain form has as many steps in a row, each of a whole step.  Lost only to the longer set-up and joining of
 //   a few key tiles (D = 128: 3 tiles 8.9 -> 9.4 us, 5 to 12 tiles 21.9 -> 15.9 and 22.7 -> 16.2; D = 64: 2 tiles 8.3 -> 6.1).
 //   Causal, one pair but more than one tile per CTA: long and short tiles even out over two rounds (16 heads x 1408 23.8 -> 19.6 us,

@@ -1,10 +1,11 @@
 """GPU parity of the two-stream form (one query tile per CTA): one and two tiles of an item, odd and even numbers of key tiles,
 items that begin in either stream, more items than SMs, rows without keys, ragged ends."""
 import pytest
+import torch
 
 from oracle import cpu_oracle as orc
 from paper_2609_33586_b200 import binding
-from paper_2609_33586_b200.inputs import Workload
+from paper_2609_33586_b200.inputs import Workload, make_inputs
 
 from parity_util import compare
 
@@ -28,6 +29,14 @@ def _device_status_is_clean():
     assert binding.device_status() == 0
 
 
+PLAIN = (binding.KERNEL_PLAIN, 1)
+
+
+def plan_of(wl, mode):
+    dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
+    return binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)
+
+
 @pytest.mark.parametrize("mode", [orc.W_EXACT, orc.W_POT, orc.W_H15])
 @pytest.mark.parametrize("wl", SHAPES, ids=lambda w: w.name)
 def test_two_streams_match_the_oracle(wl, mode):
@@ -43,3 +52,28 @@ def test_two_streams_match_the_oracle(wl, mode):
 def test_two_streams_family_members(dtype, mode):
     st = compare(Workload("streams_family", 1, 4, 4, 500, 900, 128, True, dtype, 128), mode, model_p_storage=True)
     assert st["ok"], st
+
+
+@pytest.mark.parametrize("mode", [orc.W_EXACT, orc.W_POT, orc.W_H15])
+@pytest.mark.parametrize("wl,copies", [
+    (Workload("anchor_full", 1, 12, 2, 1337, 700, 128, False, "bf16", 129), 12),
+    (Workload("anchor_causal", 1, 16, 4, 1000, 1000, 128, True, "bf16", 130, peaked_keys=True), 8),
+    (Workload("anchor_fp16_d64", 1, 8, 8, 700, 700, 64, True, "fp16", 131), 24),
+    (Workload("anchor_fp8", 1, 16, 16, 1000, 1000, 128, True, "fp8_e4m3", 132), 8)], ids=lambda x: getattr(x, "name", None))
+def test_two_streams_round_p_as_the_plain_form_does(wl, copies, mode):
+    """The same heads, alone (two streams) and among many (plain form): P has the same bits, so that O differs by fp32 sums alone.
+    Those move O by less than 2^-16 of itself before it is rounded to bf16, so at most 2 x 2^-16 / 2^-8 of its values fall on the
+    other side of a rounding and move by up to 2^-8 (2-norm sqrt(2^-7) 2^-8 = 3.5e-4).  P rounded about the maxima of a stream's own
+    tiles moves O by 2e-3 in the exact mode on 16-bit inputs."""
+    inp = make_inputs(wl)
+    q, k, v = inp.q.cuda(), inp.k.cuda(), inp.v.cuda()
+    many = [x.expand(copies, *x.shape[1:]).contiguous() if x.dtype != torch.float8_e4m3fn else
+            x.view(torch.uint8).expand(copies, *x.shape[1:]).contiguous().view(x.dtype) for x in (q, k, v)]
+    assert plan_of(wl, mode) != PLAIN and plan_of(wl.with_(B=copies), mode) == PLAIN
+    kw = dict(causal=wl.causal, softmax_scale=wl.softmax_scale, weight_mode=mode, q_descale=inp.q_descale, k_descale=inp.k_descale,
+              v_descale=inp.v_descale)
+    o, lse = binding.attn_fwd(q, k, v, **kw)
+    want, want_lse = binding.attn_fwd(*many, **kw)
+    o, want = o[0].double(), want[copies // 2].double()
+    assert ((o - want).norm() / want.norm()).item() < 3.5e-4
+    assert (lse[0] - want_lse[copies // 2]).abs().max().item() < 1e-5
