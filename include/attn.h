@@ -193,12 +193,14 @@ int attn_get_schedule(int D, int in_dtype, int weight_mode, int causal,
  * attn_get_plan — which kernel attn_fwd (or attn_fwd_pot) would take for a shape on the current device, and how many CTAs
  * would share a piece of its work.  The order in which fp32 sums are added follows from it, so O and LSE may differ in their
  * last bits between devices with other SM counts.
- *   kernel  ATTN_KERNEL_PLAIN: one CTA takes a pair of query tiles (ctas = 1); ATTN_KERNEL_SHARED: ctas CTAs share one,
- *           each with some of its keys or (2) each with one of its query tiles; ATTN_KERNEL_FEW_ROWS: few query rows per key/value head, ctas CTAs share a head
+ *   kernel  ATTN_KERNEL_PLAIN: one CTA takes a pair of query tiles (ctas = 1); ATTN_KERNEL_SHARED: ctas CTAs share one, each
+ *           with some of its keys; ATTN_KERNEL_FEW_ROWS: few query rows per key/value head, ctas CTAs share a head;
+ *           ATTN_KERNEL_STREAMS: one CTA takes one query tile (ctas = 1) and adds up its even and its odd key tiles apart
  */
 #define ATTN_KERNEL_PLAIN 0
 #define ATTN_KERNEL_SHARED 1
 #define ATTN_KERNEL_FEW_ROWS 2
+#define ATTN_KERNEL_STREAMS 3
 int attn_get_plan(int B, int Hq, int Hkv, int Sq, int Sk, int D, int causal, int weight_mode, int in_dtype,
                   int* kernel, int* ctas);
 

@@ -15,7 +15,7 @@ import torch
 W_EXACT, W_POT, W_H15, W_H15K2, W_H15K3, W_EXACT_POLY = 0, 1, 2, 3, 4, 5
 IN_BF16, IN_FP8_E4M3, IN_FP16 = 0, 1, 2
 P_BF16, P_E4M3, P_E5M2, P_FP16 = 0, 1, 2, 3
-KERNEL_PLAIN, KERNEL_SHARED, KERNEL_FEW_ROWS = 0, 1, 2
+KERNEL_PLAIN, KERNEL_SHARED, KERNEL_FEW_ROWS, KERNEL_STREAMS = 0, 1, 2, 3
 MODES = {"exact": W_EXACT, "pot": W_POT, "h15": W_H15, "h15k2": W_H15K2, "h15k3": W_H15K3,
          "exact_poly": W_EXACT_POLY}
 
@@ -142,8 +142,8 @@ def get_schedule(D: int, in_dtype: int, weight_mode: int, causal: bool) -> dict:
 
 
 def get_plan(B: int, Hq: int, Hkv: int, Sq: int, Sk: int, D: int, causal: bool, weight_mode: int, in_dtype: int) -> tuple[int, int]:
-    """(kernel, CTAs that share a piece of work) of attn_fwd for a shape on the current device: KERNEL_PLAIN, _SHARED, _FEW_ROWS.
-    `in_dtype` is in_dtype_of(q)."""
+    """(kernel, CTAs that share a piece of work) of attn_fwd for a shape on the current device: KERNEL_PLAIN, _SHARED, _FEW_ROWS,
+    _STREAMS.  `in_dtype` is in_dtype_of(q)."""
     kernel, ctas = ctypes.c_int(), ctypes.c_int()
     rc = lib().attn_get_plan(B, Hq, Hkv, Sq, Sk, D, int(causal), weight_mode, in_dtype, ctypes.addressof(kernel), ctypes.addressof(ctas))
     if rc != 0:

@@ -137,18 +137,14 @@ namespace {
 
 struct Plan {
     int kernel, ctas;
-    bool streams;     // the two-stream form: each query tile of a pair has a CTA of its own
 };
 // Which kernel a forward takes; `mode` is the kernel's.
 Plan make_plan(int D, int in_dtype, int mode, const rowmax::AttnParams& p) {
-    if (const int cs = rowmax::plan_attn_rows(D, in_dtype, mode, p)) return {ATTN_KERNEL_FEW_ROWS, cs, false};
+    if (const int cs = rowmax::plan_attn_rows(D, in_dtype, mode, p)) return {ATTN_KERNEL_FEW_ROWS, cs};
     double steps = 0.0;
     const int parts = rowmax::plan_attn_split(D, in_dtype, mode, p, &steps);
-    if (rowmax::plan_attn_streams(D, in_dtype, mode, parts, steps, p)) {
-        const bool two = p.Sq > rowmax::kTileM;
-        return {two ? ATTN_KERNEL_SHARED : ATTN_KERNEL_PLAIN, two ? 2 : 1, true};
-    }
-    return {parts > 1 ? ATTN_KERNEL_SHARED : ATTN_KERNEL_PLAIN, parts, false};
+    if (rowmax::plan_attn_streams(D, in_dtype, mode, parts, steps, p)) return {ATTN_KERNEL_STREAMS, 1};
+    return {parts > 1 ? ATTN_KERNEL_SHARED : ATTN_KERNEL_PLAIN, parts};
 }
 
 int check_shape(int B, int Hq, int Hkv, int Sq, int Sk, int D) {
@@ -228,7 +224,7 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     } else {
         if ((rc = make_tile_map(&tq, q, fp8, half_in, B, Sq, Hq, D)) != ATTN_OK) return rc;
         if (p.tau > 0.0f) e = rowmax::launch_attn_fwd_tau(D, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
-        else if (plan.streams) e = rowmax::launch_attn_fwd_streams(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
+        else if (plan.kernel == ATTN_KERNEL_STREAMS) e = rowmax::launch_attn_fwd_streams(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
         else if (plan.kernel == ATTN_KERNEL_SHARED) e = rowmax::launch_attn_fwd_split(D, in_dtype, kernel_mode, plan.ctas, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
         else e = rowmax::launch_attn_fwd(D, in_dtype, kernel_mode, tq, tk, tv, p, static_cast<cudaStream_t>(stream));
     }

@@ -511,7 +511,7 @@ def test_drawn_sizes_match_the_oracle():
         assert st["ok"], (c, st)
         dt = binding.in_dtype_of(torch.empty(0, dtype=cases.DTYPES[wl.in_dtype]))
         kernels.add(binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)[0])
-    assert kernels == {binding.KERNEL_PLAIN, binding.KERNEL_SHARED, binding.KERNEL_FEW_ROWS}
+    assert kernels == {binding.KERNEL_PLAIN, binding.KERNEL_SHARED, binding.KERNEL_FEW_ROWS, binding.KERNEL_STREAMS}
 
 
 def test_threads_with_streams_of_their_own():

@@ -33,8 +33,9 @@ SHAPES = [
     Workload("rounds_n32_fp8", 1, 8, 1, 4, 40000, 128, True, "fp8_e4m3", 93),
 ]
 
-# Shapes that the few-row kernel could take, of so few keys that the plain form is faster.
-PLAIN = {"one_key", "one_tile", "tile_plus_one", "rows_32_full", "rows_without_keys"}
+# Shapes that the few-row kernel could take, of so few keys that the plain or the two-stream form is faster.
+PLAIN = {"one_key", "one_tile", "tile_plus_one", "rows_without_keys"}
+STREAMS = {"rows_32_full"}
 
 
 @pytest.fixture(autouse=True)
@@ -49,7 +50,7 @@ def _device_status_is_clean():
 def test_few_rows_match_the_oracle(wl, mode):
     dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
     kernel, _ = binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)
-    assert kernel == (binding.KERNEL_PLAIN if wl.name in PLAIN else binding.KERNEL_FEW_ROWS), wl.name
+    assert kernel == (binding.KERNEL_PLAIN if wl.name in PLAIN else binding.KERNEL_STREAMS if wl.name in STREAMS else binding.KERNEL_FEW_ROWS), wl.name
     st = compare(wl, mode, model_p_storage=True)
     assert st["ok"], st
 

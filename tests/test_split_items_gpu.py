@@ -13,11 +13,11 @@ from parity_util import compare
 pytestmark = pytest.mark.gpu
 
 SHAPES = [
-    Workload("two_parts_chunk", 1, 32, 16, 512, 6000, 128, True, "bf16", 101),       # 64 items: 2 CTAs each
+    Workload("two_parts", 1, 64, 16, 100, 6000, 128, True, "bf16", 101),       # 64 items of one query tile: 2 CTAs each
     Workload("four_parts_fp8", 1, 16, 16, 100, 5000, 128, True, "fp8_e4m3", 102),
     Workload("eight_parts_d64", 1, 2, 2, 300, 4099, 64, False, "fp16", 103),
     Workload("causal_prompt", 1, 2, 2, 3000, 3000, 128, True, "fp8_e4m3", 104, peaked_keys=True),
-    Workload("causal_prompt_bf16", 1, 4, 2, 2304, 2304, 64, True, "bf16", 105),
+    Workload("causal_prompt_bf16", 1, 2, 1, 3000, 3000, 64, True, "bf16", 105),
     Workload("few_keys_early", 1, 1, 1, 700, 1900, 128, True, "bf16", 106),
     Workload("fp8_d64", 1, 3, 1, 257, 4500, 64, True, "fp8_e4m3", 107),
 ]
@@ -41,12 +41,20 @@ def parts_of(wl, mode):
 @pytest.mark.parametrize("mode", [orc.W_EXACT, orc.W_POT, orc.W_H15])
 @pytest.mark.parametrize("wl", SHAPES, ids=lambda w: w.name)
 def test_shared_items_match_the_oracle(wl, mode):
-    assert parts_of(wl, mode) > 1
+    assert parts_of(wl, mode) > 1 and (wl.name != "two_parts" or parts_of(wl, mode) == 2)
     rows = None
     if wl.Sq * wl.Sk * wl.Hq > 3e7:
         import numpy as np
         rows = np.unique(np.concatenate([np.arange(0, wl.Sq, 17), np.arange(max(0, wl.Sq - 130), wl.Sq)])).astype(np.int32)
     st = compare(wl, mode, rows=rows, model_p_storage=True)
+    assert st["ok"], st
+
+
+def test_two_parts_of_a_pair_of_query_tiles():
+    """Exact mode on 16-bit inputs: with a maxima pass two parts are not planned for items of two query tiles."""
+    wl = Workload("two_parts_two_tiles", 1, 48, 12, 200, 6400, 128, True, "bf16", 109)
+    assert parts_of(wl, orc.W_EXACT) == 2
+    st = compare(wl, orc.W_EXACT, rows=list(range(0, 200, 7)) + [127, 128, 199])
     assert st["ok"], st
 
 

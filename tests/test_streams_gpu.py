@@ -17,9 +17,13 @@ SHAPES = [
     Workload("rows_without_keys", 1, 2, 2, 700, 400, 64, True, "fp16", 123),
     Workload("prompt_fp8", 1, 16, 16, 1024, 1024, 128, True, "fp8_e4m3", 124),     # one item per CTA
     Workload("two_rounds", 1, 16, 16, 1500, 1500, 128, True, "bf16", 125, peaked_keys=True),   # 192 items: one or two per CTA
-    Workload("three_rounds_full", 3, 12, 2, 1337, 2803, 128, False, "bf16", 126),  # exact mode: 396 items
-    Workload("chunk_of_context", 1, 8, 2, 700, 3001, 128, True, "fp8_e4m3", 127),
+    Workload("chunk_of_context", 1, 20, 4, 700, 2000, 128, True, "fp8_e4m3", 127),
+    # more items than SMs, with two staged query tiles and four pairs of ring slots
+    Workload("two_rounds_fp8", 1, 16, 16, 1664, 1664, 128, True, "fp8_e4m3", 133),       # 13 key tiles
+    Workload("two_rounds_d64", 1, 16, 16, 1664, 1664, 64, True, "bf16", 134, peaked_keys=True),
+    Workload("two_rounds_full", 4, 64, 8, 100, 1100, 128, False, "fp8_e4m3", 135),       # 256 items of 9 key tiles
 ]
+THREE_ROUNDS = Workload("three_rounds_full", 3, 12, 2, 1337, 2803, 128, False, "bf16", 126)
 
 
 @pytest.fixture(autouse=True)
@@ -29,7 +33,7 @@ def _device_status_is_clean():
     assert binding.device_status() == 0
 
 
-PLAIN = (binding.KERNEL_PLAIN, 1)
+PLAIN, STREAMS = (binding.KERNEL_PLAIN, 1), (binding.KERNEL_STREAMS, 1)
 
 
 def plan_of(wl, mode):
@@ -40,17 +44,26 @@ def plan_of(wl, mode):
 @pytest.mark.parametrize("mode", [orc.W_EXACT, orc.W_POT, orc.W_H15])
 @pytest.mark.parametrize("wl", SHAPES, ids=lambda w: w.name)
 def test_two_streams_match_the_oracle(wl, mode):
+    assert plan_of(wl, mode) == STREAMS
     rows = None
     if wl.Sq * wl.Sk * wl.Hq * wl.B > 3e7:
-        rows = sorted(set(range(0, wl.Sq, 61)) | set(range(max(0, wl.Sq - 130), wl.Sq, 3)) | set(range(0, 130, 3)))
+        rows = sorted((set(range(0, wl.Sq, 61)) | set(range(max(0, wl.Sq - 130), wl.Sq, 3)) | set(range(0, 130, 3))) & set(range(wl.Sq)))
     st = compare(wl, mode, rows=rows, model_p_storage=True)
+    assert st["ok"], st
+
+
+def test_two_streams_over_three_rounds_of_items():
+    assert plan_of(THREE_ROUNDS, orc.W_EXACT) == STREAMS      # 396 items; the rounding maps take the plain form
+    st = compare(THREE_ROUNDS, orc.W_EXACT, rows=sorted(set(range(0, 1337, 61)) | set(range(1207, 1337, 3)) | set(range(0, 130, 3))))
     assert st["ok"], st
 
 
 @pytest.mark.parametrize("dtype", ["bf16", "fp8_e4m3"])
 @pytest.mark.parametrize("mode", [orc.W_H15K2, orc.W_H15K3])
 def test_two_streams_family_members(dtype, mode):
-    st = compare(Workload("streams_family", 1, 4, 4, 500, 900, 128, True, dtype, 128), mode, model_p_storage=True)
+    wl = Workload("streams_family", 1, 4, 4, 500, 900, 128, True, dtype, 128)
+    assert plan_of(wl, mode) == STREAMS
+    st = compare(wl, mode, model_p_storage=True)
     assert st["ok"], st
 
 
@@ -69,7 +82,7 @@ def test_two_streams_round_p_as_the_plain_form_does(wl, copies, mode):
     q, k, v = inp.q.cuda(), inp.k.cuda(), inp.v.cuda()
     many = [x.expand(copies, *x.shape[1:]).contiguous() if x.dtype != torch.float8_e4m3fn else
             x.view(torch.uint8).expand(copies, *x.shape[1:]).contiguous().view(x.dtype) for x in (q, k, v)]
-    assert plan_of(wl, mode) != PLAIN and plan_of(wl.with_(B=copies), mode) == PLAIN
+    assert plan_of(wl, mode) == STREAMS and plan_of(wl.with_(B=copies), mode) == PLAIN
     kw = dict(causal=wl.causal, softmax_scale=wl.softmax_scale, weight_mode=mode, q_descale=inp.q_descale, k_descale=inp.k_descale,
               v_descale=inp.v_descale)
     o, lse = binding.attn_fwd(q, k, v, **kw)
