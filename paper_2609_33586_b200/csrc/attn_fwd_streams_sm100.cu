@@ -61,9 +61,7 @@ bool plan_attn_streams(int D, int in_type, int mode, int parts, double split_ste
     if (p.tau > 0.0f || exact_poly_eighths(mode) > 0) return false;
     int dev = 0, sms = 0;
     if (device_and_sms(&dev, &sms) != cudaSuccess) return false;
-    const long long heads = static_cast<long long>(p.Hq) * p.B, per_head = (p.Sq + kTileM - 1) / kTileM;
-    const StreamShape s{static_cast<double>(heads * per_head), static_cast<double>(heads * ((per_head + 1) / 2)), static_cast<int>(per_head),
-                        (p.Sk + kTileN - 1) / kTileN, D, p.causal != 0, split_takes_maxima(mode, in_type == kInFP8)};
+    const StreamShape s{static_cast<long long>(p.Hq) * p.B, p.Sq, p.Sk, D, p.causal != 0, is_exact_like(mode), in_type == kInFP8};
     return streams_pay(s, parts, split_steps, sms);
 }
 

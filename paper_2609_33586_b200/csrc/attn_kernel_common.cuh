@@ -4,10 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-namespace rowmax {
+#include "plan.h"
 
-constexpr int kTileM = 128;  // query rows per tile
-constexpr int kTileN = 128;  // keys per tile
+namespace rowmax {
 
 // storage type of q, k, v (the values of ATTN_IN_* in the C interface)
 enum InType : int { kInBF16 = 0, kInFP8 = 1, kInFP16 = 2 };

@@ -6,6 +6,9 @@
 
 namespace rowmax {
 
+constexpr int kTileM = 128;  // query rows per tile
+constexpr int kTileN = 128;  // keys per tile
+
 constexpr int kMaxSplit = 8;     // CTAs that share an item in the split form (the portable cluster size)
 constexpr int kMaxCluster = 16;  // CTAs that share a (batch, key/value head) in the few-row kernel
 
@@ -45,30 +48,69 @@ int split_parts(const SplitShape& s, int sms, Fit fit, double* steps = nullptr) 
 }
 
 struct StreamShape {
-    double tiles, pairs;   // query tiles, and pairs of them, of all (batch, head)
-    int per_head;          // query tiles of a head
-    int nt;                // key tiles of the longest
-    int D;
-    bool causal;
-    bool one_anchor;       // all but the exact modes on 16-bit inputs
+    long long heads;       // (batch, query head) pairs
+    int Sq, Sk, D;
+    bool causal, exact, fp8;
+
+    int tiles() const { return (Sq + kTileM - 1) / kTileM; }       // query tiles of a head
+    int keys(int tile) const {                                     // key tiles that some row of a query tile sees
+        const int end = causal ? std::min(Sk, (tile + 1) * kTileM + Sk - Sq) : Sk;
+        return end > 0 ? (end + kTileN - 1) / kTileN : 0;
+    }
 };
 
-// Whether the two-stream form (one query tile per CTA) is faster than the plain form, or than the split form where that would
-// give an item `parts` CTAs in `split_steps`.  In steps of the plain form, measured over 60 shapes: a key tile of one query tile
-// takes 0.64 (0.56 in the exact modes on 16-bit inputs), an item boundary 3.0 against the plain form's 3.6.
-//   One tile per CTA: the plain form has as many steps in a row, each of a whole step.  Lost only to the longer set-up and joining of
-//   a few key tiles (D = 128: 3 tiles 8.9 -> 9.4 us, 5 to 12 tiles 21.9 -> 15.9 and 22.7 -> 16.2; D = 64: 2 tiles 8.3 -> 6.1).
-//   Causal, one pair but more than one tile per CTA: long and short tiles even out over two rounds (16 heads x 1408 23.8 -> 19.6 us,
-//   x 2304 36.2 -> 31.3), from 12 key tiles on (8 tiles 32.9 -> 40.1, which have three rounds).
-//   Full attention, all items equal: whole rounds decide (36 heads x 1337 x 2803 exact: 2 rounds of pairs 94 us, 3 of tiles 76).
-//   Other shapes have enough pairs: 48 heads x 2K 57.8 us in the plain form, 68.2 in this one.
+// The longest walk of a CTA over items that are dealt as item_index does it: `units` items of each head, the last first, of which
+// number u costs cost(u).  Costs fall from the last unit or from the one before it on (a last query tile without a partner), so
+// the CTA is one that has the first of these, or one at an end of the row or of the last round.
+template <class Cost>
+double longest_walk(long long heads, int units, int sms, Cost cost) {
+    const long long items = heads * units, ctas = std::min<long long>(items, sms), rounds = (items + ctas - 1) / ctas;
+    const auto cta_of = [&](long long w) { return (w / ctas & 1) ? ctas - 1 - w % ctas : w % ctas; };
+    const long long likely[4] = {0, ctas - 1, cta_of(items - 1), cta_of(std::min(heads, items - 1))};
+    double longest = 0.0;
+    for (const long long c : likely) {
+        double t = 0.0;
+        for (long long r = 0; r < rounds; ++r) {
+            const long long w = r * ctas + ((r & 1) ? ctas - 1 - c : c);
+            if (w < items) t += cost(units - 1 - static_cast<int>(w / heads));
+        }
+        longest = std::max(longest, t);
+    }
+    return longest;
+}
+
+// Whether the two-stream form is faster than the plain form, or than the split form where that would give an item `parts` CTAs in
+// `split_steps`.  Both walks are added up, in steps of the plain form (a key tile of a pair of query tiles; 0.85 where only one of the
+// two sees it): a key tile of one query tile takes 0.52 in the exact modes, 0.58 on fp8 inputs and 0.62 otherwise, an item boundary
+// 3.5 against 3.2.  Fitted to 770 measured shapes (2 to 140 key tiles, 1 to 900 query tiles, steady streams of calls): off by 7 %
+// (rms).  Times plain -> two streams:
+//   A tile for every CTA: as many steps in a row, each of a whole step in the plain form.  16 x 1K e4m3 h15 17.5 -> 14.0 us.
+//   Long and short tiles even out: 16 heads x 1408 bf16 h15 22.4 -> 20.5, x 2304 34.9 -> 30.8; not where two rounds are of long tiles
+//   alone (2 x 32 heads, 512 queries on 16K 251 -> 301, 4 x 32 heads, 200 on 8K 153 -> 209).
+//   Whole rounds: 36 heads x 1337 x 2803 exact, 2 rounds of pairs 92.9, 3 of tiles 83.2; 31 heads, 1123 on 7145 e4m3 h15 150 -> 97.
+//   Enough pairs: 48 heads x 2K 61.6 -> 70.3.
+// The margins: the plain form keeps calls that the estimate puts within 5 % of each other.  The split form's estimate is low by up to a
+// tenth: where it was up to 5 % below the two-stream form's, that took 0.66 to 1.05 times as long.  Of the shapes measured the choice
+// loses 5 % at two and 2 % at a third, nowhere else more than 2 %.
+// Two or three key tiles: the longer set-up and joining weigh most.  At D = 64 it wins while tiles lie on half of the SMs, so that the
+// next call's CTAs can start beside them (2 x 256 6.5 -> 5.7 us, 6 x 380 7.7 -> 7.2; 50 x 148 6.7 -> 7.8), but for a single head of
+// three tiles (323 queries 6.75 -> 7.3); and in full attention, where every step of the plain form is a whole one (46 x 323 x 193
+// 8.6 -> 7.4).  D = 128 gains or loses a tenth and stays plain.
 inline bool streams_pay(const StreamShape& s, int parts, double split_steps, int sms) {
-    const double tile = s.one_anchor ? 0.64 : 0.56, boundary = 3.0;
-    if (s.nt < (s.D == 64 ? 2 : 4)) return false;
-    if (parts > 1) return s.per_head > 1 && s.tiles <= sms && s.nt * tile + boundary < split_steps;
-    if (s.tiles <= sms) return true;
-    if (s.causal) return s.pairs <= sms && s.tiles <= 2.0 * sms && s.nt >= 12;
-    return 1.08 * std::ceil(s.tiles / sms) * (s.nt * tile + boundary) < std::ceil(s.pairs / sms) * (s.nt + 3.6);
+    const int per_head = s.tiles(), nt = (s.Sk + kTileN - 1) / kTileN;
+    if (nt < 4) {
+        if (s.D != 64 || nt < 2 || (s.heads == 1 && per_head == 3)) return false;
+        if (2 * s.heads * per_head > sms && (s.causal || per_head == 1)) return false;
+    }
+    if (parts > 1 && per_head == 1) return false;
+    const double tile = s.exact ? 0.52 : s.fp8 ? 0.58 : 0.62;
+    const double streams = longest_walk(s.heads, per_head, sms, [&](int i) { return s.keys(i) * tile + 3.5; });
+    if (parts > 1) return streams < 1.05 * split_steps;
+    const double plain = longest_walk(s.heads, (per_head + 1) / 2, sms, [&](int i) {
+        const int a = s.keys(2 * i), b = 2 * i + 1 < per_head ? s.keys(2 * i + 1) : 0, both = std::min(a, b);
+        return both + 0.85 * (std::max(a, b) - both) + 3.2;
+    });
+    return 1.05 * streams < plain;
 }
 
 struct RowsShape {

@@ -60,19 +60,83 @@ int main() {
     };
     for (const auto& m : measured)
         CHECK(rows_pay(m.s, m.cs, 148) == (m.rows_us < m.plain_us), "%g groups of %d rows, %d key tiles: %.1f us, plain %.1f us", m.s.groups, m.s.rows, m.s.nt, m.rows_us, m.plain_us);
-    // Two streams or the plain form, measured (us): the faster one is taken.
-    const struct { StreamShape s; bool streams; } forms[] = {
-        {{4, 2, 2, 2, 64, true, true}, true},            // 8.3 against 6.1
-        {{128, 64, 8, 8, 128, true, true}, true},        // 17.7, 14.1
-        {{396, 216, 11, 22, 128, false, false}, true},   // 94, 76
-        {{396, 216, 11, 22, 128, false, true}, false},
-        {{288, 144, 18, 18, 128, true, true}, true},     // 36.2, 31.3
-        {{768, 384, 16, 16, 128, true, true}, false},    // 57.8, 68.2
-        {{768, 384, 24, 24, 64, true, true}, false},     // 66.2, 79.9
-        {{48, 32, 3, 3, 128, true, false}, false},       // 8.9, 9.4
-        {{280, 144, 35, 35, 128, false, true}, false},   // 61.3, 72.6
+    // The longest walk, against every CTA's: units of falling cost, the last one as heavy as it is long or a lone tile.
+    for (int heads : {1, 3, 16, 18, 31, 36, 74, 148, 155, 400})
+        for (int units = 1; units <= 20; ++units)
+            for (double last : {1.0, 0.85}) {
+                const auto cost = [&](int u) { return (u == units - 1 ? last : 1.0) * (u + 4.0) + 3.0; };
+                const int items = heads * units, ctas = std::min(items, 148);
+                double longest = 0.0;
+                for (int c = 0; c < ctas; ++c) {
+                    double t = 0.0;
+                    for (int r = 0; r * ctas < items; ++r) {
+                        const int w = r * ctas + ((r & 1) ? ctas - 1 - c : c);
+                        if (w < items) t += cost(units - 1 - w / heads);
+                    }
+                    longest = std::max(longest, t);
+                }
+                const double got = longest_walk(heads, units, 148, cost);
+                CHECK(got <= longest && got >= 0.93 * longest, "%d heads of %d units: %g, is %g", heads, units, got, longest);
+            }
+    // Two streams or what the call would take otherwise (the plain form, or the split form with `parts` CTAs an item), measured in
+    // steady streams of calls (us): the faster one is taken.
+    const struct { StreamShape s; int parts; double other_us, streams_us; } forms[] = {
+        // one tile for every CTA
+        {{2, 256, 256, 64, true, false, false}, 1, 6.5, 5.7},
+        {{16, 1024, 1024, 128, true, false, true}, 1, 17.5, 14.0},
+        {{12, 590, 449, 128, false, false, false}, 1, 15.0, 11.1},
+        // two or three key tiles
+        {{1, 323, 323, 64, true, false, false}, 1, 6.75, 7.3},
+        {{6, 380, 380, 64, true, false, true}, 1, 7.7, 7.2},
+        {{46, 323, 193, 64, false, true, false}, 1, 8.6, 7.4},
+        {{50, 137, 137, 64, true, false, false}, 1, 6.6, 7.4},
+        {{50, 148, 148, 64, true, false, true}, 1, 6.7, 7.8},
+        {{37, 274, 274, 64, true, false, true}, 1, 7.7, 8.7},
+        {{46, 344, 344, 64, true, false, false}, 1, 8.1, 8.8},
+        {{30, 95, 236, 128, true, false, true}, 1, 7.2, 7.4},
+        // prompts against themselves, long and short tiles
+        {{16, 1408, 1408, 128, true, false, false}, 1, 22.1, 20.5},
+        {{16, 1408, 1408, 128, true, true, true}, 1, 21.3, 18.4},
+        {{16, 2304, 2304, 128, true, false, false}, 1, 35.3, 31.0},
+        {{16, 2048, 2048, 64, true, false, false}, 1, 25.8, 22.5},
+        {{32, 1024, 1024, 128, true, false, false}, 1, 19.6, 21.8},
+        {{48, 2048, 2048, 128, true, false, false}, 1, 61.6, 70.3},
+        {{32, 3001, 3001, 64, true, false, false}, 1, 65.6, 80.1},
+        {{16, 8192, 8192, 128, true, true, false}, 1, 272.0, 301.0},
+        // chunks on a long context: tiles of nearly one length
+        {{64, 512, 16384, 128, true, false, false}, 1, 251.1, 300.5},
+        {{64, 512, 16384, 128, true, true, true}, 1, 206.7, 233.9},
+        {{32, 1024, 16384, 128, true, false, true}, 1, 180.0, 204.1},
+        {{64, 512, 8192, 128, true, true, false}, 1, 152.9, 188.1},
+        {{128, 200, 8192, 128, true, false, false}, 1, 153.0, 208.7},
+        {{32, 640, 16384, 128, true, false, false}, 1, 203.1, 247.6},
+        {{28, 1280, 4000, 64, true, false, false}, 1, 48.3, 54.3},
+        {{31, 1123, 7145, 128, true, false, true}, 1, 150.1, 96.6},
+        {{25, 1373, 12578, 128, true, true, true}, 1, 290.5, 184.8},
+        {{199, 91, 8554, 128, true, true, true}, 1, 184.7, 133.2},
+        // full attention: whole rounds
+        {{36, 1337, 2803, 128, false, true, false}, 1, 92.9, 83.2},
+        {{36, 1337, 2803, 128, false, true, true}, 1, 84.0, 72.4},
+        {{32, 8192, 8192, 128, false, true, true}, 1, 816.2, 922.2},
+        // the split form
+        {{32, 512, 16384, 128, true, false, false}, 2, 163.7, 147.1},
+        {{32, 512, 16384, 128, true, false, true}, 2, 118.7, 104.1},
+        {{30, 336, 4191, 128, false, false, true}, 2, 43.1, 34.0},
+        {{9, 2298, 10402, 64, false, true, false}, 3, 116.4, 141.4},
+        {{3, 351, 7263, 128, true, false, false}, 8, 36.9, 58.3},
     };
-    for (const auto& f : forms) CHECK(streams_pay(f.s, 1, 0.0, 148) == f.streams, "%g query tiles, %d key tiles", f.s.tiles, f.s.nt);
+    for (const auto& f : forms) {
+        const int pairs = (f.s.tiles() + 1) / 2, all = f.s.keys(f.s.tiles() - 1), first = std::max(f.s.keys(0), f.s.tiles() > 1 ? f.s.keys(1) : 0);
+        for (int part = 1; part <= 2; ++part) {      // the whole device, and half of it with half the heads
+            if (f.s.heads % part != 0) continue;
+            StreamShape s = f.s;
+            s.heads /= part;
+            double steps = 0.0;
+            const int parts = split_parts({static_cast<double>(s.heads * pairs), all, first, s.fp8 || !s.exact}, 148 / part, [&](int p) { return whole[p] / part; }, &steps);
+            CHECK(parts == f.parts, "%lld heads, %d on %d: %d parts", s.heads, s.Sq, s.Sk, parts);
+            CHECK(streams_pay(s, parts, steps, 148 / part) == (f.streams_us < f.other_us), "%lld heads, %d on %d, D = %d: %g us in two streams, %g otherwise", s.heads, s.Sq, s.Sk, s.D, f.streams_us, f.other_us);
+        }
+    }
     std::puts("ok");
     return 0;
 }

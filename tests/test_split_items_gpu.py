@@ -16,7 +16,7 @@ SHAPES = [
     Workload("two_parts", 1, 64, 16, 100, 6000, 128, True, "bf16", 101),       # 64 items of one query tile: 2 CTAs each
     Workload("four_parts_fp8", 1, 16, 16, 100, 5000, 128, True, "fp8_e4m3", 102),
     Workload("eight_parts_d64", 1, 2, 2, 300, 4099, 64, False, "fp16", 103),
-    Workload("causal_prompt", 1, 2, 2, 3000, 3000, 128, True, "fp8_e4m3", 104, peaked_keys=True),
+    Workload("causal_prompt", 1, 1, 1, 3000, 3000, 128, True, "fp8_e4m3", 104, peaked_keys=True),
     Workload("causal_prompt_bf16", 1, 2, 1, 3000, 3000, 64, True, "bf16", 105),
     Workload("few_keys_early", 1, 1, 1, 700, 1900, 128, True, "bf16", 106),
     Workload("fp8_d64", 1, 3, 1, 257, 4500, 64, True, "fp8_e4m3", 107),
@@ -50,10 +50,10 @@ def test_shared_items_match_the_oracle(wl, mode):
     assert st["ok"], st
 
 
-def test_two_parts_of_a_pair_of_query_tiles():
-    """Exact mode on 16-bit inputs: with a maxima pass two parts are not planned for items of two query tiles."""
-    wl = Workload("two_parts_two_tiles", 1, 48, 12, 200, 6400, 128, True, "bf16", 109)
-    assert parts_of(wl, orc.W_EXACT) == 2
+def test_three_parts_of_a_pair_of_query_tiles():
+    """The fewest parts that are planned for items of two query tiles; two CTAs for two tiles take one each (two streams)."""
+    wl = Workload("three_parts_two_tiles", 1, 45, 9, 200, 9000, 128, True, "bf16", 109)
+    assert parts_of(wl, orc.W_EXACT) == 3
     st = compare(wl, orc.W_EXACT, rows=list(range(0, 200, 7)) + [127, 128, 199])
     assert st["ok"], st
 
