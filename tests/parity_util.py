@@ -28,6 +28,15 @@ EXACT_FP8_FEW_KEYS = 16
 EXACT_FP8_FEW_KEYS_TOL = 1e-1
 
 
+def plan_of(wl: Workload, mode: int):
+    """(kernel, CTAs) that attn_fwd takes for a workload on this device."""
+    dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
+    return binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)
+
+
+PLAIN, STREAMS = (binding.KERNEL_PLAIN, 1), (binding.KERNEL_STREAMS, 1)
+
+
 def run_cuda(wl: Workload, inp: Inputs, mode: int, device="cuda:0", tau=None, pot_tail=None):
     q, k, v = (t.to(device) for t in (inp.q, inp.k, inp.v))
     o, lse = binding.attn_fwd(q, k, v, causal=wl.causal, softmax_scale=wl.softmax_scale, weight_mode=mode,

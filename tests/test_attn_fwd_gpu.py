@@ -7,7 +7,7 @@ from oracle import cpu_oracle as orc
 from paper_2609_33586_b200 import binding
 from paper_2609_33586_b200.inputs import WORKLOADS, Workload, make_inputs
 
-from parity_util import compare
+from parity_util import PLAIN, STREAMS, compare, plan_of
 
 pytestmark = pytest.mark.gpu
 
@@ -52,6 +52,32 @@ def test_small_shapes(wl, mode):
 ], ids=lambda w: w.name)
 def test_h15_family_members_small_shapes(wl, mode):
     st = compare(wl, mode)
+    assert st["ok"], st
+
+
+# Several key tiles and more items than SMs, which the plain form takes (the small shapes around here go to the two-stream form).
+PLAIN_SHAPES = [
+    Workload("plain_bf16", 4, 40, 8, 500, 500, 128, True, "bf16", 47),
+    Workload("plain_d64", 4, 40, 8, 500, 600, 64, False, "bf16", 48),
+    Workload("plain_fp8", 4, 40, 8, 500, 500, 128, True, "fp8_e4m3", 49),
+    Workload("plain_fp16", 4, 40, 8, 400, 500, 128, True, "fp16", 50, peaked_keys=True),
+]
+
+
+@pytest.mark.parametrize("mode", MODES + FAMILY)
+@pytest.mark.parametrize("wl", PLAIN_SHAPES, ids=lambda w: w.name)
+def test_plain_form_with_several_key_tiles(wl, mode):
+    if wl.in_dtype == "fp16" and mode in FAMILY:
+        pytest.skip("not built")
+    assert plan_of(wl, mode) == PLAIN
+    st = compare(wl, mode, rows=_sample_rows(wl.Sq, 61)[::4], model_p_storage=True)
+    assert st["ok"], st
+
+
+@pytest.mark.parametrize("wl", PLAIN_SHAPES, ids=lambda w: w.name)
+def test_plain_form_drops_the_tail_of_pot(wl):
+    assert plan_of(wl, orc.W_POT) == PLAIN
+    st = compare(wl, orc.W_POT, rows=_sample_rows(wl.Sq, 61)[::4], pot_tail=(12, True), allow_output_rounding=True)
     assert st["ok"], st
 
 
@@ -254,13 +280,31 @@ def test_fp16_inputs_full_size_8k_on_sampled_rows(mode):
 def test_h15_fp8_clamp_tests_agree(causal, scale_up):
     # The fp8 h15 path skips its row-minimum pass when 448 * sum|q_i| already keeps every offset above
     # the clamp.  scale_up = 1: the bound holds (Gaussian inputs); 2: scores four times larger, the bound
-    # fails and the row minimum decides (no clamp needed yet).  Both must match the oracle; items of one
-    # and of several key tiles are present (the bound is used only from two key tiles on).
+    # fails and the row minimum decides (no clamp needed yet).  Both must match the oracle.  This shape has one query tile
+    # per CTA and up to 5 key tiles, of which the two-stream form takes the row minimum: the bound itself is in the next test.
     wl = Workload("floor", 1, 2, 2, 640, 640, 128, causal, "fp8_e4m3", 46)
     inp = make_inputs(wl)
     inp.q_descale *= scale_up
     inp.k_descale *= scale_up
     st = compare(wl, orc.W_H15, inp, allow_output_rounding=scale_up > 1.0)
+    assert st["ok"], st
+
+
+@pytest.mark.parametrize("scale_up", [1.0, 2.0, 8.0])
+@pytest.mark.parametrize("wl,form", [
+    (Workload("floor_plain", 4, 40, 8, 640, 1200, 128, True, "fp8_e4m3", 146), PLAIN),
+    (Workload("floor_plain_full", 4, 40, 8, 500, 1100, 64, False, "fp8_e4m3", 147), PLAIN),
+    (Workload("floor_streams", 1, 4, 2, 1200, 1200, 128, True, "fp8_e4m3", 148), STREAMS),
+    (Workload("floor_streams_rounds", 1, 16, 16, 1664, 1664, 64, True, "fp8_e4m3", 149), STREAMS),
+], ids=lambda x: getattr(x, "name", ""))
+def test_h15_fp8_bound_on_the_scores(wl, form, scale_up):
+    """The bound of the test above is taken from 4 key tiles of an item on in the plain form, from 7 or 8 on in the two-stream form.
+    1: it holds; 2: it fails and the row minimum says that no clamp is needed; 8: scores lie below the clamp."""
+    assert plan_of(wl, orc.W_H15) == form
+    inp = make_inputs(wl)
+    inp.q_descale *= scale_up
+    inp.k_descale *= scale_up
+    st = compare(wl, orc.W_H15, inp, rows=_sample_rows(wl.Sq, 61)[::4], allow_output_rounding=scale_up > 1.0)
     assert st["ok"], st
 
 
@@ -452,8 +496,10 @@ def test_output_allocations_go_through_the_dispatcher():
 
 
 def test_captured_with_copies_and_joins_around_it():
-    """The three kernels in one graph behind a copy, a fill and a join of two streams, replayed on new inputs."""
-    shapes = [(1, 2, 256, 256), (1, 2, 1, 4000), (1, 2, 300, 8192)]      # plain, few rows, shared items
+    """The four kernels in one graph behind a copy, a fill and a join of two streams, replayed on new inputs."""
+    shapes = [(1, 2, 256, 256), (1, 2, 1, 4000), (1, 2, 300, 8192), (4, 40, 500, 500)]      # two streams, few rows, shared items, plain
+    assert [binding.get_plan(B, H, H, Sq, Sk, 64, True, orc.W_H15, binding.IN_BF16)[0] for B, H, Sq, Sk in shapes] == [
+        binding.KERNEL_STREAMS, binding.KERNEL_FEW_ROWS, binding.KERNEL_SHARED, binding.KERNEL_PLAIN]
 
     def inputs(seed):
         g = torch.Generator(device="cuda").manual_seed(seed)
@@ -461,7 +507,7 @@ def test_captured_with_copies_and_joins_around_it():
 
     kw = dict(causal=True, softmax_scale=0.125, weight_mode=orc.W_H15)
     staged, bufs = inputs(1), [[torch.empty_like(x) for x in qkv] for qkv in inputs(1)]
-    outs = [(torch.empty_like(qkv[0]), torch.empty(1, 2, qkv[0].shape[1], device="cuda")) for qkv in bufs]
+    outs = [(torch.empty_like(qkv[0]), torch.empty(qkv[0].shape[0], qkv[0].shape[2], qkv[0].shape[1], device="cuda")) for qkv in bufs]
     for qkv in staged:      # set-up of the kernels outside the capture, as a program's first step does it
         binding.attn_fwd(*qkv, **kw)
     side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
@@ -480,6 +526,9 @@ def test_captured_with_copies_and_joins_around_it():
         for dst, src in zip(bufs[2], staged[2]):
             dst.copy_(src)
         binding.attn_fwd(*bufs[2], out=outs[2][0], lse=outs[2][1], **kw)
+        for dst, src in zip(bufs[3], staged[3]):
+            dst.copy_(src)
+        binding.attn_fwd(*bufs[3], out=outs[3][0], lse=outs[3][1], **kw)
         binding.attn_fwd(*bufs[0], out=outs[0][0], lse=outs[0][1], **kw)
     for seed in (2, 3):
         fresh = inputs(seed)
@@ -515,9 +564,11 @@ def test_drawn_sizes_match_the_oracle():
 
 
 def test_threads_with_streams_of_their_own():
-    """Four threads, each with its stream and its mix of the three kernels, get what one thread gets."""
+    """Four threads, each with its stream and its mix of the four kernels, get what one thread gets."""
     import threading
-    shapes = [(1, 2, 256, 256), (2, 4, 1, 4000), (1, 2, 300, 8192), (8, 16, 40, 600), (1, 16, 700, 700)]
+    shapes = [(1, 2, 256, 256), (2, 4, 1, 4000), (1, 2, 300, 8192), (8, 16, 40, 600), (1, 16, 700, 700), (4, 40, 300, 300)]
+    assert {binding.get_plan(B, H, H, Sq, Sk, 64, True, orc.W_H15, binding.IN_BF16)[0] for B, H, Sq, Sk in shapes} == {
+        binding.KERNEL_STREAMS, binding.KERNEL_FEW_ROWS, binding.KERNEL_SHARED, binding.KERNEL_PLAIN}
     kw = dict(causal=True, softmax_scale=0.125, weight_mode=orc.W_H15)
     g = torch.Generator(device="cuda").manual_seed(9)
     inputs = [[torch.randn(B, s, H, 64, device="cuda", generator=g).to(torch.bfloat16) for s in (Sq, Sk, Sk)] for B, H, Sq, Sk in shapes]

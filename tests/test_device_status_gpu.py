@@ -51,7 +51,8 @@ def test_an_expired_wait_sets_the_sticky_word_and_later_launches_store_nothing_u
 @pytest.mark.parametrize("wl", [
     Workload("one_key_tile", 1, 2, 2, 300, 100, 128, False, "bf16", 83),
     Workload("rows_without_keys", 1, 2, 2, 300, 20, 64, True, "bf16", 84),
-    Workload("several_key_tiles", 1, 2, 2, 600, 600, 128, True, "fp8_e4m3", 85)], ids=lambda w: w.name)
+    Workload("several_key_tiles", 1, 2, 2, 600, 600, 128, True, "fp8_e4m3", 85),          # two-stream form
+    Workload("several_key_tiles_plain", 4, 40, 8, 300, 500, 128, True, "fp8_e4m3", 88)], ids=lambda w: w.name)
 def test_launches_queued_behind_the_expiring_one_store_nothing(wl):
     """No synchronisation in between: the forwards may start (programmatic launch) before the word is set, and warps of one
     block may see it at different times."""

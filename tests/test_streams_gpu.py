@@ -7,7 +7,7 @@ from oracle import cpu_oracle as orc
 from paper_2609_33586_b200 import binding
 from paper_2609_33586_b200.inputs import Workload, make_inputs
 
-from parity_util import compare
+from parity_util import PLAIN, STREAMS, compare, plan_of
 
 pytestmark = pytest.mark.gpu
 
@@ -31,14 +31,6 @@ def _device_status_is_clean():
     binding.device_status_reset()
     yield
     assert binding.device_status() == 0
-
-
-PLAIN, STREAMS = (binding.KERNEL_PLAIN, 1), (binding.KERNEL_STREAMS, 1)
-
-
-def plan_of(wl, mode):
-    dt = {"bf16": binding.IN_BF16, "fp16": binding.IN_FP16, "fp8_e4m3": binding.IN_FP8_E4M3}[wl.in_dtype]
-    return binding.get_plan(wl.B, wl.Hq, wl.Hkv, wl.Sq, wl.Sk, wl.D, wl.causal, mode, dt)
 
 
 @pytest.mark.parametrize("mode", [orc.W_EXACT, orc.W_POT, orc.W_H15])
@@ -90,3 +82,48 @@ def test_two_streams_round_p_as_the_plain_form_does(wl, copies, mode):
     o, want = o[0].double(), want[copies // 2].double()
     assert ((o - want).norm() / want.norm()).item() < 3.5e-4
     assert (lse[0] - want_lse[copies // 2]).abs().max().item() < 1e-5
+
+
+@pytest.mark.parametrize("mode", [orc.W_EXACT, orc.W_H15])
+@pytest.mark.parametrize("wl", [SHAPES[1], SHAPES[3], SHAPES[6]], ids=lambda w: w.name)
+def test_two_streams_give_the_same_bits_in_a_stream_of_calls(wl, mode):
+    assert plan_of(wl, mode) == STREAMS
+    inp = make_inputs(wl)
+    q, k, v = inp.q.cuda(), inp.k.cuda(), inp.v.cuda()
+    kw = dict(causal=wl.causal, softmax_scale=wl.softmax_scale, weight_mode=mode, q_descale=inp.q_descale, k_descale=inp.k_descale,
+              v_descale=inp.v_descale)
+    o, lse = binding.attn_fwd(q, k, v, **kw)
+    for _ in range(300):
+        again, lse_again = binding.attn_fwd(q, k, v, **kw)
+    assert torch.equal(o, again) and torch.equal(lse, lse_again)
+
+
+@pytest.mark.parametrize("key", [5, 130, 990])       # in the first tile of either stream and in the last tile
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16, torch.float8_e4m3fn])
+def test_two_streams_show_a_score_that_is_no_number(dtype, key):
+    """Exact mode: the rows' O is NaN and their LSE -inf, as in the plain form."""
+    assert plan_of(Workload("nan", 1, 2, 2, 300, 1000, 64, False, {torch.bfloat16: "bf16", torch.float16: "fp16"}.get(dtype, "fp8_e4m3"), 0), orc.W_EXACT) == STREAMS
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, k, v = (torch.randn(1, s, 2, 64, device="cuda", generator=g) for s in (300, 1000, 1000))
+    k[0, key, 0, 3] = float("nan")
+    o, lse = binding.attn_fwd(q.to(dtype), k.to(dtype), v.to(dtype), causal=False, softmax_scale=0.125, weight_mode=orc.W_EXACT)
+    assert torch.isnan(o[0, :, 0]).all() and torch.isneginf(lse[0, 0]).all()
+    assert torch.isfinite(o[0, :, 1]).all() and torch.isfinite(lse[0, 1]).all()
+
+
+@pytest.mark.parametrize("mode", [orc.W_EXACT, orc.W_POT, orc.W_H15])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("key", [100, 200])
+def test_two_streams_show_a_value_that_is_not_finite_where_its_stream_weighs_nothing(key, bad, mode):
+    """The last key's score lies 700 octaves above all others, so everything before it weighs 0: 0 times the value is NaN."""
+    assert plan_of(Workload("inf", 1, 2, 2, 300, 1000, 64, False, "bf16", 0), mode) == STREAMS
+    q = torch.ones(1, 300, 2, 64, device="cuda")
+    k = torch.zeros(1, 1000, 2, 64, device="cuda")
+    v = torch.ones(1, 1000, 2, 64, device="cuda")
+    k[0, 999] = 64.0
+    v[0, key, 0, 5] = bad
+    q, k, v = (x.to(torch.bfloat16) for x in (q, k, v))
+    o, lse = binding.attn_fwd(q, k, v, causal=False, softmax_scale=0.125, weight_mode=mode)
+    assert torch.isnan(o[0, :, 0, 5]).all() and torch.isfinite(lse).all()
+    o[0, :, 0, 5] = 0.0
+    assert torch.isfinite(o).all()
