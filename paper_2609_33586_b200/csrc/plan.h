@@ -90,8 +90,10 @@ double longest_walk(long long heads, int units, int sms, Cost cost) {
 //   Whole rounds: 36 heads x 1337 x 2803 exact, 2 rounds of pairs 92.9, 3 of tiles 83.2; 31 heads, 1123 on 7145 e4m3 h15 150 -> 97.
 //   Enough pairs: 48 heads x 2K 61.6 -> 70.3.
 // The margins: the plain form keeps calls that the estimate puts within 5 % of each other.  The split form's estimate is low by up to a
-// tenth: where it was up to 5 % below the two-stream form's, that took 0.66 to 1.05 times as long.  Of the shapes measured the choice
-// loses 5 % at two and 2 % at a third, nowhere else more than 2 %.
+// tenth: where it was up to 5 % below the two-stream form's, that took 0.60 to 1.05 times as long.  The exact modes on 16-bit inputs
+// stay with it all the same: its parts round P about maxima of their own, so that O would move by 1e-3 (2-norm) with the form and
+// lie further from 64-bit results (2.23e-3 -> 2.27e-3, 20 heads, 337 on 2803).  Of the shapes measured the choice of form loses 5 % at
+// one and 2 % at another, nowhere else more than 2 %.
 // Two or three key tiles: the longer set-up and joining weigh most.  At D = 64 it wins while tiles lie on half of the SMs, so that the
 // next call's CTAs can start beside them (2 x 256 6.5 -> 5.7 us, 6 x 380 7.7 -> 7.2; 50 x 148 6.7 -> 7.8), but for a single head of
 // three tiles (323 queries 6.75 -> 7.3); and in full attention, where every step of the plain form is a whole one (46 x 323 x 193
@@ -102,7 +104,7 @@ inline bool streams_pay(const StreamShape& s, int parts, double split_steps, int
         if (s.D != 64 || nt < 2 || (s.heads == 1 && per_head == 3)) return false;
         if (2 * s.heads * per_head > sms && (s.causal || per_head == 1)) return false;
     }
-    if (parts > 1 && per_head == 1) return false;
+    if (parts > 1 && (per_head == 1 || (s.exact && !s.fp8))) return false;
     const double tile = s.exact ? 0.52 : s.fp8 ? 0.58 : 0.62;
     const double streams = longest_walk(s.heads, per_head, sms, [&](int i) { return s.keys(i) * tile + 3.5; });
     if (parts > 1) return streams < 1.05 * split_steps;

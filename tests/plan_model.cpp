@@ -137,6 +137,8 @@ int main() {
             CHECK(streams_pay(s, parts, steps, 148 / part) == (f.streams_us < f.other_us), "%lld heads, %d on %d, D = %d: %g us in two streams, %g otherwise", s.heads, s.Sq, s.Sk, s.D, f.streams_us, f.other_us);
         }
     }
+    // Exact weights on 16-bit inputs: what the split form takes stays with it.
+    CHECK(!streams_pay({32, 512, 16384, 128, true, true, false}, 2, 1e6, 148) && streams_pay({32, 512, 16384, 128, true, true, true}, 2, 1e6, 148), "exact weights");
     std::puts("ok");
     return 0;
 }

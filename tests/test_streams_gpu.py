@@ -98,13 +98,13 @@ def test_two_streams_give_the_same_bits_in_a_stream_of_calls(wl, mode):
     assert torch.equal(o, again) and torch.equal(lse, lse_again)
 
 
-@pytest.mark.parametrize("key", [5, 130, 990])       # in the first tile of either stream and in the last tile
+@pytest.mark.parametrize("key", [5, 130, 690])       # in the first tile of either stream and in the last tile
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16, torch.float8_e4m3fn])
 def test_two_streams_show_a_score_that_is_no_number(dtype, key):
     """Exact mode: the rows' O is NaN and their LSE -inf, as in the plain form."""
-    assert plan_of(Workload("nan", 1, 2, 2, 300, 1000, 64, False, {torch.bfloat16: "bf16", torch.float16: "fp16"}.get(dtype, "fp8_e4m3"), 0), orc.W_EXACT) == STREAMS
+    assert plan_of(Workload("nan", 1, 2, 2, 300, 700, 64, False, {torch.bfloat16: "bf16", torch.float16: "fp16"}.get(dtype, "fp8_e4m3"), 0), orc.W_EXACT) == STREAMS
     g = torch.Generator(device="cuda").manual_seed(5)
-    q, k, v = (torch.randn(1, s, 2, 64, device="cuda", generator=g) for s in (300, 1000, 1000))
+    q, k, v = (torch.randn(1, s, 2, 64, device="cuda", generator=g) for s in (300, 700, 700))
     k[0, key, 0, 3] = float("nan")
     o, lse = binding.attn_fwd(q.to(dtype), k.to(dtype), v.to(dtype), causal=False, softmax_scale=0.125, weight_mode=orc.W_EXACT)
     assert torch.isnan(o[0, :, 0]).all() and torch.isneginf(lse[0, 0]).all()
@@ -116,11 +116,11 @@ def test_two_streams_show_a_score_that_is_no_number(dtype, key):
 @pytest.mark.parametrize("key", [100, 200])
 def test_two_streams_show_a_value_that_is_not_finite_where_its_stream_weighs_nothing(key, bad, mode):
     """The last key's score lies 700 octaves above all others, so everything before it weighs 0: 0 times the value is NaN."""
-    assert plan_of(Workload("inf", 1, 2, 2, 300, 1000, 64, False, "bf16", 0), mode) == STREAMS
+    assert plan_of(Workload("inf", 1, 2, 2, 300, 700, 64, False, "bf16", 0), mode) == STREAMS
     q = torch.ones(1, 300, 2, 64, device="cuda")
-    k = torch.zeros(1, 1000, 2, 64, device="cuda")
-    v = torch.ones(1, 1000, 2, 64, device="cuda")
-    k[0, 999] = 64.0
+    k = torch.zeros(1, 700, 2, 64, device="cuda")
+    v = torch.ones(1, 700, 2, 64, device="cuda")
+    k[0, 699] = 64.0
     v[0, key, 0, 5] = bad
     q, k, v = (x.to(torch.bfloat16) for x in (q, k, v))
     o, lse = binding.attn_fwd(q, k, v, causal=False, softmax_scale=0.125, weight_mode=mode)
