@@ -96,13 +96,14 @@ double longest_walk(long long heads, int units, int sms, Cost cost) {
 // one and 2 % at another, nowhere else more than 2 %.
 // Two or three key tiles: the longer set-up and joining weigh most.  At D = 64 it wins while tiles lie on half of the SMs, so that the
 // next call's CTAs can start beside them (2 x 256 6.5 -> 5.7 us, 6 x 380 7.7 -> 7.2; 50 x 148 6.7 -> 7.8), but for a single head of
-// three tiles (323 queries 6.75 -> 7.3); and in full attention, where every step of the plain form is a whole one (46 x 323 x 193
-// 8.6 -> 7.4).  D = 128 gains or loses a tenth and stays plain.
+// three tiles (323 queries 6.75 -> 7.3); beyond that with the exact weights, which gain most (46 x 323 x 193 8.6 -> 7.4), and on
+// three key tiles in full attention, where every step of the plain form is a whole one (24 x 711 x 384 9.3 -> 7.9; on two 64 x 256 x
+// 256 7.0 -> 7.2).  D = 128 gains or loses a tenth and stays plain.
 inline bool streams_pay(const StreamShape& s, int parts, double split_steps, int sms) {
     const int per_head = s.tiles(), nt = (s.Sk + kTileN - 1) / kTileN;
     if (nt < 4) {
         if (s.D != 64 || nt < 2 || (s.heads == 1 && per_head == 3)) return false;
-        if (2 * s.heads * per_head > sms && (s.causal || per_head == 1)) return false;
+        if (2 * s.heads * per_head > sms && (per_head == 1 || !(s.exact || (nt == 3 && !s.causal)))) return false;
     }
     if (parts > 1 && (per_head == 1 || (s.exact && !s.fp8))) return false;
     const double tile = s.exact ? 0.52 : s.fp8 ? 0.58 : 0.62;

@@ -89,6 +89,9 @@ int main() {
         {{1, 323, 323, 64, true, false, false}, 1, 6.75, 7.3},
         {{6, 380, 380, 64, true, false, true}, 1, 7.7, 7.2},
         {{46, 323, 193, 64, false, true, false}, 1, 8.6, 7.4},
+        {{64, 256, 256, 64, false, false, false}, 1, 7.0, 7.2},
+        {{74, 237, 275, 64, true, true, true}, 1, 9.8, 8.3},
+        {{24, 711, 384, 64, false, false, true}, 1, 9.3, 7.9},
         {{50, 137, 137, 64, true, false, false}, 1, 6.6, 7.4},
         {{50, 148, 148, 64, true, false, true}, 1, 6.7, 7.8},
         {{37, 274, 274, 64, true, false, true}, 1, 7.7, 8.7},
