@@ -4,12 +4,15 @@
 // tiles.  Here both work on ONE query tile: key tiles take turns, tile G of the CTA's walk (counted over all its items) belongs
 // to stream G mod 2, which has a softmax warpgroup, a score buffer and an O accumulator of its own.
 //
-// What bounds it: at 16 bits and D = 128 shared memory (64 KB of K and V come in for every tile and 96 KB of operands are read,
-// 1700 to 2000 clocks a tile where the tensor cores need 1024), elsewhere the chain of one warpgroup, as in the plain form.  A tile
-// takes 0.56 to 0.64 of a step of the plain form, which is a tile of two query tiles; so it pays where the plain form's coarser
-// items leave SMs idle (streams_pay in plan.h).  16 x 1K e4m3 h15 17.7 -> 14.1 us, 512 queries on 16K (32/8 heads, bf16 h15)
-// 168 -> 143, cross attention 36 heads x 1337 x 2803 bf16 exact 94 -> 76.  Pairs of CTAs with cta_group::2 and half a K/V tile
-// each were no faster (16.0, 144 and 78 us): their hand-offs take longer than the operand reads that they save.
+// What bounds it: at 16 bits and D = 128 a tile takes 1700 to 2000 clocks, of which the tensor pipe is active in two thirds (nominally
+// 1024) and shared memory passes 160 KB (64 KB of K and V in, 96 KB of operands out; 1280 clocks at 128 bytes a clock), the rest
+// being hand-offs; elsewhere the chain of one warpgroup, as in the plain form.  A tile
+// takes 0.52 to 0.62 of a step of the plain form, which is a tile of two query tiles; so it pays where the plain form's coarser
+// items leave SMs idle (streams_pay in plan.h).  In steady streams of calls 16 x 1K e4m3 h15 17.5 -> 14.0 us, 512 queries on 16K
+// (32/8 heads, bf16 h15) 200 in the plain and 164 in the split form -> 147, cross attention 36 heads x 1337 x 2803 bf16 exact
+// 92.9 -> 83.2 (in short streams, at a higher clock, 143 and 76).  Pairs of CTAs with cta_group::2 and half a K/V tile each were
+// no faster (in short streams 16.0, 144 and 78 us against 14.1, 143 and 76): their hand-offs take longer than the operand reads
+// that they save.
 //
 // Semantics are those of the sequential loop: the anchor that tile g starts from is the one tile g - 1 left, handed from
 // warpgroup to warpgroup through shared memory as soon as a tile's row maximum is known, half a period before the other needs it.
@@ -87,7 +90,7 @@ __device__ __forceinline__ void wait_count(uint32_t at, int want, const WaitCtx&
 }
 
 // Rescaling, masking and weights as in the roles of the plain form, where the same code stands inline: as calls of these functions
-// it ran slower there (16K, 32/8 heads, bf16 h15: 1834 -> 1861 us; 48 heads x 2K 64.9 -> 65.4).
+// it ran slower there (16K, 32/8 heads, bf16 h15: 1834 -> 1861 us; 48 heads x 2K 64.9 -> 65.4; two runs of one side differ by up to 1 %).
 
 // Multiplies a row of an O accumulator (one row per thread, at the warp's lanes of `tO`) by alpha, unless no row of the warp moves.
 template <int D>
@@ -125,18 +128,17 @@ __device__ __forceinline__ void mask_scores(uint32_t (&s)[4][32], int limit) {
 // The weights of one row of a key tile, its scores in s and its anchor m_use: P goes to TMEM at tP, the row sum is returned.
 // LATE: post_alpha is called after the first 32 weights (else not at all).  score_floor bounds the row's scores from below
 // (h15 family on fp8 inputs).
-template <bool FP8, bool HALF, int MODE, bool TAU, bool LATE, typename PostAlpha>
+template <bool FP8, bool HALF, int MODE, bool LATE, typename PostAlpha>
 __device__ __forceinline__ float tile_weights(uint32_t (&s)[4][32], bool masked_tile, int col_limit, float m_use, float score_floor,
                                               const AttnParams& p, uint32_t tP, PostAlpha post_alpha) {
     constexpr int kFam = h15_family_k(MODE);   // h15 family: the map takes the offset times 2^kFam
     const float c_eff = static_cast<float>(1 << kFam) * p.c;
     constexpr float p_off = static_cast<float>(PFormat<FP8, MODE>::kOffLog2);  // log2 of the P / row-sum scale
     // 16-bit inputs: the h15 family uses the saturating form of weights_chunk32 (no row-minimum pass, no
-    // clamped or masked variants) whenever the anchor is always current (offsets <= 0); the deferred rescale,
-    // where a score may lie above its anchor, keeps the form with explicit clamps.  fp8 inputs keep the
-    // packed form: there a bound on the key magnitude already removes the row-minimum pass, and the
-    // scalar multiply-adds of the saturating form cost more issue slots than they save (measured 4 to 6 %).
-    constexpr bool kSatForm = kFam > 0 && !FP8 && !TAU;
+    // clamped or masked variants).  fp8 inputs keep the packed form: there a bound on the key magnitude already
+    // removes the row-minimum pass, and the scalar multiply-adds of the saturating form cost more issue slots than
+    // they save (in the plain form 4 to 6 %).
+    constexpr bool kSatForm = kFam > 0 && !FP8;
     // exact: x = s*c - m*c + P offset;  h15 family: scaled input 2^K x = s*(2^K c) - m*(2^K c);  pot: x = s*c - m*c
     RowScale rs;
     const float nmc = (is_exact_like(MODE) ? p_off : 0.0f) - m_use * c_eff;
@@ -613,7 +615,7 @@ attn_fwd_streams_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     if (lane == 0) mbar_arrive(bar_scale(t));
                 };
                 if constexpr (!kOutOfStep) post_alpha();
-                const float l_tile = tile_weights<FP8, HALF, MODE, false, kOutOfStep>(s, masked_tile, col_limit, m_use, score_floor, p, tS, post_alpha);
+                const float l_tile = tile_weights<FP8, HALF, MODE, kOutOfStep>(s, masked_tile, col_limit, m_use, score_floor, p, tS, post_alpha);
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();

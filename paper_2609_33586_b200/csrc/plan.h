@@ -24,8 +24,9 @@ struct SplitShape {
 // CTAs per item, 1 for the plain form.  fit(parts): clusters of that size that fit the device at once.  Times are in steps of the
 // loop (one key tile of a pair of query tiles), measured: a part costs its key tiles, with a maxima pass 0.65 of a step more for
 // each tile of its maxima pass (two parts share the pass, so it is half as long), and 4.5 steps + 0.5 per part for the exchange
-// and the sum of O; from two thirds of the SMs on they slow each other by a tenth.  512 queries on 16K, 32/8 heads, streams of 40
-// calls: bf16 h15 218 -> 143 us, exact 256 -> 134, e4m3 h15 203 -> 132 (2 parts); 64 queries on 8K e4m3 90 -> 45 (4 parts).
+// and the sum of O; from two thirds of the SMs on they slow each other by a tenth.  512 queries on 16K, 32/8 heads, steady
+// streams of calls: bf16 h15 200 -> 164 us, exact 228 -> 148, e4m3 h15 173 -> 119 (2 parts); in streams of 40 calls 64 queries on 8K
+// e4m3 90 -> 45 (4 parts).
 // 16 x 1K and 16 x 2K gain nothing and stay whole.
 // *steps gets the estimated time.
 template <class Fit>
@@ -178,7 +179,8 @@ inline double plain_us(const RowsShape& s, int sms) {      // one pair of query 
 // Whether the few-row kernel with clusters of cs CTAs is the faster one.  Its epilogue costs 0.18 to 0.29 us for each row of a
 // CTA, which many short heads do not earn back: 1024 heads x 64 rows x 1 key tile 174 us against 33 in the plain form, 32 x 48
 // rows x 1 tile 18.2 against 4.8.  It wins once the keys are read for long enough: 32 groups of 8 rows x 95 tiles 20 against 229.
-// Over the shapes measured the choice costs 0.6 % against always taking the better one, 29 % at most.
+// Over the shapes measured the choice costs 0.6 % against always taking the better one, 29 % at most.  (It weighs the plain form alone;
+// that the call might otherwise take the two-stream form does not enter.)
 inline bool rows_pay(const RowsShape& s, int cs, int sms) { return plain_us(s, sms) >= rows_us(s, cs, sms); }
 
 }  // namespace rowmax
